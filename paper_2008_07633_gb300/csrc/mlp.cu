@@ -140,14 +140,14 @@ __global__ void __launch_bounds__(128, 6) k_mlp_forward_tc(const float* __restri
         const __nv_bfloat16 hi = __float2bfloat16_rn(b);
         return lo ? __float2bfloat16_rn(b - __bfloat162float(hi)) : hi;
     };
-    for (int i = tid; i < kH * kKB1; i += 128) {
-        const int h = i / kKB1, k = i % kKB1;
+    for (int i = tid; i < kH * kKB1; i += 128) {  // consecutive threads take consecutive units: coalesced
+        const int h = i % kH, k = i / kH;
         sB1[core_idx<kKB1>(h, k)] = k < kF ? __float2bfloat16_rn(theta[OFF_W1 + k * kH + h])
                                   : k < kF + 2 ? split(theta[OFF_B1 + h], k == kF + 1)
                                                : __float2bfloat16_rn(0.f);
     }
     for (int i = tid; i < kH * kKA; i += 128) {
-        const int j = i / kKA, k = i % kKA;
+        const int j = i % kH, k = i / kH;
         sB2[core_idx<kKA>(j, k)] = k < kH ? __float2bfloat16_rn(theta[OFF_W2 + k * kH + j])
                                  : k < kH + 2 ? split(theta[OFF_B2 + j], k == kH + 1)
                                               : __float2bfloat16_rn(0.f);
@@ -324,12 +324,12 @@ __global__ void __launch_bounds__(128, 2)
     };
     const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
     for (int i = tid; i < kH * kTB1; i += 128) {
-        const int h = i / kTB1, k = i % kTB1;
+        const int h = i % kH, k = i / kH;
         sB1[core_idx<kTB1>(h, k)] = k < kF ? __float2bfloat16_rn(theta[OFF_W1 + k * kH + h])
                                   : k < kF + 2 ? split(theta[OFF_B1 + h], k == kF + 1) : zero;
     }
     for (int i = tid; i < kH * kTA; i += 128) {
-        const int j = i / kTA, k = i % kTA;
+        const int j = i % kH, k = i / kH;
         sB2[core_idx<kTA>(j, k)] = k < kH ? __float2bfloat16_rn(theta[OFF_W2 + k * kH + j])
                                  : (k == 80 || k == 81) ? split(theta[OFF_B2 + j], k == 81) : zero;
     }
@@ -535,15 +535,33 @@ __global__ void __launch_bounds__(128, 2)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(kTColsTmem) : "memory");
 }
 
-// grad[i] = sum over CTAs (in order) of part[cta][i]; loss = sum of squared errors / ne
-__global__ void k_mlp_fold(const float* __restrict__ part, int nparts, int64_t ne,
-                           float* __restrict__ grad, double* __restrict__ loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > NP) return;
+// grad[i] = sum over CTAs of part[cta][i] in FP64; loss2 (may be NULL) = (sum of squared errors / ne,
+// the network's error word). One CTA takes 32 entries; its kFoldWays threads per entry each add every
+// kFoldWays-th partial (32 consecutive floats a warp) and the sums are added in thread order, so
+// the order is fixed. Bound by load latency: 304 partials a thread, one after the other, on 21 CTAs
+// took 49.6 us for 65,536 rows; 38 partials a thread on 167 CTAs take 5 us.
+constexpr int kFoldWays = 8;
+__global__ void __launch_bounds__(32 * kFoldWays)
+    k_mlp_fold(const float* __restrict__ part, int nparts, int64_t ne, const int* __restrict__ err,
+               float* __restrict__ grad, double* __restrict__ loss2) {
+    __shared__ double red[kFoldWays][32];
+    const int col = threadIdx.x & 31, way = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + col;
     double s = 0.0;
-    for (int c = 0; c < nparts; ++c) s += (double)part[(size_t)c * (NP + 1) + i];
-    if (i < NP) grad[i] = (float)s;
-    else if (loss) *loss = s / (double)ne;
+    if (i <= NP) {
+#pragma unroll 8
+        for (int c = way; c < nparts; c += kFoldWays) s += (double)part[(size_t)c * (NP + 1) + i];
+    }
+    red[way][col] = s;
+    __syncthreads();
+    if (way != 0 || i > NP) return;
+    for (int w = 1; w < kFoldWays; ++w) s += red[w][col];
+    if (i < NP) {
+        grad[i] = (float)s;
+    } else if (loss2) {
+        loss2[0] = s / (double)ne;
+        loss2[1] = (double)*err;
+    }
 }
 
 __global__ void k_mlp_adam(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
@@ -620,9 +638,9 @@ static void mlp_free(sfg_mlp* n) {
     delete n;
 }
 
-// gradient (and loss) of the network on [feats, targets) into n->grad
+// gradient of the network on [feats, targets) into grad, and (loss, error word) into loss2 unless NULL
 static sfg_status mlp_grad(sfg_ctx* ctx, sfg_mlp* n, const float* feats, const float* targets,
-                           int64_t ne, double* loss_dev) {
+                           int64_t ne, float* grad, double* loss2) {
     // two CTAs per SM (each holds 256 TMEM columns and about 113 KB of shared memory)
     const auto key = std::make_tuple((const void*)k_mlp_fwdbwd_tc, 128, kTrainSmem);
     if (ctx->occupancy.find(key) == ctx->occupancy.end()) {
@@ -638,7 +656,7 @@ static sfg_status mlp_grad(sfg_ctx* ctx, sfg_mlp* n, const float* feats, const f
     k_mlp_fwdbwd_tc<<<grid, 128, kTrainSmem, ctx->stream>>>(n->theta, feats, targets, ne, part, n->err,
                                                              ctx->withhold_mma ? 1 : 0);
     sfg_toc(ctx);
-    k_mlp_fold<<<ceil_div_u(NP + 1, 256), 256, 0, ctx->stream>>>(part, grid, ne, n->grad, loss_dev);
+    k_mlp_fold<<<ceil_div_u(NP + 1, 32), 32 * kFoldWays, 0, ctx->stream>>>(part, grid, ne, n->err, grad, loss2);
     ctx->launches += 2;
     SFG_LAUNCH_CHECK(ctx, "k_mlp_fwdbwd_tc");
     return SFG_OK;
@@ -692,6 +710,15 @@ sfg_status sfg_mlp_check_impl(sfg_ctx* ctx, const sfg_mlp* net) {
         return sfg_fail(ctx, SFG_ETIMEOUT, "a tensor-core completion wait of the network ran out");
     }
     return SFG_OK;
+}
+
+// Read back the loss and the error word that k_mlp_fold wrote side by side: one copy, one wait.
+static sfg_status mlp_read_loss(sfg_ctx* ctx, const sfg_mlp* net, const double* loss2, double* loss_host) {
+    double h[2] = {0.0, 0.0};
+    SFG_CUDA(ctx, cudaMemcpyAsync(h, loss2, sizeof h, cudaMemcpyDeviceToHost, ctx->stream));
+    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    *loss_host = h[0];
+    return h[1] != 0.0 ? sfg_mlp_check_impl(ctx, net) : SFG_OK;  // reports and clears the word
 }
 
 sfg_status sfg_edge_features_impl(sfg_ctx* ctx, const sfg_graph* LG, const sfg_graph* LP, int K,
@@ -782,18 +809,12 @@ sfg_status sfg_mlp_gradient(sfg_ctx* ctx, sfg_mlp* net, const float* feats, cons
     if (ne < 1) return sfg_fail(ctx, SFG_EINVAL, "ne must be >= 1");
     SFG_TRY(sfg_check_dev(ctx, feats, "feats"));
     SFG_TRY(sfg_check_dev(ctx, targets, "targets"));
+    if (grad_out) SFG_TRY(sfg_check_dev(ctx, grad_out, "grad_out"));
     Scratch s(ctx);
-    double* loss;
-    SFG_TRY(s.get(&loss, 1));
-    SFG_TRY(mlp_grad(ctx, net, feats, targets, ne, loss));
-    if (grad_out) {
-        SFG_TRY(sfg_check_dev(ctx, grad_out, "grad_out"));
-        SFG_CUDA(ctx, cudaMemcpyAsync(grad_out, net->grad, 4 * NP, cudaMemcpyDeviceToDevice, ctx->stream));
-    }
-    if (loss_host) {
-        SFG_CUDA(ctx, cudaMemcpyAsync(loss_host, loss, 8, cudaMemcpyDeviceToHost, ctx->stream));
-        SFG_TRY(sfg_mlp_check_impl(ctx, net));
-    }
+    double* loss2;
+    SFG_TRY(s.get(&loss2, 2));
+    SFG_TRY(mlp_grad(ctx, net, feats, targets, ne, grad_out ? grad_out : net->grad, loss2));
+    if (loss_host) SFG_TRY(mlp_read_loss(ctx, net, loss2, loss_host));
     return SFG_OK;
 }
 
@@ -809,7 +830,7 @@ sfg_status sfg_mlp_train(sfg_ctx* ctx, sfg_mlp* net, const float* feats, const f
     for (int ep = 0; ep < epochs; ++ep)
         for (int64_t i = 0; i < ne; i += batch) {
             const int64_t nb = std::min(batch, ne - i);
-            SFG_TRY(mlp_grad(ctx, net, feats + i * kF, targets + i, nb, nullptr));
+            SFG_TRY(mlp_grad(ctx, net, feats + i * kF, targets + i, nb, net->grad, nullptr));
             net->step += 1;
             const float c1 = 1.f - powf(b1, (float)net->step), c2 = 1.f - powf(b2, (float)net->step);
             k_mlp_adam<<<ceil_div_u(NP, 256), 256, 0, ctx->stream>>>(net->theta, net->m, net->v,
@@ -820,11 +841,10 @@ sfg_status sfg_mlp_train(sfg_ctx* ctx, sfg_mlp* net, const float* feats, const f
         }
     if (loss_host) {
         Scratch s(ctx);
-        double* loss;
-        SFG_TRY(s.get(&loss, 1));
-        SFG_TRY(mlp_grad(ctx, net, feats, targets, ne, loss));
-        SFG_CUDA(ctx, cudaMemcpyAsync(loss_host, loss, 8, cudaMemcpyDeviceToHost, ctx->stream));
-        SFG_TRY(sfg_mlp_check_impl(ctx, net));
+        double* loss2;
+        SFG_TRY(s.get(&loss2, 2));
+        SFG_TRY(mlp_grad(ctx, net, feats, targets, ne, net->grad, loss2));
+        SFG_TRY(mlp_read_loss(ctx, net, loss2, loss_host));
     }
     return SFG_OK;
 }
