@@ -9,6 +9,7 @@
 #include <mutex>
 
 #include "sfg_internal.cuh"
+#include "dot64.cuh"
 
 namespace {
 
@@ -24,21 +25,17 @@ __device__ __align__(256) double g_rownorm_scratch[SFG_AFFINITY_NOALLOC_MAX_N];
 std::mutex g_mu;
 double* g_scratch_dev[kMaxDevices] = {};
 
-// ||X_p||^2 in FP64, increasing k, no fused multiply-add (same arithmetic as sfg_affinity).
+// ||X_p||^2 in FP64, increasing k (same arithmetic as sfg_affinity: dot64.cuh).
+template <bool VEC>
 __global__ void k_rownorm_static(int32_t n, const float* __restrict__ X, int K,
                                  double* __restrict__ nn) {
     for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * kBlock) {
-        double s = 0.0;
-        for (int k = 0; k < K; ++k) {
-            const double x = (double)X[p * K + k];
-            s = __dadd_rn(s, __dmul_rn(x, x));
-        }
-        nn[p] = s;
-    }
+         p += (int64_t)gridDim.x * kBlock)
+        nn[p] = norm2_seq<float, VEC>(X + p * K, K);
 }
 
-// delta_e = 1 - (X_p . X_q)^2 / (||X_p||^2 ||X_q||^2), FP64, no fused multiply-add.
+// delta_e = 1 - (X_p . X_q)^2 / (||X_p||^2 ||X_q||^2), as k_affinity.
+template <bool VEC>
 __global__ void k_affinity_static(int64_t m, const int32_t* __restrict__ eu,
                                   const int32_t* __restrict__ ev, const float* __restrict__ X,
                                   int K, const double* __restrict__ nn,
@@ -46,12 +43,25 @@ __global__ void k_affinity_static(int64_t m, const int32_t* __restrict__ eu,
     for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m;
          e += (int64_t)gridDim.x * kBlock) {
         const int64_t p = eu[e], q = ev[e];
-        double dot = 0.0;
-        for (int k = 0; k < K; ++k)
-            dot = __dadd_rn(dot, __dmul_rn((double)X[p * K + k], (double)X[q * K + k]));
-        const double den = __dmul_rn(nn[p], nn[q]);
-        delta[e] = den > 0.0 ? __dsub_rn(1.0, __ddiv_rn(__dmul_rn(dot, dot), den)) : 1.0;
+        delta[e] = affinity_delta(dot_seq<float, VEC>(X + p * K, X + q * K, K), nn[p], nn[q]);
     }
+}
+
+template <bool VEC>
+sfg_status launch_static(sfg_ctx* ctx, const sfg_graph* L, const float* X, int K, double* nn,
+                         double* delta) {
+    // every entry of nn[0, n) is rewritten below before it is read: nothing needs clearing
+    k_rownorm_static<VEC><<<sfg_grid(ctx, (const void*)k_rownorm_static<VEC>, kBlock, 0, L->n), kBlock, 0,
+                            ctx->stream>>>(L->n, X, K, nn);
+    ++ctx->launches;
+    SFG_LAUNCH_CHECK(ctx, "k_rownorm_static");
+    if (L->m > 0) {
+        k_affinity_static<VEC><<<sfg_grid(ctx, (const void*)k_affinity_static<VEC>, kBlock, 0, L->m), kBlock,
+                                 0, ctx->stream>>>(L->m, L->eu, L->ev, X, K, nn, delta);
+        ++ctx->launches;
+        SFG_LAUNCH_CHECK(ctx, "k_affinity_static");
+    }
+    return SFG_OK;
 }
 
 }  // namespace
@@ -99,16 +109,6 @@ extern "C" sfg_status sfg_affinity_noalloc(sfg_ctx* ctx, const sfg_graph* L, con
     if (L->m > 0) SFG_TRY(sfg_check_dev(ctx, delta_out, "delta_out"));
     double* nn = nullptr;
     SFG_TRY(scratch_address(ctx, &nn));
-    // every entry of nn[0, n) is rewritten below before it is read: nothing needs clearing
-    k_rownorm_static<<<sfg_grid(ctx, (const void*)k_rownorm_static, kBlock, 0, L->n), kBlock, 0,
-                       ctx->stream>>>(L->n, X, K, nn);
-    ++ctx->launches;
-    SFG_LAUNCH_CHECK(ctx, "k_rownorm_static");
-    if (L->m > 0) {
-        k_affinity_static<<<sfg_grid(ctx, (const void*)k_affinity_static, kBlock, 0, L->m), kBlock,
-                            0, ctx->stream>>>(L->m, L->eu, L->ev, X, K, nn, delta_out);
-        ++ctx->launches;
-        SFG_LAUNCH_CHECK(ctx, "k_affinity_static");
-    }
-    return SFG_OK;
+    return rows_vectorised(X, K) ? launch_static<true>(ctx, L, X, K, nn, delta_out)
+                                 : launch_static<false>(ctx, L, X, K, nn, delta_out);
 }

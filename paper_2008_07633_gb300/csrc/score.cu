@@ -7,6 +7,7 @@
 // both blocks (one 32-byte load per row and lane), forms the two squared distances in FP32 and
 // folds them with xor-shuffles inside the group.
 #include "sfg_internal.cuh"
+#include "dot64.cuh"
 #include "vec.cuh"
 
 namespace {
@@ -189,38 +190,25 @@ __global__ void __launch_bounds__(kBlock, MINB)
     }
 }
 
-// Stored block entry widened to FP64 (exact for FP32 and BF16).
-__device__ __forceinline__ double widen(float x) { return (double)x; }
-__device__ __forceinline__ double widen(__nv_bfloat16 x) { return (double)__bfloat162float(x); }
-
-// ||X_p||^2 in FP64, increasing k, no fused multiply-add.
-template <typename T>
+// ||X_p||^2 in FP64, increasing k (dot64.cuh).
+template <typename T, bool VEC>
 __global__ void k_rownorm(int32_t n, const T* __restrict__ X, int K, double* __restrict__ nn) {
     for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * kBlock) {
-        double s = 0.0;
-        for (int k = 0; k < K; ++k) {
-            const double x = widen(X[p * K + k]);
-            s = __dadd_rn(s, __dmul_rn(x, x));
-        }
-        nn[p] = s;
-    }
+         p += (int64_t)gridDim.x * kBlock)
+        nn[p] = norm2_seq<T, VEC>(X + p * K, K);
 }
 
 // delta_e = 1 - (X_p . X_q)^2 / (||X_p||^2 ||X_q||^2) in FP64, same operation order as the
-// definition, no fused multiply-add; a zero row gives 1.
-template <typename T>
+// definition (dot64.cuh); a zero row gives 1. One thread per edge: the order fixes one chain of K
+// sums an edge, and there are edges enough to fill the FP64 pipe.
+template <typename T, bool VEC>
 __global__ void k_affinity(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
                            const T* __restrict__ X, int K, const double* __restrict__ nn,
                            double* __restrict__ delta) {
     for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m;
          e += (int64_t)gridDim.x * kBlock) {
         const int64_t p = eu[e], q = ev[e];
-        double dot = 0.0;
-        for (int k = 0; k < K; ++k)
-            dot = __dadd_rn(dot, __dmul_rn(widen(X[p * K + k]), widen(X[q * K + k])));
-        const double den = __dmul_rn(nn[p], nn[q]);
-        delta[e] = den > 0.0 ? __dsub_rn(1.0, __ddiv_rn(__dmul_rn(dot, dot), den)) : 1.0;
+        delta[e] = affinity_delta(dot_seq<T, VEC>(X + p * K, X + q * K, K), nn[p], nn[q]);
     }
 }
 
@@ -353,24 +341,31 @@ sfg_status sfg_score_impl(sfg_ctx* ctx, const sfg_graph* LG, const void* XG, con
 }
 
 namespace {
-template <typename T>
-sfg_status affinity_t(sfg_ctx* ctx, const sfg_graph* L, const T* X, int K, double* delta) {
+template <typename T, bool VEC>
+sfg_status affinity_launch(sfg_ctx* ctx, const sfg_graph* L, const T* X, int K, double* delta) {
     Scratch s(ctx);
     double* nn;
     SFG_TRY(s.get(&nn, (size_t)L->n));
-    k_rownorm<T><<<sfg_grid(ctx, (const void*)k_rownorm<T>, kBlock, 0, L->n), kBlock, 0,
-                   ctx->stream>>>(L->n, X, K, nn);
+    k_rownorm<T, VEC><<<sfg_grid(ctx, (const void*)k_rownorm<T, VEC>, kBlock, 0, L->n), kBlock, 0,
+                        ctx->stream>>>(L->n, X, K, nn);
     ++ctx->launches;
     SFG_LAUNCH_CHECK(ctx, "k_rownorm");
     if (L->m > 0) {
         sfg_tic(ctx, "affinity");
-        k_affinity<T><<<sfg_grid(ctx, (const void*)k_affinity<T>, kBlock, 0, L->m), kBlock, 0,
-                        ctx->stream>>>(L->m, L->eu, L->ev, X, K, nn, delta);
+        k_affinity<T, VEC><<<sfg_grid(ctx, (const void*)k_affinity<T, VEC>, kBlock, 0, L->m), kBlock, 0,
+                             ctx->stream>>>(L->m, L->eu, L->ev, X, K, nn, delta);
         ++ctx->launches;
         sfg_toc(ctx);
         SFG_LAUNCH_CHECK(ctx, "k_affinity");
     }
     return SFG_OK;
+}
+
+// Rows that cannot be read by 16-byte vectors (any K and any alignment are accepted) go entry by entry.
+template <typename T>
+sfg_status affinity_t(sfg_ctx* ctx, const sfg_graph* L, const T* X, int K, double* delta) {
+    return rows_vectorised(X, K) ? affinity_launch<T, true>(ctx, L, X, K, delta)
+                                 : affinity_launch<T, false>(ctx, L, X, K, delta);
 }
 }  // namespace
 
