@@ -1,11 +1,13 @@
 // Graph canonicalisation and the CSR Laplacian (Sec. 2.1: A(p,q) = w(p,q), D(p,p) = sum_t w(p,t),
 // L = D - A; Sec. 4: positive weights).
 //
-// One stable radix sort of the 2m directed entries keyed by (row, column) gives, in order, the
-// CSR rows sorted by column with parallel edges adjacent and in input order. Runs of equal keys
-// are merged by an FP64 sum rounded once to FP32; the upper-triangle runs, in order, are the
-// canonical edge list (edge id = rank among them); a lower-triangle entry finds its edge id by a
-// binary search in the mirrored row.
+// By rows (the usual path): every directed entry (column, input position) is placed in its row by
+// a counting pass and each row is then sorted on chip, so an entry crosses HBM a few times instead
+// of once per radix digit (see build_by_rows). By sort (graphs with a row of more than kRowCap raw
+// entries, or 2m >= 2^31): one stable radix sort of the 2m directed entries keyed by (row, column).
+// Both give the CSR rows sorted by column with parallel edges merged by an FP64 sum in input order
+// rounded once to FP32; the upper-triangle entries, in order, are the canonical edge list (edge id
+// = rank among them), and a lower-triangle entry takes the id of its mirror.
 #include <cmath>
 
 #include "sfg_internal.cuh"
@@ -55,8 +57,28 @@ __global__ void k_lap_runs(const uint64_t* __restrict__ keys, const uint32_t* __
          i += (int64_t)gridDim.x * blockDim.x) {
         if (!head[i]) continue;
         const uint64_t k = keys[i];
-        double s = 0.0;  // parallel edges: FP64 sum in input order, rounded once
-        for (int64_t t = i; t < len && keys[t] == k; ++t) s += (double)w[vals[t]];
+        // parallel edges: FP64 sum in input order, rounded once; a coarse graph's hub pair can have
+        // thousands, so eight entries are loaded at a time
+        double s = (double)w[vals[i]];
+        if (i + 1 < len && keys[i + 1] == k)
+            for (int64_t t = i + 1;; t += 8) {
+                uint64_t kk[8];
+                float ww[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int64_t j = min(t + q, len - 1);
+                    kk[q] = t + q < len ? keys[j] : ~k;
+                    ww[q] = w[vals[j]];
+                }
+                int q = 0;
+#pragma unroll
+                for (int b = 0; b < 8; ++b)
+                    if (q == b && kk[b] == k) {
+                        s += (double)ww[b];
+                        q = b + 1;
+                    }
+                if (q < 8) break;
+            }
         const int64_t j = run_off[i];
         const int32_t row = (int32_t)(k >> bits), col = (int32_t)(k & cmask);
         row_of_run[j] = row;
@@ -127,6 +149,604 @@ __global__ void k_lap_f2c(const uint64_t* __restrict__ keys, const uint32_t* __r
         if (keys[i] == sent) continue;
         const int64_t j = run_off[i + 1] - 1;  // run holding position i
         if (upper[j]) f2c[vals[i]] = (int32_t)up_off[j];
+    }
+}
+
+// ---- canonical form by rows -------------------------------------------------------------------
+// What bounds it: 4-byte and 8-byte accesses at random rows (counting, placing, mirrors), so the
+// passes are few: count, place, sort rows, index. Rows are sorted where their entries fit on chip: up
+// to kRowSmall entries, four rows a warp, and up to kRowWarp, one row a warp, each entry ranked
+// against its row in shared memory (quadratic, but no barrier but the warp's); up to kRowMid and up
+// to kRowCap entries, one CTA a row, bitonic. The keys (column, input position) are unique, so the
+// order does not depend on the order in which atomics placed them. Measured against the radix path,
+// which moves 24 bytes an entry for each of 5-6 digits (GB300, kernels of one build): 2^20-node
+// Chung-Lu graph (15.7M entries) 2.54 -> 1.75 ms, 128^3 grid (12.5M entries) 1.47 -> 0.57 ms. What is
+// left of the first is the 390 us of counting (atomics on random rows) and 346 us of placing.
+constexpr int kRowSmall = 32, kRowWarp = 256, kRowMid = 4096, kRowCap = 16384;
+
+// Words the build reads back: input error, longest raw row, rows of the three larger classes, merged
+// rows over SFG_HEAVY_ROW, raw entries, merged entries, canonical edges.
+enum { kWErr, kWMax, kWWarp, kWMid, kWLarge, kWHeavy, kWRaw, kWNnz, kWEdges, kWCount };
+
+// Raw row lengths and each entry's place within its row (slot.x in row u, slot.y in row v; -1 for
+// self-loops and bad edges). A warp whose edges all share an endpoint (a hub's edges in a sorted
+// list) adds once; MATCH: lanes that share an endpoint always add once (coarse graphs, whose sorted
+// lists hold runs of parallel edges and hubs of thousands of entries).
+template <bool MATCH>
+__global__ void __launch_bounds__(kBlock)
+    k_row_count(int32_t n, int64_t m, const int32_t* __restrict__ u, const int32_t* __restrict__ v,
+                const float* __restrict__ w, int32_t* __restrict__ cnt, int2* __restrict__ slot,
+                unsigned long long* __restrict__ words) {
+    constexpr int Q = 4;
+    const int lane = threadIdx.x & 31;
+    auto place = [&](int32_t r, bool ok) {
+        if (MATCH) {
+            const unsigned peers = __match_any_sync(0xffffffffu, ok ? r : -1);
+            const int first = __ffs(peers) - 1;
+            int32_t at = 0;
+            if (ok && lane == first) at = atomicAdd(&cnt[r], __popc(peers));
+            at = __shfl_sync(0xffffffffu, at, first) + __popc(peers & ((1u << lane) - 1u));
+            return ok ? at : -1;
+        }
+        const int32_t r0 = __shfl_sync(0xffffffffu, r, 0);
+        if (__all_sync(0xffffffffu, ok && r == r0)) {
+            int32_t at = 0;
+            if (lane == 0) at = atomicAdd(&cnt[r], 32);
+            return __shfl_sync(0xffffffffu, at, 0) + lane;
+        }
+        return ok ? atomicAdd(&cnt[r], 1) : -1;
+    };
+    for (int64_t i0 = (int64_t)blockIdx.x * (kBlock * Q); i0 < m; i0 += (int64_t)gridDim.x * (kBlock * Q)) {
+        int32_t a[Q], b[Q];
+        bool bad = false;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int64_t e = i0 + q * kBlock + threadIdx.x;
+            a[q] = b[q] = -1;
+            if (e < m) {
+                a[q] = u[e];
+                b[q] = v[e];
+                const float ww = w[e];
+                if (a[q] < 0 || a[q] >= n || b[q] < 0 || b[q] >= n || !isfinite(ww) || !(ww > 0.0f)) {
+                    bad = true;
+                    a[q] = b[q] = -1;
+                }
+            }
+        }
+        if (bad) atomicOr(words + kWErr, 1ull);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int64_t e = i0 + q * kBlock + threadIdx.x;
+            const bool ok = a[q] >= 0 && a[q] != b[q];
+            const int32_t x = place(a[q], ok), y = place(b[q], ok);
+            if (e < m) slot[e] = make_int2(x, y);
+        }
+    }
+}
+
+// The rows of the three larger classes (in no particular order) and the longest row.
+__global__ void k_row_classify(int32_t n, const int32_t* __restrict__ cnt, int32_t* __restrict__ lwarp,
+                               int32_t* __restrict__ mid, int32_t* __restrict__ large,
+                               unsigned long long* __restrict__ words) {
+    int32_t top = 0;
+    for (int64_t r0 = (int64_t)blockIdx.x * kBlock; r0 < n; r0 += (int64_t)gridDim.x * kBlock) {
+        const int64_t r = r0 + threadIdx.x;
+        const int32_t c = r < n ? cnt[r] : 0;
+        top = max(top, c);
+        const bool w = c > kRowSmall && c <= kRowWarp;
+        const unsigned ws = __ballot_sync(0xffffffffu, w);
+        if (ws) {
+            const int lane = threadIdx.x & 31, first = __ffs(ws) - 1;
+            unsigned long long at = 0;
+            if (lane == first) at = atomicAdd(words + kWWarp, (unsigned long long)__popc(ws));
+            at = __shfl_sync(0xffffffffu, at, first);
+            if (w) lwarp[at + __popc(ws & ((1u << lane) - 1u))] = (int32_t)r;
+        }
+        if (c > kRowWarp) {
+            if (c <= kRowMid) mid[atomicAdd(words + kWMid, 1ull)] = (int32_t)r;
+            else large[atomicAdd(words + kWLarge, 1ull)] = (int32_t)r;
+        }
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0 && top > 0) atomicMax(words + kWMax, (unsigned long long)top);
+}
+
+__global__ void __launch_bounds__(kBlock)
+    k_row_place(int64_t m, const int32_t* __restrict__ u, const int32_t* __restrict__ v,
+                const int2* __restrict__ slot, const int64_t* __restrict__ off, uint64_t* __restrict__ raw) {
+    constexpr int Q = 4;  // edges in flight a thread: slot and endpoints, then both offsets, then the stores
+    for (int64_t i0 = (int64_t)blockIdx.x * (kBlock * Q) + threadIdx.x; i0 < m; i0 += (int64_t)gridDim.x * (kBlock * Q)) {
+        int2 at[Q];
+        int32_t a[Q], b[Q];
+        int64_t oa[Q], ob[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int64_t e = i0 + q * kBlock;
+            at[q] = e < m ? slot[e] : make_int2(-1, -1);
+            a[q] = e < m ? u[e] : 0;
+            b[q] = e < m ? v[e] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            oa[q] = at[q].x >= 0 ? off[a[q]] + at[q].x : -1;
+            ob[q] = at[q].x >= 0 ? off[b[q]] + at[q].y : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const uint32_t e = (uint32_t)(i0 + q * kBlock);
+            if (oa[q] < 0) continue;
+            raw[oa[q]] = ((uint64_t)(uint32_t)b[q] << 32) | e;
+            raw[ob[q]] = ((uint64_t)(uint32_t)a[q] << 32) | e;
+        }
+    }
+}
+
+// Per-row results at the row's raw offset: rcv / re / rrow = merged entries (column, weight), the
+// first input position of each and its row (-1 past the row's merged entries); rpos[e] = raw-space
+// place of input edge e's entry in its upper row; and the row's merged length, entries above the
+// diagonal, degree and its reciprocal.
+struct RowOut {
+    int2* rcv;
+    int32_t* re;
+    int32_t* rrow;
+    int32_t* rpos;
+    int32_t* nnz;
+    int32_t* up;
+    double* deg;
+    double* invdeg;
+    unsigned long long* words;
+};
+
+__device__ __forceinline__ void row_finish(const RowOut& o, int64_t r, int32_t nnz, int32_t up, double s) {
+    o.nnz[r] = nnz;
+    o.up[r] = up;
+    o.deg[r] = s;
+    o.invdeg[r] = s > 0.0 ? 1.0 / s : 0.0;
+    if (nnz > SFG_HEAVY_ROW) atomicAdd(o.words + kWHeavy, 1ull);
+}
+
+__device__ __forceinline__ int32_t key_col(uint64_t k) { return (int32_t)(k >> 32); }
+__device__ __forceinline__ uint32_t key_pos(uint64_t k) { return (uint32_t)k; }
+
+__device__ __forceinline__ void row_entry(const RowOut& o, int64_t p, int32_t r, uint64_t k, float w) {
+    o.rcv[p] = make_int2(key_col(k), __float_as_int(w));
+    o.re[p] = (int32_t)key_pos(k);
+    o.rrow[p] = r;
+}
+
+// FP64 sum over the run of equal columns that starts at sorted position i (end b), input order.
+__device__ __forceinline__ float run_weight(const uint64_t* key, const float* sw, int i, int b) {
+    const int32_t c = key_col(key[i]);
+    double s = (double)sw[i];
+    for (int t = i + 1; t < b && key_col(key[t]) == c; ++t) s += (double)sw[t];
+    return (float)s;
+}
+
+// Whether FP64 sums of nnz FP32 weights whose exponent fields span [lo, hi] are exact in any order:
+// every partial sum is a multiple of the smallest weight's unit below 2^53 of them.
+__device__ __forceinline__ bool sums_exact(int lo, int hi, int nnz) {
+    const int lg = nnz > 1 ? 32 - __clz(nnz - 1) : 0;
+    return 24 + (hi - lo) + lg <= 53;
+}
+__device__ __forceinline__ int exponent_of(float w) { return max(1, (int)((__float_as_uint(w) >> 23) & 0xffu)); }
+
+// Four consecutive rows a warp (one or two entries a lane on meshes); rows longer than kRowSmall
+// are left to the kernels below. The degrees come last, one lane a row of the CTA's 32: an FP64
+// instruction holds the pipe for 16 clocks whether one lane needs it or all (with eight rows a
+// warp adding their own degrees the 128^3 grid took 410 us here, bound by that).
+constexpr int kRowsPerWarp = 4, kRowWarps = kBlock / 32;
+__global__ void __launch_bounds__(kBlock, 5)
+    k_rows_small(int32_t n, const int32_t* __restrict__ cnt, const int64_t* __restrict__ off,
+                 const uint64_t* __restrict__ raw, const float* __restrict__ w, RowOut o) {
+    constexpr int CAP = kRowsPerWarp * kRowSmall, PER = CAP / 32;
+    __shared__ uint64_t skey[kRowWarps][CAP];
+    __shared__ float ssw[kRowWarps][CAP];
+    __shared__ int32_t sstart[kRowWarps][kRowsPerWarp + 1];
+    __shared__ unsigned sdup[kRowWarps];
+    static_assert(kRowWarps * kRowsPerWarp == 32, "one warp adds the degrees");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint64_t* key = skey[warp];
+    float* sw = ssw[warp];
+    int32_t* start = sstart[warp];
+    const int64_t r0 = ((int64_t)blockIdx.x * kRowWarps + warp) * kRowsPerWarp;
+    // lane l < kRowsPerWarp: row r0 + l
+    const int64_t rl = r0 + lane;
+    const bool have = lane < kRowsPerWarp && rl < n;
+    int32_t c = have ? cnt[rl] : 0;
+    const int64_t ol = have ? off[rl] : 0;
+    const bool longer = c > kRowSmall;
+    if (longer) c = 0;
+    int32_t inc = c;
+#pragma unroll
+    for (int d = 1; d < kRowsPerWarp; d <<= 1) {
+        const int32_t q = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += q;
+    }
+    if (lane < kRowsPerWarp) start[lane] = inc - c;
+    if (lane == kRowsPerWarp - 1) start[kRowsPerWarp] = inc;
+    __syncwarp();
+    const int total = start[kRowsPerWarp];
+    uint64_t mine[PER];
+    float wv[PER];
+    int lr[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (q * 32 >= total) break;  // warp-uniform
+        const int i = q * 32 + lane;
+        int l = 0;
+#pragma unroll
+        for (int s = kRowsPerWarp / 2; s > 0; s >>= 1)
+            if (start[l + s] <= i) l += s;
+        const int64_t base = __shfl_sync(0xffffffffu, ol, l);
+        lr[q] = l;
+        mine[q] = ~0ull;
+        wv[q] = 0.f;
+        if (i < total) {
+            mine[q] = raw[base + (i - start[l])];
+            key[i] = mine[q];
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (q * 32 >= total) break;
+        if (q * 32 + lane < total) wv[q] = w[key_pos(mine[q])];
+    }
+    __syncwarp();
+    int to[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (q * 32 >= total) break;
+        const int a = start[lr[q]], b = start[lr[q] + 1];
+        int rank = 0;
+        if (q * 32 + lane < total)
+            for (int t = a; t < b; ++t) rank += key[t] < mine[q];
+        to[q] = a + rank;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (q * 32 >= total) break;
+        if (q * 32 + lane < total) {
+            key[to[q]] = mine[q];
+            sw[to[q]] = wv[q];
+        }
+    }
+    __syncwarp();
+    unsigned dups = 0;  // rows of this warp that hold parallel edges
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (q * 32 >= total) break;
+        const int i = q * 32 + lane;
+        if (i < total && i > start[lr[q]] && key_col(key[i - 1]) == key_col(key[i])) dups |= 1u << lr[q];
+    }
+    dups = __reduce_or_sync(0xffffffffu, dups);
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (q * 32 >= total) break;
+        const int i = q * 32 + lane;
+        const int64_t base = __shfl_sync(0xffffffffu, ol, lr[q]);
+        if (i >= total) continue;
+        const int a = start[lr[q]], b = start[lr[q] + 1];
+        const int32_t r = (int32_t)(r0 + lr[q]);
+        const uint64_t k = key[i];
+        const int32_t cc = key_col(k);
+        int at = i - a;
+        bool head = true;
+        float ww = sw[i];
+        if (dups >> lr[q] & 1u) {  // place among the merged entries: runs started up to here, less one
+            at = 0;
+            for (int t = a + 1; t <= i; ++t) at += key_col(key[t - 1]) != key_col(key[t]);
+            head = i == a || key_col(key[i - 1]) != cc;
+            if (head) ww = run_weight(key, sw, i, b);
+        }
+        if (head) row_entry(o, base + at, r, k, ww);
+        if (cc > r) o.rpos[key_pos(k)] = (int32_t)(base + at);
+    }
+    if (lane == 0) sdup[warp] = dups;
+    __syncthreads();
+    // degree (FP64, column order), merged length and upper entries
+    const int64_t r = (int64_t)blockIdx.x * 32 + lane;
+    if (warp != 0 || r >= n || cnt[r] > kRowSmall) return;
+    const int w4 = lane / kRowsPerWarp, l4 = lane % kRowsPerWarp;
+    const int a = sstart[w4][l4], b = sstart[w4][l4 + 1];
+    const bool merge = sdup[w4] >> l4 & 1u;
+    key = skey[w4];
+    sw = ssw[w4];
+    double s = 0.0;
+    int32_t nnz = 0, up = 0;
+    for (int t = a; t < b;) {
+        const int32_t cc = key_col(key[t]);
+        float ww = sw[t];
+        int e = t + 1;
+        if (merge) {
+            ww = run_weight(key, sw, t, b);
+            while (e < b && key_col(key[e]) == cc) ++e;
+        }
+        s += (double)ww;
+        ++nnz;
+        up += cc > (int32_t)r;
+        t = e;
+    }
+    for (int t = nnz; t < b - a; ++t) o.rrow[off[r] + t] = -1;
+    row_finish(o, r, nnz, up, s);
+}
+
+// One warp a listed row of at most kRowWarp raw entries.
+__global__ void __launch_bounds__(kBlock)
+    k_rows_warp(int32_t nrows, const int32_t* __restrict__ rows, const int32_t* __restrict__ cnt,
+                const int64_t* __restrict__ off, const uint64_t* __restrict__ raw,
+                const float* __restrict__ w, RowOut o) {
+    constexpr int PER = kRowWarp / 32;
+    __shared__ __align__(16) uint64_t skey[kRowWarps][kRowWarp];
+    __shared__ float ssw[kRowWarps][kRowWarp];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint64_t* key = skey[warp];
+    float* sw = ssw[warp];
+    for (int32_t h = blockIdx.x * kRowWarps + warp; h < nrows; h += gridDim.x * kRowWarps) {
+        const int32_t r = rows[h], d = cnt[r];
+        const int64_t base = off[r];
+        uint64_t mine[PER];
+        float wv[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int i = q * 32 + lane;
+            mine[q] = i < d ? raw[base + i] : ~0ull;
+            key[i] = mine[q];  // past the end: larger than every key
+        }
+#pragma unroll
+        for (int q = 0; q < PER; ++q) wv[q] = q * 32 + lane < d ? w[key_pos(mine[q])] : 0.f;
+        __syncwarp();
+        int rank[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) rank[q] = 0;
+        for (int t = 0; t < d; t += 2) {  // two keys a load, the same for every lane
+            const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(key + t);
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                if (q * 32 >= d) break;  // warp-uniform
+                rank[q] += (int)(kk.x < mine[q]) + (int)(kk.y < mine[q]);
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if (q * 32 + lane < d) {
+                key[rank[q]] = mine[q];
+                sw[rank[q]] = wv[q];
+            }
+        __syncwarp();
+        int nnz = 0, up = 0, lo = 255, hi = 0;
+        double s = 0.0;
+        for (int i0 = 0; i0 < d; i0 += 32) {
+            const int i = i0 + lane;
+            bool head = false, upper = false;
+            uint64_t k = 0;
+            if (i < d) {
+                k = key[i];
+                head = i == 0 || key_col(key[i - 1]) != key_col(k);
+                upper = key_col(k) > r;
+            }
+            const unsigned hb = __ballot_sync(0xffffffffu, head);
+            const int at = nnz + __popc(hb & ((2u << lane) - 1u)) - 1;
+            if (head) {
+                const float ww = run_weight(key, sw, i, d);
+                row_entry(o, base + at, r, k, ww);
+                const int ex = exponent_of(ww);
+                lo = min(lo, ex);
+                hi = max(hi, ex);
+                s += (double)ww;
+            }
+            if (upper) o.rpos[key_pos(k)] = (int32_t)(base + at);
+            nnz += __popc(hb);
+            up += __popc(__ballot_sync(0xffffffffu, head && upper));
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (sums_exact(lo, hi, nnz)) {
+#pragma unroll
+            for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+        } else if (lane == 0) {
+            s = 0.0;
+            for (int i = 0; i < d; ++i)
+                if (i == 0 || key_col(key[i - 1]) != key_col(key[i])) s += (double)run_weight(key, sw, i, d);
+        }
+        for (int i = nnz + lane; i < d; i += 32) o.rrow[base + i] = -1;
+        if (lane == 0) row_finish(o, r, nnz, up, s);
+        __syncwarp();  // the next row reuses shared memory
+    }
+}
+
+// One CTA a listed row of at most CAP raw entries: bitonic sort of the keys in shared memory.
+// The degree is the FP64 sum in column order; where every partial sum is exact (sums_exact), any
+// order gives the same bits and the CTA adds in parallel, else one thread adds in order.
+template <int THREADS, int CAP>
+__global__ void __launch_bounds__(THREADS)
+    k_rows_cta(int32_t nrows, const int32_t* __restrict__ rows, const int32_t* __restrict__ cnt,
+               const int64_t* __restrict__ off, const uint64_t* __restrict__ raw,
+               const float* __restrict__ w, RowOut o) {
+    extern __shared__ __align__(16) unsigned char s_rows[];
+    uint64_t* key = reinterpret_cast<uint64_t*>(s_rows);
+    float* sw = reinterpret_cast<float*>(key + CAP);
+    __shared__ int32_t wsum[THREADS / 32];
+    __shared__ double dsum[THREADS / 32];
+    __shared__ int32_t smin, smax, scarry, sup;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int32_t h = blockIdx.x; h < nrows; h += gridDim.x) {
+        const int32_t r = rows[h], d = cnt[r];
+        const int64_t base = off[r];
+        int N = 64;
+        while (N < d) N <<= 1;  // <= CAP
+        for (int i = tid; i < N; i += THREADS) key[i] = i < d ? raw[base + i] : ~0ull;
+        if (tid == 0) {
+            smin = 255;
+            smax = 0;
+            scarry = 0;
+            sup = 0;
+        }
+        __syncthreads();
+        for (int k = 2; k <= N; k <<= 1)
+            for (int j = k >> 1; j > 0;) {
+                if (j >= 2) {  // two steps (distances j and j / 2) on four keys in registers
+                    const int g = j >> 1;
+                    for (int t = tid; t < N / 4; t += THREADS) {
+                        const int i = ((t & ~(g - 1)) << 2) | (t & (g - 1));
+                        const bool asc = (i & k) == 0;
+                        uint64_t x0 = key[i], x1 = key[i + g], x2 = key[i + j], x3 = key[i + j + g];
+                        auto order = [&](uint64_t& a, uint64_t& b) {
+                            if ((a > b) == asc) {
+                                const uint64_t q = a;
+                                a = b;
+                                b = q;
+                            }
+                        };
+                        order(x0, x2);
+                        order(x1, x3);
+                        order(x0, x1);
+                        order(x2, x3);
+                        key[i] = x0;
+                        key[i + g] = x1;
+                        key[i + j] = x2;
+                        key[i + j + g] = x3;
+                    }
+                    j >>= 2;
+                } else {
+                    for (int t = tid; t < N / 2; t += THREADS) {
+                        const int i = 2 * t;
+                        const uint64_t a = key[i], b = key[i + 1];
+                        if ((a > b) == ((i & k) == 0)) {
+                            key[i] = b;
+                            key[i + 1] = a;
+                        }
+                    }
+                    j = 0;
+                }
+                __syncthreads();
+            }
+        for (int i = tid; i < d; i += THREADS) sw[i] = w[key_pos(key[i])];
+        __syncthreads();
+        // merged entries, THREADS positions at a time: place = runs started before
+        for (int i0 = 0; i0 < d; i0 += THREADS) {
+            const int i = i0 + tid;
+            bool head = false, upper = false;
+            uint64_t k = 0;
+            float ww = 0.f;
+            if (i < d) {
+                k = key[i];
+                head = i == 0 || key_col(key[i - 1]) != key_col(k);
+                upper = key_col(k) > r;
+                if (head) ww = run_weight(key, sw, i, d);
+            }
+            const unsigned hb = __ballot_sync(0xffffffffu, head);
+            const unsigned ub = __ballot_sync(0xffffffffu, head && upper);
+            if (lane == 0) wsum[warp] = __popc(hb);
+            __syncthreads();
+            int before = scarry;
+            for (int q = 0; q < warp; ++q) before += wsum[q];
+            const int at = before + __popc(hb & ((2u << lane) - 1u)) - 1;
+            if (head) {
+                sw[at] = ww;  // at <= i: every run that starts in this stretch has been read
+                const int ex = exponent_of(ww);
+                atomicMin(&smin, ex);
+                atomicMax(&smax, ex);
+                row_entry(o, base + at, r, k, ww);
+            }
+            if (i < d && upper) o.rpos[key_pos(k)] = (int32_t)(base + at);
+            if (lane == 0 && ub) atomicAdd(&sup, __popc(ub));
+            __syncthreads();
+            if (tid == THREADS - 1) scarry = before + __popc(hb);
+            __syncthreads();
+        }
+        const int nnz = scarry;
+        for (int i = nnz + tid; i < d; i += THREADS) o.rrow[base + i] = -1;
+        double s = 0.0;
+        if (sums_exact(smin, smax, nnz)) {
+            for (int i = tid; i < nnz; i += THREADS) s += (double)sw[i];
+#pragma unroll
+            for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+            if (lane == 0) dsum[warp] = s;
+            __syncthreads();
+            s = 0.0;
+            if (tid == 0)
+                for (int q = 0; q < THREADS / 32; ++q) s += dsum[q];
+        } else if (tid == 0) {
+            for (int i = 0; i < nnz; ++i) s += (double)sw[i];
+        }
+        if (tid == 0) row_finish(o, r, nnz, sup, s);
+        __syncthreads();  // the next row reuses shared memory
+    }
+}
+
+// row_ptr; D[c] such that an edge whose upper entry sits at raw place p of row c has id p + D[c]; and
+// move[r], from a row's raw places to its final ones.
+__global__ void k_row_index(int32_t n, const int64_t* __restrict__ off, const int64_t* __restrict__ row_off,
+                            const int64_t* __restrict__ up_off, const int32_t* __restrict__ nnz,
+                            const int32_t* __restrict__ up, int32_t* __restrict__ row_ptr,
+                            int32_t* __restrict__ D, int32_t* __restrict__ move,
+                            unsigned long long* __restrict__ words) {
+    for (int64_t r = (int64_t)blockIdx.x * kBlock + threadIdx.x; r <= n; r += (int64_t)gridDim.x * kBlock) {
+        row_ptr[r] = (int32_t)row_off[r];
+        if (r < n) {
+            D[r] = (int32_t)(up_off[r] - (int64_t)(nnz[r] - up[r]) - off[r]);
+            move[r] = (int32_t)(row_off[r] - off[r]);
+        } else {
+            words[kWRaw] = (unsigned long long)off[n];
+            words[kWNnz] = (unsigned long long)row_off[n];
+            words[kWEdges] = (unsigned long long)up_off[n];
+        }
+    }
+}
+
+// Edge ids, the edge list, and (MOVE) the entries themselves at their final places. An upper entry's
+// id comes from its own place, a lower entry's from its mirror's.
+template <bool MOVE>
+__global__ void __launch_bounds__(kBlock)
+    k_entries_write(int64_t len, const int32_t* __restrict__ rrow, const int2* __restrict__ rcv,
+                    const int32_t* __restrict__ re, const int32_t* __restrict__ rpos,
+                    const int32_t* __restrict__ D, const int32_t* __restrict__ move, int2* __restrict__ colval,
+                    int32_t* __restrict__ eid, int32_t* __restrict__ eu, int32_t* __restrict__ ev,
+                    float* __restrict__ ew) {
+    constexpr int Q = 4;  // entries in flight a thread
+    for (int64_t j0 = (int64_t)blockIdx.x * (kBlock * Q) + threadIdx.x; j0 < len; j0 += (int64_t)gridDim.x * (kBlock * Q)) {
+        int32_t r[Q], e[Q], id[Q];
+        int2 cv[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int64_t j = j0 + q * kBlock;
+            r[q] = j < len ? rrow[j] : -1;
+            cv[q] = j < len ? rcv[j] : make_int2(0, 0);
+            e[q] = j < len ? re[j] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            id[q] = 0;
+            if (r[q] < 0) continue;
+            const int32_t place = cv[q].x > r[q] ? (int32_t)(j0 + q * kBlock) : rpos[e[q]];
+            id[q] = place + D[min(r[q], cv[q].x)];
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            if (r[q] < 0) continue;
+            int64_t dst = j0 + q * kBlock;
+            if (MOVE) {
+                dst += move[r[q]];
+                colval[dst] = cv[q];
+            }
+            eid[dst] = id[q];
+            if (cv[q].x > r[q]) {
+                eu[id[q]] = r[q];
+                ev[id[q]] = cv[q].x;
+                ew[id[q]] = __int_as_float(cv[q].y);
+            }
+        }
+    }
+}
+
+__global__ void k_row_f2c(int64_t m, const int32_t* __restrict__ u, const int32_t* __restrict__ v,
+                          const int32_t* __restrict__ rpos, const int32_t* __restrict__ D,
+                          int32_t* __restrict__ f2c) {
+    for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m; e += (int64_t)gridDim.x * kBlock) {
+        const int32_t a = u[e], b = v[e];
+        f2c[e] = a == b ? -1 : rpos[e] + D[min(a, b)];
     }
 }
 
@@ -237,8 +857,10 @@ sfg_status sfg_alloc_graph(sfg_ctx* ctx, int32_t n, int64_t m, sfg_graph** out) 
     return SFG_OK;
 }
 
-sfg_status sfg_build_graph(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
-                           const float* w, bool validate, sfg_graph** out, int32_t* f2c) {
+// Canonical form by one radix sort of the directed entries: graphs with a row over kRowCap raw
+// entries, and lists whose 2m entries do not fit int32 places.
+static sfg_status build_by_sort(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
+                                const float* w, bool validate, sfg_graph** out, int32_t* f2c) {
     *out = nullptr;
     const int bits = bits_for(n);
     const uint64_t sent = (bits * 2 >= 64) ? ~0ull : ((1ull << (2 * bits)) - 1);
@@ -333,6 +955,153 @@ sfg_status sfg_build_graph(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u,
     }
     *out = g;
     return SFG_OK;
+}
+
+// Canonical form by rows (see k_row_count). *fits = false (and nothing built) when a raw row is
+// longer than kRowCap. Two host waits: the input check with the longest row, and the merged sizes.
+static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
+                                const float* w, bool validate, sfg_graph** out, int32_t* f2c, bool* fits) {
+    *out = nullptr;
+    *fits = true;
+    const int64_t len = 2 * m;
+    Scratch s(ctx);
+    int32_t *cnt, *lwarp, *mid, *large, *re, *rrow, *rpos, *nnz, *up, *D, *move;
+    int2 *slot, *rcv;
+    uint64_t* raw;
+    int64_t *off, *row_off, *up_off;
+    unsigned long long* words;
+    SFG_TRY(s.get(&cnt, n));
+    SFG_TRY(s.get(&lwarp, n));
+    SFG_TRY(s.get(&mid, (size_t)(len / kRowWarp) + 1));  // longer rows are at most so many
+    SFG_TRY(s.get(&large, (size_t)(len / kRowMid) + 1));
+    SFG_TRY(s.get(&slot, m));
+    SFG_TRY(s.get(&words, kWCount));
+    int* hw32 = nullptr;
+    SFG_TRY(sfg_host_word(ctx, kSfgHostBuild, &hw32));
+    unsigned long long* hw = reinterpret_cast<unsigned long long*>(hw32);
+    SFG_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)n, ctx->stream));
+    SFG_CUDA(ctx, cudaMemsetAsync(words, 0, sizeof(unsigned long long) * kWCount, ctx->stream));
+    if (m > 0) {
+        auto* count = validate ? k_row_count<false> : k_row_count<true>;
+        count<<<grid_of(ctx, count, (m + 3) / 4), kBlock, 0, ctx->stream>>>(n, m, u, v, w, cnt, slot, words);
+        k_row_classify<<<grid_of(ctx, k_row_classify, n), kBlock, 0, ctx->stream>>>(n, cnt, lwarp, mid, large, words);
+        ctx->launches += 2;
+        SFG_LAUNCH_CHECK(ctx, "k_row_count");
+    }
+    SFG_CUDA(ctx, cudaMemcpyAsync(hw, words, sizeof(unsigned long long) * kWCount, cudaMemcpyDeviceToHost,
+                                  ctx->stream));
+    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (validate && hw[kWErr])
+        return sfg_fail(ctx, SFG_EINVAL,
+                        "edge list: endpoint outside [0, n) or weight not finite and > 0");
+    if (hw[kWMax] > (unsigned long long)kRowCap) {
+        *fits = false;
+        return SFG_OK;
+    }
+    const int32_t nwarp = (int32_t)hw[kWWarp], nmid = (int32_t)hw[kWMid], nlarge = (int32_t)hw[kWLarge];
+
+    sfg_graph* g = new sfg_graph();
+    struct Owner { sfg_graph* g; ~Owner() { sfg_graph_free(g); } } own{g};
+    g->device = ctx->device;
+    g->n = n;
+    g->stream = ctx->stream;
+    SFG_TRY(sfg_alloc(ctx, (void**)&g->row_ptr, sizeof(int32_t) * ((size_t)n + 1)));
+    SFG_TRY(sfg_alloc(ctx, (void**)&g->deg, sizeof(double) * (size_t)n));
+    SFG_TRY(sfg_alloc(ctx, (void**)&g->invdeg, sizeof(double) * (size_t)n));
+    SFG_TRY(s.get(&off, (size_t)n + 1));
+    SFG_TRY(s.get(&row_off, (size_t)n + 1));
+    SFG_TRY(s.get(&up_off, (size_t)n + 1));
+    SFG_TRY(s.get(&raw, len));
+    SFG_TRY(s.get(&rcv, len));
+    SFG_TRY(s.get(&re, len));
+    SFG_TRY(s.get(&rrow, len));
+    SFG_TRY(s.get(&rpos, m));
+    SFG_TRY(s.get(&nnz, n));
+    SFG_TRY(s.get(&up, n));
+    SFG_TRY(s.get(&D, n));
+    SFG_TRY(s.get(&move, n));
+    SFG_TRY(sfg_scan_i32(ctx, cnt, off, n));
+    if (m > 0) {
+        k_row_place<<<grid_of(ctx, k_row_place, (m + 3) / 4), kBlock, 0, ctx->stream>>>(m, u, v, slot, off, raw);
+        ++ctx->launches;
+    }
+    const RowOut ro{rcv, re, rrow, rpos, nnz, up, g->deg, g->invdeg, words};
+    k_rows_small<<<ceil_div_u(n, kRowsPerWarp * kRowWarps), kBlock, 0, ctx->stream>>>(n, cnt, off, raw, w, ro);
+    ++ctx->launches;
+    if (nwarp > 0) {
+        k_rows_warp<<<sfg_grid(ctx, (const void*)k_rows_warp, kBlock, 0, (int64_t)nwarp * 32), kBlock, 0, ctx->stream>>>(
+            nwarp, lwarp, cnt, off, raw, w, ro);
+        ++ctx->launches;
+    }
+    auto rows_cta = [&](auto* k, int threads, int cap, int32_t count, const int32_t* list) -> sfg_status {
+        const size_t sm = (size_t)cap * (sizeof(uint64_t) + sizeof(float));  // 48 and 192 KB: opt in once
+        const auto key = std::make_tuple((const void*)k, -threads, sm);
+        if (ctx->occupancy.find(key) == ctx->occupancy.end()) {
+            SFG_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+            ctx->occupancy.emplace(key, 1);
+        }
+        k<<<sfg_grid(ctx, (const void*)k, threads, sm, (int64_t)count * threads), threads, sm, ctx->stream>>>(
+            count, list, cnt, off, raw, w, ro);
+        ++ctx->launches;
+        return SFG_OK;
+    };
+    if (nmid > 0) SFG_TRY(rows_cta(k_rows_cta<256, kRowMid>, 256, kRowMid, nmid, mid));
+    if (nlarge > 0) SFG_TRY(rows_cta(k_rows_cta<1024, kRowCap>, 1024, kRowCap, nlarge, large));
+    SFG_LAUNCH_CHECK(ctx, "k_rows");
+    SFG_TRY(sfg_scan_i32(ctx, nnz, row_off, n));
+    SFG_TRY(sfg_scan_i32(ctx, up, up_off, n));
+    k_row_index<<<grid_of(ctx, k_row_index, (int64_t)n + 1), kBlock, 0, ctx->stream>>>(
+        n, off, row_off, up_off, nnz, up, g->row_ptr, D, move, words);
+    ++ctx->launches;
+    SFG_LAUNCH_CHECK(ctx, "k_row_index");
+    SFG_CUDA(ctx, cudaMemcpyAsync(hw, words, sizeof(unsigned long long) * kWCount, cudaMemcpyDeviceToHost,
+                                  ctx->stream));
+    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    const int64_t entries = (int64_t)hw[kWNnz], mc = (int64_t)hw[kWEdges];
+    g->m = mc;
+    SFG_TRY(sfg_alloc(ctx, (void**)&g->eu, sizeof(int32_t) * mc + 16));
+    SFG_TRY(sfg_alloc(ctx, (void**)&g->ev, sizeof(int32_t) * mc + 16));
+    SFG_TRY(sfg_alloc(ctx, (void**)&g->ew, sizeof(float) * mc + 16));
+    SFG_TRY(sfg_alloc(ctx, (void**)&g->eid, sizeof(int32_t) * entries + 16));
+    const bool moved = entries != len;  // else nothing was merged or dropped: the sorted rows are the CSR rows
+    if (!moved && len > 0) {
+        s.release(rcv);
+        g->colval = rcv;
+    } else {
+        SFG_TRY(sfg_alloc(ctx, (void**)&g->colval, sizeof(int2) * entries + 16));
+    }
+    if (entries > 0) {
+        auto* write = moved ? k_entries_write<true> : k_entries_write<false>;
+        // raw places end where the rows do: self-loops were never placed
+        write<<<grid_of(ctx, write, (len + 3) / 4), kBlock, 0, ctx->stream>>>(
+            (int64_t)hw[kWRaw], rrow, rcv, re, rpos, D, move, g->colval, g->eid, g->eu, g->ev, g->ew);
+        ++ctx->launches;
+    }
+    if (f2c && m > 0) {
+        k_row_f2c<<<grid_of(ctx, k_row_f2c, m), kBlock, 0, ctx->stream>>>(m, u, v, rpos, D, f2c);
+        ++ctx->launches;
+    }
+    SFG_LAUNCH_CHECK(ctx, "k_entries_write");
+    // the sweep's heavy-row lists are built with the graph, so that later calls (which may be
+    // captured into a CUDA graph) never synchronise for them
+    if (hw[kWHeavy] == 0) {
+        g->hv_nseg = 0;
+        g->hv_n = 0;
+    }
+    SFG_TRY(sfg_heavy_prepare(ctx, g));
+    own.g = nullptr;
+    *out = g;
+    return SFG_OK;
+}
+
+sfg_status sfg_build_graph(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
+                           const float* w, bool validate, sfg_graph** out, int32_t* f2c) {
+    if (n > 0 && m < (1ll << 30)) {
+        bool fits = false;
+        SFG_TRY(build_by_rows(ctx, n, m, u, v, w, validate, out, f2c, &fits));
+        if (fits) return SFG_OK;
+    }
+    return build_by_sort(ctx, n, m, u, v, w, validate, out, f2c);
 }
 
 sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* mask,

@@ -150,8 +150,9 @@ struct Scratch {
 
 // The context's pinned host ints (allocated on first use): a stream-ordered copy into one costs no
 // synchronisation, and the host reads it after the next one. Slots: 0 spanning-forest round
-// flag, 1 pointer-jumping flag.
-constexpr int kSfgHostWords = 4;
+// flag, 1 pointer-jumping flag, 3 breadth-first flag; from kSfgHostBuild on, the 64-bit words of a
+// graph build.
+constexpr int kSfgHostBuild = 8, kSfgHostWords = 32;
 sfg_status sfg_host_word(sfg_ctx* ctx, int slot, int** out);
 
 // Kernel timing (no-ops unless ctx->timing).
