@@ -123,7 +123,7 @@ static sfg_status aggregate(sfg_ctx* ctx, const sfg_graph* L, const double* delt
     k_hook<<<gn, kBlock, 0, ctx->stream>>>(n, L->row_ptr, L->colval, L->eid, delta, hook); ++ctx->launches;
     k_hook_forest<<<gn, kBlock, 0, ctx->stream>>>(n, hook, root); ++ctx->launches;
     SFG_LAUNCH_CHECK(ctx, "k_hook");
-    SFG_TRY(sfg_pointer_jump(ctx, n, nullptr, root));
+    SFG_TRY(sfg_pointer_jump(ctx, n, root));
     SFG_CUDA(ctx, cudaMemsetAsync(minm, 0x7f, sizeof(int32_t) * n, ctx->stream));
     k_min_member<<<gn, kBlock, 0, ctx->stream>>>(n, root, minm); ++ctx->launches;
     k_is_first<<<gn, kBlock, 0, ctx->stream>>>(n, root, minm, first); ++ctx->launches;

@@ -3,11 +3,11 @@
 //
 // Boruvka rounds under the strict order (weight descending, edge id ascending): every edge key is
 // (FP32 weight bits << 32) | ~id, unique and ordered like that order, so the forest is unique and
-// equal to Kruskal's. A round: (1) each component takes the largest key among edges leaving it
-// (per row over its CSR entries, then one 64-bit atomicMax per row or per segment of a long
-// row), (2) marks that edge and hooks to the component across it, (3) the 2-cycles
-// that mutual choices create are broken toward the smaller label, (4) pointer jumping flattens the
-// hook forest, (5) nodes are relabelled. Rounds repeat until no component has an outgoing edge.
+// equal to Kruskal's. A round: (1) each component takes the largest key among edges leaving it,
+// (2) marks that edge and hooks to the component across it, the smaller label of a mutual pair
+// staying a root, (3) pointer jumping flattens the hook forest, (4) nodes are relabelled. Rounds
+// repeat until no component has an outgoing edge. All rounds run in one cooperative launch.
+#include "gridbar.cuh"
 #include "sfg_internal.cuh"
 
 namespace {
@@ -20,174 +20,221 @@ __global__ void k_mst_init(int32_t n, int32_t* __restrict__ comp) {
         comp[p] = (int32_t)p;
 }
 
-__global__ void k_mst_reset(int32_t n, unsigned long long* __restrict__ best, int* __restrict__ flag) {
-    for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * kBlock)
-        best[p] = 0ull;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
-}
+// What bounds a round: a node's largest key leaving its component is a gather of its neighbours'
+// labels, 8 + 4 + 4 bytes an entry. An edge inside a component stays inside for good, so a node
+// keeps its best edge and looks through its row again only when that edge has become internal, and
+// never again once no edge leaves; a component's maximum is compared before the 64-bit atomicMax, so
+// most nodes of a large component only read it. With the launches and host waits of separate round
+// kernels gone as well, the forest of the 128^3 grid takes 1,220 us (11 rounds of 6 launches and a
+// wait, every row rescanned: 1,490 us of kernels and about 170 us of waits) and that of a 64 x 64
+// grid 95 us (290 us with the waits).
+//
+// Items are the rows [0, n), rows longer than SFG_HEAVY_ROW excepted, and then the fixed segments
+// of those rows. A warp takes 32 items: one lane each checks the kept edge; the items to look
+// through again are dealt to four 8-lane groups, kMstItems at a time so that as many independent
+// load chains (entry -> neighbour's label) are in flight.
+constexpr int kMstLanes = 8, kMstGroups = 32 / kMstLanes, kMstItems = 4;
 
-// Each component's largest key among the edges leaving it, from the CSR rows: a group of 8 lanes
-// takes kMstItems rows at a time, its lanes stride over each row's entries (the first entry of all
-// rows is loaded before any later one), the group folds the largest key that leaves the row's
-// component and issues one atomicMax for that component. Every
-// edge leaving a component sits in the row of its endpoint inside it. SEG = false: rows
-// [0, n), skipping rows longer than SFG_HEAVY_ROW; SEG = true: the fixed segments of those rows.
-constexpr int kMstLanes = 8, kMstItems = 4;
+// Words of one launch: barrier count, error, edges taken, last pointer-jumping pass with work left.
+enum { kMwBar, kMwErr, kMwTree, kMwJump, kMwCount };
 
-struct MstItem {
-    int32_t a, b, cp;
-    unsigned long long best;
+struct MstArgs {
+    int32_t n;
+    int64_t nseg;
+    const int32_t* row_ptr;
+    const int4* seg;
+    const int2* colval;
+    const int32_t* eid;
+    const int32_t* eu;
+    const int32_t* ev;
+    const uint8_t* allow;
+    const int32_t* key_id;
+    const int32_t* key_inv;
+    int32_t* comp;              // written by the kernel from here on
+    int32_t* parent;
+    unsigned long long* best;   // per component label
+    unsigned long long* ckey;   // per item: its kept edge's key and the node across it (-1: none left)
+    int32_t* cnbr;
+    uint8_t* mask;
+    unsigned long long* words;
 };
 
-// Candidate key of CSR entry j of a row in component cp (0 if the entry stays inside it or the
-// edge is not allowed).
-__device__ __forceinline__ unsigned long long mst_key(int32_t j, int32_t cp, const int2* __restrict__ colval,
-                                                      const int32_t* __restrict__ eid,
-                                                      const uint8_t* __restrict__ allow,
-                                                      const int32_t* __restrict__ comp,
-                                                      const int32_t* __restrict__ key_id) {
-    const int2 cv = colval[j];
-    if (comp[cv.x] == cp) return 0ull;
-    const int32_t e = eid[j];
-    if (allow && !allow[e]) return 0ull;
-    const uint32_t id = key_id ? (uint32_t)key_id[e] : (uint32_t)e;
-    return ((unsigned long long)(uint32_t)cv.y << 32) | (unsigned long long)(~id);
+// Pointer jumping in place: every node climbs up to kHops parents and stores the ancestor it
+// reached. Other threads' stores are read as they land: every stored value is an ancestor of its
+// node, so any mix of old and new values is a valid forest with the same roots, and a node whose
+// ancestors were already shortened climbs further.
+constexpr int kHops = 8;
+__device__ __forceinline__ bool jump_node(volatile int32_t* par, int64_t r) {  // true: not at a root yet
+    int32_t p = par[r];
+#pragma unroll 1
+    for (int h = 0; h < kHops; ++h) {
+        const int32_t pp = par[p];
+        if (pp == p) break;
+        p = pp;
+    }
+    par[r] = p;
+    return par[p] != p;
 }
 
-template <bool SEG>
-__global__ void __launch_bounds__(kBlock) k_mst_rows(int64_t nitems, const int32_t* __restrict__ row_ptr,
-                                                     const int4* __restrict__ seg,
-                                                     const int2* __restrict__ colval,
-                                                     const int32_t* __restrict__ eid,
-                                                     const uint8_t* __restrict__ allow,
-                                                     const int32_t* __restrict__ comp,
-                                                     const int32_t* __restrict__ key_id,
-                                                     unsigned long long* __restrict__ best) {
-    const int sub = threadIdx.x % kMstLanes;
-    const int64_t g0 = ((int64_t)blockIdx.x * kBlock + threadIdx.x) / kMstLanes;
-    const int64_t ng = (int64_t)gridDim.x * kBlock / kMstLanes;
-    const int64_t lg = g0 % (32 / kMstLanes);
-    // kMstItems rows per group and iteration, so that as many independent load chains are in
-    // flight; the same trip count for the whole warp, so the group folds below run converged
-    for (int64_t i0 = g0 - lg; i0 < nitems; i0 += ng * kMstItems) {
-        MstItem it[kMstItems];
-        int32_t p[kMstItems];
-#pragma unroll
-        for (int u = 0; u < kMstItems; ++u) {
-            const int64_t k = i0 + lg + (int64_t)u * ng;
-            it[u].a = it[u].b = 0;
-            p[u] = 0;
-            if (k < nitems) {
-                if (SEG) {
-                    const int4 sg = seg[k];
-                    p[u] = sg.x, it[u].a = sg.y, it[u].b = sg.z;
-                } else {
-                    p[u] = (int32_t)k, it[u].a = row_ptr[k], it[u].b = row_ptr[k + 1];
-                    if (it[u].b - it[u].a > SFG_HEAVY_ROW) it[u].b = it[u].a;  // swept by segments
+__device__ __forceinline__ void mst_offer(unsigned long long* best, int32_t c, unsigned long long key) {
+    if (key > *(volatile unsigned long long*)(best + c)) atomicMax(best + c, key);
+}
+
+__global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
+    __shared__ uint8_t s_list[kBlock / 32][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % kMstLanes, grp = lane / kMstLanes;
+    const int64_t t0 = (int64_t)blockIdx.x * kBlock + threadIdx.x, nt = (int64_t)gridDim.x * kBlock;
+    const int64_t items = (int64_t)A.n + A.nseg;
+    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kMwBar), reinterpret_cast<int*>(A.words + kMwErr)};
+    unsigned passed = 0;
+    for (int64_t p = t0; p < A.n; p += nt) {
+        A.comp[p] = (int32_t)p;
+        A.best[p] = 0ull;
+    }
+    if (!grid_barrier(bar, passed)) return;
+    unsigned long long tree = 0, jump_pass = 0;
+    // each round at least halves the number of components that still have outgoing edges
+    for (int round = 0; round < 64; ++round) {
+        // (1) the largest key leaving each component
+        for (int64_t base = t0 - lane; base < items; base += nt) {
+            const int64_t i = base + lane;
+            int32_t cp = -1, a = 0, b = 0;
+            bool need = false;
+            if (i < items) {
+                const int32_t nb = round == 0 ? 0 : A.cnbr[i];
+                if (nb >= 0) {
+                    int4 sg = make_int4((int32_t)i, 0, 0, 0);
+                    if (i >= A.n) sg = A.seg[i - A.n];
+                    cp = A.comp[sg.x];
+                    need = round == 0 || A.comp[nb] == cp;
+                    if (need) {
+                        a = sg.y;
+                        b = sg.z;
+                        if (i < A.n) {
+                            a = A.row_ptr[i];
+                            b = A.row_ptr[i + 1];
+                            if (b - a > SFG_HEAVY_ROW) b = a;  // looked through by segments
+                        }
+                    } else {
+                        mst_offer(A.best, cp, A.ckey[i]);
+                    }
                 }
             }
-        }
-        // the row's own label and its first entry (most rows of meshes and k-NN graphs have no
-        // second) with the entry's edge id, all issued before any of them is used: the chain is
-        // row bounds -> entry -> neighbour's label
-        int2 cv[kMstItems];
-        int32_t e[kMstItems];
+            const unsigned todo = __ballot_sync(0xffffffffu, need);
+            if (need) s_list[warp][__popc(todo & ((1u << lane) - 1u))] = (uint8_t)lane;
+            __syncwarp();
+            const int cnt = __popc(todo);
+            for (int k0 = 0; k0 < cnt; k0 += kMstGroups * kMstItems) {
+                int src[kMstItems];
+                int32_t ra[kMstItems], rb[kMstItems], rc[kMstItems], nbr[kMstItems], e[kMstItems];
+                int2 cv[kMstItems];
+                unsigned long long top[kMstItems];
 #pragma unroll
-        for (int u = 0; u < kMstItems; ++u) {
-            it[u].cp = comp[p[u]];
-            const int32_t j = it[u].a + sub;
-            cv[u] = j < it[u].b ? colval[j] : make_int2(p[u], 0);
-            e[u] = j < it[u].b ? eid[j] : 0;
-        }
+                for (int u = 0; u < kMstItems; ++u) {
+                    const int k = k0 + u * kMstGroups + grp;
+                    src[u] = k < cnt ? s_list[warp][k] : -1;
+                    const int from = src[u] < 0 ? 0 : src[u];
+                    ra[u] = __shfl_sync(0xffffffffu, a, from);
+                    rb[u] = __shfl_sync(0xffffffffu, b, from);
+                    rc[u] = __shfl_sync(0xffffffffu, cp, from);
+                    if (src[u] < 0) rb[u] = ra[u];
+                    const int32_t j = ra[u] + sub;
+                    cv[u] = j < rb[u] ? A.colval[j] : make_int2(-1, 0);
+                    e[u] = j < rb[u] ? A.eid[j] : 0;
+                }
 #pragma unroll
-        for (int u = 0; u < kMstItems; ++u) {
-            const bool out = comp[cv[u].x] != it[u].cp && (!allow || allow[e[u]]);
-            const uint32_t id = key_id ? (uint32_t)key_id[e[u]] : (uint32_t)e[u];
-            it[u].best = out ? ((unsigned long long)(uint32_t)cv[u].y << 32) |
-                                   (unsigned long long)(~id)
-                             : 0ull;
-        }
+                for (int u = 0; u < kMstItems; ++u) {
+                    top[u] = 0ull;
+                    nbr[u] = -1;
+                    for (int32_t j = ra[u] + sub;;) {
+                        if (cv[u].x >= 0 && A.comp[cv[u].x] != rc[u] && (!A.allow || A.allow[e[u]])) {
+                            const uint32_t id = A.key_id ? (uint32_t)A.key_id[e[u]] : (uint32_t)e[u];
+                            const unsigned long long key = ((unsigned long long)(uint32_t)cv[u].y << 32) |
+                                                           (unsigned long long)(~id);
+                            if (key > top[u]) {
+                                top[u] = key;
+                                nbr[u] = cv[u].x;
+                            }
+                        }
+                        j += kMstLanes;
+                        if (j >= rb[u]) break;
+                        cv[u] = A.colval[j];
+                        e[u] = A.eid[j];
+                    }
+                }
 #pragma unroll
-        for (int u = 0; u < kMstItems; ++u)
-            for (int32_t j = it[u].a + sub + kMstLanes; j < it[u].b; j += kMstLanes) {
-                const unsigned long long key = mst_key(j, it[u].cp, colval, eid, allow, comp, key_id);
-                it[u].best = key > it[u].best ? key : it[u].best;
+                for (int u = 0; u < kMstItems; ++u) {
+                    unsigned long long m = top[u];
+#pragma unroll
+                    for (int o = 1; o < kMstLanes; o <<= 1) {
+                        const unsigned long long q = __shfl_xor_sync(0xffffffffu, m, o);
+                        m = q > m ? q : m;
+                    }
+                    if (src[u] < 0) continue;
+                    const int64_t it = base + src[u];
+                    if (m == 0ull) {
+                        if (sub == 0) A.cnbr[it] = -1;
+                    } else if (top[u] == m) {  // keys are unique: one lane holds it
+                        A.cnbr[it] = nbr[u];
+                        A.ckey[it] = m;
+                        mst_offer(A.best, rc[u], m);
+                    }
+                }
             }
-#pragma unroll
-        for (int u = 0; u < kMstItems; ++u) {
-            unsigned long long local = it[u].best;
-#pragma unroll
-            for (int o = 1; o < kMstLanes; o <<= 1) {
-                const unsigned long long q = __shfl_xor_sync(0xffffffffu, local, o);
-                local = q > local ? q : local;
+            __syncwarp();
+        }
+        if (!grid_barrier(bar, passed)) return;
+        // (2) hooks across the chosen edges
+        unsigned taken = 0;
+        for (int64_t r = t0; r < A.n; r += nt) {
+            if (A.comp[r] != r) continue;  // only component labels act
+            const unsigned long long k = A.best[r];
+            int32_t up = (int32_t)r;
+            if (k != 0ull) {
+                const uint32_t id = ~(uint32_t)(k & 0xffffffffull);
+                const uint32_t e = A.key_inv ? (uint32_t)A.key_inv[id] : id;
+                A.mask[e] = 1;
+                const int32_t c0 = A.comp[A.eu[e]], c1 = A.comp[A.ev[e]];
+                const int32_t other = c0 == (int32_t)r ? c1 : c0;
+                if (!(A.best[other] == k && (int32_t)r < other)) {
+                    up = other;
+                    ++taken;
+                }
             }
-            if (sub == 0 && local) atomicMax(&best[it[u].cp], local);
+            A.parent[r] = up;
         }
-    }
-}
-
-__global__ void k_mst_hook(int32_t n, const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-                           const int32_t* __restrict__ comp, const unsigned long long* __restrict__ best,
-                           const int32_t* __restrict__ key_inv, int32_t* __restrict__ parent,
-                           uint8_t* __restrict__ mask, int* __restrict__ flag) {
-    for (int64_t r = (int64_t)blockIdx.x * kBlock + threadIdx.x; r < n;
-         r += (int64_t)gridDim.x * kBlock) {
-        if (comp[r] != r) continue;  // only component labels act
-        const unsigned long long b = best[r];
-        if (b == 0ull) {
-            parent[r] = (int32_t)r;
-            continue;
+        taken = __reduce_add_sync(0xffffffffu, taken);
+        if (lane == 0 && taken) atomicAdd(A.words + kMwTree, (unsigned long long)taken);
+        if (!grid_barrier(bar, passed)) return;
+        const unsigned long long now = *(volatile unsigned long long*)(A.words + kMwTree);
+        if (now == tree) return;  // no component has an outgoing edge
+        tree = now;
+        // (3) flatten; a pass with work left leaves its number (a later pass only starts if it did)
+        for (;;) {
+            ++jump_pass;
+            bool left = false;
+            for (int64_t r = t0; r < A.n; r += nt)
+                if (A.comp[r] == r) left |= jump_node(A.parent, r);
+            if (left) atomicMax(A.words + kMwJump, jump_pass);
+            if (!grid_barrier(bar, passed)) return;
+            if (*(volatile unsigned long long*)(A.words + kMwJump) < jump_pass) break;
         }
-        const uint32_t id = ~(uint32_t)(b & 0xffffffffull);
-        const uint32_t e = key_inv ? (uint32_t)key_inv[id] : id;
-        mask[e] = 1;
-        const int32_t a = comp[eu[e]], c = comp[ev[e]];
-        parent[r] = (a == r) ? c : a;
-        *flag = 1;
-    }
-}
-
-__global__ void k_mst_break(int32_t n, const int32_t* __restrict__ comp, int32_t* __restrict__ parent) {
-    for (int64_t r = (int64_t)blockIdx.x * kBlock + threadIdx.x; r < n;
-         r += (int64_t)gridDim.x * kBlock) {
-        if (comp[r] != r) continue;
-        const int32_t p = parent[r];
-        // only the smaller label of a mutual pair writes, and it writes only its own entry
-        if (p != r && p > r && parent[p] == (int32_t)r) parent[r] = (int32_t)r;
-    }
-}
-
-// Pointer jumping in place on a forest (roots point to themselves): every node climbs up to
-// kHops parents and stores the ancestor it reached; flag set while some node does not point at
-// a root yet. Other threads' stores are read as they land: every stored value is an ancestor of
-// its node, so any mix of old and new values is a valid forest with the same roots, and a node
-// whose ancestors were already shortened climbs further (the reach grows geometrically from one
-// launch to the next). Only component labels take part when comp != NULL.
-constexpr int kHops = 8;
-
-__global__ void k_jump_inplace(int32_t n, const int32_t* __restrict__ comp, int32_t* parent,
-                               int* __restrict__ flag) {
-    volatile int32_t* par = parent;
-    for (int64_t r = (int64_t)blockIdx.x * kBlock + threadIdx.x; r < n;
-         r += (int64_t)gridDim.x * kBlock) {
-        if (comp && comp[r] != r) continue;
-        int32_t p = par[r];
-#pragma unroll 1
-        for (int h = 0; h < kHops; ++h) {
-            const int32_t pp = par[p];
-            if (pp == p) break;
-            p = pp;
+        // (4) relabel; the labels that remain start the next round with no edge
+        for (int64_t p = t0; p < A.n; p += nt) {
+            const int32_t c = A.parent[A.comp[p]];
+            A.comp[p] = c;
+            if (c == (int32_t)p) A.best[p] = 0ull;
         }
-        par[r] = p;
-        if (par[p] != p) *flag = 1;
+        if (!grid_barrier(bar, passed)) return;
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(reinterpret_cast<int*>(A.words + kMwErr), 1);
 }
 
-__global__ void k_mst_relabel(int32_t n, int32_t* __restrict__ comp, const int32_t* __restrict__ parent) {
-    for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * kBlock)
-        comp[p] = parent[comp[p]];
+// One jumping pass over a forest of all nodes (roots point to themselves); flag set while some node
+// does not point at a root yet.
+__global__ void k_jump_inplace(int32_t n, int32_t* parent, int* __restrict__ flag) {
+    for (int64_t r = (int64_t)blockIdx.x * kBlock + threadIdx.x; r < n; r += (int64_t)gridDim.x * kBlock)
+        if (jump_node(parent, r)) *flag = 1;
 }
 
 __global__ void k_count_u8(int64_t m, const uint8_t* __restrict__ mask,
@@ -205,7 +252,7 @@ __global__ void k_count_u8(int64_t m, const uint8_t* __restrict__ mask,
 // Flatten a forest given by parent pointers (roots point to themselves) so that every entry
 // points at its root: in-place jumping launches until no node moves (one launch when no path is
 // longer than kHops; the reach multiplies by about kHops per launch otherwise).
-sfg_status sfg_pointer_jump(sfg_ctx* ctx, int32_t n, const int32_t* comp, int32_t* parent) {
+sfg_status sfg_pointer_jump(sfg_ctx* ctx, int32_t n, int32_t* parent) {
     if (n <= 0) return SFG_OK;
     Scratch s(ctx);
     int* flag;
@@ -216,7 +263,7 @@ sfg_status sfg_pointer_jump(sfg_ctx* ctx, int32_t n, const int32_t* comp, int32_
     for (int it = 0; it < 64; ++it) {
         SFG_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), ctx->stream));
         sfg_tic(ctx, "jump");
-        k_jump_inplace<<<grid, kBlock, 0, ctx->stream>>>(n, comp, parent, flag); ++ctx->launches;
+        k_jump_inplace<<<grid, kBlock, 0, ctx->stream>>>(n, parent, flag); ++ctx->launches;
         sfg_toc(ctx);
         SFG_LAUNCH_CHECK(ctx, "k_jump_inplace");
         SFG_CUDA(ctx, cudaMemcpyAsync(h, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
@@ -255,66 +302,49 @@ sfg_status sfg_mst_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* allow, 
         }
         return SFG_OK;
     }
-    Scratch s(ctx);
-    int32_t *comp, *parent;
-    unsigned long long* best;
-    int* flag;
-    SFG_TRY(s.get(&comp, n));
-    SFG_TRY(s.get(&parent, n));
-    SFG_TRY(s.get(&best, n));
-    SFG_TRY(s.get(&flag, 1));
-    int* hflag = nullptr;  // pinned, written by the stream, read after a synchronisation
-    SFG_TRY(sfg_host_word(ctx, 0, &hflag));
-    const int gn = sfg_grid(ctx, (const void*)k_mst_hook, kBlock, 0, n);
     SFG_TRY(sfg_heavy_prepare(ctx, g));
-    const int gr = sfg_grid(ctx, (const void*)k_mst_rows<false>, kBlock, 0, (int64_t)n * kMstLanes);
-    const int gs = g->hv_n > 0 ? sfg_grid(ctx, (const void*)k_mst_rows<true>, kBlock, 0,
-                                          g->hv_nseg * kMstLanes)
-                               : 0;
-    k_mst_init<<<gn, kBlock, 0, ctx->stream>>>(n, comp); ++ctx->launches;
-    SFG_LAUNCH_CHECK(ctx, "k_mst_init");
-    // each round at least halves the number of components that still have outgoing edges
-    for (int round = 0; round < 64; ++round) {
-        sfg_tic(ctx, "mst_reset");
-        k_mst_reset<<<gn, kBlock, 0, ctx->stream>>>(n, best, flag); ++ctx->launches;
-        sfg_toc(ctx);
-        sfg_tic(ctx, "mst_rows");
-        k_mst_rows<false><<<gr, kBlock, 0, ctx->stream>>>(n, g->row_ptr, nullptr, g->colval, g->eid,
-                                                          allow, comp, key_id, best);
-        ++ctx->launches;
-        if (gs > 0) {
-            k_mst_rows<true><<<gs, kBlock, 0, ctx->stream>>>(g->hv_nseg, nullptr, g->hv_seg, g->colval,
-                                                             g->eid, allow, comp, key_id, best);
-            ++ctx->launches;
-        }
-        sfg_toc(ctx);
-        sfg_tic(ctx, "mst_hook");
-        k_mst_hook<<<gn, kBlock, 0, ctx->stream>>>(n, g->eu, g->ev, comp, best, key_inv, parent, mask,
-                                                   flag);
-        ++ctx->launches;
-        sfg_toc(ctx);
-        SFG_LAUNCH_CHECK(ctx, "k_mst_round");
-        // The round's "any hook" flag travels with the pointer-jumping readback: a round in
-        // which nothing hooks leaves every label its own parent, so break, jumping and relabel
-        // change nothing and the check can wait for the next synchronisation.
-        SFG_CUDA(ctx, cudaMemcpyAsync(hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-        sfg_tic(ctx, "mst_break");
-        k_mst_break<<<gn, kBlock, 0, ctx->stream>>>(n, comp, parent); ++ctx->launches;
-        sfg_toc(ctx);
-        SFG_TRY(sfg_pointer_jump(ctx, n, comp, parent));
-        if (!*hflag) {
-            if (n_tree) SFG_TRY(sfg_count_mask(ctx, mask, m, n_tree));
-            if (comp_out)
-                SFG_CUDA(ctx, cudaMemcpyAsync(comp_out, comp, sizeof(int32_t) * n,
-                                              cudaMemcpyDeviceToDevice, ctx->stream));
-            return SFG_OK;
-        }
-        sfg_tic(ctx, "mst_relabel");
-        k_mst_relabel<<<gn, kBlock, 0, ctx->stream>>>(n, comp, parent); ++ctx->launches;
-        sfg_toc(ctx);
-        SFG_LAUNCH_CHECK(ctx, "k_mst_relabel");
-    }
-    return sfg_fail(ctx, SFG_ETIMEOUT, "spanning forest did not converge in 64 rounds");
+    const int64_t items = (int64_t)n + (g->hv_n > 0 ? g->hv_nseg : 0);
+    Scratch s(ctx);
+    MstArgs a{};
+    SFG_TRY(s.get(&a.comp, n));
+    SFG_TRY(s.get(&a.parent, n));
+    SFG_TRY(s.get(&a.best, n));
+    SFG_TRY(s.get(&a.ckey, items));
+    SFG_TRY(s.get(&a.cnbr, items));
+    SFG_TRY(s.get(&a.words, kMwCount));
+    int* hw32 = nullptr;
+    SFG_TRY(sfg_host_word(ctx, kSfgHostBuild, &hw32));
+    unsigned long long* hw = reinterpret_cast<unsigned long long*>(hw32);
+    SFG_CUDA(ctx, cudaMemsetAsync(a.words, 0, sizeof(unsigned long long) * kMwCount, ctx->stream));
+    a.n = n;
+    a.nseg = items - n;
+    a.row_ptr = g->row_ptr;
+    a.seg = g->hv_seg;
+    a.colval = g->colval;
+    a.eid = g->eid;
+    a.eu = g->eu;
+    a.ev = g->ev;
+    a.allow = allow;
+    a.key_id = key_id;
+    a.key_inv = key_inv;
+    a.mask = mask;
+    void* args[] = {(void*)&a};
+    const int grid = sfg_grid(ctx, (const void*)k_mst, kBlock, 0, items);
+    sfg_tic(ctx, "mst");
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_mst, dim3(grid), dim3(kBlock), args, 0,
+                                                      ctx->stream);
+    sfg_toc(ctx);
+    if (e != cudaSuccess) return sfg_cuda_fail(ctx, e, "k_mst");
+    ++ctx->launches;
+    if (comp_out)
+        SFG_CUDA(ctx, cudaMemcpyAsync(comp_out, a.comp, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice,
+                                      ctx->stream));
+    SFG_CUDA(ctx, cudaMemcpyAsync(hw, a.words, sizeof(unsigned long long) * kMwCount, cudaMemcpyDeviceToHost,
+                                  ctx->stream));
+    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (hw[kMwErr]) return sfg_fail(ctx, SFG_ETIMEOUT, "spanning forest did not converge in 64 rounds");
+    if (n_tree) *n_tree = (int64_t)hw[kMwTree];
+    return SFG_OK;
 }
 
 extern "C" sfg_status sfg_spanning_tree(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* allow,

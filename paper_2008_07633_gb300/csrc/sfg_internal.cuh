@@ -286,7 +286,7 @@ __global__ void k_gs_weights_heavy(int32_t nh, const int32_t* __restrict__ hrow,
                                    const int32_t* __restrict__ color, double omega, double* __restrict__ y);
 sfg_status sfg_smooth_gs_impl(sfg_ctx* ctx, const sfg_graph* L, int K, int steps, double omega,
                               uint64_t seed, sfg_dtype storage, void* X_out);
-sfg_status sfg_pointer_jump(sfg_ctx* ctx, int32_t n, const int32_t* comp, int32_t* parent);
+sfg_status sfg_pointer_jump(sfg_ctx* ctx, int32_t n, int32_t* parent);
 sfg_status sfg_count_mask(sfg_ctx* ctx, const uint8_t* mask, int64_t m, int64_t* count_host);
 sfg_status sfg_affinity_impl(sfg_ctx* ctx, const sfg_graph* L, const void* X, int K,
                              sfg_dtype storage, double* delta);
