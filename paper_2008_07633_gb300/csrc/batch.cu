@@ -113,19 +113,6 @@ __global__ void k_seg_count(int64_t m, const uint8_t* __restrict__ mask, int ng,
     }
 }
 
-__global__ void k_not(int64_t m, const uint8_t* __restrict__ mask, uint8_t* __restrict__ out) {
-    for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * kBlock)
-        out[e] = mask[e] == 0;
-}
-
-__global__ void k_compact(int64_t m, const uint8_t* __restrict__ flag, const int64_t* __restrict__ pos,
-                          int32_t* __restrict__ ids) {
-    for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * kBlock)
-        if (flag[e]) ids[pos[e]] = (int32_t)e;
-}
-
 __global__ void k_mark(int64_t k, const int32_t* __restrict__ ids, uint8_t* __restrict__ mask) {
     for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < k;
          i += (int64_t)gridDim.x * kBlock)
@@ -489,17 +476,7 @@ static sfg_status batch_build(sfg_ctx* ctx, int ng, const sfg_graph* const* gs, 
     SFG_CUDA(ctx, cudaMemcpyAsync(b->d_coff, coff.data(), 8 * (ng + 1), cudaMemcpyHostToDevice, ctx->stream));
     SFG_CUDA(ctx, cudaMemcpyAsync(b->d_k, kk.data(), 8 * ng, cudaMemcpyHostToDevice, ctx->stream));
     if (b->k_total > 0) {
-        uint8_t* flag;
-        int64_t* pos;
-        SFG_TRY(s.get(&flag, m));
-        SFG_TRY(s.get(&pos, m + 1));
-        SFG_TRY(sfg_alloc(ctx, (void**)&b->cand, 4 * (size_t)b->ncand + 16));
-        k_not<<<grid_of(ctx, k_not, m), kBlock, 0, ctx->stream>>>(m, b->forest, flag);
-        ++ctx->launches;
-        SFG_TRY(sfg_scan_u8(ctx, flag, pos, m));
-        k_compact<<<grid_of(ctx, k_compact, m), kBlock, 0, ctx->stream>>>(m, flag, pos, b->cand);
-        ++ctx->launches;
-        SFG_LAUNCH_CHECK(ctx, "k_compact");
+        SFG_TRY(sfg_subgraph_impl(ctx, b->U, b->forest, &b->PU, &b->cand));
         if (b->orig_edge) {  // the candidates under their original ids, for the selection
             SFG_TRY(sfg_alloc(ctx, (void**)&b->cand_orig, 4 * (size_t)b->ncand + 16));
             k_gather_ids<<<grid_of(ctx, k_gather_ids, b->ncand), kBlock, 0, ctx->stream>>>(
@@ -507,7 +484,6 @@ static sfg_status batch_build(sfg_ctx* ctx, int ng, const sfg_graph* const* gs, 
             ++ctx->launches;
             SFG_LAUNCH_CHECK(ctx, "k_gather_ids");
         }
-        SFG_TRY(sfg_subgraph_impl(ctx, b->U, b->forest, &b->PU));
         // one-time per-graph structures the sweeps use, built here so that runs never synchronise
         SFG_TRY(sfg_heavy_prepare(ctx, b->U));
         SFG_TRY(sfg_heavy_prepare(ctx, b->PU));

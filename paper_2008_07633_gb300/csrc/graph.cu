@@ -129,14 +129,74 @@ __global__ void k_lap_lower(const int2* __restrict__ colval, const int32_t* __re
     }
 }
 
+// Degrees of the rows of at most hmax entries: FP64 sum in column order, one thread a row.
 __global__ void k_lap_deg(const int32_t* __restrict__ row_ptr, const int2* __restrict__ colval,
-                          int32_t n, double* __restrict__ deg, double* __restrict__ invdeg) {
+                          int32_t n, int32_t hmax, double* __restrict__ deg, double* __restrict__ invdeg) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
          p += (int64_t)gridDim.x * blockDim.x) {
-        double s = 0.0;  // in column order
-        for (int32_t j = row_ptr[p]; j < row_ptr[p + 1]; ++j) s += (double)__int_as_float(colval[j].y);
+        const int32_t a = row_ptr[p], b = row_ptr[p + 1];
+        if (b - a > hmax) continue;
+        double s = 0.0;
+        for (int32_t j = a; j < b; ++j) s += (double)__int_as_float(colval[j].y);
         deg[p] = s;
         invdeg[p] = s > 0.0 ? 1.0 / s : 0.0;
+    }
+}
+
+// Whether FP64 sums of cnt FP32 weights whose exponent fields span [lo, hi] are exact in any order:
+// every partial sum is a multiple of the smallest weight's unit below 2^53 of them.
+__device__ __forceinline__ bool sums_exact(int lo, int hi, int cnt) {
+    const int lg = cnt > 1 ? 32 - __clz(cnt - 1) : 0;
+    return 24 + (hi - lo) + lg <= 53;
+}
+__device__ __forceinline__ int exponent_of(float w) { return max(1, (int)((__float_as_uint(w) >> 23) & 0xffu)); }
+
+// Degrees of the listed rows that have more than SFG_HEAVY_ROW entries, one CTA a row: in parallel
+// where every order gives the column order's bits, else one thread in order (a 4,000-entry row took
+// one thread 0.7 ms).
+__global__ void __launch_bounds__(kBlock) k_lap_deg_heavy(int32_t nh, const int32_t* __restrict__ hrow,
+                                                          const int32_t* __restrict__ row_ptr,
+                                                          const int2* __restrict__ colval,
+                                                          double* __restrict__ deg, double* __restrict__ invdeg) {
+    __shared__ int slo, shi;
+    __shared__ double ws[kBlock / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int32_t h = blockIdx.x; h < nh; h += gridDim.x) {
+        const int32_t p = hrow[h], a = row_ptr[p], b = row_ptr[p + 1];
+        if (b - a <= SFG_HEAVY_ROW) continue;
+        if (threadIdx.x == 0) {
+            slo = 255;
+            shi = 0;
+        }
+        __syncthreads();
+        int lo = 255, hi = 0;
+        double s = 0.0;
+        for (int32_t j = a + threadIdx.x; j < b; j += kBlock) {
+            const float w = __int_as_float(colval[j].y);
+            lo = min(lo, exponent_of(w));
+            hi = max(hi, exponent_of(w));
+            s += (double)w;
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+        if (lane == 0) {
+            atomicMin(&slo, lo);
+            atomicMax(&shi, hi);
+            ws[warp] = s;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s = 0.0;
+            if (sums_exact(slo, shi, b - a))
+                for (int q = 0; q < kBlock / 32; ++q) s += ws[q];
+            else
+                for (int32_t j = a; j < b; ++j) s += (double)__int_as_float(colval[j].y);
+            deg[p] = s;
+            invdeg[p] = s > 0.0 ? 1.0 / s : 0.0;
+        }
+        __syncthreads();
     }
 }
 
@@ -321,14 +381,6 @@ __device__ __forceinline__ float run_weight(const uint64_t* key, const float* sw
     for (int t = i + 1; t < b && key_col(key[t]) == c; ++t) s += (double)sw[t];
     return (float)s;
 }
-
-// Whether FP64 sums of nnz FP32 weights whose exponent fields span [lo, hi] are exact in any order:
-// every partial sum is a multiple of the smallest weight's unit below 2^53 of them.
-__device__ __forceinline__ bool sums_exact(int lo, int hi, int nnz) {
-    const int lg = nnz > 1 ? 32 - __clz(nnz - 1) : 0;
-    return 24 + (hi - lo) + lg <= 53;
-}
-__device__ __forceinline__ int exponent_of(float w) { return max(1, (int)((__float_as_uint(w) >> 23) & 0xffu)); }
 
 // Four consecutive rows a warp (one or two entries a lane on meshes); rows longer than kRowSmall
 // are left to the kernels below. The degrees come last, one lane a row of the CTA's 32: an FP64
@@ -751,49 +803,84 @@ __global__ void k_row_f2c(int64_t m, const int32_t* __restrict__ u, const int32_
 }
 
 // ---- subgraph ----------------------------------------------------------------------------------
-__global__ void k_sub_flags(const int32_t* __restrict__ eid, const uint8_t* __restrict__ mask,
-                            int64_t nnz, uint8_t* __restrict__ keep) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nnz;
-         j += (int64_t)gridDim.x * blockDim.x)
-        keep[j] = mask[eid[j]] != 0;
+// Kept edges and kept entries as one bit each with a running count per 32-bit word: an item's place
+// in the subgraph is its word's count plus the bits below it, so the scans run over 1/32 of the
+// items and the ranks of 12.5M entries are 3 MB of L2-resident words instead of 100 MB of 64-bit
+// offsets. Bound by reading the entries. On the spanning forest of the 128^3 grid the kernels of one
+// subgraph (with its degrees and the list of the other edges) and four host waits took about 0.55 ms of
+// an end-to-end call, of which 0.24 ms are gone.
+__device__ __forceinline__ int64_t bit_rank(const unsigned* __restrict__ bits, const int64_t* __restrict__ woff,
+                                            int64_t i) {
+    const int64_t w = i >> 5;
+    return woff[w] + __popc(bits[w] & ((1u << (i & 31)) - 1u));
 }
 
-__global__ void k_mask01(const uint8_t* __restrict__ mask, int64_t m, uint8_t* __restrict__ out) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * blockDim.x)
-        out[e] = mask[e] != 0;
+// IDS: item i is kept when mask[ids[i]] is set, else when mask[i] is. Whole words of 32 items a warp.
+template <bool IDS>
+__global__ void k_sub_bits(int64_t count, const int32_t* __restrict__ ids, const uint8_t* __restrict__ mask,
+                           unsigned* __restrict__ bits, int32_t* __restrict__ pop) {
+    constexpr int Q = 4;
+    const int lane = threadIdx.x & 31;
+    const int64_t nwords = (count + 31) / 32;
+    const int64_t w0 = ((int64_t)blockIdx.x * kBlock + threadIdx.x) >> 5, nw = (int64_t)gridDim.x * (kBlock / 32);
+    for (int64_t wb = w0 * Q; wb < nwords; wb += nw * Q) {
+        int64_t at[Q];
+        bool keep[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int64_t i = (wb + q) * 32 + lane;
+            at[q] = i < count ? (IDS ? (int64_t)ids[i] : i) : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) keep[q] = at[q] >= 0 && mask[at[q]] != 0;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const unsigned b = __ballot_sync(0xffffffffu, keep[q]);
+            if (lane == 0 && wb + q < nwords) {
+                bits[wb + q] = b;
+                pop[wb + q] = __popc(b);
+            }
+        }
+    }
 }
 
+// The kept edges, and (out != NULL) the ids of the others in ascending order.
 __global__ void k_sub_edges(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-                            const float* __restrict__ ew, const uint8_t* __restrict__ keep_e,
-                            const int64_t* __restrict__ escan, int64_t m, int32_t* __restrict__ su,
-                            int32_t* __restrict__ sv, float* __restrict__ sw) {
+                            const float* __restrict__ ew, const unsigned* __restrict__ bits,
+                            const int64_t* __restrict__ woff, int64_t m, int32_t* __restrict__ su,
+                            int32_t* __restrict__ sv, float* __restrict__ sw, int32_t* __restrict__ out) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
          e += (int64_t)gridDim.x * blockDim.x) {
-        if (!keep_e[e]) continue;
-        const int64_t t = escan[e];
-        su[t] = eu[e]; sv[t] = ev[e]; sw[t] = ew[e];
+        const int64_t t = bit_rank(bits, woff, e);
+        if (bits[e >> 5] >> (e & 31) & 1u) {
+            su[t] = eu[e]; sv[t] = ev[e]; sw[t] = ew[e];
+        } else if (out) {
+            out[e - t] = (int32_t)e;
+        }
     }
 }
 
 __global__ void k_sub_csr(const int2* __restrict__ colval, const int32_t* __restrict__ eid,
-                          const uint8_t* __restrict__ keep, const int64_t* __restrict__ jscan,
-                          const int64_t* __restrict__ escan, int64_t nnz, int2* __restrict__ scv,
-                          int32_t* __restrict__ seid) {
+                          const unsigned* __restrict__ jbits, const int64_t* __restrict__ jwoff,
+                          const unsigned* __restrict__ ebits, const int64_t* __restrict__ ewoff, int64_t nnz,
+                          int2* __restrict__ scv, int32_t* __restrict__ seid) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nnz;
          j += (int64_t)gridDim.x * blockDim.x) {
-        if (!keep[j]) continue;
-        const int64_t t = jscan[j];
+        if (!(jbits[j >> 5] >> (j & 31) & 1u)) continue;
+        const int64_t t = bit_rank(jbits, jwoff, j);
         scv[t] = colval[j];
-        seid[t] = (int32_t)escan[eid[j]];
+        seid[t] = (int32_t)bit_rank(ebits, ewoff, eid[j]);
     }
 }
 
-__global__ void k_sub_rowptr(const int32_t* __restrict__ row_ptr, const int64_t* __restrict__ jscan,
-                             int32_t n, int32_t* __restrict__ srp) {
+__global__ void k_sub_rowptr(const int32_t* __restrict__ row_ptr, const unsigned* __restrict__ jbits,
+                             const int64_t* __restrict__ jwoff, int64_t nnz, int32_t n,
+                             int32_t* __restrict__ srp) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p <= n;
-         p += (int64_t)gridDim.x * blockDim.x)
-        srp[p] = (int32_t)jscan[row_ptr[p]];
+         p += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = row_ptr[p];
+        srp[p] = (int32_t)(j < nnz ? bit_rank(jbits, jwoff, j) : jwoff[(nnz + 31) / 32]);
+    }
 }
 
 __global__ void k_split_colval(const int2* __restrict__ cv, int64_t nnz, int32_t* __restrict__ col,
@@ -854,6 +941,24 @@ sfg_status sfg_alloc_graph(sfg_ctx* ctx, int32_t n, int64_t m, sfg_graph** out) 
         return st;
     }
     *out = g;
+    return SFG_OK;
+}
+
+// Degrees of a graph whose rows are in place. The sweep's heavy-row lists are built with the graph, so
+// that later calls (which may be captured into a CUDA graph) never synchronise for them.
+static sfg_status row_degrees(sfg_ctx* ctx, sfg_graph* g) {
+    SFG_TRY(sfg_heavy_prepare(ctx, g));
+    if (g->n == 0) return SFG_OK;
+    const int32_t hmax = g->hv_n > 0 ? SFG_HEAVY_ROW : INT32_MAX;
+    k_lap_deg<<<grid_of(ctx, k_lap_deg, g->n), kBlock, 0, ctx->stream>>>(g->row_ptr, g->colval, g->n, hmax, g->deg,
+                                                                         g->invdeg);
+    ++ctx->launches;
+    if (g->hv_n > 0) {
+        k_lap_deg_heavy<<<std::min(g->hv_n, 8 * ctx->num_sms), kBlock, 0, ctx->stream>>>(g->hv_n, g->hv_rows, g->row_ptr,
+                                                                                         g->colval, g->deg, g->invdeg);
+        ++ctx->launches;
+    }
+    SFG_LAUNCH_CHECK(ctx, "k_lap_deg");
     return SFG_OK;
 }
 
@@ -933,10 +1038,12 @@ static sfg_status build_by_sort(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
             g->colval, row_of_run, upper, g->row_ptr, nnz, g->eid); ++ctx->launches;
         SFG_LAUNCH_CHECK(ctx, "k_lap_lower");
     }
-    if (n > 0) {
-        k_lap_deg<<<grid_of(ctx, k_lap_deg, n), kBlock, 0, ctx->stream>>>(g->row_ptr, g->colval, n,
-                                                                          g->deg, g->invdeg); ++ctx->launches;
-        SFG_LAUNCH_CHECK(ctx, "k_lap_deg");
+    {
+        const sfg_status ds = row_degrees(ctx, g);
+        if (ds != SFG_OK) {
+            sfg_graph_free(g);
+            return ds;
+        }
     }
     if (f2c && m > 0) {
         SFG_CUDA(ctx, cudaMemsetAsync(f2c, 0xff, sizeof(int32_t) * m, ctx->stream));
@@ -945,13 +1052,6 @@ static sfg_status build_by_sort(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
                 keys, vals, len, sent, run_off, upper, up_off, f2c); ++ctx->launches;
             SFG_LAUNCH_CHECK(ctx, "k_lap_f2c");
         }
-    }
-    // the sweep's heavy-row lists are built with the graph, so that later calls (which may be
-    // captured into a CUDA graph) never synchronise for them
-    const sfg_status hs = sfg_heavy_prepare(ctx, g);
-    if (hs != SFG_OK) {
-        sfg_graph_free(g);
-        return hs;
     }
     *out = g;
     return SFG_OK;
@@ -1105,52 +1205,58 @@ sfg_status sfg_build_graph(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u,
 }
 
 sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* mask,
-                             sfg_graph** out) {
+                             sfg_graph** out, int32_t** off_ids) {
     *out = nullptr;
-    const int64_t nnz = 2 * g->m;
+    if (off_ids) *off_ids = nullptr;
+    const int64_t m = g->m, nnz = 2 * m, ewords = (m + 31) / 32, jwords = (nnz + 31) / 32;
     Scratch s(ctx);
-    uint8_t *keep, *keep_e;
-    int64_t *jscan, *escan;
-    SFG_TRY(s.get(&keep, nnz));
-    SFG_TRY(s.get(&keep_e, g->m));
-    SFG_TRY(s.get(&jscan, nnz + 1));
-    SFG_TRY(s.get(&escan, g->m + 1));
+    unsigned *ebits, *jbits;
+    int32_t *epop, *jpop;
+    int64_t *ewoff, *jwoff;
+    SFG_TRY(s.get(&ebits, ewords));
+    SFG_TRY(s.get(&jbits, jwords));
+    SFG_TRY(s.get(&epop, ewords));
+    SFG_TRY(s.get(&jpop, jwords));
+    SFG_TRY(s.get(&ewoff, ewords + 1));
+    SFG_TRY(s.get(&jwoff, jwords + 1));
     int64_t ms = 0;
-    if (g->m > 0) {
-        k_mask01<<<grid_of(ctx, k_mask01, g->m), kBlock, 0, ctx->stream>>>(mask, g->m, keep_e); ++ctx->launches;
-        SFG_LAUNCH_CHECK(ctx, "k_mask01");
-        k_sub_flags<<<grid_of(ctx, k_sub_flags, nnz), kBlock, 0, ctx->stream>>>(g->eid, mask, nnz,
-                                                                                keep); ++ctx->launches;
-        SFG_LAUNCH_CHECK(ctx, "k_sub_flags");
-        SFG_TRY(sfg_scan_u8(ctx, keep_e, escan, g->m));
-        SFG_TRY(sfg_scan_u8(ctx, keep, jscan, nnz));
-        SFG_TRY(sfg_read_i64(ctx, escan + g->m, &ms));
+    if (m > 0) {
+        k_sub_bits<false><<<grid_of(ctx, k_sub_bits<false>, (m + 3) / 4), kBlock, 0, ctx->stream>>>(m, nullptr, mask, ebits, epop);
+        SFG_TRY(sfg_scan_i32(ctx, epop, ewoff, ewords));
+        k_sub_bits<true><<<grid_of(ctx, k_sub_bits<true>, (nnz + 3) / 4), kBlock, 0, ctx->stream>>>(nnz, g->eid, mask, jbits, jpop);
+        SFG_TRY(sfg_scan_i32(ctx, jpop, jwoff, jwords));
+        ctx->launches += 2;
+        SFG_LAUNCH_CHECK(ctx, "k_sub_bits");
+        SFG_TRY(sfg_read_i64(ctx, ewoff + ewords, &ms));
     } else {
-        SFG_CUDA(ctx, cudaMemsetAsync(jscan, 0, sizeof(int64_t), ctx->stream));
+        SFG_CUDA(ctx, cudaMemsetAsync(jwoff, 0, sizeof(int64_t), ctx->stream));
     }
     sfg_graph* p = nullptr;
     SFG_TRY(sfg_alloc_graph(ctx, g->n, ms, &p));
-    if (g->m > 0) {
-        k_sub_edges<<<grid_of(ctx, k_sub_edges, g->m), kBlock, 0, ctx->stream>>>(
-            g->eu, g->ev, g->ew, keep_e, escan, g->m, p->eu, p->ev, p->ew); ++ctx->launches;
+    struct Owner { sfg_graph* g; ~Owner() { sfg_graph_free(g); } } own{p};
+    int32_t* rest = nullptr;
+    if (off_ids) SFG_TRY(s.get(&rest, m - ms));
+    if (m > 0) {
+        k_sub_edges<<<grid_of(ctx, k_sub_edges, m), kBlock, 0, ctx->stream>>>(
+            g->eu, g->ev, g->ew, ebits, ewoff, m, p->eu, p->ev, p->ew, rest); ++ctx->launches;
         SFG_LAUNCH_CHECK(ctx, "k_sub_edges");
         k_sub_csr<<<grid_of(ctx, k_sub_csr, nnz), kBlock, 0, ctx->stream>>>(
-            g->colval, g->eid, keep, jscan, escan, nnz, p->colval, p->eid); ++ctx->launches;
+            g->colval, g->eid, jbits, jwoff, ebits, ewoff, nnz, p->colval, p->eid); ++ctx->launches;
         SFG_LAUNCH_CHECK(ctx, "k_sub_csr");
     }
     k_sub_rowptr<<<grid_of(ctx, k_sub_rowptr, (int64_t)g->n + 1), kBlock, 0, ctx->stream>>>(
-        g->row_ptr, jscan, g->n, p->row_ptr); ++ctx->launches;
+        g->row_ptr, jbits, jwoff, nnz, g->n, p->row_ptr); ++ctx->launches;
     SFG_LAUNCH_CHECK(ctx, "k_sub_rowptr");
-    if (g->n > 0) {
-        k_lap_deg<<<grid_of(ctx, k_lap_deg, g->n), kBlock, 0, ctx->stream>>>(p->row_ptr, p->colval,
-                                                                             g->n, p->deg, p->invdeg); ++ctx->launches;
-        SFG_LAUNCH_CHECK(ctx, "k_lap_deg");
+    if (g->hv_n == 0) {  // rows only lose entries: no heavy row here either
+        p->hv_nseg = 0;
+        p->hv_n = 0;
     }
-    const sfg_status hs = sfg_heavy_prepare(ctx, p);
-    if (hs != SFG_OK) {
-        sfg_graph_free(p);
-        return hs;
+    SFG_TRY(row_degrees(ctx, p));
+    if (off_ids) {
+        s.release(rest);
+        *off_ids = rest;
     }
+    own.g = nullptr;
     *out = p;
     return SFG_OK;
 }

@@ -142,6 +142,7 @@ struct Scratch {
         *p = static_cast<T*>(q);
         return SFG_OK;
     }
+    void adopt(void* p) { ptrs.push_back(p); }  // take ownership from the caller
     void release(void* p) {  // hand ownership to the caller
         for (auto& q : ptrs)
             if (q == p) q = nullptr;
@@ -188,8 +189,10 @@ sfg_status sfg_read_i64(sfg_ctx* ctx, const int64_t* dev, int64_t* host);
 sfg_status sfg_build_graph(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u,
                            const int32_t* v, const float* w, bool validate, sfg_graph** out,
                            int32_t* fine2coarse_out);
+// off_ids (may be NULL) receives the ids of the edges outside the mask, ascending, in an allocation
+// of the context (at least m - kept entries) that the caller frees.
 sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* mask,
-                             sfg_graph** out);
+                             sfg_graph** out, int32_t** off_ids = nullptr);
 // comp_out (optional, n entries): each node's component label, a node of that component.
 // key_id (m entries, may be NULL): the id that breaks weight ties for edge e (default e), with
 // key_inv its inverse; a relabelled copy of a graph passes its original edge ids, so that its

@@ -13,19 +13,6 @@ namespace {
 
 constexpr int kBlock = 256;
 
-__global__ void k_not_mask(int64_t m, const uint8_t* __restrict__ mask, uint8_t* __restrict__ out) {
-    for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * kBlock)
-        out[e] = mask[e] == 0;
-}
-
-__global__ void k_compact_ids(int64_t m, const uint8_t* __restrict__ flag,
-                              const int64_t* __restrict__ pos, int32_t* __restrict__ ids) {
-    for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * kBlock)
-        if (flag[e]) ids[pos[e]] = (int32_t)e;
-}
-
 __global__ void k_f32_to_bf16(int64_t n, const float* __restrict__ x, __nv_bfloat16* __restrict__ y) {
     for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * kBlock)
@@ -61,14 +48,14 @@ size_t elem_size(sfg_dtype dt) { return dt == SFG_BF16 ? 2 : 4; }
 // Edge recovery at one level (Sec. 3.5; the embedding, scoring and selection steps of
 // Algorithm 1). `mask` holds the current sparsifier of g and receives the added edges. XG_f32: the
 // FP32 embedding of g from this level's seed, cached from coarsening (may be NULL: computed here
-// in the requested storage).
+// in the requested storage). count: the mask's edges on entry (-1: not known) and on return.
 sfg_status recover(sfg_ctx* ctx, const sfg_graph* g, const sfg_params* P, uint64_t seed,
-                   int64_t forest, const float* XG_f32, uint8_t* mask) {
+                   int64_t forest, const float* XG_f32, uint8_t* mask, int64_t* count) {
     const int64_t m = g->m;
     const int64_t base = P->budget_unit == 0 ? (int64_t)g->n : m - forest;
     const int64_t target = round_half_up(P->budget_frac * (double)base);
-    int64_t in_p = 0;
-    SFG_TRY(sfg_count_mask(ctx, mask, m, &in_p));
+    if (*count < 0) SFG_TRY(sfg_count_mask(ctx, mask, m, count));
+    const int64_t in_p = *count;
     const int64_t ncand = m - in_p;
     int64_t k = target - (in_p - forest);
     if (k < 0) k = 0;
@@ -76,24 +63,13 @@ sfg_status recover(sfg_ctx* ctx, const sfg_graph* g, const sfg_params* P, uint64
     if (k == 0) return SFG_OK;
 
     Scratch s(ctx);
-    uint8_t* flag;
-    int64_t* pos;
     int32_t *cand, *sel;
     float* scores;
-    SFG_TRY(s.get(&flag, m));
-    SFG_TRY(s.get(&pos, m + 1));
-    SFG_TRY(s.get(&cand, ncand));
     SFG_TRY(s.get(&scores, ncand));
     SFG_TRY(s.get(&sel, k));
-    const int gm = sfg_grid(ctx, (const void*)k_not_mask, kBlock, 0, m);
-    k_not_mask<<<gm, kBlock, 0, ctx->stream>>>(m, mask, flag); ++ctx->launches;
-    SFG_LAUNCH_CHECK(ctx, "k_not_mask");
-    SFG_TRY(sfg_scan_u8(ctx, flag, pos, m));
-    k_compact_ids<<<gm, kBlock, 0, ctx->stream>>>(m, flag, pos, cand); ++ctx->launches;
-    SFG_LAUNCH_CHECK(ctx, "k_compact_ids");
-
     sfg_graph* pg = nullptr;
-    SFG_TRY(sfg_subgraph_impl(ctx, g, mask, &pg));
+    SFG_TRY(sfg_subgraph_impl(ctx, g, mask, &pg, &cand));
+    s.adopt(cand);
     struct Guard { sfg_graph* g; ~Guard() { sfg_graph_free(g); } } guard{pg};
 
     if (P->smoother == SFG_SMOOTH_GAUSS_SEIDEL) {  // the paper's smoother: embed both, then score
@@ -136,6 +112,7 @@ sfg_status recover(sfg_ctx* ctx, const sfg_graph* g, const sfg_params* P, uint64
     k_set_mask<<<sfg_grid(ctx, (const void*)k_set_mask, kBlock, 0, k), kBlock, 0, ctx->stream>>>(
         k, sel, mask); ++ctx->launches;
     SFG_LAUNCH_CHECK(ctx, "k_set_mask");
+    *count = in_p + k;
     return SFG_OK;
 }
 
@@ -229,7 +206,8 @@ extern "C" sfg_status sfg_sparsify(sfg_ctx* ctx, const sfg_graph* G, const sfg_p
     int64_t n_tree = 0;
     SFG_TRY(sfg_mst_impl(ctx, gc, nullptr, pm, &n_tree));
     const int64_t comps = (int64_t)gc->n - n_tree;  // same at every level: aggregates are connected
-    SFG_TRY(recover(ctx, gc, P, level_seed(P->seed, lf), n_tree, nullptr, pm));
+    int64_t count = n_tree;
+    SFG_TRY(recover(ctx, gc, P, level_seed(P->seed, lf), n_tree, nullptr, pm, &count));
 
     // Algorithm 1, level loop: map back and recover edges level by level
     for (int l = lf; l >= 1; --l) {
@@ -237,14 +215,18 @@ extern "C" sfg_status sfg_sparsify(sfg_ctx* ctx, const sfg_graph* G, const sfg_p
         SFG_TRY(sfg_alloc(ctx, (void**)&lv[l - 1].pmask, (size_t)f->m + 16));
         uint8_t* pf = lv[l - 1].pmask;
         SFG_TRY(sfg_backward_impl(ctx, f, lv[l].agg, lv[l].f2c, lv[l].g, pm, pf));
+        count = -1;
         SFG_TRY(recover(ctx, f, P, level_seed(P->seed, l - 1), (int64_t)f->n - comps, lv[l - 1].xg,
-                        pf));
+                        pf, &count));
         pm = pf;
     }
     for (Level& v : lv) v.xg = nullptr;  // scratch, freed with s
     if (G->m > 0)
         SFG_CUDA(ctx, cudaMemcpyAsync(mask_out, pm, G->m, cudaMemcpyDeviceToDevice, ctx->stream));
-    if (n_selected_host) SFG_TRY(sfg_count_mask(ctx, mask_out, G->m, n_selected_host));
+    if (n_selected_host) {
+        SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        *n_selected_host = count;
+    }
     if (hier_out) {
         *hier_out = h;
         owner.h = nullptr;
@@ -334,27 +316,16 @@ extern "C" sfg_status sfg_sparsify_learned(sfg_ctx* ctx, const sfg_graph* G, con
         if (nprop < k) nprop = k;
         if (nprop > ncand) nprop = ncand;
         Scratch s(ctx);
-        uint8_t* flag;
-        int64_t* pos;
         int32_t *cand, *prop, *sel;
         float *feats, *pred, *scores;
-        SFG_TRY(s.get(&flag, m));
-        SFG_TRY(s.get(&pos, m + 1));
-        SFG_TRY(s.get(&cand, ncand));
         SFG_TRY(s.get(&feats, (size_t)ncand * SFG_MLP_NFEAT));
         SFG_TRY(s.get(&pred, ncand));
         SFG_TRY(s.get(&prop, nprop));
         SFG_TRY(s.get(&scores, nprop));
         SFG_TRY(s.get(&sel, k));
-        const int gm = sfg_grid(ctx, (const void*)k_not_mask, kBlock, 0, m);
-        k_not_mask<<<gm, kBlock, 0, ctx->stream>>>(m, mask_out, flag);
-        ++ctx->launches;
-        SFG_TRY(sfg_scan_u8(ctx, flag, pos, m));
-        k_compact_ids<<<gm, kBlock, 0, ctx->stream>>>(m, flag, pos, cand);
-        ++ctx->launches;
-        SFG_LAUNCH_CHECK(ctx, "k_compact_ids");
         sfg_graph* pg = nullptr;
-        SFG_TRY(sfg_subgraph_impl(ctx, G, mask_out, &pg));
+        SFG_TRY(sfg_subgraph_impl(ctx, G, mask_out, &pg, &cand));
+        s.adopt(cand);
         struct Guard { sfg_graph* g; ~Guard() { sfg_graph_free(g); } } guard{pg};
         SFG_TRY(sfg_edge_features_impl(ctx, G, pg, P->K, feat_steps, P->omega, P->seed, P->storage,
                                        cand, ncand, feats));
@@ -399,21 +370,23 @@ extern "C" sfg_status sfg_sparsify_to_kappa(sfg_ctx* ctx, const sfg_graph* G, co
     if (G->m > 0) SFG_TRY(sfg_check_dev(ctx, mask_out, "mask_out"));
     int64_t forest = 0;
     SFG_TRY(sfg_mst_impl(ctx, G, nullptr, mask_out, &forest));
+    int64_t count = forest;
     int r = 0;
     for (;; ++r) {
         double kap = 1.0;
         SFG_TRY(sfg_kappa_impl(ctx, G, mask_out, kappa_steps, P->seed ^ 0x6b617070ull, &kap, nullptr));
         if (kappa_trace_host) kappa_trace_host[r] = kap;
         if (kap <= kappa_target || r == max_rounds) break;
-        int64_t before = 0, after = 0;
-        SFG_TRY(sfg_count_mask(ctx, mask_out, G->m, &before));
+        const int64_t before = count;
         sfg_params Pr = *P;
         Pr.budget_frac = (double)(r + 1) * batch_frac;
-        SFG_TRY(recover(ctx, G, &Pr, P->seed, forest, nullptr, mask_out));
-        SFG_TRY(sfg_count_mask(ctx, mask_out, G->m, &after));
-        if (after == before) break;  // nothing left to add
+        SFG_TRY(recover(ctx, G, &Pr, P->seed, forest, nullptr, mask_out, &count));
+        if (count == before) break;  // nothing left to add
     }
     if (rounds_host) *rounds_host = r;
-    if (n_selected_host) SFG_TRY(sfg_count_mask(ctx, mask_out, G->m, n_selected_host));
+    if (n_selected_host) {
+        SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        *n_selected_host = count;
+    }
     return SFG_OK;
 }
