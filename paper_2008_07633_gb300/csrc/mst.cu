@@ -24,19 +24,25 @@ __global__ void k_mst_init(int32_t n, int32_t* __restrict__ comp) {
 // labels, 8 + 4 + 4 bytes an entry. An edge inside a component stays inside for good, so a node
 // keeps its best edge and looks through its row again only when that edge has become internal, and
 // never again once no edge leaves; a component's maximum is compared before the 64-bit atomicMax, so
-// most nodes of a large component only read it. With the launches and host waits of separate round
-// kernels gone as well, the forest of the 128^3 grid takes 1,220 us (11 rounds of 6 launches and a
-// wait, every row rescanned: 1,490 us of kernels and about 170 us of waits) and that of a 64 x 64
-// grid 95 us (290 us with the waits).
+// most nodes of a large component only read it. Hooking and jumping go over a list of the labels that
+// are left. Separate round kernels that rescanned every row took 1,490 us and 11 host waits on the
+// 128^3 grid and 200 us and 7 waits on a 64 x 64 grid.
 //
 // Items are the rows [0, n), rows longer than SFG_HEAVY_ROW excepted, and then the fixed segments
-// of those rows. A warp takes 32 items: one lane each checks the kept edge; the items to look
-// through again are dealt to four 8-lane groups, kMstItems at a time so that as many independent
-// load chains (entry -> neighbour's label) are in flight.
+// of those rows. A warp takes kMstTiles x 32 items at once (the tiles a whole grid apart, so that the hubs
+// of a graph numbered by degree spread over the warps), one lane each checking the kept edges. The
+// items to look through again go through shared memory: up to kMstLong entries to four 8-lane groups,
+// kMstItems at a time, longer ones to the whole warp, four entries a lane in flight. Every step is a
+// chain of dependent loads, so the chains in flight set the time: with one tile a warp and every row
+// in 8-lane groups the 128^3 grid took 1,220 us, and a coarsened power-law graph, whose consecutive
+// hub rows then shared a warp, more than the separate kernels (two-level sparsify of a 249,480-node
+// Chung-Lu graph 9.6 ms instead of 6.9).
+constexpr int kMstTiles = 4, kMstLong = 32;
 constexpr int kMstLanes = 8, kMstGroups = 32 / kMstLanes, kMstItems = 4;
 
-// Words of one launch: barrier count, error, edges taken, last pointer-jumping pass with work left.
-enum { kMwBar, kMwErr, kMwTree, kMwJump, kMwCount };
+// Words of one launch: barrier count, error, edges taken, last pointer-jumping pass with work left,
+// lengths of the two label lists.
+enum { kMwBar, kMwErr, kMwTree, kMwJump, kMwLabels0, kMwLabels1, kMwCount };
 
 struct MstArgs {
     int32_t n;
@@ -55,6 +61,7 @@ struct MstArgs {
     unsigned long long* best;   // per component label
     unsigned long long* ckey;   // per item: its kept edge's key and the node across it (-1: none left)
     int32_t* cnbr;
+    int32_t* labels[2];         // labels of the components that still had an edge, this round's and the next's
     uint8_t* mask;
     unsigned long long* words;
 };
@@ -81,7 +88,9 @@ __device__ __forceinline__ void mst_offer(unsigned long long* best, int32_t c, u
 }
 
 __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
-    __shared__ uint8_t s_list[kBlock / 32][32];
+    constexpr int LIST = kMstTiles * 32;
+    __shared__ uint8_t s_list[kBlock / 32][LIST];
+    __shared__ int32_t s_a[kBlock / 32][LIST], s_b[kBlock / 32][LIST], s_c[kBlock / 32][LIST];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % kMstLanes, grp = lane / kMstLanes;
     const int64_t t0 = (int64_t)blockIdx.x * kBlock + threadIdx.x, nt = (int64_t)gridDim.x * kBlock;
     const int64_t items = (int64_t)A.n + A.nseg;
@@ -96,48 +105,66 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
     // each round at least halves the number of components that still have outgoing edges
     for (int round = 0; round < 64; ++round) {
         // (1) the largest key leaving each component
-        for (int64_t base = t0 - lane; base < items; base += nt) {
-            const int64_t i = base + lane;
-            int32_t cp = -1, a = 0, b = 0;
-            bool need = false;
-            if (i < items) {
-                const int32_t nb = round == 0 ? 0 : A.cnbr[i];
-                if (nb >= 0) {
-                    int4 sg = make_int4((int32_t)i, 0, 0, 0);
-                    if (i >= A.n) sg = A.seg[i - A.n];
-                    cp = A.comp[sg.x];
-                    need = round == 0 || A.comp[nb] == cp;
-                    if (need) {
+        for (int64_t base = t0 - lane; base < items; base += nt * kMstTiles) {
+            int32_t nb[kMstTiles], row[kMstTiles], cp[kMstTiles];
+#pragma unroll
+            for (int q = 0; q < kMstTiles; ++q) {
+                const int64_t i = base + q * nt + lane;
+                nb[q] = i < items ? (round == 0 ? 0 : A.cnbr[i]) : -1;
+                row[q] = (int32_t)i;
+                if (i >= A.n && nb[q] >= 0) row[q] = A.seg[i - A.n].x;
+            }
+#pragma unroll
+            for (int q = 0; q < kMstTiles; ++q) {
+                cp[q] = nb[q] >= 0 ? A.comp[row[q]] : -1;
+                // the label across the kept edge (round 0: nothing kept, look)
+                nb[q] = nb[q] >= 0 ? (round == 0 ? cp[q] : A.comp[nb[q]]) : -1;
+            }
+            int cnt = 0, longs = 0;  // short items from the front of the lists, long ones from the back
+#pragma unroll
+            for (int q = 0; q < kMstTiles; ++q) {
+                const int64_t i = base + q * nt + lane;
+                const bool need = cp[q] >= 0 && nb[q] == cp[q];
+                if (cp[q] >= 0 && !need) mst_offer(A.best, cp[q], A.ckey[i]);
+                int32_t a = 0, b = 0;
+                if (need) {
+                    if (i < A.n) {
+                        a = A.row_ptr[i];
+                        b = A.row_ptr[i + 1];
+                        if (b - a > SFG_HEAVY_ROW) b = a;  // looked through by segments
+                    } else {
+                        const int4 sg = A.seg[i - A.n];
                         a = sg.y;
                         b = sg.z;
-                        if (i < A.n) {
-                            a = A.row_ptr[i];
-                            b = A.row_ptr[i + 1];
-                            if (b - a > SFG_HEAVY_ROW) b = a;  // looked through by segments
-                        }
-                    } else {
-                        mst_offer(A.best, cp, A.ckey[i]);
                     }
                 }
+                const bool big = b - a > kMstLong;
+                const unsigned low = (1u << lane) - 1u;
+                const unsigned todo = __ballot_sync(0xffffffffu, need && !big), wide = __ballot_sync(0xffffffffu, big);
+                if (need) {
+                    const int at = big ? LIST - 1 - (longs + __popc(wide & low)) : cnt + __popc(todo & low);
+                    s_list[warp][at] = (uint8_t)(q * 32 + lane);
+                    s_a[warp][at] = a;
+                    s_b[warp][at] = b;
+                    s_c[warp][at] = cp[q];
+                }
+                cnt += __popc(todo);
+                longs += __popc(wide);
             }
-            const unsigned todo = __ballot_sync(0xffffffffu, need);
-            if (need) s_list[warp][__popc(todo & ((1u << lane) - 1u))] = (uint8_t)lane;
             __syncwarp();
-            const int cnt = __popc(todo);
             for (int k0 = 0; k0 < cnt; k0 += kMstGroups * kMstItems) {
-                int src[kMstItems];
-                int32_t ra[kMstItems], rb[kMstItems], rc[kMstItems], nbr[kMstItems], e[kMstItems];
+                int32_t ra[kMstItems], rb[kMstItems], rc[kMstItems], across[kMstItems], e[kMstItems];
                 int2 cv[kMstItems];
                 unsigned long long top[kMstItems];
 #pragma unroll
                 for (int u = 0; u < kMstItems; ++u) {
                     const int k = k0 + u * kMstGroups + grp;
-                    src[u] = k < cnt ? s_list[warp][k] : -1;
-                    const int from = src[u] < 0 ? 0 : src[u];
-                    ra[u] = __shfl_sync(0xffffffffu, a, from);
-                    rb[u] = __shfl_sync(0xffffffffu, b, from);
-                    rc[u] = __shfl_sync(0xffffffffu, cp, from);
-                    if (src[u] < 0) rb[u] = ra[u];
+                    ra[u] = rb[u] = rc[u] = 0;
+                    if (k < cnt) {
+                        ra[u] = s_a[warp][k];
+                        rb[u] = s_b[warp][k];
+                        rc[u] = s_c[warp][k];
+                    }
                     const int32_t j = ra[u] + sub;
                     cv[u] = j < rb[u] ? A.colval[j] : make_int2(-1, 0);
                     e[u] = j < rb[u] ? A.eid[j] : 0;
@@ -145,7 +172,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
 #pragma unroll
                 for (int u = 0; u < kMstItems; ++u) {
                     top[u] = 0ull;
-                    nbr[u] = -1;
+                    across[u] = -1;
                     for (int32_t j = ra[u] + sub;;) {
                         if (cv[u].x >= 0 && A.comp[cv[u].x] != rc[u] && (!A.allow || A.allow[e[u]])) {
                             const uint32_t id = A.key_id ? (uint32_t)A.key_id[e[u]] : (uint32_t)e[u];
@@ -153,7 +180,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
                                                            (unsigned long long)(~id);
                             if (key > top[u]) {
                                 top[u] = key;
-                                nbr[u] = cv[u].x;
+                                across[u] = cv[u].x;
                             }
                         }
                         j += kMstLanes;
@@ -170,33 +197,80 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
                         const unsigned long long q = __shfl_xor_sync(0xffffffffu, m, o);
                         m = q > m ? q : m;
                     }
-                    if (src[u] < 0) continue;
-                    const int64_t it = base + src[u];
+                    const int k = k0 + u * kMstGroups + grp;
+                    if (k >= cnt) continue;
+                    const int64_t it = base + (s_list[warp][k] >> 5) * nt + (s_list[warp][k] & 31);
                     if (m == 0ull) {
                         if (sub == 0) A.cnbr[it] = -1;
                     } else if (top[u] == m) {  // keys are unique: one lane holds it
-                        A.cnbr[it] = nbr[u];
+                        A.cnbr[it] = across[u];
                         A.ckey[it] = m;
                         mst_offer(A.best, rc[u], m);
                     }
                 }
             }
+            for (int k = LIST - longs; k < LIST; ++k) {
+                const int32_t a = s_a[warp][k], b = s_b[warp][k], c = s_c[warp][k];
+                unsigned long long top = 0ull;
+                int32_t across = -1;
+                for (int32_t j0 = a; j0 < b; j0 += 128) {
+                    int2 cv[4];
+                    int32_t e[4], other[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int32_t j = j0 + u * 32 + lane;
+                        cv[u] = j < b ? A.colval[j] : make_int2(-1, 0);
+                        e[u] = j < b ? A.eid[j] : 0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) other[u] = cv[u].x >= 0 ? A.comp[cv[u].x] : c;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (other[u] == c || (A.allow && !A.allow[e[u]])) continue;
+                        const uint32_t id = A.key_id ? (uint32_t)A.key_id[e[u]] : (uint32_t)e[u];
+                        const unsigned long long key = ((unsigned long long)(uint32_t)cv[u].y << 32) |
+                                                       (unsigned long long)(~id);
+                        if (key > top) {
+                            top = key;
+                            across = cv[u].x;
+                        }
+                    }
+                }
+                unsigned long long m = top;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned long long q = __shfl_xor_sync(0xffffffffu, m, o);
+                    m = q > m ? q : m;
+                }
+                const int64_t it = base + (s_list[warp][k] >> 5) * nt + (s_list[warp][k] & 31);
+                if (m == 0ull) {
+                    if (lane == 0) A.cnbr[it] = -1;
+                } else if (top == m) {
+                    A.cnbr[it] = across;
+                    A.ckey[it] = m;
+                    mst_offer(A.best, c, m);
+                }
+            }
             __syncwarp();
         }
         if (!grid_barrier(bar, passed)) return;
-        // (2) hooks across the chosen edges
+        // (2) hooks across the chosen edges; round 0: every node is a label
+        const int32_t* list = A.labels[round & 1];
+        const int64_t nlab = round == 0 ? (int64_t)A.n
+                                        : (int64_t)*(volatile unsigned long long*)(A.words + kMwLabels0 + (round & 1));
+        if (blockIdx.x == 0 && threadIdx.x == 0) A.words[kMwLabels0 + ((round + 1) & 1)] = 0ull;
         unsigned taken = 0;
-        for (int64_t r = t0; r < A.n; r += nt) {
-            if (A.comp[r] != r) continue;  // only component labels act
+        for (int64_t i = t0; i < nlab; i += nt) {
+            const int32_t r = round == 0 ? (int32_t)i : list[i];
             const unsigned long long k = A.best[r];
-            int32_t up = (int32_t)r;
+            int32_t up = r;
             if (k != 0ull) {
                 const uint32_t id = ~(uint32_t)(k & 0xffffffffull);
                 const uint32_t e = A.key_inv ? (uint32_t)A.key_inv[id] : id;
                 A.mask[e] = 1;
                 const int32_t c0 = A.comp[A.eu[e]], c1 = A.comp[A.ev[e]];
-                const int32_t other = c0 == (int32_t)r ? c1 : c0;
-                if (!(A.best[other] == k && (int32_t)r < other)) {
+                const int32_t other = c0 == r ? c1 : c0;
+                if (!(A.best[other] == k && r < other)) {
                     up = other;
                     ++taken;
                 }
@@ -213,17 +287,35 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
         for (;;) {
             ++jump_pass;
             bool left = false;
-            for (int64_t r = t0; r < A.n; r += nt)
-                if (A.comp[r] == r) left |= jump_node(A.parent, r);
+            for (int64_t i = t0; i < nlab; i += nt) left |= jump_node(A.parent, round == 0 ? i : (int64_t)list[i]);
             if (left) atomicMax(A.words + kMwJump, jump_pass);
             if (!grid_barrier(bar, passed)) return;
             if (*(volatile unsigned long long*)(A.words + kMwJump) < jump_pass) break;
         }
-        // (4) relabel; the labels that remain start the next round with no edge
-        for (int64_t p = t0; p < A.n; p += nt) {
-            const int32_t c = A.parent[A.comp[p]];
-            A.comp[p] = c;
-            if (c == (int32_t)p) A.best[p] = 0ull;
+        // (4) relabel; the next round's labels are the roots that had an edge in this one
+        for (int64_t p0 = t0; p0 < A.n; p0 += nt * kMstTiles) {
+            int32_t c[kMstTiles];
+#pragma unroll
+            for (int q = 0; q < kMstTiles; ++q) c[q] = p0 + q * nt < A.n ? A.comp[p0 + q * nt] : 0;
+#pragma unroll
+            for (int q = 0; q < kMstTiles; ++q) c[q] = A.parent[c[q]];
+#pragma unroll
+            for (int q = 0; q < kMstTiles; ++q)
+                if (p0 + q * nt < A.n) A.comp[p0 + q * nt] = c[q];
+        }
+        for (int64_t i0 = t0 - lane; i0 < nlab; i0 += nt) {
+            const int64_t i = i0 + lane;
+            const int32_t r = i < nlab ? (round == 0 ? (int32_t)i : list[i]) : -1;
+            const bool stays = r >= 0 && A.parent[r] == r && A.best[r] != 0ull;
+            const unsigned b = __ballot_sync(0xffffffffu, stays);
+            if (!b) continue;
+            unsigned long long at = 0;
+            if (lane == __ffs(b) - 1) at = atomicAdd(A.words + kMwLabels0 + ((round + 1) & 1), (unsigned long long)__popc(b));
+            at = __shfl_sync(0xffffffffu, at, __ffs(b) - 1);
+            if (stays) {
+                A.labels[(round + 1) & 1][at + __popc(b & ((1u << lane) - 1u))] = r;
+                A.best[r] = 0ull;
+            }
         }
         if (!grid_barrier(bar, passed)) return;
     }
@@ -311,6 +403,8 @@ sfg_status sfg_mst_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* allow, 
     SFG_TRY(s.get(&a.best, n));
     SFG_TRY(s.get(&a.ckey, items));
     SFG_TRY(s.get(&a.cnbr, items));
+    SFG_TRY(s.get(&a.labels[0], n));
+    SFG_TRY(s.get(&a.labels[1], n));
     SFG_TRY(s.get(&a.words, kMwCount));
     int* hw32 = nullptr;
     SFG_TRY(sfg_host_word(ctx, kSfgHostBuild, &hw32));
