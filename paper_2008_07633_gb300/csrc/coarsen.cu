@@ -13,22 +13,82 @@ namespace {
 
 constexpr int kBlock = 256;
 
-__global__ void k_hook(int32_t n, const int32_t* __restrict__ row_ptr, const int2* __restrict__ colval,
-                       const int32_t* __restrict__ eid, const double* __restrict__ delta,
-                       int32_t* __restrict__ hook) {
-    for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * kBlock) {
-        int32_t best = -1;
-        double bd = 0.0;
-        for (int32_t j = row_ptr[p]; j < row_ptr[p + 1]; ++j) {
-            const double d = delta[eid[j]];
-            const int32_t q = colval[j].x;
-            if (best < 0 || d < bd || (d == bd && q < best)) {
-                best = q;
-                bd = d;
-            }
+// Distances compared as integers in their numerical order (-0 as +0): FP64 comparisons share the slow
+// FP64 pipe. A scan of the row that keeps the first entry until a smaller distance comes never
+// replaces a NaN it started with and never takes a NaN later: first entry below, others above all.
+__device__ __forceinline__ int64_t hook_key(double d, bool first) {
+    int64_t b = __double_as_longlong(d);
+    if ((b & INT64_MAX) > 0x7ff0000000000000ll) return first ? INT64_MIN : INT64_MAX;
+    if ((b & INT64_MAX) == 0) b = 0;
+    return b < 0 ? b ^ INT64_MAX : b;
+}
+
+__device__ __forceinline__ void hook_take(int64_t& bk, int32_t& bq, int64_t k, int32_t q) {
+    if (k < bk || (k == bk && q < bq)) {
+        bk = k;
+        bq = q;
+    }
+}
+
+// Each node's neighbour of smallest (distance, id): eight lanes a row, the loads of a lane's entries
+// independent; rows over SFG_HEAVY_ROW entries (listed) are left to k_hook_heavy, one CTA each. A
+// thread a row chained distance gathers one after the other: 126 us on the 128^3 grid and its coarse
+// graph together, 1,190 us on a coarsened power-law graph whose hub rows held one thread each.
+constexpr int kHookLanes = 8;
+__global__ void __launch_bounds__(kBlock) k_hook(int32_t n, int32_t hmax, const int32_t* __restrict__ row_ptr,
+                                                 const int2* __restrict__ colval, const int32_t* __restrict__ eid,
+                                                 const double* __restrict__ delta, int32_t* __restrict__ hook) {
+    const int sub = threadIdx.x % kHookLanes;
+    const int64_t ng = (int64_t)gridDim.x * kBlock / kHookLanes;
+    for (int64_t p0 = ((int64_t)blockIdx.x * kBlock + threadIdx.x) / 32 * (32 / kHookLanes); p0 < n; p0 += ng) {
+        const int64_t p = p0 + (threadIdx.x & 31) / kHookLanes;
+        int32_t a = 0, b = 0;
+        if (p < n) {
+            a = row_ptr[p];
+            b = row_ptr[p + 1];
         }
-        hook[p] = best < 0 ? (int32_t)p : best;
+        const bool heavy = b - a > hmax;
+        int64_t bk = INT64_MAX;
+        int32_t bq = INT32_MAX;
+        if (!heavy)
+            for (int32_t j = a + sub; j < b; j += kHookLanes) hook_take(bk, bq, hook_key(delta[eid[j]], j == a), colval[j].x);
+#pragma unroll
+        for (int o = 1; o < kHookLanes; o <<= 1) {
+            const int64_t k = __shfl_xor_sync(0xffffffffu, bk, o);
+            const int32_t q = __shfl_xor_sync(0xffffffffu, bq, o);
+            hook_take(bk, bq, k, q);
+        }
+        if (sub == 0 && p < n && !heavy) hook[p] = b > a ? bq : (int32_t)p;
+    }
+}
+
+__global__ void __launch_bounds__(kBlock) k_hook_heavy(int32_t nh, const int32_t* __restrict__ hrow,
+                                                       const int32_t* __restrict__ row_ptr,
+                                                       const int2* __restrict__ colval, const int32_t* __restrict__ eid,
+                                                       const double* __restrict__ delta, int32_t* __restrict__ hook) {
+    __shared__ int64_t sk[kBlock / 32];
+    __shared__ int32_t sq[kBlock / 32];
+    for (int32_t h = blockIdx.x; h < nh; h += gridDim.x) {
+        const int32_t p = hrow[h], a = row_ptr[p], b = row_ptr[p + 1];
+        int64_t bk = INT64_MAX;
+        int32_t bq = INT32_MAX;
+        for (int32_t j = a + threadIdx.x; j < b; j += kBlock) hook_take(bk, bq, hook_key(delta[eid[j]], j == a), colval[j].x);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t k = __shfl_xor_sync(0xffffffffu, bk, o);
+            const int32_t q = __shfl_xor_sync(0xffffffffu, bq, o);
+            hook_take(bk, bq, k, q);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            sk[threadIdx.x >> 5] = bk;
+            sq[threadIdx.x >> 5] = bq;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kBlock / 32; ++w) hook_take(bk, bq, sk[w], sq[w]);
+            hook[p] = bq;
+        }
+        __syncthreads();
     }
 }
 
@@ -119,8 +179,14 @@ static sfg_status aggregate(sfg_ctx* ctx, const sfg_graph* L, const double* delt
     SFG_TRY(s.get(&minm, n));
     SFG_TRY(s.get(&first, n));
     SFG_TRY(s.get(&rank, (size_t)n + 1));
-    const int gn = grid_of(ctx, k_hook, n);
-    k_hook<<<gn, kBlock, 0, ctx->stream>>>(n, L->row_ptr, L->colval, L->eid, delta, hook); ++ctx->launches;
+    const int gn = grid_of(ctx, k_hook_forest, n);
+    SFG_TRY(sfg_heavy_prepare(ctx, L));
+    k_hook<<<grid_of(ctx, k_hook, (int64_t)n * kHookLanes), kBlock, 0, ctx->stream>>>(
+        n, L->hv_n > 0 ? SFG_HEAVY_ROW : INT32_MAX, L->row_ptr, L->colval, L->eid, delta, hook); ++ctx->launches;
+    if (L->hv_n > 0) {
+        k_hook_heavy<<<std::min(L->hv_n, 8 * ctx->num_sms), kBlock, 0, ctx->stream>>>(
+            L->hv_n, L->hv_rows, L->row_ptr, L->colval, L->eid, delta, hook); ++ctx->launches;
+    }
     k_hook_forest<<<gn, kBlock, 0, ctx->stream>>>(n, hook, root); ++ctx->launches;
     SFG_LAUNCH_CHECK(ctx, "k_hook");
     SFG_TRY(sfg_pointer_jump(ctx, n, root));
