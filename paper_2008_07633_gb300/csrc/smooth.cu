@@ -29,6 +29,15 @@ constexpr int kBlock = 256;
 struct JVariant { int tpi, minb; };
 constexpr JVariant kJVariants[] = {{1, 4}, {2, 4}, {4, 4}, {1, 3}, {2, 3}, {4, 3}};
 constexpr int kJNumVariants = 6, kJDefault = 1;
+// Untuned sweeps: rows of up to 8 lanes take one tile a turn, longer ones two (GB300, us a sweep, one /
+// two tiles: 2048^2 power grid K = 64 BF16 274 / 284, 128^3 grid K = 16 85 / 87, K = 32 129 / 129; 1000^2
+// power grid K = 64 FP32 140 / 124). Sweeps with statistics keep kJDefault: their sums are per CTA.
+__host__ __device__ constexpr int plain_variant(int lpr) { return lpr <= 8 ? 0 : kJDefault; }
+// Graphs with hub rows get kHubWaves CTAs a resident slot: their rows differ in length by hundreds, and
+// rows of one length tend to be neighbours (degree order), so CTAs that finish early must find more
+// (2^20-node Chung-Lu graph, K = 32, one wave / eight: 333 / 323 us on L_G, 186 / 154 on its forest,
+// 369 / 241 with two tiles a turn). Meshes lose 10-30% from the extra starts and keep one wave.
+constexpr int kHubWaves = 8;
 
 // Gaussian entries 2p and 2p+1 of the counter-based generator (see sfg.h): SplitMix64 output
 // p + 1 of the stream started in state splitmix64(seed), both Box-Muller branches in FP32 (logf,
@@ -965,21 +974,31 @@ struct Smoother {
 
     template <bool A, bool B>
     static void* kern() {
-        return (void*)k_jacobi<T, LPR, A, B, kJVariants[kJDefault].tpi, kJVariants[kJDefault].minb>;
+        constexpr int v = B ? kJDefault : plain_variant(LPR);
+        return (void*)k_jacobi<T, LPR, A, B, kJVariants[v].tpi, kJVariants[v].minb>;
     }
     static void* plain_kern(int v) {  // the tuned variants of the plain sweep
         switch (v) {
             case 0: return (void*)k_jacobi<T, LPR, false, false, 1, 4>;
+            case 1: return (void*)k_jacobi<T, LPR, false, false, 2, 4>;
             case 2: return (void*)k_jacobi<T, LPR, false, false, 4, 4>;
             case 3: return (void*)k_jacobi<T, LPR, false, false, 1, 3>;
             case 4: return (void*)k_jacobi<T, LPR, false, false, 2, 3>;
             case 5: return (void*)k_jacobi<T, LPR, false, false, 4, 3>;
-            default: return (void*)k_jacobi<T, LPR, false, false, 2, 4>;
+            default: return kern<false, false>();
         }
     }
 
+    // CTAs of a seeded block and of a sweep with statistics (one statistics slot each).
     static int grid_jacobi(sfg_ctx* ctx, int32_t n) {
-        return sfg_grid(ctx, kern<false, false>(), kBlock, 0, (int64_t)n * LPR);
+        return sfg_grid(ctx, plain_kern(kJDefault), kBlock, 0, (int64_t)n * LPR);
+    }
+
+    // CTAs of a sweep without statistics.
+    static int grid_plain(sfg_ctx* ctx, const void* k, const sfg_graph* L) {
+        const int64_t lanes = (int64_t)L->n * LPR;
+        const int g = sfg_grid(ctx, k, kBlock, 0, lanes);
+        return L->hv_n > 0 ? (int)std::min<int64_t>((int64_t)g * kHubWaves, (lanes + kBlock - 1) / kBlock) : g;
     }
 
     // Statistics slots a sweep of L with `grid` tile CTAs writes (the heavy rows add theirs).
@@ -995,14 +1014,9 @@ struct Smoother {
         const int32_t hmax = L->hv_n > 0 ? kHeavy : INT32_MAX;
         void* k = sub_mu ? (stats ? kern<true, true>() : kern<true, false>())
                          : (stats ? kern<false, true>() : kern<false, false>());
-        int g = grid;
-        if (!sub_mu && !stats) {  // the plain sweep takes the tuned tile shape, if any
-            const int v = sfg_tuned_variant(ctx, K, Vec<T>::E == 4 ? SFG_F32 : SFG_BF16, L);
-            if (v >= 0 && v != kJDefault) {
-                k = plain_kern(v);
-                g = sfg_grid(ctx, k, kBlock, 0, (int64_t)n * LPR);
-            }
-        }
+        if (!sub_mu && !stats)  // the plain sweep takes the tuned tile shape, if any
+            k = plain_kern(sfg_tuned_variant(ctx, K, Vec<T>::E == 4 ? SFG_F32 : SFG_BF16, L));
+        const int g = stats ? grid : grid_plain(ctx, k, L);
         void* args[] = {(void*)&n, (void*)&hmax, (void*)&L->row_ptr, (void*)&L->colval, (void*)&coef,
                         (void*)&a_self, (void*)&X, (void*)&Y, (void*)&mu, (void*)&part};
         sfg_tic(ctx, "jacobi");
@@ -1325,14 +1339,14 @@ struct Smoother {
         SFG_CUDA(ctx, cudaEventCreate(&e1));
         SFG_TRY(heavy_prepare(ctx, L));  // the tile kernel is timed as the sweep runs it
         const int32_t hmax = L->hv_n > 0 ? kHeavy : INT32_MAX;
-        int best = kJDefault;
+        int best = plain_variant(LPR);
         float best_ms = 1e30f;
         const float a_self = 0.3f;
         const float* mu = nullptr;
         double* pp = nullptr;
         for (int v = 0; v < kJNumVariants; ++v) {
             void* k = plain_kern(v);
-            const int g = sfg_grid(ctx, k, kBlock, 0, (int64_t)n * LPR);
+            const int g = grid_plain(ctx, k, L);
             const T* X = x;
             T* Y = y;
             void* args[] = {(void*)&n, (void*)&hmax, (void*)&L->row_ptr, (void*)&L->colval, (void*)&coef,
