@@ -3,100 +3,280 @@
 //
 // Each candidate becomes a unique 64-bit key: the order-preserving image of its FP32 score in the
 // high word and the complement of its id in the low word, so "larger key" is exactly the strict
-// order (score descending, id ascending). An MSB-first radix select (8 passes of 8-bit digits,
-// histogram in shared memory, the digit pick done on the device) finds the k-th largest key
-// without any host round trip; one compaction pass keeps the keys at or above it and a small
-// radix sort returns the chosen ids in ascending order.
+// order (score descending, id ascending). One cooperative launch does the whole selection (k_topk):
+// an MSB-first radix select finds the k-th largest key, the kept candidates are written in list
+// order, and they are sorted by id only when the list was not in id order already.
+#include "gridbar.cuh"
 #include "sfg_internal.cuh"
 
 namespace {
 
 constexpr int kBlock = 256;
 
-__device__ __forceinline__ uint64_t sel_key(float s, int32_t id) {
+__device__ __forceinline__ uint32_t score_bits(float s) {
     const uint32_t b = __float_as_uint(s);
-    const uint32_t o = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-    return ((uint64_t)o << 32) | (uint64_t)(~(uint32_t)id);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-struct SelState {
-    unsigned long long prefix;
-    long long krem;
-    unsigned long long hist[256];
+__device__ __forceinline__ uint64_t sel_key(float s, int32_t id) {
+    return ((uint64_t)score_bits(s) << 32) | (uint64_t)(~(uint32_t)id);
+}
+
+// ---- one list ----------------------------------------------------------------------------------
+// Bound by launches and, for long lists, by reading the scores: the digits are 11, 11 and 10 bits, so
+// three passes over the scores alone settle the threshold (the ids are read only when more
+// candidates tie at the threshold score than are wanted, and for the kept ones); every CTA picks the
+// digit from the global histogram itself, so a pass costs one barrier. Sixteen histogram and pick
+// launches, flags, scan, compaction and a four-digit radix sort of the ids took about 130 us more on a 64 x 64
+// grid (3,969 candidates) and 210 us more on the 128^3 grid (4.1M).
+constexpr int kTkPasses = 6, kTkBins = 2048, kTkUnroll = 8;
+__host__ __device__ constexpr int tk_shift(int pass) { return pass % 3 == 0 ? 21 : pass % 3 == 1 ? 10 : 0; }
+__host__ __device__ constexpr int tk_width(int pass) { return pass % 3 == 2 ? 10 : 11; }
+
+// Words of one launch: barrier count, error, ids out of order.
+enum { kTwBar, kTwErr, kTwOrder, kTwCount };
+
+struct TkArgs {
+    int64_t ne, k;
+    const float* scores;
+    const int32_t* ids;
+    unsigned long long* hist;   // kTkPasses x kTkBins, zero at launch
+    unsigned long long* words;  // zero at launch
+    unsigned* keep;             // one bit a candidate, written by the kernel from here on
+    long long* cta_kept;        // one count a CTA
+    unsigned* cnt;              // digit counts of the id sort, 256 x sort_ctas
+    int sort_ctas;
+    int32_t* tmp;               // k
+    int32_t* out;               // k
 };
 
-__global__ void k_sel_init(SelState* st, int64_t k) {
-    st->prefix = 0ull;
-    st->krem = k;
-    for (int d = threadIdx.x; d < 256; d += blockDim.x) st->hist[d] = 0ull;
-}
+struct TkPick {
+    int digit;
+    long long krem, in_bin;
+};
 
-__global__ void __launch_bounds__(kBlock)
-    k_sel_hist(int64_t ne, const float* __restrict__ scores, const int32_t* __restrict__ ids,
-               int shift, SelState* __restrict__ st) {
-    __shared__ unsigned int h[256];
-    h[threadIdx.x] = 0;
+// The digit that holds the krem-th largest candidate: bins from the top, thread t holds bins
+// [top - 8 t - 7, top - 8 t].
+__device__ __forceinline__ TkPick tk_pick(const unsigned long long* hist, int nb, long long krem) {
+    __shared__ long long ws[kBlock / 32];
+    __shared__ TkPick res;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int PER = kTkBins / kBlock;
+    long long c[PER], sum = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const int b = nb - 1 - (tid * PER + q);
+        c[q] = b >= 0 ? (long long)__ldcg(hist + b) : 0;
+        sum += c[q];
+    }
+    long long inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+    }
+    if (lane == 31) ws[warp] = inc;
+    if (tid == 0) res = TkPick{0, krem, 0};
     __syncthreads();
-    const uint64_t prefix = st->prefix;
-    const int hi = shift + 8;  // bits at and above `hi` must match the prefix
-    for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < ne;
-         i += (int64_t)gridDim.x * kBlock) {
-        const uint64_t key = sel_key(scores[i], ids[i]);
-        if (hi >= 64 || (key >> hi) == (prefix >> hi)) atomicAdd(&h[(key >> shift) & 0xff], 1u);
+    long long above = inc - sum;
+    for (int q = 0; q < warp; ++q) above += ws[q];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (above < krem && above + c[q] >= krem) res = TkPick{nb - 1 - (tid * PER + q), krem - above, c[q]};
+        above += c[q];
     }
     __syncthreads();
-    if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], (unsigned long long)h[threadIdx.x]);
-}
-
-// Pick the digit holding the k-th largest key: suffix sums over the 256 buckets by a block scan
-// (thread d holds bucket 255 - d), then the first bucket whose suffix reaches krem.
-__global__ void k_sel_pick(int shift, SelState* st) {
-    __shared__ long long suf[256];
-    const int d = 255 - (int)threadIdx.x;
-    const long long c = (long long)st->hist[d];
-    suf[threadIdx.x] = c;
+    const TkPick r = res;
     __syncthreads();
-    for (int o = 1; o < 256; o <<= 1) {  // inclusive scan from the top bucket down
-        const long long v = threadIdx.x >= o ? suf[threadIdx.x - o] : 0;
-        __syncthreads();
-        suf[threadIdx.x] += v;
-        __syncthreads();
+    return r;
+}
+
+// Exclusive scan of one int per thread over the CTA; total in *all.
+__device__ __forceinline__ int tk_scan(int v, int* all) {
+    __shared__ int ws[kBlock / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int q = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += q;
     }
-    const long long krem = st->krem;
-    const long long incl = suf[threadIdx.x], above = incl - c;
-    const bool pick = (above < krem && incl >= krem) || (d == 0 && incl < krem);
+    if (lane == 31) ws[warp] = inc;
     __syncthreads();
-    if (pick) {
-        st->prefix |= (unsigned long long)d << shift;
-        st->krem = krem - above;
+    int before = 0, tot = 0;
+#pragma unroll
+    for (int q = 0; q < kBlock / 32; ++q) {
+        if (q < warp) before += ws[q];
+        tot += ws[q];
     }
-    st->hist[d] = 0ull;
+    __syncthreads();
+    *all = tot;
+    return before + inc - v;
 }
 
-__global__ void k_sel_flags(int64_t ne, const float* __restrict__ scores,
-                            const int32_t* __restrict__ ids, const SelState* __restrict__ st,
-                            uint8_t* __restrict__ flag) {
-    const uint64_t thr = st->prefix;
-    for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < ne;
-         i += (int64_t)gridDim.x * kBlock)
-        flag[i] = sel_key(scores[i], ids[i]) >= thr;
-}
-
-__global__ void k_sel_compact(int64_t ne, const int32_t* __restrict__ ids,
-                              const uint8_t* __restrict__ flag, const int64_t* __restrict__ pos,
-                              uint64_t* __restrict__ out_keys, uint32_t* __restrict__ out_vals) {
-    for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < ne;
-         i += (int64_t)gridDim.x * kBlock)
-        if (flag[i]) {
-            out_keys[pos[i]] = (uint64_t)(uint32_t)ids[i];
-            out_vals[pos[i]] = 0u;
+// Stable sort of out[0, k) by id (as unsigned words): four 8-bit digits, CTA c of the first
+// sort_ctas owning one contiguous range.
+__device__ bool tk_sort_ids(const TkArgs& A, const GridBar& bar, unsigned& passed) {
+    __shared__ unsigned base[256], wcnt[kBlock / 32][256];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nc = A.sort_ctas;
+    const int64_t per = (A.k + nc - 1) / nc;
+    const int64_t lo = min(A.k, (int64_t)blockIdx.x * per), hi = min(A.k, lo + per);
+    const bool mine = (int)blockIdx.x < nc;
+    int32_t *from = A.out, *to = A.tmp;
+    for (int shift = 0; shift < 32; shift += 8) {
+        if (mine) {
+            base[tid] = 0;
+            __syncthreads();
+            for (int64_t i = lo + tid; i < hi; i += kBlock) atomicAdd(&base[((uint32_t)__ldcg(from + i) >> shift) & 0xff], 1u);
+            __syncthreads();
+            A.cnt[(size_t)tid * nc + blockIdx.x] = base[tid];
         }
+        if (!grid_barrier(bar, passed)) return false;
+        if (mine) {
+            // first place of digit tid in this CTA's range: smaller digits, then earlier CTAs
+            unsigned total = 0, before = 0;
+            for (int c = 0; c < nc; ++c) {
+                const unsigned v = __ldcg(A.cnt + (size_t)tid * nc + c);
+                if (c < (int)blockIdx.x) before += v;
+                total += v;
+            }
+            int all;
+            const int first = tk_scan((int)total, &all);
+            base[tid] = (unsigned)first + before;
+            for (int64_t t0 = lo; t0 < hi; t0 += kBlock) {
+#pragma unroll
+                for (int q = 0; q < kBlock / 32; ++q) wcnt[q][tid] = 0;
+                __syncthreads();
+                const int64_t i = t0 + tid;
+                const bool ok = i < hi;
+                const uint32_t x = ok ? (uint32_t)__ldcg(from + i) : 0u;
+                const int d = ok ? (int)((x >> shift) & 0xff) : 256;
+                const unsigned peers = __match_any_sync(0xffffffffu, d);
+                const int rank = __popc(peers & ((1u << lane) - 1u));
+                if (ok && rank == 0) wcnt[warp][d] = __popc(peers);
+                __syncthreads();
+                if (ok) {
+                    unsigned p = base[d] + rank;
+                    for (int q = 0; q < warp; ++q) p += wcnt[q][d];
+                    to[p] = (int32_t)x;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < kBlock / 32; ++q) base[tid] += wcnt[q][tid];
+                __syncthreads();
+            }
+        }
+        if (!grid_barrier(bar, passed)) return false;
+        int32_t* t = from;
+        from = to;
+        to = t;
+    }
+    return true;  // an even number of passes: the result is in out
 }
 
-__global__ void k_sel_emit(int64_t k, const uint64_t* __restrict__ keys, int32_t* __restrict__ out) {
-    for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < k;
-         i += (int64_t)gridDim.x * kBlock)
-        out[i] = (int32_t)keys[i];
+// A barrier ran out: no selection; every CTA leaves -1 in its share of the list.
+__device__ void tk_give_up(const TkArgs& A) {
+    for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < A.k; i += (int64_t)gridDim.x * kBlock)
+        A.out[i] = -1;
+}
+
+__global__ void __launch_bounds__(kBlock, 4) k_topk(TkArgs A) {
+    __shared__ unsigned h[kTkBins];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t t0 = (int64_t)blockIdx.x * kBlock + tid, nt = (int64_t)gridDim.x * kBlock;
+    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kTwBar), reinterpret_cast<int*>(A.words + kTwErr)};
+    unsigned passed = 0;
+    long long krem = A.k;
+    uint32_t word[2] = {0u, 0u};  // the threshold key's score image and complemented id
+    for (int pass = 0; pass < kTkPasses; ++pass) {
+        const int shift = tk_shift(pass), nb = 1 << tk_width(pass);
+        const uint32_t digit_mask = (uint32_t)nb - 1u;
+        const uint32_t prefix = word[pass / 3];
+        const int up = shift + tk_width(pass);  // bits at and above `up` match the prefix
+        for (int b = tid; b < nb; b += kBlock) h[b] = 0;
+        __syncthreads();
+        for (int64_t i0 = t0; i0 < A.ne; i0 += nt * kTkUnroll) {
+            float sc[kTkUnroll];
+#pragma unroll
+            for (int q = 0; q < kTkUnroll; ++q) {
+                const int64_t i = i0 + q * nt;
+                sc[q] = i < A.ne ? A.scores[i] : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < kTkUnroll; ++q) {
+                const int64_t i = i0 + q * nt;
+                if (i >= A.ne) break;
+                uint32_t x = score_bits(sc[q]);
+                if (pass >= 3) {
+                    if (x != word[0]) continue;
+                    x = ~(uint32_t)A.ids[i];
+                }
+                if (up == 32 || (x >> up) == (prefix >> up)) atomicAdd(&h[(x >> shift) & digit_mask], 1u);
+            }
+        }
+        __syncthreads();
+        unsigned long long* gh = A.hist + (size_t)pass * kTkBins;
+        for (int b = tid; b < nb; b += kBlock)
+            if (h[b]) atomicAdd(gh + b, (unsigned long long)h[b]);
+        if (!grid_barrier(bar, passed)) return tk_give_up(A);
+        const TkPick p = tk_pick(gh, nb, krem);
+        word[pass / 3] |= (uint32_t)p.digit << shift;
+        krem = p.krem;
+        if (pass == 2 && p.in_bin == krem) break;  // every candidate at the threshold score is wanted
+    }
+    const uint64_t thr = ((uint64_t)word[0] << 32) | word[1];
+    // kept bits and counts of this CTA's contiguous range of 32-candidate words
+    const int64_t nwords = (A.ne + 31) / 32, per = (nwords + gridDim.x - 1) / gridDim.x;
+    const int64_t w0 = min(nwords, (int64_t)blockIdx.x * per), w1 = min(nwords, w0 + per);
+    int kept = 0;
+    for (int64_t w = w0 + (tid >> 5); w < w1; w += kBlock / 32) {
+        const int64_t i = w * 32 + lane;
+        bool take = false;
+        if (i < A.ne) {
+            const uint32_t x = score_bits(A.scores[i]);
+            take = x > word[0] || (x == word[0] && (word[1] == 0u || sel_key(A.scores[i], A.ids[i]) >= thr));
+        }
+        const unsigned bits = __ballot_sync(0xffffffffu, take);
+        if (lane == 0) A.keep[w] = bits;
+        kept += __popc(bits);
+    }
+    int all;
+    tk_scan(lane == 0 ? kept : 0, &all);
+    if (tid == 0) A.cta_kept[blockIdx.x] = all;
+    if (!grid_barrier(bar, passed)) return tk_give_up(A);
+    __shared__ long long s_before;
+    if (tid == 0) s_before = 0;
+    __syncthreads();
+    {
+        long long b = 0;
+        for (int c = tid; c < (int)blockIdx.x; c += kBlock) b += __ldcg(A.cta_kept + c);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+        if (lane == 0 && b) atomicAdd((unsigned long long*)&s_before, (unsigned long long)b);
+    }
+    __syncthreads();
+    int64_t at = s_before;
+    for (int64_t wb = w0; wb < w1; wb += kBlock) {
+        const int64_t w = wb + tid;
+        unsigned bits = w < w1 ? __ldcg(A.keep + w) : 0u;
+        int64_t p = at + tk_scan(__popc(bits), &all);
+        at += all;
+        while (bits) {
+            const int b = __ffs(bits) - 1;
+            bits &= bits - 1;
+            if (p < A.k) A.out[p] = A.ids[w * 32 + b];
+            ++p;
+        }
+    }
+    if (!grid_barrier(bar, passed)) return tk_give_up(A);
+    bool wrong = false;
+    for (int64_t i = t0; i + 1 < A.k; i += nt)
+        wrong |= (uint32_t)__ldcg(A.out + i) > (uint32_t)__ldcg(A.out + i + 1);
+    if (wrong) atomicExch((unsigned long long*)(A.words + kTwOrder), 1ull);
+    if (!grid_barrier(bar, passed)) return tk_give_up(A);
+    if (*(volatile unsigned long long*)(A.words + kTwOrder) != 0ull && !tk_sort_ids(A, bar, passed))
+        tk_give_up(A);
 }
 
 }  // namespace
@@ -104,36 +284,34 @@ __global__ void k_sel_emit(int64_t k, const uint64_t* __restrict__ keys, int32_t
 sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, int64_t ne,
                          int64_t k, int32_t* out) {
     if (k == 0) return SFG_OK;
+    // at least 1,024 candidates a CTA: fewer CTAs make the barriers cheaper
+    const int grid = sfg_grid(ctx, (const void*)k_topk, kBlock, 0, (ne + 3) / 4);
+    const int sort_ctas = (int)std::min<int64_t>(grid, (k + 4095) / 4096);
     Scratch s(ctx);
-    SelState* st;
-    uint8_t* flag;
-    int64_t* pos;
-    uint64_t *ka, *kb;
-    uint32_t *va, *vb;
-    SFG_TRY(s.get(&st, 1));
-    SFG_TRY(s.get(&flag, ne));
-    SFG_TRY(s.get(&pos, ne + 1));
-    SFG_TRY(s.get(&ka, k));
-    SFG_TRY(s.get(&kb, k));
-    SFG_TRY(s.get(&va, k));
-    SFG_TRY(s.get(&vb, k));
-    const int grid = sfg_grid(ctx, (const void*)k_sel_hist, kBlock, 0, ne);
+    TkArgs a{};
+    unsigned long long* zeroed;  // histograms, then the words
+    SFG_TRY(s.get(&zeroed, (size_t)kTkPasses * kTkBins + kTwCount));
+    SFG_TRY(s.get(&a.keep, (size_t)(ne + 31) / 32));
+    SFG_TRY(s.get(&a.cta_kept, grid));
+    SFG_TRY(s.get(&a.cnt, (size_t)256 * sort_ctas));
+    SFG_TRY(s.get(&a.tmp, k));
+    SFG_CUDA(ctx, cudaMemsetAsync(zeroed, 0, sizeof(unsigned long long) * ((size_t)kTkPasses * kTkBins + kTwCount),
+                                  ctx->stream));
+    a.ne = ne;
+    a.k = k;
+    a.scores = scores;
+    a.ids = ids;
+    a.hist = zeroed;
+    a.words = zeroed + (size_t)kTkPasses * kTkBins;
+    a.sort_ctas = sort_ctas;
+    a.out = out;
+    void* args[] = {(void*)&a};
     sfg_tic(ctx, "topk");
-    k_sel_init<<<1, kBlock, 0, ctx->stream>>>(st, k); ++ctx->launches;
-    for (int shift = 56; shift >= 0; shift -= 8) {
-        k_sel_hist<<<grid, kBlock, 0, ctx->stream>>>(ne, scores, ids, shift, st); ++ctx->launches;
-        k_sel_pick<<<1, 256, 0, ctx->stream>>>(shift, st); ++ctx->launches;
-    }
-    k_sel_flags<<<grid, kBlock, 0, ctx->stream>>>(ne, scores, ids, st, flag); ++ctx->launches;
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_topk, dim3(grid), dim3(kBlock), args, 0,
+                                                      ctx->stream);
     sfg_toc(ctx);
-    SFG_LAUNCH_CHECK(ctx, "k_sel");
-    SFG_TRY(sfg_scan_u8(ctx, flag, pos, ne));
-    k_sel_compact<<<grid, kBlock, 0, ctx->stream>>>(ne, ids, flag, pos, ka, va); ++ctx->launches;
-    SFG_LAUNCH_CHECK(ctx, "k_sel_compact");
-    SFG_TRY(sfg_radix_sort_pairs(ctx, &ka, &va, &kb, &vb, k, 32));
-    k_sel_emit<<<sfg_grid(ctx, (const void*)k_sel_emit, kBlock, 0, k), kBlock, 0, ctx->stream>>>(
-        k, ka, out); ++ctx->launches;
-    SFG_LAUNCH_CHECK(ctx, "k_sel_emit");
+    if (e != cudaSuccess) return sfg_cuda_fail(ctx, e, "k_topk");
+    ++ctx->launches;
     return SFG_OK;
 }
 
