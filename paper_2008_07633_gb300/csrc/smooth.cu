@@ -17,6 +17,7 @@
 // The first sweep also removes the initial column means (A-form sweeps map a constant column to
 // itself, so J(X - 1 mu^T) = J(X) - 1 mu^T), and the last sweep accumulates the column sums and
 // sums of squares the projection needs, so neither costs an extra pass over the block.
+#include "gridbar.cuh"
 #include "sfg_internal.cuh"
 #include "vec.cuh"
 
@@ -97,12 +98,10 @@ __device__ __forceinline__ void block_column_partials(float (&s1)[E], float (&s2
 // the block free of a constant that the final projection would otherwise have to cancel in FP32;
 // the two choices differ by a constant vector only, which the projection removes either way.
 template <typename T, int LPR, bool WEIGHTED>
-__global__ void __launch_bounds__(kBlock) k_init(int32_t n, uint64_t seed, const double* __restrict__ deg,
-                                                 T* __restrict__ X, double* __restrict__ part) {
+__device__ __forceinline__ void init_rows(int32_t n, uint64_t seed, const double* deg, int64_t g0, int64_t ng,
+                                          T* X, double* part) {
     constexpr int E = Vec<T>::E, K = LPR * E;
     const int lane = threadIdx.x & 31, sub = lane % LPR;
-    const int64_t g0 = ((int64_t)blockIdx.x * kBlock + threadIdx.x) / LPR;
-    const int64_t ng = (int64_t)gridDim.x * kBlock / LPR;
     float s1[E], s2[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) s1[e] = s2[e] = 0.f;
@@ -129,6 +128,13 @@ __global__ void __launch_bounds__(kBlock) k_init(int32_t n, uint64_t seed, const
         Vec<T>::store(X + row * K + sub * E, x);
     }
     block_column_partials<LPR, E>(s1, s2, part);
+}
+
+template <typename T, int LPR, bool WEIGHTED>
+__global__ void __launch_bounds__(kBlock) k_init(int32_t n, uint64_t seed, const double* __restrict__ deg,
+                                                 T* __restrict__ X, double* __restrict__ part) {
+    init_rows<T, LPR, WEIGHTED>(n, seed, deg, ((int64_t)blockIdx.x * kBlock + threadIdx.x) / LPR,
+                                (int64_t)gridDim.x * kBlock / LPR, X, part);
 }
 
 template <typename V>
@@ -734,12 +740,9 @@ __global__ void __launch_bounds__(kBlock) k_col_stats(int32_t n, const T* __rest
 // blocks, then a fixed-shape tree, so the result does not depend on scheduling.
 // proj = 0: mean only (mu = S1 / n). proj = 1: mean and scale = 1 / RMS of the centred column
 // (1 if the column is zero). proj = 2: D-weighted mean S1 / S2 of k_init<WEIGHTED>.
-__global__ void __launch_bounds__(kBlock) k_finalize(const double* __restrict__ part, int nblocks,
-                                                     int K, int32_t n, int proj,
-                                                     float* __restrict__ mean,
-                                                     float* __restrict__ scale) {
+__device__ __forceinline__ void finalize_column(const double* part, int nblocks, int K, int k, int32_t n,
+                                                int proj, float* mean, float* scale) {
     __shared__ double r1[kBlock], r2[kBlock];
-    const int k = blockIdx.x;
     double s1 = 0.0, s2 = 0.0;
     for (int b = threadIdx.x; b < nblocks; b += kBlock) {
         s1 += part[(size_t)b * 2 * K + k];
@@ -770,6 +773,13 @@ __global__ void __launch_bounds__(kBlock) k_finalize(const double* __restrict__ 
     }
 }
 
+__global__ void __launch_bounds__(kBlock) k_finalize(const double* __restrict__ part, int nblocks,
+                                                     int K, int32_t n, int proj,
+                                                     float* __restrict__ mean,
+                                                     float* __restrict__ scale) {
+    finalize_column(part, nblocks, K, blockIdx.x, n, proj, mean, scale);
+}
+
 template <typename T, int LPR>
 __global__ void __launch_bounds__(kBlock) k_project(int32_t n, const T* __restrict__ X,
                                                     T* __restrict__ Y, const float* __restrict__ mean,
@@ -794,6 +804,149 @@ __global__ void k_coef(int32_t n, const double* __restrict__ invdeg, double omeg
     for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < n;
          p += (int64_t)gridDim.x * kBlock)
         coef[p] = (float)(omega * invdeg[p]);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Small graphs: the whole embedding in one cooperative launch. A sweep of a block whose lane groups
+// all fit on the chip at once takes 2-3 us, of which one gather round is work and the rest is the
+// end of one launch and the start of the next; here every warp keeps its tile's rows and first
+// entries in registers, and a barrier over the grid (gridbar.cuh) separates the sweeps. L_G and L_P
+// are swept side by side by the two halves of the grid. Rows, statistics slots and orders of
+// summation are those of k_init, k_jacobi (default shape) and k_finalize, so the bits are theirs.
+// Taken when both halves are resident together (see small_fits) and no row is a hub row: beyond
+// that the separate launches overlap their ends well enough. Filter + score + select of a 17,280-node
+// mesh (K = 16, 15 steps): 192 us with separate launches, 113 us so.
+// ------------------------------------------------------------------------------------------------
+template <typename T>
+struct SmallArgs {
+    int32_t n;
+    int grid;       // CTAs of one side; the launch has sides * grid
+    int sides;      // 2: filter (L_G, L_P); 1: smooth (projected into out)
+    int steps;      // >= 1
+    double omega;
+    uint64_t seed;
+    const double* deg;            // of L_G: weights of the first mean
+    const int32_t* row_ptr[2];
+    const int2* colval[2];
+    const double* invdeg[2];
+    T* x0;                        // written by the kernel from here on
+    T* buf[2][2];
+    T* out;
+    double* part;                 // sides * grid slots
+    float* mu;
+    float* mean[2];
+    float* scale[2];
+    unsigned* words;              // barrier count and error, zero at launch
+};
+
+template <typename T, int LPR>
+__global__ void __launch_bounds__(kBlock, 4) k_small(SmallArgs<T> A) {
+    constexpr int E = Vec<T>::E, K = LPR * E, GPW = 32 / LPR, C = Chunk<LPR>::C;
+    const int lane = threadIdx.x & 31, grp = lane / LPR, sub = lane % LPR;
+    const unsigned gm = group_mask<LPR>(lane);
+    const int side = (int)blockIdx.x >= A.grid ? 1 : 0, cta = (int)blockIdx.x - side * A.grid;
+    const int32_t wid = (int32_t)((cta * kBlock + threadIdx.x) >> 5);
+    const int32_t ntiles = (A.n + GPW - 1) / GPW;
+    const GridBar bar{A.words, reinterpret_cast<int*>(A.words + 1)};
+    unsigned passed = 0;
+    const int32_t* row_ptr = A.row_ptr[side];
+    const int2* colval = A.colval[side];
+    auto give_up = [&] {  // a barrier ran out: the scales, and with them every result, become NaN
+        for (int k = threadIdx.x; k < K; k += kBlock) A.scale[side][k] = __int_as_float(0x7fffffff);
+    };
+    // this group's row in tile t
+    struct Row { int32_t r, a, b; float cp; };
+    auto load_row = [&](int32_t t) {
+        Row w{t * GPW + grp, 0, 0, 0.f};
+        if (t < ntiles && w.r < A.n) {
+            w.a = row_ptr[w.r];
+            w.b = row_ptr[w.r + 1];
+            w.cp = (float)(A.omega * A.invdeg[side][w.r]);
+        }
+        return w;
+    };
+    Row row = load_row(wid);
+    Chunk<LPR> ch;
+    ch.load(colval, row.a, row.b, min(row.r, A.n - 1), sub);
+    if (side == 0)
+        init_rows<T, LPR, true>(A.n, A.seed, A.deg, ((int64_t)cta * kBlock + threadIdx.x) / LPR,
+                                (int64_t)A.grid * kBlock / LPR, A.x0, A.part);
+    if (!grid_barrier(bar, passed)) return give_up();
+    if (side == 0)
+        for (int k = cta; k < K; k += A.grid) {
+            finalize_column(A.part, A.grid, K, k, A.n, 2, A.mu, nullptr);
+            __syncthreads();
+        }
+    if (!grid_barrier(bar, passed)) return give_up();
+    const float a_self = (float)(1.0 - A.omega);
+    float s1[E], s2[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) s1[e] = s2[e] = 0.f;
+    auto tile = [&](const Row& w, const Chunk<LPR>& c, const T* X, T* Y, bool sub_mu, bool stats) {
+        const bool live = w.r < A.n;
+        const int32_t self = live ? w.r : 0, deg = w.b - w.a;
+        const int32_t maxdeg = __reduce_max_sync(0xffffffffu, deg);
+        const T* Xl = X + sub * E;
+        float acc[E];
+        const uint4 xr = Vec<T>::load_raw(Xl + (int64_t)self * K);
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[e] = 0.f;
+        gather_chunk<T, LPR>(c, min(maxdeg, C), gm, Xl, acc);
+        for (int32_t j0 = C; j0 < maxdeg; j0 += C) {
+            Chunk<LPR> cx;
+            cx.load(colval, w.a + j0, w.b, self, sub);
+            gather_chunk<T, LPR>(cx, min(maxdeg - j0, C), gm, Xl, acc);
+        }
+        if (!live) return;
+        float xs[E], y[E];
+        Vec<T>::unpack(xr, xs);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            y[e] = deg > 0 ? fmaf(w.cp, acc[e], a_self * xs[e]) : xs[e];
+            if (sub_mu) y[e] = y[e] - A.mu[sub * E + e];
+        }
+        Vec<T>::store(Y + (int64_t)w.r * K + sub * E, y);
+        if (stats)
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const float q = Vec<T>::round(y[e]);
+                s1[e] += q;
+                s2[e] = fmaf(q, q, s2[e]);
+            }
+    };
+    const T* cur = A.x0;
+    for (int t = 1; t < A.steps; ++t) {
+        T* nxt = A.buf[side][(t - 1) & 1];
+        tile(row, ch, cur, nxt, t == 1, false);
+        if (!grid_barrier(bar, passed)) return give_up();
+        cur = nxt;
+    }
+    // the last sweep with its statistics, in the tile order of k_jacobi's default shape
+    T* last = A.buf[side][(A.steps - 1) & 1];
+    constexpr int TPI = kJVariants[kJDefault].tpi;
+    for (int q = 0; q < TPI; ++q) {
+        const int32_t t = wid * TPI + q;
+        if (t >= ntiles) break;
+        const Row w = load_row(t);
+        Chunk<LPR> c;
+        c.load(colval, w.a, w.b, min(w.r, A.n - 1), sub);
+        tile(w, c, cur, last, A.steps == 1, true);
+    }
+    block_column_partials<LPR, E>(s1, s2, A.part);
+    if (!grid_barrier(bar, passed)) return give_up();
+    for (int k = cta; k < K; k += A.grid) {
+        finalize_column(A.part + (size_t)side * A.grid * 2 * K, A.grid, K, k, A.n, 1, A.mean[side], A.scale[side]);
+        __syncthreads();
+    }
+    if (A.sides == 2) return;
+    if (!grid_barrier(bar, passed)) return give_up();
+    if (row.r < A.n) {
+        float x[E];
+        Vec<T>::load(last + (int64_t)row.r * K + sub * E, x);
+#pragma unroll
+        for (int e = 0; e < E; ++e) x[e] = (x[e] - A.mean[0][sub * E + e]) * A.scale[0][sub * E + e];
+        Vec<T>::store(A.out + (int64_t)row.r * K + sub * E, x);
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1001,6 +1154,26 @@ struct Smoother {
         return L->hv_n > 0 ? (int)std::min<int64_t>((int64_t)g * kHubWaves, (lanes + kBlock - 1) / kBlock) : g;
     }
 
+    // Whether `sides` copies of one side's grid are resident at once, with one tile a warp and no hub rows.
+    static bool small_fits(sfg_ctx* ctx, int sides, int steps, int grid, const sfg_graph* LG, const sfg_graph* LP) {
+        if (steps < 1 || (int64_t)grid * kBlock < (int64_t)LG->n * LPR) return false;
+        if (LG->hv_n != 0 || (LP && LP->hv_n != 0)) return false;
+        const int64_t lanes = (int64_t)sides * grid * kBlock;
+        return sfg_grid(ctx, (const void*)k_small<T, LPR>, kBlock, 0, lanes) == sides * grid;
+    }
+
+    static sfg_status launch_small(sfg_ctx* ctx, SmallArgs<T>& a) {
+        void* args[] = {(void*)&a};
+        SFG_CUDA(ctx, cudaMemsetAsync(a.words, 0, 2 * sizeof(unsigned), ctx->stream));
+        sfg_tic(ctx, "small");
+        const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_small<T, LPR>, dim3(a.sides * a.grid),
+                                                          dim3(kBlock), args, 0, ctx->stream);
+        sfg_toc(ctx);
+        if (e != cudaSuccess) return sfg_cuda_fail(ctx, e, "k_small");
+        ++ctx->launches;
+        return SFG_OK;
+    }
+
     // Statistics slots a sweep of L with `grid` tile CTAs writes (the heavy rows add theirs).
     static int part_slots(const sfg_graph* L, int grid) {
         return grid + (L->hv_n > 0 ? kHeavyGrid : 0);
@@ -1059,10 +1232,21 @@ struct Smoother {
         float *coef, *mu, *scale;
         double* part;
         SFG_TRY(s.get(&buf, (size_t)n * K));
-        SFG_TRY(s.get(&coef, (size_t)n));
         SFG_TRY(s.get(&mu, K));
         SFG_TRY(s.get(&scale, K));
         SFG_TRY(s.get(&part, (size_t)(grid + kHeavyGrid) * 2 * K));
+        SFG_TRY(heavy_prepare(ctx, L));
+        if (small_fits(ctx, 1, steps, grid, L, nullptr)) {
+            SmallArgs<T> a{};
+            SFG_TRY(s.get(&a.words, 2));
+            SFG_TRY(s.get(&a.mean[0], K));
+            a.n = n, a.grid = grid, a.sides = 1, a.steps = steps, a.omega = omega, a.seed = seed;
+            a.deg = L->deg, a.row_ptr[0] = L->row_ptr, a.colval[0] = L->colval, a.invdeg[0] = L->invdeg;
+            a.x0 = buf, a.buf[0][0] = X_out, a.buf[0][1] = buf, a.out = X_out;
+            a.part = part, a.mu = mu, a.scale[0] = scale;
+            return launch_small(ctx, a);
+        }
+        SFG_TRY(s.get(&coef, (size_t)n));
         k_coef<<<sfg_grid(ctx, (const void*)k_coef, kBlock, 0, n), kBlock, 0, ctx->stream>>>(
             n, L->invdeg, omega, coef); ++ctx->launches;
         SFG_LAUNCH_CHECK(ctx, "k_coef");
@@ -1226,6 +1410,26 @@ struct Smoother {
         SFG_TRY(s.get(&sg, K));
         SFG_TRY(s.get(&mp, K));
         SFG_TRY(s.get(&sp, K));
+        SFG_TRY(heavy_prepare(ctx, LG));
+        SFG_TRY(heavy_prepare(ctx, LP));
+        if (small_fits(ctx, 2, steps, grid, LG, LP)) {
+            SmallArgs<T> a{};
+            SFG_TRY(s.get(&a.words, 2));
+            SFG_TRY(s.get(&a.part, (size_t)2 * grid * 2 * K));
+            a.n = n, a.grid = grid, a.sides = 2, a.steps = steps, a.omega = omega, a.seed = seed;
+            a.deg = LG->deg, a.x0 = x0, a.mu = mu;
+            const sfg_graph* L[2] = {LG, LP};
+            T* b[2][2] = {{g0, g1}, {p0, p1}};
+            float *m[2] = {mg, mp}, *sc[2] = {sg, sp};
+            for (int q = 0; q < 2; ++q) {
+                a.row_ptr[q] = L[q]->row_ptr, a.colval[q] = L[q]->colval, a.invdeg[q] = L[q]->invdeg;
+                a.buf[q][0] = b[q][0], a.buf[q][1] = b[q][1], a.mean[q] = m[q], a.scale[q] = sc[q];
+            }
+            SFG_TRY(launch_small(ctx, a));
+            const int l = (steps - 1) & 1;
+            return sfg_score_impl(ctx, LG, b[0][l], b[1][l], K, Vec<T>::E == 4 ? SFG_F32 : SFG_BF16, ids, ne,
+                                  mode, scores, sg, sp);
+        }
         SFG_TRY(s.get(&part, (size_t)(grid + kHeavyGrid) * 2 * K));
         sfg_tic(ctx, "init");
         // the D-weighted mean is taken on L_G; L_P has the same nodes, and any constant left in
