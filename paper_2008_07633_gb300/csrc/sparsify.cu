@@ -22,7 +22,7 @@ __global__ void k_f32_to_bf16(int64_t n, const float* __restrict__ x, __nv_bfloa
 __global__ void k_set_mask(int64_t k, const int32_t* __restrict__ ids, uint8_t* __restrict__ mask) {
     for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < k;
          i += (int64_t)gridDim.x * kBlock)
-        mask[ids[i]] = 1;
+        if (ids[i] >= 0) mask[ids[i]] = 1;  // -1: the selection gave up
 }
 
 // Smoother choice and its omega range: weighted Jacobi (0, 1], Gauss-Seidel / SOR (0, 2).
