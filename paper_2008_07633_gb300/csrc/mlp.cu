@@ -168,23 +168,25 @@ __global__ void __launch_bounds__(128, 6) k_mlp_forward_tc(const float* __restri
     uint32_t phase = 0;
     bool ok = true;
     const int64_t ntiles = (ne + 127) / 128;
-    // this thread's feature row of the next tile, loaded one tile ahead so that the global
+    // this thread's feature pieces of the next tile, loaded one tile ahead so that the global
     // latency overlaps the current tile's MMAs
     float4 f[4];
+    // four lanes a row: each load instruction reads 512 consecutive bytes (one lane a row and 64 bytes
+    // between lanes cost four times the L1 cycles, which bound the inference kernel)
+    const int frow = warp * 32 + ((tid & 31) >> 2), fcol = (tid & 3) * 4;
     auto load_row = [&](int64_t tile) {
-        const float4* xr = reinterpret_cast<const float4*>(x + min(tile * 128 + tid, ne - 1) * kF);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) f[c] = xr[c];
+        for (int c = 0; c < 4; ++c)
+            f[c] = *reinterpret_cast<const float4*>(x + min(tile * 128 + frow + 8 * c, ne - 1) * kF + fcol);
     };
     if ((int64_t)blockIdx.x < ntiles) load_row(blockIdx.x);
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t row = tile * 128 + tid;
         // features -> BF16 in chunk 0 (the previous tile's layer 2 has completed)
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-            *reinterpret_cast<uint4*>(&sA[core_idx<kKA>(tid, 8 * c)]) =
-                make_uint4(pack_bf16(f[2 * c].x, f[2 * c].y), pack_bf16(f[2 * c].z, f[2 * c].w),
-                           pack_bf16(f[2 * c + 1].x, f[2 * c + 1].y), pack_bf16(f[2 * c + 1].z, f[2 * c + 1].w));
+        for (int c = 0; c < 4; ++c)
+            *reinterpret_cast<uint2*>(&sA[core_idx<kKA>(frow + 8 * c, fcol)]) =
+                make_uint2(pack_bf16(f[c].x, f[c].y), pack_bf16(f[c].z, f[c].w));
         if (tile + gridDim.x < ntiles) load_row(tile + gridDim.x);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_sync();  // also orders the previous tile's TMEM reads before this tile's MMAs
@@ -363,10 +365,13 @@ __global__ void __launch_bounds__(128, 2)
     float gb3 = 0.f, sse = 0.f;
     const int64_t ntiles = (ne + 127) / 128;
     float4 f[4];
+    // four lanes a row: each load instruction reads 512 consecutive bytes (one lane a row and 64 bytes
+    // between lanes cost four times the L1 cycles, which bound the inference kernel)
+    const int frow = warp * 32 + ((tid & 31) >> 2), fcol = (tid & 3) * 4;
     auto load_row = [&](int64_t tile) {
-        const float4* xr = reinterpret_cast<const float4*>(x + min(tile * 128 + tid, ne - 1) * kF);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) f[c] = xr[c];
+        for (int c = 0; c < 4; ++c)
+            f[c] = *reinterpret_cast<const float4*>(x + min(tile * 128 + frow + 8 * c, ne - 1) * kF + fcol);
     };
     auto step = [&](auto&& issue) {  // one MMA group: issue, commit, bounded wait (CTA-wide)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -388,10 +393,9 @@ __global__ void __launch_bounds__(128, 2)
         const float tgt = valid ? target[row] : 0.f;
         // features -> BF16 at columns 64-79 (the previous tile's gradient product has completed)
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-            *reinterpret_cast<uint4*>(&sA[core_idx<kTA>(tid, 64 + 8 * c)]) =
-                make_uint4(pack_bf16(f[2 * c].x, f[2 * c].y), pack_bf16(f[2 * c].z, f[2 * c].w),
-                           pack_bf16(f[2 * c + 1].x, f[2 * c + 1].y), pack_bf16(f[2 * c + 1].z, f[2 * c + 1].w));
+        for (int c = 0; c < 4; ++c)
+            *reinterpret_cast<uint2*>(&sA[core_idx<kTA>(frow + 8 * c, 64 + fcol)]) =
+                make_uint2(pack_bf16(f[c].x, f[c].y), pack_bf16(f[c].z, f[c].w));
         if (tile + gridDim.x < ntiles) load_row(tile + gridDim.x);
         // layer 1: [X | 1] [W1; b1]
         if (!step([&] {
@@ -714,8 +718,10 @@ sfg_status sfg_mlp_check_impl(sfg_ctx* ctx, const sfg_mlp* net) {
 
 // Read back the loss and the error word that k_mlp_fold wrote side by side: one copy, one wait.
 static sfg_status mlp_read_loss(sfg_ctx* ctx, const sfg_mlp* net, const double* loss2, double* loss_host) {
-    double h[2] = {0.0, 0.0};
-    SFG_CUDA(ctx, cudaMemcpyAsync(h, loss2, sizeof h, cudaMemcpyDeviceToHost, ctx->stream));
+    int* hw = nullptr;
+    SFG_TRY(sfg_host_word(ctx, kSfgHostBuild, &hw));  // pinned: no staging copy
+    double* h = reinterpret_cast<double*>(hw);
+    SFG_CUDA(ctx, cudaMemcpyAsync(h, loss2, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     *loss_host = h[0];
     return h[1] != 0.0 ? sfg_mlp_check_impl(ctx, net) : SFG_OK;  // reports and clears the word
