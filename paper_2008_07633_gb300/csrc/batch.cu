@@ -113,12 +113,6 @@ __global__ void k_seg_count(int64_t m, const uint8_t* __restrict__ mask, int ng,
     }
 }
 
-__global__ void k_mark(int64_t k, const int32_t* __restrict__ ids, uint8_t* __restrict__ mask) {
-    for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < k;
-         i += (int64_t)gridDim.x * kBlock)
-        mask[ids[i]] = 1;
-}
-
 __global__ void k_split(int64_t m, const uint8_t* __restrict__ mask, int ng,
                         const int64_t* __restrict__ eoff, uint8_t* const* __restrict__ outs) {
     for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m;
@@ -509,20 +503,15 @@ static sfg_status batch_run(sfg_ctx* ctx, const sfg_batch* b, uint64_t seed, uin
     }
     if (b->k_total == 0) return SFG_OK;
     Scratch s(ctx);
-    int32_t* sel;
     float* scores;
     SFG_TRY(s.get(&scores, b->ncand));
-    SFG_TRY(s.get(&sel, b->k_total));
     const sfg_params& P = b->P;
     SFG_TRY(sfg_filter_score_batched_impl(ctx, b->U, b->PU, b->orig_local, b->ng, b->d_noff, P.K,
                                           P.steps, P.omega, seed, P.storage, b->cand, b->ncand,
                                           P.mode, scores));
     // selection under original edge ids (ties and the output order as without the reordering)
-    SFG_TRY(sfg_topk_segmented_impl(ctx, scores, b->cand_orig ? b->cand_orig : b->cand, b->ncand,
-                                    b->ng, b->d_coff, b->d_k, b->k_total, sel));
-    k_mark<<<grid_of(ctx, k_mark, b->k_total), kBlock, 0, ctx->stream>>>(b->k_total, sel, mask);
-    ++ctx->launches;
-    SFG_LAUNCH_CHECK(ctx, "k_mark");
+    SFG_TRY(sfg_topk_segmented_mark(ctx, scores, b->cand_orig ? b->cand_orig : b->cand, b->ncand,
+                                    b->ng, b->d_coff, b->d_k, mask));
     return SFG_OK;
 }
 

@@ -330,16 +330,39 @@ extern "C" sfg_status sfg_select_topk(sfg_ctx* ctx, const float* scores, const i
 }
 
 // ------------------------------------------------------------------------------------------------
-// Segmented top-k (one selection per graph of a batch): the same MSB-first radix select, with one
-// histogram and one (prefix, remaining k) state per segment. Candidates are contiguous per
-// segment; each warp sweeps one contiguous range of them, 32 at a time, so its segment (found once
-// by a binary search) advances by a few steps at most and its state stays in registers.
+// Segmented top-k (one selection per graph of a batch): the same MSB-first radix select with one
+// histogram and one state per segment, in one cooperative launch. Candidates are contiguous per
+// segment and each CTA owns one contiguous range of them, so its shared histogram serves a segment at
+// a time; the digits have 9 bits (2 KB of histogram a segment). The chosen candidates' mask entries
+// are set directly, which needs no order. On 5.9M candidates of 64 graphs this takes 170 us less than
+// sixteen histogram and pick launches, flags, a scan, a compaction and a marking pass (250 us of kernels).
 // ------------------------------------------------------------------------------------------------
 namespace {
 
+constexpr int kSgBits = 9, kSgBins = 1 << kSgBits, kSgPasses = 8;  // four digits of the score, four of the id
+__host__ __device__ constexpr int sg_shift(int pass) { return pass % 4 == 3 ? 0 : 32 - kSgBits * (pass % 4 + 1); }
+__host__ __device__ constexpr int sg_width(int pass) { return pass % 4 == 3 ? 32 - 3 * kSgBits : kSgBits; }
+
 struct SegSel {
-    unsigned long long prefix;
+    uint32_t word[2];  // threshold key so far: score image, complemented id
+    int32_t wanted;    // 0: the segment keeps nothing
+    int32_t open;      // id digits still needed
     long long krem;
+};
+
+enum { kSwBar, kSwErr, kSwOpen, kSwCount };
+
+struct SegArgs {
+    int64_t ne;
+    const float* scores;
+    const int32_t* ids;
+    int nseg;
+    const int64_t* off;
+    const int64_t* k;
+    SegSel* st;                 // written by the kernel from here on
+    unsigned* hist;             // nseg x kSgBins, zero at launch
+    unsigned long long* words;  // zero at launch
+    uint8_t* mask;
 };
 
 __device__ __forceinline__ int seg_of(const int64_t* __restrict__ off, int nseg, int64_t i) {
@@ -351,143 +374,130 @@ __device__ __forceinline__ int seg_of(const int64_t* __restrict__ off, int nseg,
     return lo;
 }
 
-__global__ void k_segsel_init(int nseg, const int64_t* __restrict__ k, SegSel* __restrict__ st,
-                              unsigned long long* __restrict__ hist) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)nseg * 256;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        hist[i] = 0ull;
-        if ((i & 255) == 0) st[i >> 8] = SegSel{0ull, (long long)k[i >> 8]};
-    }
-}
-
-// The contiguous item range [lo, hi) of this warp: ne split into equal chunks of whole 32-item steps.
-__device__ __forceinline__ void warp_range(int64_t ne, int64_t& lo, int64_t& hi) {
-    const int64_t nw = (int64_t)gridDim.x * (kBlock / 32);
-    const int64_t w = ((int64_t)blockIdx.x * kBlock + threadIdx.x) >> 5;
-    const int64_t steps = (ne + 31) / 32, per = (steps + nw - 1) / nw;
-    lo = min(ne, w * per * 32);
-    hi = min(ne, (w + 1) * per * 32);
-}
-
-__global__ void __launch_bounds__(kBlock)
-    k_segsel_hist(int64_t ne, const float* __restrict__ scores, const int32_t* __restrict__ ids,
-                  int nseg, const int64_t* __restrict__ off, const SegSel* __restrict__ st,
-                  int shift, unsigned long long* __restrict__ hist) {
-    const int hi = shift + 8;
-    int64_t lo_i, hi_i;
-    warp_range(ne, lo_i, hi_i);
-    if (lo_i >= hi_i) return;
-    int s = seg_of(off, nseg, lo_i);  // this lane's segment, advanced as the range moves on
-    int64_t s_end = off[s + 1];
-    SegSel ss = st[s];
-    for (int64_t base = lo_i; base < hi_i; base += 32) {
-        const int64_t i = base + (threadIdx.x & 31);
-        bool take = false;
-        int digit = 0;
-        if (i < hi_i) {
-            if (i >= s_end) {
-                do ++s; while (off[s + 1] <= i);
-                s_end = off[s + 1];
-                ss = st[s];
+__global__ void __launch_bounds__(kBlock, 4) k_topk_seg(SegArgs A) {
+    __shared__ unsigned h[kSgBins];
+    __shared__ long long ws[kBlock / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kSwBar), reinterpret_cast<int*>(A.words + kSwErr)};
+    unsigned passed = 0;
+    const int64_t per = (A.ne + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = min(A.ne, (int64_t)blockIdx.x * per), hi = min(A.ne, lo + per);
+    const int s0 = lo < hi ? seg_of(A.off, A.nseg, lo) : A.nseg;
+    for (int64_t s = (int64_t)blockIdx.x * kBlock + tid; s < A.nseg; s += (int64_t)gridDim.x * kBlock)
+        A.st[s] = SegSel{{0u, 0u}, A.k[s] > 0 ? 1 : 0, 0, (long long)A.k[s]};
+    if (!grid_barrier(bar, passed)) return;
+    for (int pass = 0; pass < kSgPasses; ++pass) {
+        const int shift = sg_shift(pass), nb = 1 << sg_width(pass), up = shift + sg_width(pass), which = pass / 4;
+        for (int s = s0; s < A.nseg && A.off[s] < hi; ++s) {
+            const int64_t a = max(lo, A.off[s]), b = min(hi, A.off[s + 1]);
+            const SegSel st = A.st[s];
+            if (a >= b || !st.wanted || (which && !st.open)) continue;  // the same for the whole CTA
+            for (int d = tid; d < nb; d += kBlock) h[d] = 0;
+            __syncthreads();
+            const uint32_t prefix = st.word[which];
+            for (int64_t i0 = a + tid; i0 < b; i0 += kBlock * 4) {
+                float sc[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) sc[q] = i0 + q * kBlock < b ? A.scores[i0 + q * kBlock] : 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (i0 + q * kBlock >= b) break;
+                    uint32_t x = score_bits(sc[q]);
+                    if (which) {
+                        if (x != st.word[0]) continue;
+                        x = ~(uint32_t)A.ids[i0 + q * kBlock];
+                    }
+                    if (up == 32 || (x >> up) == (prefix >> up)) atomicAdd(&h[(x >> shift) & (uint32_t)(nb - 1)], 1u);
+                }
             }
-            const uint64_t key = sel_key(scores[i], ids[i]);
-            take = ss.krem > 0 && (hi >= 64 || (key >> hi) == (ss.prefix >> hi));
-            digit = (int)((key >> shift) & 0xff);
+            __syncthreads();
+            for (int d = tid; d < nb; d += kBlock)
+                if (h[d]) atomicAdd(A.hist + (size_t)s * kSgBins + d, h[d]);
+            __syncthreads();
         }
-        const unsigned bin = take ? (unsigned)s * 256u + (unsigned)digit : 0xffffffffu;
-        const unsigned peers = __match_any_sync(0xffffffffu, bin);
-        if (take && (__ffs(peers) - 1) == (int)(threadIdx.x & 31))
-            atomicAdd(&hist[bin], (unsigned long long)__popc(peers));
-    }
-}
-
-// one CTA of 256 threads per segment (see k_sel_pick)
-__global__ void k_segsel_pick(int shift, SegSel* __restrict__ st, unsigned long long* __restrict__ hist) {
-    __shared__ long long suf[256];
-    const int sgi = blockIdx.x;
-    unsigned long long* h = hist + (size_t)sgi * 256;
-    const long long krem = st[sgi].krem;
-    const int d = 255 - (int)threadIdx.x;
-    const long long c = (long long)h[d];
-    suf[threadIdx.x] = c;
-    __syncthreads();
-    for (int o = 1; o < 256; o <<= 1) {
-        const long long v = threadIdx.x >= o ? suf[threadIdx.x - o] : 0;
-        __syncthreads();
-        suf[threadIdx.x] += v;
-        __syncthreads();
-    }
-    const long long incl = suf[threadIdx.x], above = incl - c;
-    const bool pick = krem > 0 && ((above < krem && incl >= krem) || (d == 0 && incl < krem));
-    __syncthreads();
-    if (pick) {
-        st[sgi].prefix |= (unsigned long long)d << shift;
-        st[sgi].krem = krem - above;
-    }
-    h[d] = 0ull;
-}
-
-__global__ void __launch_bounds__(kBlock)
-    k_segsel_flags(int64_t ne, const float* __restrict__ scores, const int32_t* __restrict__ ids,
-                   int nseg, const int64_t* __restrict__ off, const SegSel* __restrict__ st,
-                   const int64_t* __restrict__ k, uint8_t* __restrict__ flag) {
-    int64_t lo_i, hi_i;
-    warp_range(ne, lo_i, hi_i);
-    if (lo_i >= hi_i) return;
-    int s = seg_of(off, nseg, lo_i);
-    int64_t s_end = off[s + 1];
-    bool on = k[s] > 0;
-    uint64_t thr = st[s].prefix;
-    for (int64_t i = lo_i + (threadIdx.x & 31); i < hi_i; i += 32) {
-        if (i >= s_end) {
-            do ++s; while (off[s + 1] <= i);
-            s_end = off[s + 1];
-            on = k[s] > 0;
-            thr = st[s].prefix;
+        if (!grid_barrier(bar, passed)) return;
+        // picks, a CTA a segment: thread t holds the bins nb - 1 - 2t and nb - 2 - 2t, from the top
+        for (int s = blockIdx.x; s < A.nseg; s += gridDim.x) {
+            const SegSel st = A.st[s];
+            if (!st.wanted || (which && !st.open)) continue;
+            unsigned* gh = A.hist + (size_t)s * kSgBins;
+            long long c[2], sum = 0;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int d = nb - 1 - (2 * tid + q);
+                c[q] = d >= 0 ? (long long)__ldcg(gh + d) : 0;
+                if (d >= 0) gh[d] = 0u;
+                sum += c[q];
+            }
+            long long inc = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += v;
+            }
+            if (lane == 31) ws[warp] = inc;
+            __syncthreads();
+            long long above = inc - sum;
+            for (int q = 0; q < warp; ++q) above += ws[q];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (above < st.krem && above + c[q] >= st.krem) {
+                    SegSel nx = st;
+                    nx.word[which] |= (uint32_t)(nb - 1 - (2 * tid + q)) << shift;
+                    nx.krem = st.krem - above;
+                    if (pass == 3 && c[q] > nx.krem) {  // more candidates at the threshold score than wanted
+                        nx.open = 1;
+                        atomicExch(A.words + kSwOpen, 1ull);
+                    }
+                    A.st[s] = nx;
+                }
+                above += c[q];
+            }
+            __syncthreads();
         }
-        flag[i] = on && sel_key(scores[i], ids[i]) >= thr;
+        if (!grid_barrier(bar, passed)) return;
+        if (pass == 3 && *(volatile unsigned long long*)(A.words + kSwOpen) == 0ull) break;
     }
-}
-
-__global__ void k_segsel_emit(int64_t ne, const int32_t* __restrict__ ids,
-                              const uint8_t* __restrict__ flag, const int64_t* __restrict__ pos,
-                              int32_t* __restrict__ out) {
-    for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < ne;
-         i += (int64_t)gridDim.x * kBlock)
-        if (flag[i]) out[pos[i]] = ids[i];
+    for (int s = s0; s < A.nseg && A.off[s] < hi; ++s) {
+        const int64_t a = max(lo, A.off[s]), b = min(hi, A.off[s + 1]);
+        const SegSel st = A.st[s];
+        if (!st.wanted) continue;
+        for (int64_t i = a + tid; i < b; i += kBlock) {
+            const uint32_t x = score_bits(A.scores[i]);
+            if (x < st.word[0]) continue;
+            const int32_t id = A.ids[i];
+            if (x > st.word[0] || ~(uint32_t)id >= st.word[1]) A.mask[id] = 1;
+        }
+    }
 }
 
 }  // namespace
 
-sfg_status sfg_topk_segmented_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids,
+sfg_status sfg_topk_segmented_mark(sfg_ctx* ctx, const float* scores, const int32_t* ids,
                                    int64_t ne, int nseg, const int64_t* seg_off,
-                                   const int64_t* k_dev, int64_t k_total, int32_t* out) {
-    if (k_total == 0 || ne == 0) return SFG_OK;
+                                   const int64_t* k_dev, uint8_t* mask) {
+    if (ne == 0 || nseg == 0) return SFG_OK;
     Scratch s(ctx);
-    SegSel* st;
-    unsigned long long* hist;
-    uint8_t* flag;
-    int64_t* pos;
-    SFG_TRY(s.get(&st, nseg));
-    SFG_TRY(s.get(&hist, (size_t)nseg * 256));
-    SFG_TRY(s.get(&flag, ne));
-    SFG_TRY(s.get(&pos, ne + 1));
-    const int grid = sfg_grid(ctx, (const void*)k_segsel_hist, kBlock, 0, ne);
+    SegArgs a{};
+    SFG_TRY(s.get(&a.st, nseg));
+    SFG_TRY(s.get(&a.words, kSwCount));
+    SFG_TRY(s.get(&a.hist, (size_t)nseg * kSgBins));
+    SFG_CUDA(ctx, cudaMemsetAsync(a.words, 0, sizeof(unsigned long long) * kSwCount, ctx->stream));
+    SFG_CUDA(ctx, cudaMemsetAsync(a.hist, 0, sizeof(unsigned) * (size_t)nseg * kSgBins, ctx->stream));
+    a.ne = ne;
+    a.scores = scores;
+    a.ids = ids;
+    a.nseg = nseg;
+    a.off = seg_off;
+    a.k = k_dev;
+    a.mask = mask;
+    void* args[] = {(void*)&a};
+    const int grid = sfg_grid(ctx, (const void*)k_topk_seg, kBlock, 0, (ne + 3) / 4);
     sfg_tic(ctx, "topk");
-    k_segsel_init<<<ceil_div_u((int64_t)nseg * 256, kBlock), kBlock, 0, ctx->stream>>>(nseg, k_dev, st, hist);
-    ++ctx->launches;
-    for (int shift = 56; shift >= 0; shift -= 8) {
-        k_segsel_hist<<<grid, kBlock, 0, ctx->stream>>>(ne, scores, ids, nseg, seg_off, st, shift, hist);
-        k_segsel_pick<<<nseg, 256, 0, ctx->stream>>>(shift, st, hist);
-        ctx->launches += 2;
-    }
-    k_segsel_flags<<<grid, kBlock, 0, ctx->stream>>>(ne, scores, ids, nseg, seg_off, st, k_dev, flag);
-    ++ctx->launches;
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_topk_seg, dim3(grid), dim3(kBlock), args, 0,
+                                                      ctx->stream);
     sfg_toc(ctx);
-    SFG_LAUNCH_CHECK(ctx, "k_segsel");
-    SFG_TRY(sfg_scan_u8(ctx, flag, pos, ne));
-    k_segsel_emit<<<grid, kBlock, 0, ctx->stream>>>(ne, ids, flag, pos, out);
+    if (e != cudaSuccess) return sfg_cuda_fail(ctx, e, "k_topk_seg");
     ++ctx->launches;
-    SFG_LAUNCH_CHECK(ctx, "k_segsel_emit");
     return SFG_OK;
 }

@@ -219,11 +219,11 @@ sfg_status sfg_filter_score_batched_impl(sfg_ctx* ctx, const sfg_graph* U, const
                                          double omega, uint64_t seed, sfg_dtype storage,
                                          const int32_t* ids, int64_t ne, sfg_score_mode mode,
                                          float* scores);
-// Top-k per segment: candidates [seg_off[s], seg_off[s+1]) of segment s keep their k_dev[s]
-// largest; the chosen ids of all segments are written in ascending order (out has sum k entries).
-sfg_status sfg_topk_segmented_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids,
+// Top-k per segment: of the candidates [seg_off[s], seg_off[s+1]) of segment s the k_dev[s] largest
+// get mask[id] = 1.
+sfg_status sfg_topk_segmented_mark(sfg_ctx* ctx, const float* scores, const int32_t* ids,
                                    int64_t ne, int nseg, const int64_t* seg_off,
-                                   const int64_t* k_dev, int64_t k_total, int32_t* out);
+                                   const int64_t* k_dev, uint8_t* mask);
 typedef struct sfg_mlp sfg_mlp;
 sfg_status sfg_mlp_forward_impl(sfg_ctx* ctx, const sfg_mlp* net, const float* feats, int64_t ne,
                                 float* out);
