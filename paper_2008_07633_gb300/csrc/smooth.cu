@@ -19,6 +19,7 @@
 // sums of squares the projection needs, so neither costs an extra pass over the block.
 #include "gridbar.cuh"
 #include "sfg_internal.cuh"
+#include "dot64.cuh"
 #include "vec.cuh"
 
 namespace {
@@ -991,10 +992,13 @@ __global__ void __launch_bounds__(kBlock) k_init_batched(int32_t n, uint64_t see
 
 // Per-graph column sums and sums of squares (FP64) of X. Every graph's rows are cut into
 // kSegSlices equal contiguous slices, one CTA per (graph, slice): each LPR-lane group folds 64-row
-// chunks in FP32 (the chunk's rows loaded 8 at a time, accumulated in row order) into FP64, then a
-// fixed-shape tree across the CTA gives the slice's partials; k_seg_reduce adds a graph's slices in
+// chunks in FP32 (the chunk's rows loaded 8 at a time, accumulated in row order) into FP64, the groups'
+// sums are added in a fixed order through shared memory, and k_seg_finalize adds a graph's slices in
 // slice order. The partition does not depend on the launch, so the sums are deterministic.
 // deg != NULL: sums of d_i x_ik and of d_i instead (the D-weighted means, see k_init).
+// The FP64 pipe takes 16 clocks a warp instruction whatever lanes are active, and folding the lanes by
+// shuffles made it the bound: 54 us for 1.25M rows of 16 FP32, about 45 with full warps adding columns
+// and integer widening.
 constexpr int kSegSlices = 32;
 
 template <typename T, int LPR>
@@ -1002,16 +1006,18 @@ __global__ void __launch_bounds__(kBlock) k_seg_stats(const T* __restrict__ X,
                                                       const int32_t* __restrict__ node_off,
                                                       const double* __restrict__ deg,
                                                       double* __restrict__ part) {
-    constexpr int E = Vec<T>::E, K = LPR * E, GPB = kBlock / LPR, NB = 8;
-    __shared__ double red[kBlock / 32][2 * K];
+    constexpr int E = Vec<T>::E, K = LPR * E, GPB = kBlock / LPR, NB = 8, COLS = 2 * K, WAYS = kBlock / COLS;
+    __shared__ double sd[GPB][COLS];
+    __shared__ double sw[WAYS][COLS];
     const int g = blockIdx.x / kSegSlices, q = blockIdx.x % kSegSlices;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % LPR;
+    const int sub = threadIdx.x % LPR, grp = threadIdx.x / LPR;
     const int64_t g0 = node_off[g], rows = node_off[g + 1] - g0;
     const int64_t r0 = g0 + rows * q / kSegSlices, r1 = g0 + rows * (q + 1) / kSegSlices;
     double d1[E], d2[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) d1[e] = d2[e] = 0.0;
-    for (int64_t base = r0 + threadIdx.x / LPR; base < r1; base += (int64_t)GPB * 64) {
+    bool first = true;
+    for (int64_t base = r0 + grp; base < r1; base += (int64_t)GPB * 64) {
         float f1[E], f2[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) f1[e] = f2[e] = 0.f;
@@ -1040,55 +1046,49 @@ __global__ void __launch_bounds__(kBlock) k_seg_stats(const T* __restrict__ X,
                 }
             }
         }
+        double w1[E], w2[E];
+        widen_vec<E>(f1, w1);
+        widen_vec<E>(f2, w2);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            d1[e] += f1[e];
-            d2[e] += f2[e];
+            d1[e] = first ? w1[e] : d1[e] + w1[e];
+            d2[e] = first ? w2[e] : d2[e] + w2[e];
         }
+        first = false;
     }
 #pragma unroll
-    for (int o = LPR; o < 32; o <<= 1)
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            d1[e] += __shfl_xor_sync(0xffffffffu, d1[e], o);
-            d2[e] += __shfl_xor_sync(0xffffffffu, d2[e], o);
-        }
-    if (lane < LPR)
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            red[warp][sub * E + e] = d1[e];
-            red[warp][K + sub * E + e] = d2[e];
-        }
+    for (int e = 0; e < E; ++e) {
+        sd[grp][sub * E + e] = d1[e];
+        sd[grp][K + sub * E + e] = d2[e];
+    }
     __syncthreads();
-    for (int t = threadIdx.x; t < 2 * K; t += kBlock) {
-        double acc = 0.0;
-#pragma unroll
-        for (int w = 0; w < kBlock / 32; ++w) acc += red[w][t];
-        part[(size_t)blockIdx.x * 2 * K + t] = acc;
+    const int col = threadIdx.x % COLS, way = threadIdx.x / COLS;
+    double acc = 0.0;
+    for (int h = way; h < GPB; h += WAYS) acc += sd[h][col];
+    sw[way][col] = acc;
+    __syncthreads();
+    if (way == 0) {
+        for (int w = 1; w < WAYS; ++w) acc += sw[w][col];
+        part[(size_t)blockIdx.x * COLS + col] = acc;
     }
 }
 
-// stats[g][t] = sum over the slices of graph g, in slice order, of their partials
-__global__ void k_seg_reduce(int ng, int K2, const double* __restrict__ part,
-                             double* __restrict__ stats) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)ng * K2) return;
-    const int64_t g = i / K2, t = i % K2;
-    double acc = 0.0;
-    for (int q = 0; q < kSegSlices; ++q) acc += part[((size_t)g * kSegSlices + q) * K2 + t];
-    stats[i] = acc;
-}
-
-// mean[g][k], scale[g][k] (scale = 1 / RMS of the centred column, 1 if zero) from the stats.
+// mean[g][k], scale[g][k] (scale = 1 / RMS of the centred column, 1 if zero) from the slices' sums.
 // weighted: mean = s1 / s2 of k_seg_stats with degrees (no scale).
-__global__ void k_seg_finalize(const double* __restrict__ stats, const int32_t* __restrict__ node_off,
+__global__ void k_seg_finalize(const double* __restrict__ part, const int32_t* __restrict__ node_off,
                                int ng, int K, int weighted, float* __restrict__ mean,
                                float* __restrict__ scale) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)ng * K) return;
     const int g = (int)(i / K), k = (int)(i % K);
     const double n = (double)(node_off[g + 1] - node_off[g]);
-    const double s1 = stats[(size_t)g * 2 * K + k], s2 = stats[(size_t)g * 2 * K + K + k];
+    double s1 = 0.0, s2 = 0.0;
+#pragma unroll 8
+    for (int q = 0; q < kSegSlices; ++q) {
+        const double* p = part + ((size_t)g * kSegSlices + q) * 2 * K;
+        s1 += p[k];
+        s2 += p[K + k];
+    }
     if (weighted) {
         mean[i] = s2 > 0.0 ? (float)(s1 / s2) : 0.f;
         return;
@@ -1466,7 +1466,6 @@ struct Smoother {
         Scratch s(ctx);
         T *x0, *g0, *g1, *p0, *p1;
         float *coef, *mean, *sg, *sp;
-        double* stats;
         SFG_TRY(s.get(&x0, (size_t)n * K));
         SFG_TRY(s.get(&g0, (size_t)n * K));
         SFG_TRY(s.get(&g1, (size_t)n * K));
@@ -1476,20 +1475,17 @@ struct Smoother {
         SFG_TRY(s.get(&mean, (size_t)ng * K));
         SFG_TRY(s.get(&sg, (size_t)ng * K));
         SFG_TRY(s.get(&sp, (size_t)ng * K));
-        SFG_TRY(s.get(&stats, (size_t)ng * 2 * K));
         double* spart;
         SFG_TRY(s.get(&spart, (size_t)ng * kSegSlices * 2 * K));
-        const unsigned fin_grid = ceil_div_u((int64_t)ng * K, kBlock);
-        const unsigned red_grid = ceil_div_u((int64_t)ng * 2 * K, kBlock);
+        const unsigned fin_grid = ceil_div_u((int64_t)ng * K, 64);
         auto seg_stats = [&](const T* X, const double* deg) {
             k_seg_stats<T, LPR><<<ng * kSegSlices, kBlock, 0, ctx->stream>>>(X, node_off, deg, spart);
-            k_seg_reduce<<<red_grid, kBlock, 0, ctx->stream>>>(ng, 2 * K, spart, stats);
-            ctx->launches += 2;
+            ++ctx->launches;
         };
         k_init_batched<T, LPR><<<grid, kBlock, 0, ctx->stream>>>(n, seed, node_off, ng, orig_local, x0);
         const bool weighted = steps > 0;
         seg_stats(x0, weighted ? U->deg : nullptr);
-        k_seg_finalize<<<fin_grid, kBlock, 0, ctx->stream>>>(stats, node_off, ng, K, weighted ? 1 : 0,
+        k_seg_finalize<<<fin_grid, 64, 0, ctx->stream>>>(spart, node_off, ng, K, weighted ? 1 : 0,
                                                              mean, nullptr);
         k_center_batched<T, LPR><<<grid, kBlock, 0, ctx->stream>>>(n, node_off, ng, mean, x0);
         ctx->launches += 3;
@@ -1513,7 +1509,7 @@ struct Smoother {
             }
             xr[w] = cur;
             seg_stats(cur, nullptr);
-            k_seg_finalize<<<fin_grid, kBlock, 0, ctx->stream>>>(stats, node_off, ng, K, 0, mean, sc[w]);
+            k_seg_finalize<<<fin_grid, 64, 0, ctx->stream>>>(spart, node_off, ng, K, 0, mean, sc[w]);
             ++ctx->launches;
             SFG_LAUNCH_CHECK(ctx, "k_seg_stats");
         }
