@@ -8,6 +8,7 @@
 // kernel, so no selection ever sees a colour written in the same round). Selected nodes are
 // never adjacent, so the colouring is deterministic and proper.
 #include "sfg_internal.cuh"
+#include "dot64.cuh"
 
 namespace {
 
@@ -99,22 +100,26 @@ __global__ void k_color_bounds(int32_t n, int32_t ncolors, const uint64_t* __res
 // converges to the constant (y . x0) / (y . 1); removing that y-weighted mean first keeps the
 // block free of a constant the final projection would otherwise cancel in FP32.
 // One thread per row (rows of meshes and k-NN graphs are short, and eight-lane groups measured
-// slower there); rows longer than SFG_HEAVY_ROW are left to k_gs_weights_heavy.
+// slower there); rows longer than SFG_HEAVY_ROW are left to k_gs_weights_heavy. d_p is the row's
+// degree, summed in the same order when the graph was built; the FP64 pipe (two lanes a clock) bounds
+// the rest, so the weights are widened by integer moves (dot64.cuh).
 __global__ void k_gs_weights(int32_t n, const int32_t* __restrict__ row_ptr,
                              const int2* __restrict__ colval, const int32_t* __restrict__ color,
-                             double omega, double* __restrict__ y) {
+                             const double* __restrict__ deg, double omega, double* __restrict__ y) {
     for (int64_t p = blockIdx.x * (int64_t)256 + threadIdx.x; p < n; p += (int64_t)gridDim.x * 256) {
         const int32_t a = row_ptr[p], b = row_ptr[p + 1];
         if (b - a > SFG_HEAVY_ROW) continue;
         const int32_t cp = color[p];
-        double d = 0.0, later = 0.0;
+        double later = 0.0;
         for (int32_t j = a; j < b; ++j) {
-            const int32_t q = colval[j].x;
-            const double w = (double)__int_as_float(colval[j].y);
-            d += w;
-            if (color[q] > cp || (color[q] == cp && q > (int32_t)p)) later += w;
+            const int2 cv = colval[j];
+            const int32_t cq = color[cv.x];
+            if (cq > cp || (cq == cp && cv.x > (int32_t)p)) {
+                const float w = __int_as_float(cv.y);
+                later += is_normal32(w) ? widen_normal(w) : (double)w;
+            }
         }
-        y[p] = d - omega * later;
+        y[p] = deg[p] - omega * later;
     }
 }
 

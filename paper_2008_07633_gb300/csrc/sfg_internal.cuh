@@ -283,7 +283,7 @@ sfg_status sfg_gs_inherit(sfg_ctx* ctx, const sfg_graph* P, const sfg_graph* G);
 // quantity y^T x that the colour-ordered SOR sweep conserves (color.cu).
 __global__ void k_gs_weights(int32_t n, const int32_t* __restrict__ row_ptr,
                              const int2* __restrict__ colval, const int32_t* __restrict__ color,
-                             double omega, double* __restrict__ y);
+                             const double* __restrict__ deg, double omega, double* __restrict__ y);
 __global__ void k_gs_weights_heavy(int32_t nh, const int32_t* __restrict__ hrow,
                                    const int32_t* __restrict__ row_ptr, const int2* __restrict__ colval,
                                    const int32_t* __restrict__ color, double omega, double* __restrict__ y);

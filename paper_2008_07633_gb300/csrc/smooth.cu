@@ -543,8 +543,11 @@ sfg_status heavy_prepare(sfg_ctx* ctx, const sfg_graph* Lc) {
 // Gauss-Seidel): rows[0, cnt) are pairwise non-adjacent, so each is updated in place from the
 // current values of its neighbours, x_p <- (1 - omega) x_p + (omega / D(p,p)) (A x)_p, which is the
 // sequential sweep restricted to this class. Same group layout and gathers as the Jacobi sweep;
-// the tile's rows come from the class list, one tile at a time. X is read and written through
-// plain pointers (rows of this class are written, only rows of other classes are gathered).
+// the tile's rows come from the class list. X is read and written through plain pointers (rows of this
+// class are written, only rows of other classes are gathered). A tile is a chain of four dependent
+// loads (row id -> bounds -> entries -> neighbour rows); while one tile gathers, the next one's entries
+// and the row ids of the one after are on their way, so one gather round is exposed (128 x 128 x 64 mesh,
+// K = 32: 32 us a class one tile at a time, about 26 so).
 template <typename T, int LPR>
 __global__ void __launch_bounds__(kBlock, 4)
     k_gs(int32_t cnt, const int32_t* __restrict__ rows, const int32_t* __restrict__ row_ptr,
@@ -557,45 +560,69 @@ __global__ void __launch_bounds__(kBlock, 4)
     const int32_t nw = (int32_t)(gridDim.x * (kBlock / 32));
     const int32_t ntiles = (cnt + GPW - 1) / GPW;
     const T* Xl = X + sub * E;
-    for (int32_t t = wid; t < ntiles; t += nw) {
+    // lane l < GPW: row l of a tile, its bounds and coefficient
+    struct Meta { int32_t r, lo, hi; float cf; };
+    auto load_rows = [&](int32_t t) -> int32_t {
         const int32_t i = t * GPW + lane;
-        int32_t r = -1, lo = 0, hi = 0;
-        float cf = 0.f;
-        if (lane < GPW && i < cnt) {
-            r = rows[i];
-            lo = row_ptr[r];
-            hi = row_ptr[r + 1];
-            cf = coef[r];
-            if (hi - lo > hmax) hi = lo - 1;  // updated by the heavy-row kernels of this class
+        return t < ntiles && lane < GPW && i < cnt ? rows[i] : -1;
+    };
+    auto load_meta = [&](int32_t r) {
+        Meta m{r, 0, 0, 0.f};
+        if (r >= 0) {
+            m.lo = row_ptr[r];
+            m.hi = row_ptr[r + 1];
+            m.cf = coef[r];
         }
-        const int32_t row = __shfl_sync(0xffffffffu, r, grp);
-        const int32_t a = __shfl_sync(0xffffffffu, lo, grp);
-        const int32_t b = __shfl_sync(0xffffffffu, hi, grp);
-        const float cp = __shfl_sync(0xffffffffu, cf, grp);
-        const bool live = row >= 0;
-        const int32_t first = __shfl_sync(0xffffffffu, r, 0);  // all lanes: the tile's first row
-        const int32_t self = live ? row : first;
-        const int32_t deg = b - a;
+        return m;
+    };
+    // this group's row; b < a: a heavy row, updated by the heavy-row kernels of this class
+    struct Row { int32_t row, self, a, b; float cp; };
+    auto own = [&](const Meta& m) {
+        Row w;
+        w.row = __shfl_sync(0xffffffffu, m.r, grp);
+        w.a = __shfl_sync(0xffffffffu, m.lo, grp);
+        w.b = __shfl_sync(0xffffffffu, m.hi, grp);
+        w.cp = __shfl_sync(0xffffffffu, m.cf, grp);
+        if (w.b - w.a > hmax) w.b = w.a - 1;
+        const int32_t first = __shfl_sync(0xffffffffu, m.r, 0);  // the tile's first row
+        w.self = w.row >= 0 ? w.row : max(first, 0);
+        return w;
+    };
+    int32_t t = wid;
+    if (t >= ntiles) return;
+    Row cur = own(load_meta(load_rows(t)));
+    Chunk<LPR> ch;
+    ch.load(colval, cur.a, cur.b, cur.self, sub);
+    Meta m1 = load_meta(load_rows(t + nw));
+    while (t < ntiles) {
+        const Row nxt = own(m1);
+        Chunk<LPR> ch1;
+        ch1.load(colval, nxt.a, nxt.b, nxt.self, sub);
+        const int32_t r2 = load_rows(t + 2 * nw);
+        const int32_t deg = cur.b - cur.a;
         const int32_t maxdeg = __reduce_max_sync(0xffffffffu, deg);
-        Chunk<LPR> ch;
-        ch.load(colval, a, b, self, sub);
+        T* xp = X + (int64_t)cur.self * K + sub * E;
+        const uint4 xr = Vec<T>::load_raw(xp);
         float acc[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) acc[e] = 0.f;
         gather_chunk<T, LPR>(ch, min(maxdeg, C), gm, Xl, acc);
         for (int32_t j0 = C; j0 < maxdeg; j0 += C) {
             Chunk<LPR> cx;
-            cx.load(colval, a + j0, b, self, sub);
+            cx.load(colval, cur.a + j0, cur.b, cur.self, sub);
             gather_chunk<T, LPR>(cx, min(maxdeg - j0, C), gm, Xl, acc);
         }
-        if (live && deg > 0) {
-            T* xp = X + (int64_t)self * K + sub * E;
+        m1 = load_meta(r2);
+        if (cur.row >= 0 && deg > 0) {
             float xs[E], y[E];
-            Vec<T>::load(xp, xs);
+            Vec<T>::unpack(xr, xs);
 #pragma unroll
-            for (int e = 0; e < E; ++e) y[e] = fmaf(cp, acc[e], a_self * xs[e]);
+            for (int e = 0; e < E; ++e) y[e] = fmaf(cur.cp, acc[e], a_self * xs[e]);
             Vec<T>::store(xp, y);
         }
+        t += nw;
+        cur = nxt;
+        ch = ch1;
     }
 }
 
@@ -1306,7 +1333,7 @@ struct Smoother {
         k_coef<<<sfg_grid(ctx, (const void*)k_coef, kBlock, 0, n), kBlock, 0, ctx->stream>>>(
             n, L->invdeg, omega, coef);
         k_gs_weights<<<sfg_grid(ctx, (const void*)k_gs_weights, kBlock, 0, n), kBlock, 0,
-                       ctx->stream>>>(n, L->row_ptr, L->colval, L->gs_color, omega, yw);
+                       ctx->stream>>>(n, L->row_ptr, L->colval, L->gs_color, L->deg, omega, yw);
         if (L->hv_n > 0) {
             k_gs_weights_heavy<<<std::min(L->hv_n, 4 * ctx->num_sms), 256, 0, ctx->stream>>>(
                 L->hv_n, L->hv_rows, L->row_ptr, L->colval, L->gs_color, omega, yw);
