@@ -216,17 +216,19 @@ __global__ void k_lap_f2c(const uint64_t* __restrict__ keys, const uint32_t* __r
 // What bounds it: 4-byte and 8-byte accesses at random rows (counting, placing, mirrors), so the
 // passes are few: count, place, sort rows, index. Rows are sorted where their entries fit on chip: up
 // to kRowSmall entries, four rows a warp, and up to kRowWarp, one row a warp, each entry ranked
-// against its row in shared memory (quadratic, but no barrier but the warp's); up to kRowMid and up
-// to kRowCap entries, one CTA a row, bitonic. The keys (column, input position) are unique, so the
+// against its row in shared memory (quadratic, but no barrier but the warp's); up to kRowMid, kRowBig
+// and kRowCap entries, one CTA of 128, 256 or 1,024 threads a row, bitonic (three classes, because a
+// CTA's shared memory is its class's largest row: rows of 257-4,096 entries in one class of 48 KB took
+// 302 us on the Chung-Lu graph below, about 270 in two). The keys (column, input position) are unique, so the
 // order does not depend on the order in which atomics placed them. Measured against the radix path,
 // which moves 24 bytes an entry for each of 5-6 digits (GB300, kernels of one build): 2^20-node
 // Chung-Lu graph (15.7M entries) 2.54 -> 1.75 ms, 128^3 grid (12.5M entries) 1.47 -> 0.57 ms. What is
 // left of the first is the 390 us of counting (atomics on random rows) and 346 us of placing.
-constexpr int kRowSmall = 32, kRowWarp = 256, kRowMid = 4096, kRowCap = 16384;
+constexpr int kRowSmall = 32, kRowWarp = 256, kRowMid = 1024, kRowBig = 4096, kRowCap = 16384;
 
-// Words the build reads back: input error, longest raw row, rows of the three larger classes, merged
+// Words the build reads back: input error, longest raw row, rows of the four larger classes, merged
 // rows over SFG_HEAVY_ROW, raw entries, merged entries, canonical edges.
-enum { kWErr, kWMax, kWWarp, kWMid, kWLarge, kWHeavy, kWRaw, kWNnz, kWEdges, kWCount };
+enum { kWErr, kWMax, kWWarp, kWMid, kWBig, kWLarge, kWHeavy, kWRaw, kWNnz, kWEdges, kWCount };
 
 // Raw row lengths and each entry's place within its row (slot.x in row u, slot.y in row v; -1 for
 // self-loops and bad edges). A warp whose edges all share an endpoint (a hub's edges in a sorted
@@ -284,9 +286,9 @@ __global__ void __launch_bounds__(kBlock)
     }
 }
 
-// The rows of the three larger classes (in no particular order) and the longest row.
+// The rows of the four larger classes (in no particular order) and the longest row.
 __global__ void k_row_classify(int32_t n, const int32_t* __restrict__ cnt, int32_t* __restrict__ lwarp,
-                               int32_t* __restrict__ mid, int32_t* __restrict__ large,
+                               int32_t* __restrict__ mid, int32_t* __restrict__ big, int32_t* __restrict__ large,
                                unsigned long long* __restrict__ words) {
     int32_t top = 0;
     for (int64_t r0 = (int64_t)blockIdx.x * kBlock; r0 < n; r0 += (int64_t)gridDim.x * kBlock) {
@@ -304,6 +306,7 @@ __global__ void k_row_classify(int32_t n, const int32_t* __restrict__ cnt, int32
         }
         if (c > kRowWarp) {
             if (c <= kRowMid) mid[atomicAdd(words + kWMid, 1ull)] = (int32_t)r;
+            else if (c <= kRowBig) big[atomicAdd(words + kWBig, 1ull)] = (int32_t)r;
             else large[atomicAdd(words + kWLarge, 1ull)] = (int32_t)r;
         }
     }
@@ -1065,7 +1068,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     *fits = true;
     const int64_t len = 2 * m;
     Scratch s(ctx);
-    int32_t *cnt, *lwarp, *mid, *large, *re, *rrow, *rpos, *nnz, *up, *D, *move;
+    int32_t *cnt, *lwarp, *mid, *big, *large, *re, *rrow, *rpos, *nnz, *up, *D, *move;
     int2 *slot, *rcv;
     uint64_t* raw;
     int64_t *off, *row_off, *up_off;
@@ -1073,7 +1076,8 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     SFG_TRY(s.get(&cnt, n));
     SFG_TRY(s.get(&lwarp, n));
     SFG_TRY(s.get(&mid, (size_t)(len / kRowWarp) + 1));  // longer rows are at most so many
-    SFG_TRY(s.get(&large, (size_t)(len / kRowMid) + 1));
+    SFG_TRY(s.get(&big, (size_t)(len / kRowMid) + 1));
+    SFG_TRY(s.get(&large, (size_t)(len / kRowBig) + 1));
     SFG_TRY(s.get(&slot, m));
     SFG_TRY(s.get(&words, kWCount));
     int* hw32 = nullptr;
@@ -1084,7 +1088,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     if (m > 0) {
         auto* count = validate ? k_row_count<false> : k_row_count<true>;
         count<<<grid_of(ctx, count, (m + 3) / 4), kBlock, 0, ctx->stream>>>(n, m, u, v, w, cnt, slot, words);
-        k_row_classify<<<grid_of(ctx, k_row_classify, n), kBlock, 0, ctx->stream>>>(n, cnt, lwarp, mid, large, words);
+        k_row_classify<<<grid_of(ctx, k_row_classify, n), kBlock, 0, ctx->stream>>>(n, cnt, lwarp, mid, big, large, words);
         ctx->launches += 2;
         SFG_LAUNCH_CHECK(ctx, "k_row_count");
     }
@@ -1098,7 +1102,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
         *fits = false;
         return SFG_OK;
     }
-    const int32_t nwarp = (int32_t)hw[kWWarp], nmid = (int32_t)hw[kWMid], nlarge = (int32_t)hw[kWLarge];
+    const int32_t nwarp = (int32_t)hw[kWWarp], nmid = (int32_t)hw[kWMid], nbig = (int32_t)hw[kWBig], nlarge = (int32_t)hw[kWLarge];
 
     sfg_graph* g = new sfg_graph();
     struct Owner { sfg_graph* g; ~Owner() { sfg_graph_free(g); } } own{g};
@@ -1134,7 +1138,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
         ++ctx->launches;
     }
     auto rows_cta = [&](auto* k, int threads, int cap, int32_t count, const int32_t* list) -> sfg_status {
-        const size_t sm = (size_t)cap * (sizeof(uint64_t) + sizeof(float));  // 48 and 192 KB: opt in once
+        const size_t sm = (size_t)cap * (sizeof(uint64_t) + sizeof(float));  // up to 192 KB: opt in once
         const auto key = std::make_tuple((const void*)k, -threads, sm);
         if (ctx->occupancy.find(key) == ctx->occupancy.end()) {
             SFG_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
@@ -1145,7 +1149,8 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
         ++ctx->launches;
         return SFG_OK;
     };
-    if (nmid > 0) SFG_TRY(rows_cta(k_rows_cta<256, kRowMid>, 256, kRowMid, nmid, mid));
+    if (nmid > 0) SFG_TRY(rows_cta(k_rows_cta<128, kRowMid>, 128, kRowMid, nmid, mid));
+    if (nbig > 0) SFG_TRY(rows_cta(k_rows_cta<256, kRowBig>, 256, kRowBig, nbig, big));
     if (nlarge > 0) SFG_TRY(rows_cta(k_rows_cta<1024, kRowCap>, 1024, kRowCap, nlarge, large));
     SFG_LAUNCH_CHECK(ctx, "k_rows");
     SFG_TRY(sfg_scan_i32(ctx, nnz, row_off, n));

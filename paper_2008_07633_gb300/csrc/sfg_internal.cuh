@@ -153,7 +153,7 @@ struct Scratch {
 // synchronisation, and the host reads it after the next one. Slots: 0 spanning-forest round
 // flag, 1 pointer-jumping flag, 3 breadth-first flag; from kSfgHostBuild on, the 64-bit words of a
 // graph build.
-constexpr int kSfgHostBuild = 8, kSfgHostWords = 32;
+constexpr int kSfgHostBuild = 8, kSfgHostWords = 64;
 sfg_status sfg_host_word(sfg_ctx* ctx, int slot, int** out);
 
 // Kernel timing (no-ops unless ctx->timing).

@@ -36,7 +36,7 @@ def star_lists(lengths, dup, wide, order, seed):
     return n, u[p].astype(np.int32), v[p].astype(np.int32), w.astype(np.float32)
 
 
-@pytest.mark.parametrize("lengths", [(1, 2, 31, 32, 33, 64), (255, 256, 257, 1023, 1024, 1025, 1500), (4095, 4096, 4097, 33), (5000, 16384, 40),
+@pytest.mark.parametrize("lengths", [(1, 2, 31, 32, 33, 64), (255, 256, 257, 1023, 1024, 1025, 1500), (4095, 4096, 4097, 33), (5000, 16384, 40), (257, 1024, 1025),
                                      (16385, 33, 8)])
 @pytest.mark.parametrize("dup,wide,order", [(False, False, "random"), (True, True, "random"), (True, False, "sorted")])
 def test_rows_bit_exact(lengths, dup, wide, order):
