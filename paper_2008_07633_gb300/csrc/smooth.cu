@@ -31,10 +31,32 @@ constexpr int kBlock = 256;
 struct JVariant { int tpi, minb; };
 constexpr JVariant kJVariants[] = {{1, 4}, {2, 4}, {4, 4}, {1, 3}, {2, 3}, {4, 3}};
 constexpr int kJNumVariants = 6, kJDefault = 1;
-// Untuned sweeps: rows of up to 8 lanes take one tile a turn, longer ones two (GB300, us a sweep, one /
-// two tiles: 2048^2 power grid K = 64 BF16 274 / 284, 128^3 grid K = 16 85 / 87, K = 32 129 / 129; 1000^2
-// power grid K = 64 FP32 140 / 124). Sweeps with statistics keep kJDefault: their sums are per CTA.
-__host__ __device__ constexpr int plain_variant(int lpr) { return lpr <= 8 ? 0 : kJDefault; }
+// Untuned sweeps without statistics take one of three forms (sweeps with statistics keep kJDefault: their
+// sums are per CTA). AHEAD: each tile also prefetches into L2 the rows kAheadBytes after its own, past
+// the rows that the running CTAs gather, so that first touches come from L2; the distance is in the
+// instruction and costs no register. It pays where the gathers leave the L1 pipe room for one more
+// request a row: low degrees (spanning forests) or other widths than 8 FP32 lanes. Measured (GB300, us a
+// sweep on the graph, on its spanning forest: two tiles a turn / one tile / two tiles AHEAD / one AHEAD):
+//   128^3 grid K = 4 FP32 (1 lane)       48/48/48/48      42/42/42/41
+//   300k mesh K = 4 FP32                 11/11/11/11      10.9/9.4/10.9/9.6
+//   128^3 grid K = 8 FP32 (2 lanes)      57/59/54/54      48/51/46/48
+//   128^3 grid K = 16 FP32 (4 lanes)     87/85/81/81      69/69/65/67
+//   128^3 grid K = 32 BF16 (4 lanes)     87/112/89/105    78/96/77/91
+//   128^3 grid K = 32 FP32 (8 lanes)     130/129/140/141  120/120/111/115
+//   2048^2 power grid K = 64 BF16 (8)    284/274/298/273  274/268/284/259
+//   1000^2 power grid K = 64 FP32 (16)   124/140/114/132  118/134/107/128
+//   2^20-node Chung-Lu K = 32 FP32       327/325/346/343  212/153/210/154
+constexpr int64_t kAheadBytes = 4 << 20;
+enum { kFormTwo, kFormOne, kFormTwoAhead, kFormOneAhead };
+template <typename T, int LPR>
+int plain_form(const sfg_graph* L) {
+    if (L->hv_n > 0) return LPR <= 8 ? kFormOne : kFormTwo;
+    const bool bf16 = sizeof(T) == 2, sparse = L->m < 2 * (int64_t)L->n;
+    if (LPR == 1) return kFormOne;
+    if (LPR == 4 && bf16) return kFormTwo;
+    if (LPR == 8) return bf16 ? kFormOneAhead : sparse ? kFormTwoAhead : kFormOne;
+    return kFormTwoAhead;
+}
 // Graphs with hub rows get kHubWaves CTAs a resident slot: their rows differ in length by hundreds, and
 // rows of one length tend to be neighbours (degree order), so CTAs that finish early must find more
 // (2^20-node Chung-Lu graph, K = 32, one wave / eight: 333 / 323 us on L_G, 186 / 154 on its forest,
@@ -211,7 +233,7 @@ __device__ __forceinline__ void gather_chunk(const Chunk<LPR>& ch, int need, uns
 // per tile. Gathers go in warp-uniform batches sized by the tile's longest row. Rows with more
 // than hmax entries are left to the heavy-row kernels below (their group idles through the tile
 // and stores nothing), so one hub row cannot serialise a warp for the whole sweep.
-template <typename T, int LPR, bool SUB_MU, bool STATS, int TPI, int MINB>
+template <typename T, int LPR, bool SUB_MU, bool STATS, int TPI, int MINB, bool AHEAD = false>
 __global__ void __launch_bounds__(kBlock, MINB)
     k_jacobi(int32_t n, int32_t hmax, const int32_t* __restrict__ row_ptr, const int2* __restrict__ colval,
              const float* __restrict__ coef, float a_self, const T* __restrict__ X,
@@ -262,6 +284,11 @@ __global__ void __launch_bounds__(kBlock, MINB)
         const int32_t maxdeg = __reduce_max_sync(0xffffffffu, deg);
         float acc[E];
         const uint4 xr = Vec<T>::load_raw(Xl + (int64_t)self * K);  // widened at use
+        if (AHEAD) {  // only rows of the block are prefetched
+            constexpr int rows = (int)(kAheadBytes / (K * sizeof(T)));
+            if (self < n - rows)
+                asm volatile("prefetch.global.L2 [%0+%1];" ::"l"(Xl + (int64_t)self * K), "n"((int)kAheadBytes));
+        }
 #pragma unroll
         for (int e = 0; e < E; ++e) acc[e] = 0.f;
         gather_chunk<T, LPR>(ch, min(maxdeg, C), gm, Xl, acc);
@@ -1153,25 +1180,36 @@ struct Smoother {
     static constexpr int E = Vec<T>::E, K = LPR * E;
 
     template <bool A, bool B>
-    static void* kern() {
-        constexpr int v = B ? kJDefault : plain_variant(LPR);
-        return (void*)k_jacobi<T, LPR, A, B, kJVariants[v].tpi, kJVariants[v].minb>;
+    static void* kern() {  // with the first mean removed (A), with statistics (B)
+        return (void*)k_jacobi<T, LPR, A, B, kJVariants[kJDefault].tpi, kJVariants[kJDefault].minb>;
     }
-    static void* plain_kern(int v) {  // the tuned variants of the plain sweep
+    template <bool A>
+    static void* form_kern(int form) {  // untuned, without statistics
+        switch (form) {
+            case kFormOne: return (void*)k_jacobi<T, LPR, A, false, 1, 4>;
+            case kFormTwoAhead: return (void*)k_jacobi<T, LPR, A, false, 2, 4, true>;
+            case kFormOneAhead: return (void*)k_jacobi<T, LPR, A, false, 1, 4, true>;
+            default: return (void*)k_jacobi<T, LPR, A, false, 2, 4>;
+        }
+    }
+    // The tuned variants of the plain sweep; those of one and two tiles a turn prefetch where the graph's
+    // untuned form does.
+    static void* plain_kern(int v, const sfg_graph* L) {
+        const int form = plain_form<T, LPR>(L);
+        const bool ahead = form == kFormTwoAhead || form == kFormOneAhead;
         switch (v) {
-            case 0: return (void*)k_jacobi<T, LPR, false, false, 1, 4>;
-            case 1: return (void*)k_jacobi<T, LPR, false, false, 2, 4>;
+            case 0: return form_kern<false>(ahead ? kFormOneAhead : kFormOne);
             case 2: return (void*)k_jacobi<T, LPR, false, false, 4, 4>;
             case 3: return (void*)k_jacobi<T, LPR, false, false, 1, 3>;
             case 4: return (void*)k_jacobi<T, LPR, false, false, 2, 3>;
             case 5: return (void*)k_jacobi<T, LPR, false, false, 4, 3>;
-            default: return kern<false, false>();
+            default: return form_kern<false>(ahead ? kFormTwoAhead : kFormTwo);
         }
     }
 
     // CTAs of a seeded block and of a sweep with statistics (one statistics slot each).
     static int grid_jacobi(sfg_ctx* ctx, int32_t n) {
-        return sfg_grid(ctx, plain_kern(kJDefault), kBlock, 0, (int64_t)n * LPR);
+        return sfg_grid(ctx, form_kern<false>(kFormTwo), kBlock, 0, (int64_t)n * LPR);
     }
 
     // CTAs of a sweep without statistics.
@@ -1212,10 +1250,14 @@ struct Smoother {
         const int32_t n = L->n;
         SFG_TRY(heavy_prepare(ctx, L));
         const int32_t hmax = L->hv_n > 0 ? kHeavy : INT32_MAX;
-        void* k = sub_mu ? (stats ? kern<true, true>() : kern<true, false>())
-                         : (stats ? kern<false, true>() : kern<false, false>());
-        if (!sub_mu && !stats)  // the plain sweep takes the tuned tile shape, if any
-            k = plain_kern(sfg_tuned_variant(ctx, K, Vec<T>::E == 4 ? SFG_F32 : SFG_BF16, L));
+        void* k;
+        if (stats) {
+            k = sub_mu ? kern<true, true>() : kern<false, true>();
+        } else {  // the plain sweep takes the tuned tile shape, if any
+            const int v = sub_mu ? -1 : sfg_tuned_variant(ctx, K, Vec<T>::E == 4 ? SFG_F32 : SFG_BF16, L);
+            const int form = plain_form<T, LPR>(L);
+            k = v >= 0 ? plain_kern(v, L) : sub_mu ? form_kern<true>(form) : form_kern<false>(form);
+        }
         const int g = stats ? grid : grid_plain(ctx, k, L);
         void* args[] = {(void*)&n, (void*)&hmax, (void*)&L->row_ptr, (void*)&L->colval, (void*)&coef,
                         (void*)&a_self, (void*)&X, (void*)&Y, (void*)&mu, (void*)&part};
@@ -1566,13 +1608,13 @@ struct Smoother {
         SFG_CUDA(ctx, cudaEventCreate(&e1));
         SFG_TRY(heavy_prepare(ctx, L));  // the tile kernel is timed as the sweep runs it
         const int32_t hmax = L->hv_n > 0 ? kHeavy : INT32_MAX;
-        int best = plain_variant(LPR);
+        int best = kJDefault;
         float best_ms = 1e30f;
         const float a_self = 0.3f;
         const float* mu = nullptr;
         double* pp = nullptr;
         for (int v = 0; v < kJNumVariants; ++v) {
-            void* k = plain_kern(v);
+            void* k = plain_kern(v, L);
             const int g = grid_plain(ctx, k, L);
             const T* X = x;
             T* Y = y;
