@@ -5,8 +5,9 @@
 // (FP32 weight bits << 32) | ~id, unique and ordered like that order, so the forest is unique and
 // equal to Kruskal's. A round: (1) each component takes the largest key among edges leaving it,
 // (2) marks that edge and hooks to the component across it, the smaller label of a mutual pair
-// staying a root, (3) pointer jumping flattens the hook forest, (4) nodes are relabelled. Rounds
-// repeat until no component has an outgoing edge. All rounds run in one cooperative launch.
+// staying a root, (3) nodes are relabelled with the roots of the hook forest (flattened by pointer jumping
+// first where a path is long). Rounds repeat until no component has an outgoing edge. All rounds run in
+// one cooperative launch.
 #include "gridbar.cuh"
 #include "sfg_internal.cuh"
 
@@ -25,19 +26,25 @@ __global__ void k_mst_init(int32_t n, int32_t* __restrict__ comp) {
 // keeps its best edge and looks through its row again only when that edge has become internal, and
 // never again once no edge leaves; a component's maximum is compared before the 64-bit atomicMax, so
 // most nodes of a large component only read it. Hooking and jumping go over a list of the labels that
-// are left. Separate round kernels that rescanned every row took 1,490 us and 11 host waits on the
-// 128^3 grid and 200 us and 7 waits on a 64 x 64 grid.
+// are left, and relabelling climbs the hooks itself, so a round has three phases. Separate round kernels
+// that rescanned every row took 1,490 us and 11 host waits on the 128^3 grid and 200 us and 7 waits on a
+// 64 x 64 grid.
 //
 // Items are the rows [0, n), rows longer than SFG_HEAVY_ROW excepted, and then the fixed segments
 // of those rows. A warp takes kMstTiles x 32 items at once (the tiles a whole grid apart, so that the hubs
 // of a graph numbered by degree spread over the warps), one lane each checking the kept edges. The
 // items to look through again go through shared memory: up to kMstLong entries to four 8-lane groups,
-// kMstItems at a time, longer ones to the whole warp, four entries a lane in flight. Every step is a
-// chain of dependent loads, so the chains in flight set the time: with one tile a warp and every row
-// in 8-lane groups the 128^3 grid took 1,220 us, and a coarsened power-law graph, whose consecutive
-// hub rows then shared a warp, more than the separate kernels (two-level sparsify of a 249,480-node
-// Chung-Lu graph 9.6 ms instead of 6.9).
-constexpr int kMstTiles = 4, kMstLong = 32;
+// kMstItems at a time, longer ones to the whole warp, four entries a lane in flight. Rows of up to
+// kMstSorted entries are looked through once: the first round ranks their entries by key, one lane a
+// row, and later rounds only step on while the current entry is internal, one lane a row and kMstAhead
+// entries at once (the order is one 64-bit word a row: 4 bits a remaining entry, best first, above a 4-bit
+// count). Every step is a chain of dependent loads, so the chains in flight set the time. Kernel time on
+// the 128^3 grid and a 64 x 64 grid: every row in 8-lane groups each time 1,220 and 95 us, four tiles in
+// flight and label lists 1,080 and 90, short rows stepped 880 and 72, two tiles and five entries ahead 826
+// and 64 (one tile: 913 and 61). With hub rows in 8-lane groups a coarsened power-law graph, whose
+// consecutive hub rows then shared a warp, took longer than the separate kernels (two-level sparsify of a
+// 249,480-node Chung-Lu graph 9.6 ms instead of 6.9).
+constexpr int kMstTiles = 2, kMstLong = 32, kMstSorted = 15, kMstAhead = 5;
 constexpr int kMstLanes = 8, kMstGroups = 32 / kMstLanes, kMstItems = 4;
 
 // Words of one launch: barrier count, error, edges taken, last pointer-jumping pass with work left,
@@ -61,6 +68,7 @@ struct MstArgs {
     unsigned long long* best;   // per component label
     unsigned long long* ckey;   // per item: its kept edge's key and the node across it (-1: none left)
     int32_t* cnbr;
+    unsigned long long* order;  // per row: the remaining entries of a short row (0: not a short row)
     int32_t* labels[2];         // labels of the components that still had an edge, this round's and the next's
     uint8_t* mask;
     unsigned long long* words;
@@ -83,14 +91,18 @@ __device__ __forceinline__ bool jump_node(volatile int32_t* par, int64_t r) {  /
     return par[p] != p;
 }
 
+// Offer a key to a component: the maximum so far is read first (from L2), so that most nodes of a large
+// component only read. Folding a warp's offers first (by match and reduce, or along runs of lanes) cost
+// more than the atomics it saved on every graph tried.
 __device__ __forceinline__ void mst_offer(unsigned long long* best, int32_t c, unsigned long long key) {
-    if (key > *(volatile unsigned long long*)(best + c)) atomicMax(best + c, key);
+    if (key > __ldcg(best + c)) atomicMax(best + c, key);
 }
 
 __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
     constexpr int LIST = kMstTiles * 32;
     __shared__ uint8_t s_list[kBlock / 32][LIST];
     __shared__ int32_t s_a[kBlock / 32][LIST], s_b[kBlock / 32][LIST], s_c[kBlock / 32][LIST];
+    __shared__ unsigned long long s_rank[kBlock / 32][kMstSorted][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % kMstLanes, grp = lane / kMstLanes;
     const int64_t t0 = (int64_t)blockIdx.x * kBlock + threadIdx.x, nt = (int64_t)gridDim.x * kBlock;
     const int64_t items = (int64_t)A.n + A.nseg;
@@ -120,12 +132,76 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
                 // the label across the kept edge (round 0: nothing kept, look)
                 nb[q] = nb[q] >= 0 ? (round == 0 ? cp[q] : A.comp[nb[q]]) : -1;
             }
+            // short rows whose kept entry has become internal: step on
+            bool offer[kMstTiles];
+            if (round > 0) {
+                unsigned long long w[kMstTiles];  // remaining entries after the current one, best first
+                int32_t first[kMstTiles], left[kMstTiles], j[kMstTiles];
+                bool step[kMstTiles], any = false;
+#pragma unroll
+                for (int q = 0; q < kMstTiles; ++q) {
+                    const int64_t i = base + q * nt + lane;
+                    offer[q] = cp[q] >= 0 && nb[q] != cp[q];
+                    step[q] = cp[q] >= 0 && !offer[q] && i < A.n;
+                    w[q] = step[q] ? A.order[i] : 0ull;
+                    first[q] = step[q] ? A.row_ptr[i] : 0;
+                    step[q] = w[q] != 0ull;
+                    left[q] = (int)(w[q] & 15ull) - 1;
+                    w[q] >>= 8;
+                    any |= step[q];
+                    j[q] = step[q] ? -2 : -1;  // -2: looking, or found nothing
+                }
+                while (any) {  // kMstAhead entries of every row at once: one turn is two loads deep
+                    any = false;
+                    int32_t col[kMstTiles][kMstAhead];
+#pragma unroll
+                    for (int q = 0; q < kMstTiles; ++q)
+#pragma unroll
+                        for (int d = 0; d < kMstAhead; ++d)
+                            col[q][d] = step[q] && d < left[q] ? A.colval[first[q] + (int32_t)((w[q] >> (4 * d)) & 15ull)].x : -1;
+#pragma unroll
+                    for (int q = 0; q < kMstTiles; ++q)
+#pragma unroll
+                        for (int d = 0; d < kMstAhead; ++d)
+                            if (col[q][d] >= 0) col[q][d] = A.comp[col[q][d]] != cp[q] ? 1 : 0;
+#pragma unroll
+                    for (int q = 0; q < kMstTiles; ++q)
+                        if (step[q]) {
+                            int drop = kMstAhead;
+#pragma unroll
+                            for (int d = kMstAhead - 1; d >= 0; --d)
+                                if (col[q][d] != 0) drop = d;  // external (1), or past the last one (-1)
+                            w[q] >>= 4 * drop;
+                            left[q] -= drop;
+                            const bool found = drop < kMstAhead && left[q] > 0;
+                            if (found) j[q] = first[q] + (int32_t)(w[q] & 15ull);
+                            step[q] = !found && left[q] > 0;
+                            any |= step[q];
+                        }
+                }
+#pragma unroll
+                for (int q = 0; q < kMstTiles; ++q) {
+                    const int64_t i = base + q * nt + lane;
+                    if (j[q] >= 0) {
+                        const int2 cv = A.colval[j[q]];
+                        const int32_t e = A.eid[j[q]];
+                        const uint32_t id = A.key_id ? (uint32_t)A.key_id[e] : (uint32_t)e;
+                        A.order[i] = (w[q] << 4) | (unsigned long long)left[q];
+                        A.cnbr[i] = cv.x;
+                        A.ckey[i] = ((unsigned long long)(uint32_t)cv.y << 32) | (unsigned long long)(~id);
+                        offer[q] = true;
+                    } else if (j[q] == -2) {
+                        A.cnbr[i] = -1;  // its last entry is internal
+                        cp[q] = -1;
+                    }
+                }
+            }
             int cnt = 0, longs = 0;  // short items from the front of the lists, long ones from the back
 #pragma unroll
             for (int q = 0; q < kMstTiles; ++q) {
                 const int64_t i = base + q * nt + lane;
-                const bool need = cp[q] >= 0 && nb[q] == cp[q];
-                if (cp[q] >= 0 && !need) mst_offer(A.best, cp[q], A.ckey[i]);
+                bool need = cp[q] >= 0 && !(round > 0 && offer[q]);
+                if (round > 0 && cp[q] >= 0 && offer[q]) mst_offer(A.best, cp[q], A.ckey[i]);
                 int32_t a = 0, b = 0;
                 if (need) {
                     if (i < A.n) {
@@ -137,6 +213,55 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
                         a = sg.y;
                         b = sg.z;
                     }
+                }
+                if (round == 0) {  // short rows: rank their entries (every allowed entry leaves its node)
+                    const bool shortrow = need && i < A.n && b - a <= kMstSorted;
+                    const int len = shortrow ? b - a : 0;
+                    int live = 0;
+                    unsigned long long top = 0ull, word = 0ull;
+                    int32_t across = -1;
+                    for (int x0 = 0; x0 < len; x0 += 4) {
+                        int2 cv[4];
+                        int32_t e[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (x0 + u < len) {
+                                cv[u] = A.colval[a + x0 + u];
+                                e[u] = A.eid[a + x0 + u];
+                            }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (x0 + u < len) {
+                                unsigned long long key = 0ull;
+                                if (!A.allow || A.allow[e[u]]) {
+                                    const uint32_t id = A.key_id ? (uint32_t)A.key_id[e[u]] : (uint32_t)e[u];
+                                    key = ((unsigned long long)(uint32_t)cv[u].y << 32) | (unsigned long long)(~id);
+                                    ++live;
+                                    if (key > top) {
+                                        top = key;
+                                        across = cv[u].x;
+                                    }
+                                }
+                                s_rank[warp][x0 + u][lane] = key;
+                            }
+                    }
+                    for (int x = 0; x < len; ++x) {
+                        const unsigned long long key = s_rank[warp][x][lane];
+                        if (key == 0ull) continue;
+                        int rank = 0;
+                        for (int y = 0; y < len; ++y) rank += s_rank[warp][y][lane] > key;
+                        word |= (unsigned long long)x << (4 * rank + 4);
+                    }
+                    if (shortrow) {
+                        A.order[i] = live ? word | (unsigned long long)live : 0ull;
+                        A.cnbr[i] = across;
+                        A.ckey[i] = top;
+                        if (top) atomicMax(A.best + cp[q], top);
+                        need = false;
+                    } else if (need && i < A.n) {
+                        A.order[i] = 0ull;
+                    }
+                    if (!need) a = b = 0;
                 }
                 const bool big = b - a > kMstLong;
                 const unsigned low = (1u << lane) - 1u;
@@ -283,25 +408,35 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
         const unsigned long long now = *(volatile unsigned long long*)(A.words + kMwTree);
         if (now == tree) return;  // no component has an outgoing edge
         tree = now;
-        // (3) flatten; a pass with work left leaves its number (a later pass only starts if it did)
-        for (;;) {
-            ++jump_pass;
-            bool left = false;
-            for (int64_t i = t0; i < nlab; i += nt) left |= jump_node(A.parent, round == 0 ? i : (int64_t)list[i]);
-            if (left) atomicMax(A.words + kMwJump, jump_pass);
-            if (!grid_barrier(bar, passed)) return;
-            if (*(volatile unsigned long long*)(A.words + kMwJump) < jump_pass) break;
-        }
-        // (4) relabel; the next round's labels are the roots that had an edge in this one
+        // (3) relabel: every node climbs from its label up to kHops hooks (nothing writes them here); a
+        // node that stops short of a root leaves the pass's number, and the hooks are then flattened and
+        // the nodes, which hold some ancestor of their label, relabelled once more. The next round's
+        // labels are the roots that had an edge in this one.
+        ++jump_pass;
+        bool left = false;
         for (int64_t p0 = t0; p0 < A.n; p0 += nt * kMstTiles) {
-            int32_t c[kMstTiles];
+            int32_t c[kMstTiles], up[kMstTiles];
 #pragma unroll
             for (int q = 0; q < kMstTiles; ++q) c[q] = p0 + q * nt < A.n ? A.comp[p0 + q * nt] : 0;
 #pragma unroll
-            for (int q = 0; q < kMstTiles; ++q) c[q] = A.parent[c[q]];
+            for (int q = 0; q < kMstTiles; ++q) up[q] = A.parent[c[q]];
+            for (int h = 0; h < kHops; ++h) {
+                bool moved = false;
+#pragma unroll
+                for (int q = 0; q < kMstTiles; ++q)
+                    if (up[q] != c[q]) {
+                        c[q] = up[q];
+                        up[q] = A.parent[c[q]];
+                        moved = true;
+                    }
+                if (!moved) break;
+            }
 #pragma unroll
             for (int q = 0; q < kMstTiles; ++q)
-                if (p0 + q * nt < A.n) A.comp[p0 + q * nt] = c[q];
+                if (p0 + q * nt < A.n) {
+                    A.comp[p0 + q * nt] = c[q];
+                    left |= up[q] != c[q];
+                }
         }
         for (int64_t i0 = t0 - lane; i0 < nlab; i0 += nt) {
             const int64_t i = i0 + lane;
@@ -317,6 +452,18 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
                 A.best[r] = 0ull;
             }
         }
+        if (left) atomicMax(A.words + kMwJump, jump_pass);
+        if (!grid_barrier(bar, passed)) return;
+        if (*(volatile unsigned long long*)(A.words + kMwJump) < jump_pass) continue;
+        for (;;) {
+            ++jump_pass;
+            left = false;
+            for (int64_t i = t0; i < nlab; i += nt) left |= jump_node(A.parent, round == 0 ? i : (int64_t)list[i]);
+            if (left) atomicMax(A.words + kMwJump, jump_pass);
+            if (!grid_barrier(bar, passed)) return;
+            if (*(volatile unsigned long long*)(A.words + kMwJump) < jump_pass) break;
+        }
+        for (int64_t p = t0; p < A.n; p += nt) A.comp[p] = A.parent[A.comp[p]];
         if (!grid_barrier(bar, passed)) return;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(reinterpret_cast<int*>(A.words + kMwErr), 1);
@@ -403,6 +550,7 @@ sfg_status sfg_mst_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* allow, 
     SFG_TRY(s.get(&a.best, n));
     SFG_TRY(s.get(&a.ckey, items));
     SFG_TRY(s.get(&a.cnbr, items));
+    SFG_TRY(s.get(&a.order, n));
     SFG_TRY(s.get(&a.labels[0], n));
     SFG_TRY(s.get(&a.labels[1], n));
     SFG_TRY(s.get(&a.words, kMwCount));
