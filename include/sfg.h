@@ -73,9 +73,11 @@ SFG_API sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream);
 SFG_API void sfg_ctx_destroy(sfg_ctx* ctx);
 /* Device memory: every allocation of the library (graphs, scratch) comes stream-ordered from one
  * pool per device, shared by the contexts on that device and kept for the life of the process,
- * which holds freed memory for reuse instead of returning it at each synchronisation.
- * sfg_ctx_trim synchronises the context stream and returns the pool's unused memory to the
- * device (an allocation that fails also trims and retries once). */
+ * which holds freed memory for reuse instead of returning it at each synchronisation. A context
+ * keeps scratch blocks of its last calls (at most 1/128 of the device's memory, and the contexts
+ * of a device together 1/32) for its next call on the same stream. sfg_ctx_trim synchronises the context stream and
+ * returns what the context keeps and the pool's unused memory to the device (an allocation that
+ * fails also trims and retries once); sfg_ctx_set_stream gives the kept blocks back to the pool. */
 SFG_API sfg_status sfg_ctx_trim(sfg_ctx* ctx);
 SFG_API sfg_status sfg_ctx_set_stream(sfg_ctx* ctx, void* cuda_stream);
 /* Text of the last error on this context ("" if none). Valid until the next call on ctx. */
@@ -166,7 +168,8 @@ SFG_API sfg_status sfg_jacobi(sfg_ctx* ctx, const sfg_graph* L, int K, int steps
 
 /* Tile-shape autotuning of the sweep and the scorer (not in the paper). Variant v of the plain
  * sweep: a warp sweeps TPI = {1, 2, 4, 1, 2, 4}[v] consecutive row tiles before its grid-stride
- * jump, with {4, 4, 4, 3, 3, 3}[v] CTAs per SM requested from the compiler; default v = 1. Shape s
+ * jump, with {4, 4, 4, 3, 3, 3}[v] CTAs per SM requested from the compiler; without an entry the
+ * shape follows from the width, the storage and the degrees. Shape s
  * of the scorer (sfg_score_edges, sfg_filter_score and the batched forms): a warp scores
  * {1, 2, 1}[s] edge tiles per iteration with {4, 2, 4}[s] CTAs per SM, shape 2 reading rows with
  * loads cached in L2 only; default s = 0 below an average degree of 8, else 1. sfg_autotune times all sweep variants on L (three sweeps each) and both

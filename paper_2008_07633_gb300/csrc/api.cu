@@ -1,4 +1,5 @@
 // Context, status, allocation and timing plumbing of libsfg.
+#include <atomic>
 #include <cstdarg>
 #include <cstdlib>
 #include <cstring>
@@ -27,16 +28,18 @@ sfg_status sfg_cuda_fail(sfg_ctx* ctx, cudaError_t e, const char* where) {
                     where);
 }
 
-sfg_status sfg_alloc(sfg_ctx* ctx, void** p, size_t bytes) {
-    *p = nullptr;
+// Counts an allocation; true when this one has to fail (SFG_FAULT_ALLOC).
+static bool alloc_fails(sfg_ctx* ctx) {
     ctx->alloc_count++;
-    if (ctx->fail_alloc_at >= 0 && ctx->alloc_count == ctx->fail_alloc_at)
-        return sfg_fail(ctx, SFG_ENOMEM, "injected allocation failure (allocation %lld)",
-                        (long long)ctx->alloc_count);
+    return ctx->fail_alloc_at >= 0 && ctx->alloc_count == ctx->fail_alloc_at;
+}
+
+static sfg_status pool_alloc(sfg_ctx* ctx, void** p, size_t bytes) {
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
     if (e == cudaErrorMemoryAllocation) {
         // the pool keeps freed memory; hand it back to the device and try once more
         cudaGetLastError();
+        sfg_scratch_flush(ctx);
         cudaStreamSynchronize(ctx->stream);
         cudaMemPoolTrimTo(ctx->pool, 0);
         e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
@@ -48,6 +51,96 @@ sfg_status sfg_alloc(sfg_ctx* ctx, void** p, size_t bytes) {
                         cudaGetErrorString(e));
     }
     return SFG_OK;
+}
+
+static sfg_status alloc_injected(sfg_ctx* ctx) {
+    return sfg_fail(ctx, SFG_ENOMEM, "injected allocation failure (allocation %lld)", (long long)ctx->alloc_count);
+}
+
+sfg_status sfg_alloc(sfg_ctx* ctx, void** p, size_t bytes) {
+    *p = nullptr;
+    if (alloc_fails(ctx)) return alloc_injected(ctx);
+    return pool_alloc(ctx, p, bytes);
+}
+
+bool sfg_capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {  // the legacy stream while another one is captured
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+constexpr size_t kKeptBlocks = 96;
+constexpr int kKeptDevices = 64;
+constexpr int64_t kKeptShare = 128, kKeptDeviceShare = 32;  // of a device's memory: a context's, all contexts' together
+static std::atomic<int64_t> kept_room[kKeptDevices];  // bytes that the contexts of a device may still keep
+
+static int64_t kept_all[kKeptDevices];                // the same before any is kept
+
+static void kept_room_init(int device) {  // once per device
+    static std::once_flag once[kKeptDevices];
+    if (device >= kKeptDevices) return;
+    std::call_once(once[device], [device] {
+        size_t unused = 0, total = 0;
+        if (cudaMemGetInfo(&unused, &total) == cudaSuccess) kept_room[device] = kept_all[device] = (int64_t)total / kKeptDeviceShare;
+        else cudaGetLastError();
+    });
+}
+
+static bool kept_reserve(sfg_ctx* ctx, int64_t bytes) {
+    const int device = ctx->device;
+    if (device >= kKeptDevices || ctx->kept_bytes + bytes > kept_all[device] / (kKeptShare / kKeptDeviceShare)) return false;
+    if (kept_room[device].fetch_sub(bytes) < bytes) {
+        kept_room[device].fetch_add(bytes);
+        return false;
+    }
+    ctx->kept_bytes += bytes;
+    return true;
+}
+
+static SfgKept kept_remove(sfg_ctx* ctx, size_t i) {
+    const SfgKept b = ctx->kept[i];
+    kept_room[ctx->device].fetch_add((int64_t)b.bytes);
+    ctx->kept_bytes -= (int64_t)b.bytes;
+    ctx->kept.erase(ctx->kept.begin() + i);
+    return b;
+}
+
+// Frees kept block i in its stream's order; not while that stream is being captured.
+static bool kept_drop(sfg_ctx* ctx, size_t i) {
+    if (sfg_capturing(ctx->kept[i].stream)) return false;
+    const SfgKept b = kept_remove(ctx, i);
+    cudaFreeAsync(b.p, b.stream);
+    return true;
+}
+
+void sfg_scratch_flush(sfg_ctx* ctx) {
+    for (size_t i = ctx->kept.size(); i-- > 0;) kept_drop(ctx, i);
+}
+
+sfg_status sfg_scratch_take(sfg_ctx* ctx, void** p, size_t* bytes) {
+    *p = nullptr;
+    if (alloc_fails(ctx)) return alloc_injected(ctx);
+    size_t best = 0, size = SIZE_MAX;  // the smallest block that is large enough, if it is not much larger
+    for (size_t i = 0; i < ctx->kept.size(); ++i) {
+        const SfgKept& b = ctx->kept[i];
+        if (b.stream == ctx->stream && b.bytes >= *bytes && b.bytes < size) best = i, size = b.bytes;
+    }
+    if (size > *bytes + *bytes / 4 + 4096) return pool_alloc(ctx, p, *bytes);
+    const SfgKept b = kept_remove(ctx, best);
+    *p = b.p;
+    *bytes = b.bytes;
+    return SFG_OK;
+}
+
+void sfg_scratch_give(sfg_ctx* ctx, void* p, size_t bytes) {
+    if (ctx->kept.size() >= kKeptBlocks) kept_drop(ctx, 0);  // the oldest goes first
+    bool room = ctx->kept.size() < kKeptBlocks && kept_reserve(ctx, (int64_t)bytes);
+    while (!room && !ctx->kept.empty() && kept_drop(ctx, 0)) room = kept_reserve(ctx, (int64_t)bytes);
+    if (room) ctx->kept.push_back({p, bytes, ctx->stream});
+    else sfg_free(ctx, p);
 }
 
 void sfg_free(sfg_ctx* ctx, void* p) {
@@ -192,6 +285,7 @@ sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream) {
     c->stream = (cudaStream_t)cuda_stream;
     cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (c->num_sms < 1) c->num_sms = 1;
+    kept_room_init(device);
     if (const char* f = std::getenv("SFG_FAULT_ALLOC")) c->fail_alloc_at = std::atoll(f);
     if (const char* f = std::getenv("SFG_FAULT_MMA_WAIT")) c->withhold_mma = std::atoi(f) != 0;
     c->pool = device_pool(device);
@@ -213,6 +307,7 @@ sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream) {
 sfg_status sfg_ctx_trim(sfg_ctx* ctx) {
     if (!ctx) return SFG_EINVAL;
     SFG_DEVICE(ctx);
+    sfg_scratch_flush(ctx);
     SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     SFG_CUDA(ctx, cudaMemPoolTrimTo(ctx->pool, 0));
     return SFG_OK;
@@ -231,6 +326,7 @@ void sfg_ctx_destroy(sfg_ctx* ctx) {
         cudaFreeHost(ctx->host_word);
     }
     if (ctx->pool) {
+        sfg_scratch_flush(ctx);
         // unused memory goes back to the device; memory of live graphs stays valid
         cudaStreamSynchronize(ctx->stream);
         cudaMemPoolTrimTo(ctx->pool, 0);
@@ -241,6 +337,7 @@ void sfg_ctx_destroy(sfg_ctx* ctx) {
 sfg_status sfg_ctx_set_stream(sfg_ctx* ctx, void* cuda_stream) {
     if (!ctx) return SFG_EINVAL;
     SFG_DEVICE(ctx);
+    if (ctx->stream != (cudaStream_t)cuda_stream) sfg_scratch_flush(ctx);
     ctx->stream = (cudaStream_t)cuda_stream;
     return SFG_OK;
 }

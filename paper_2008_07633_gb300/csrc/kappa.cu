@@ -1132,7 +1132,7 @@ struct CompMean {
         SFG_TRY(sfg_radix_sort_pairs(ctx, &k1, &order, &k2, &v2, n, 64));
         if (order == alt) {  // sorted values ended in the temporary buffer: keep it with s
             t.release(alt);
-            s.ptrs.push_back(alt);
+            s.adopt(alt);
         }
         k_comp_heads<<<grid_of(ctx, k_comp_heads, n), kBlock, 0, st>>>(n, k1, head);
         ++ctx->launches;

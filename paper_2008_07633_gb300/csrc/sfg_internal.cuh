@@ -22,6 +22,13 @@ struct sfg_timer_rec {
     cudaEvent_t start, stop;
 };
 
+// A scratch block that a context keeps after the call that used it, free for work on its stream.
+struct SfgKept {
+    void* p;
+    size_t bytes;
+    cudaStream_t stream;
+};
+
 struct sfg_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -36,6 +43,8 @@ struct sfg_ctx {
     std::map<uint32_t, int> tune;          // (K, dtype, degree bucket) -> sweep variant
     std::map<uint32_t, int> score_tune;    // (K, dtype, degree bucket) -> scorer launch shape
     std::map<std::tuple<const void*, int, size_t>, int> occupancy;  // resident CTAs per SM
+    std::vector<SfgKept> kept;             // scratch kept for the next call, oldest first
+    int64_t kept_bytes = 0;
     int64_t alloc_count = 0;               // for the allocation-failure injection hook
     int64_t fail_alloc_at = -1;            // SFG_FAULT_ALLOC=<n>: the n-th allocation fails
     bool withhold_mma = false;             // SFG_FAULT_MMA_WAIT=1: tensor-core kernels issue no
@@ -125,27 +134,45 @@ sfg_status sfg_cuda_fail(sfg_ctx* ctx, cudaError_t e, const char* where);
 sfg_status sfg_alloc(sfg_ctx* ctx, void** p, size_t bytes);
 void sfg_free(sfg_ctx* ctx, void* p);
 
-// Scoped list of scratch allocations released (stream-ordered) at scope exit.
+// Scratch from the blocks the context keeps from its earlier calls, else from the pool; *bytes becomes the
+// block's size. A kept block is reused on the stream it was given back on only. What a context keeps is bounded
+// (kKeptBlocks, and 1/128 of the device's memory; 1/32 over all contexts of a device); sfg_ctx_trim,
+// sfg_ctx_set_stream, sfg_ctx_destroy and an allocation that fails give it back to the pool.
+// Why: the pool took 45-190 us for each of the four large blocks of an end-to-end call on the 128^3 grid, with the
+// GPU idle, and about 1 us for each small one (GB300, all scratch from the pool / kept: that call
+// 7,347 / 7,084 us, two-level 14,170 / 13,970, a 64 x 64 grid 257 / 241, a gradient over 65,536 rows 74 / 61).
+sfg_status sfg_scratch_take(sfg_ctx* ctx, void** p, size_t* bytes);
+void sfg_scratch_give(sfg_ctx* ctx, void* p, size_t bytes);
+void sfg_scratch_flush(sfg_ctx* ctx);
+bool sfg_capturing(cudaStream_t stream);
+
+// Scoped list of scratch allocations released (stream-ordered) at scope exit. A captured call takes and
+// frees its own (nodes of the graph being captured); any other call goes through the kept blocks.
 struct Scratch {
     sfg_ctx* ctx;
-    std::vector<void*> ptrs;
-    explicit Scratch(sfg_ctx* c) : ctx(c) {}
+    bool keep;
+    std::vector<std::pair<void*, size_t>> ptrs;  // size 0: not to be kept
+    explicit Scratch(sfg_ctx* c) : ctx(c), keep(!sfg_capturing(c->stream)) {}
     ~Scratch() {
-        for (void* p : ptrs) sfg_free(ctx, p);
+        for (auto& q : ptrs) {
+            if (!q.first) continue;
+            if (keep && q.second > 0) sfg_scratch_give(ctx, q.first, q.second);
+            else sfg_free(ctx, q.first);
+        }
     }
     template <typename T>
     sfg_status get(T** p, size_t count) {
         void* q = nullptr;
-        sfg_status s = sfg_alloc(ctx, &q, count * sizeof(T) > 0 ? count * sizeof(T) : 16);
-        if (s != SFG_OK) return s;
-        ptrs.push_back(q);
+        size_t bytes = count * sizeof(T) > 0 ? count * sizeof(T) : 16;
+        SFG_TRY(keep ? sfg_scratch_take(ctx, &q, &bytes) : sfg_alloc(ctx, &q, bytes));
+        ptrs.emplace_back(q, keep ? bytes : 0);
         *p = static_cast<T*>(q);
         return SFG_OK;
     }
-    void adopt(void* p) { ptrs.push_back(p); }  // take ownership from the caller
+    void adopt(void* p) { ptrs.emplace_back(p, 0); }  // take ownership from the caller
     void release(void* p) {  // hand ownership to the caller
         for (auto& q : ptrs)
-            if (q == p) q = nullptr;
+            if (q.first == p) q.first = nullptr;
     }
 };
 
