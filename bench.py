@@ -768,7 +768,8 @@ def cpu_baseline():
 # ------------------------------------------------------------------------------------------------
 def run_ours(args):
     world, rank, local = dist_env()
-    extra = rank == 0 and not args.profile and not args.headline_only
+    # --mlp-only starts no generators: exiting while they run can leave the process waiting for them
+    extra = rank == 0 and not (args.profile or args.headline_only or args.mlp_only)
     pool, jobs = start_generators() if extra and not args.no_workloads else (None, None)
 
     import torch
