@@ -147,6 +147,11 @@ void sfg_free(sfg_ctx* ctx, void* p) {
     if (p) cudaFreeAsync(p, ctx->stream);
 }
 
+sfg_status sfg_wait(sfg_ctx* ctx) {
+    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    return SFG_OK;
+}
+
 sfg_status sfg_host_word(sfg_ctx* ctx, int slot, int** out) {
     if (!ctx->host_word)
         SFG_CUDA(ctx, cudaMallocHost((void**)&ctx->host_word, sizeof(int) * kSfgHostWords));

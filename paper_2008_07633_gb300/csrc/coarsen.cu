@@ -268,7 +268,13 @@ sfg_status sfg_coarsen(sfg_ctx* ctx, const sfg_graph* L, const void* X, int K, s
     Scratch s(ctx);
     int32_t* f2c = fine2coarse_out;
     if (!f2c) SFG_TRY(s.get(&f2c, L->m));
-    return sfg_coarsen_impl(ctx, L, X, K, storage, agg_out, f2c, n_coarse_host, coarse_out);
+    SFG_TRY(sfg_coarsen_impl(ctx, L, X, K, storage, agg_out, f2c, n_coarse_host, coarse_out));
+    const sfg_status st = sfg_wait(ctx);  // the coarse graph and the maps are complete
+    if (st != SFG_OK) {
+        sfg_graph_free(*coarse_out);
+        *coarse_out = nullptr;
+    }
+    return st;
 }
 
 sfg_status sfg_backward_map(sfg_ctx* ctx, const sfg_graph* fine, const int32_t* agg,
@@ -283,7 +289,8 @@ sfg_status sfg_backward_map(sfg_ctx* ctx, const sfg_graph* fine, const int32_t* 
         SFG_TRY(sfg_check_dev(ctx, pmask_f, "pmask_f"));
     }
     if (coarse->m > 0) SFG_TRY(sfg_check_dev(ctx, pmask_c, "pmask_c"));
-    return sfg_backward_impl(ctx, fine, agg, fine2coarse, coarse, pmask_c, pmask_f);
+    SFG_TRY(sfg_backward_impl(ctx, fine, agg, fine2coarse, coarse, pmask_c, pmask_f));
+    return sfg_wait(ctx);
 }
 
 }  // extern "C"

@@ -288,6 +288,7 @@ extern "C" sfg_status sfg_coloring(sfg_ctx* ctx, const sfg_graph* L, int32_t* co
     if (color_out && L->n > 0)
         SFG_CUDA(ctx, cudaMemcpyAsync(color_out, L->gs_color, sizeof(int32_t) * L->n,
                                       cudaMemcpyDeviceToDevice, ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     if (ncolors_host) *ncolors_host = (int32_t)L->gs_off.size() - 1;
     return SFG_OK;
 }

@@ -1266,6 +1266,17 @@ sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* ma
     return SFG_OK;
 }
 
+// The build's last kernels are still at work when the builders return: no graph leaves the library before
+// they have finished.
+static sfg_status wait_for_graph(sfg_ctx* ctx, sfg_graph** out) {
+    const sfg_status st = sfg_wait(ctx);
+    if (st != SFG_OK) {
+        sfg_graph_free(*out);
+        *out = nullptr;
+    }
+    return st;
+}
+
 extern "C" {
 
 sfg_status sfg_laplacian(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
@@ -1280,7 +1291,8 @@ sfg_status sfg_laplacian(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, c
         SFG_TRY(sfg_check_dev(ctx, v, "v"));
         SFG_TRY(sfg_check_dev(ctx, w, "w"));
     }
-    return sfg_build_graph(ctx, n, m, u, v, w, true, out, nullptr);
+    SFG_TRY(sfg_build_graph(ctx, n, m, u, v, w, true, out, nullptr));
+    return wait_for_graph(ctx, out);
 }
 
 void sfg_graph_destroy(sfg_graph* g) { sfg_graph_free(g); }
@@ -1330,7 +1342,8 @@ sfg_status sfg_graph_subgraph(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* m
     SFG_DEVICE(ctx);
     *out = nullptr;
     if (g->m > 0) SFG_TRY(sfg_check_dev(ctx, mask, "mask"));
-    return sfg_subgraph_impl(ctx, g, mask, out);
+    SFG_TRY(sfg_subgraph_impl(ctx, g, mask, out));
+    return wait_for_graph(ctx, out);
 }
 
 }  // extern "C"

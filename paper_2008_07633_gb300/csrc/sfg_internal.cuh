@@ -206,6 +206,9 @@ sfg_status sfg_scan_i64(sfg_ctx* ctx, const int64_t* in, int64_t* out, int64_t n
 // ends in (*keys, *vals); the pointers may be swapped with the alternate buffers.
 sfg_status sfg_radix_sort_pairs(sfg_ctx* ctx, uint64_t** keys, uint32_t** vals,
                                 uint64_t** keys_alt, uint32_t** vals_alt, int64_t n, int bits);
+// Wait for the context's stream: the last step of every entry point that is documented to synchronise, so
+// that what it made may be used from any stream, and its inputs released, when it returns.
+sfg_status sfg_wait(sfg_ctx* ctx);
 // Copy scalars back (synchronises the stream).
 sfg_status sfg_read_i64(sfg_ctx* ctx, const int64_t* dev, int64_t* host);
 

@@ -223,10 +223,8 @@ extern "C" sfg_status sfg_sparsify(sfg_ctx* ctx, const sfg_graph* G, const sfg_p
     for (Level& v : lv) v.xg = nullptr;  // scratch, freed with s
     if (G->m > 0)
         SFG_CUDA(ctx, cudaMemcpyAsync(mask_out, pm, G->m, cudaMemcpyDeviceToDevice, ctx->stream));
-    if (n_selected_host) {
-        SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-        *n_selected_host = count;
-    }
+    SFG_TRY(sfg_wait(ctx));
+    if (n_selected_host) *n_selected_host = count;
     if (hier_out) {
         *hier_out = h;
         owner.h = nullptr;
@@ -384,9 +382,7 @@ extern "C" sfg_status sfg_sparsify_to_kappa(sfg_ctx* ctx, const sfg_graph* G, co
         if (count == before) break;  // nothing left to add
     }
     if (rounds_host) *rounds_host = r;
-    if (n_selected_host) {
-        SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-        *n_selected_host = count;
-    }
+    SFG_TRY(sfg_wait(ctx));
+    if (n_selected_host) *n_selected_host = count;
     return SFG_OK;
 }
