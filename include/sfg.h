@@ -214,7 +214,7 @@ SFG_API sfg_status sfg_filter_score(sfg_ctx* ctx, const sfg_graph* LG, const sfg
 
 /* ids_out[0..k) = the ids of the k largest entries under the strict order (score descending,
  * id ascending), written in ascending id order. ids must be distinct; 0 <= k <= ne else
- * SFG_EINVAL. */
+ * SFG_EINVAL. ids_out may overlap ids or scores (their other entries keep their values). */
 SFG_API sfg_status sfg_select_topk(sfg_ctx* ctx, const float* scores, const int32_t* ids, int64_t ne,
                            int64_t k, int32_t* ids_out);
 

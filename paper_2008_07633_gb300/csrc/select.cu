@@ -279,6 +279,11 @@ __global__ void __launch_bounds__(kBlock, 4) k_topk(TkArgs A) {
         tk_give_up(A);
 }
 
+bool ranges_overlap(const void* a, size_t na, const void* b, size_t nb) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x < y + nb && y < x + na;
+}
+
 }  // namespace
 
 sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, int64_t ne,
@@ -288,6 +293,12 @@ sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, 
     const int grid = sfg_grid(ctx, (const void*)k_topk, kBlock, 0, (ne + 3) / 4);
     const int sort_ctas = (int)std::min<int64_t>(grid, (k + 4095) / 4096);
     Scratch s(ctx);
+    // The kept ids are written while other CTAs still read the lists: a list over its own inputs (an
+    // in-place selection) is made beside them first.
+    int32_t* list = out;
+    const bool aside = ranges_overlap(out, sizeof(int32_t) * (size_t)k, ids, sizeof(int32_t) * (size_t)ne) ||
+                       ranges_overlap(out, sizeof(int32_t) * (size_t)k, scores, sizeof(float) * (size_t)ne);
+    if (aside) SFG_TRY(s.get(&list, k));
     TkArgs a{};
     unsigned long long* zeroed;  // histograms, then the words
     SFG_TRY(s.get(&zeroed, (size_t)kTkPasses * kTkBins + kTwCount));
@@ -304,7 +315,7 @@ sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, 
     a.hist = zeroed;
     a.words = zeroed + (size_t)kTkPasses * kTkBins;
     a.sort_ctas = sort_ctas;
-    a.out = out;
+    a.out = list;
     void* args[] = {(void*)&a};
     sfg_tic(ctx, "topk");
     const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_topk, dim3(grid), dim3(kBlock), args, 0,
@@ -312,6 +323,8 @@ sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, 
     sfg_toc(ctx);
     if (e != cudaSuccess) return sfg_cuda_fail(ctx, e, "k_topk");
     ++ctx->launches;
+    if (aside)
+        SFG_CUDA(ctx, cudaMemcpyAsync(out, list, sizeof(int32_t) * (size_t)k, cudaMemcpyDeviceToDevice, ctx->stream));
     return SFG_OK;
 }
 
