@@ -796,13 +796,13 @@ __global__ void __launch_bounds__(kBlock)
     }
 }
 
+// Edges that were not placed (self-loops, and edges that an unvalidated list may hold with a weight that is not
+// finite, such as merged weights past the FP32 range) belong to no canonical edge.
 __global__ void k_row_f2c(int64_t m, const int32_t* __restrict__ u, const int32_t* __restrict__ v,
-                          const int32_t* __restrict__ rpos, const int32_t* __restrict__ D,
-                          int32_t* __restrict__ f2c) {
-    for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m; e += (int64_t)gridDim.x * kBlock) {
-        const int32_t a = u[e], b = v[e];
-        f2c[e] = a == b ? -1 : rpos[e] + D[min(a, b)];
-    }
+                          const int2* __restrict__ slot, const int32_t* __restrict__ rpos,
+                          const int32_t* __restrict__ D, int32_t* __restrict__ f2c) {
+    for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < m; e += (int64_t)gridDim.x * kBlock)
+        f2c[e] = slot[e].x < 0 ? -1 : rpos[e] + D[min(u[e], v[e])];
 }
 
 // ---- subgraph ----------------------------------------------------------------------------------
@@ -1183,7 +1183,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
         ++ctx->launches;
     }
     if (f2c && m > 0) {
-        k_row_f2c<<<grid_of(ctx, k_row_f2c, m), kBlock, 0, ctx->stream>>>(m, u, v, rpos, D, f2c);
+        k_row_f2c<<<grid_of(ctx, k_row_f2c, m), kBlock, 0, ctx->stream>>>(m, u, v, slot, rpos, D, f2c);
         ++ctx->launches;
     }
     SFG_LAUNCH_CHECK(ctx, "k_entries_write");
