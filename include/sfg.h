@@ -41,7 +41,7 @@ typedef enum {
     SFG_EINVAL = 1,       /* bad argument: range, NULL, size, non-finite or non-positive weight */
     SFG_ENOMEM = 2,       /* device allocation failed */
     SFG_ECUDA = 3,        /* a CUDA runtime call failed */
-    SFG_ETIMEOUT = 4,     /* an iteration limit ran out before convergence */
+    SFG_ETIMEOUT = 4,     /* an iteration limit ran out before convergence, or a bounded wait on the GPU */
     SFG_ECAPACITY = 5,    /* an output buffer is too small */
     SFG_EUNSUPPORTED = 6  /* valid but not implemented (e.g. an unsupported K / dtype pair) */
 } sfg_status;
@@ -80,6 +80,11 @@ SFG_API void sfg_ctx_destroy(sfg_ctx* ctx);
  * fails also trims and retries once); sfg_ctx_set_stream gives the kept blocks back to the pool. */
 SFG_API sfg_status sfg_ctx_trim(sfg_ctx* ctx);
 SFG_API sfg_status sfg_ctx_set_stream(sfg_ctx* ctx, void* cuda_stream);
+/* Calls whose kernels wait for one another across the GPU (the spanning forest, top-k and batched selection, the
+ * embedding of graphs that fit on chip) bound every wait by a clock of two seconds. A wait that runs out is
+ * reported as SFG_ETIMEOUT (once): by the call itself if it synchronises, else by the next call on the
+ * context that does (sfg_ctx_trim always does, so it can serve as a check). The results of the call in
+ * question are then not valid; a selection may hold ids of -1. */
 /* Text of the last error on this context ("" if none). Valid until the next call on ctx. */
 SFG_API const char* sfg_last_error(const sfg_ctx* ctx);
 

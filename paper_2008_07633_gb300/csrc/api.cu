@@ -147,9 +147,49 @@ void sfg_free(sfg_ctx* ctx, void* p) {
     if (p) cudaFreeAsync(p, ctx->stream);
 }
 
+// Status words of the grid barriers, one a context, in page-locked host memory that is never freed: a captured
+// launch may be replayed after its context is gone (its word may then belong to a later context).
+static std::mutex status_mu;
+static std::vector<int*> status_free;
+
+static int* status_take() {
+    std::lock_guard<std::mutex> lock(status_mu);
+    if (status_free.empty()) {
+        constexpr int kWords = 1024;
+        int* page = nullptr;
+        if (cudaHostAlloc((void**)&page, sizeof(int) * kWords, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        for (int i = 0; i < kWords; ++i) status_free.push_back(page + i);
+    }
+    int* w = status_free.back();
+    status_free.pop_back();
+    *(volatile int*)w = 0;
+    return w;
+}
+
+static void status_give(int* w) {
+    std::lock_guard<std::mutex> lock(status_mu);
+    if (w) status_free.push_back(w);
+}
+
+GridWait sfg_grid_wait(const sfg_ctx* ctx, const char* kernel) {
+    if (ctx->fault_barrier && ctx->fault_grid == kernel) return GridWait{ctx->grid_status, 20000000ull, ctx->fault_barrier};
+    return GridWait{ctx->grid_status, 2000000000ull, 0u};
+}
+
+sfg_status sfg_grid_check(sfg_ctx* ctx) {
+    volatile int* w = ctx->grid_status;
+    if (!*w) return SFG_OK;
+    *w = 0;
+    return sfg_fail(ctx, SFG_ETIMEOUT, "a launch whose CTAs wait for one another gave up: its results, or those of "
+                                       "an earlier call that did not synchronise, are not valid");
+}
+
 sfg_status sfg_wait(sfg_ctx* ctx) {
     SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return SFG_OK;
+    return sfg_grid_check(ctx);
 }
 
 sfg_status sfg_host_word(sfg_ctx* ctx, int slot, int** out) {
@@ -294,8 +334,17 @@ sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream) {
     c->kept.reserve(kKeptBlocks);  // giving a block back never allocates
     if (const char* f = std::getenv("SFG_FAULT_ALLOC")) c->fail_alloc_at = std::atoll(f);
     if (const char* f = std::getenv("SFG_FAULT_MMA_WAIT")) c->withhold_mma = std::atoi(f) != 0;
+    if (const char* f = std::getenv("SFG_FAULT_GRID_WAIT")) {
+        const char* colon = std::strchr(f, ':');
+        if (colon) {
+            c->fault_grid.assign(f, colon - f);
+            c->fault_barrier = (unsigned)std::atoi(colon + 1);
+        }
+    }
     c->pool = device_pool(device);
-    if (!c->pool) {
+    c->grid_status = status_take();
+    if (!c->pool || !c->grid_status) {
+        status_give(c->grid_status);
         delete c;
         return SFG_ECUDA;
     }
@@ -303,6 +352,7 @@ sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream) {
     // that holds it is loaded (and its memory taken) when a context is created, never inside
     // one of those calls.
     if (sfg_noalloc_prepare(c) != SFG_OK) {
+        status_give(c->grid_status);
         delete c;
         return SFG_ECUDA;
     }
@@ -314,7 +364,7 @@ sfg_status sfg_ctx_trim(sfg_ctx* ctx) {
     if (!ctx) return SFG_EINVAL;
     SFG_DEVICE(ctx);
     sfg_scratch_flush(ctx);
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     SFG_CUDA(ctx, cudaMemPoolTrimTo(ctx->pool, 0));
     return SFG_OK;
 }
@@ -337,6 +387,7 @@ void sfg_ctx_destroy(sfg_ctx* ctx) {
         cudaStreamSynchronize(ctx->stream);
         cudaMemPoolTrimTo(ctx->pool, 0);
     }
+    status_give(ctx->grid_status);
     delete ctx;
 }
 
@@ -353,7 +404,7 @@ const char* sfg_last_error(const sfg_ctx* ctx) { return ctx ? ctx->last_error.c_
 sfg_status sfg_ctx_timing(sfg_ctx* ctx, int on) {
     if (!ctx) return SFG_EINVAL;
     SFG_DEVICE(ctx);
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     for (auto& r : ctx->timers) {
         ctx->event_pool.push_back(r.start);
         ctx->event_pool.push_back(r.stop);
@@ -367,7 +418,7 @@ sfg_status sfg_ctx_kernel_time(sfg_ctx* ctx, const char* prefix, int64_t* launch
                                double* ms_host) {
     if (!ctx || !prefix || !launches_host || !ms_host) return SFG_EINVAL;
     SFG_DEVICE(ctx);
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     int64_t n = 0;
     double total = 0.0;
     size_t len = std::strlen(prefix);

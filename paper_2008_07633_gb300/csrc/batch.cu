@@ -332,7 +332,7 @@ static sfg_status batch_reorder(sfg_ctx* ctx, sfg_batch* b, int32_t* f2c) {
             k_bfs_step<<<gn, kBlock, 0, ctx->stream>>>(n, U->row_ptr, U->colval, depth, level, flag);
             ++ctx->launches;
             SFG_CUDA(ctx, cudaMemcpyAsync(hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-            SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+            SFG_TRY(sfg_wait(ctx));
             if (!*hflag) break;
         }
         if (pass == 0) {
@@ -449,7 +449,7 @@ static sfg_status batch_build(sfg_ctx* ctx, int ng, const sfg_graph* const* gs, 
         SFG_LAUNCH_CHECK(ctx, "k_seg_count");
     }
     SFG_CUDA(ctx, cudaMemcpyAsync(tree.data(), d_cnt, 8 * ng, cudaMemcpyDeviceToHost, ctx->stream));
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
 
     // per-graph budgets (each graph's P starts as its forest: no edge is over budget)
     std::vector<int64_t> kk(ng), coff(ng + 1, 0);
@@ -486,7 +486,7 @@ static sfg_status batch_build(sfg_ctx* ctx, int ng, const sfg_graph* const* gs, 
             SFG_TRY(sfg_autotune_impl(ctx, b->PU, P->K, P->storage, nullptr, nullptr));
         }
     }
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     return SFG_OK;
 }
 
@@ -587,7 +587,7 @@ sfg_status sfg_sparsify_batched(sfg_ctx* ctx, int ng, const sfg_graph* const* gs
         ++ctx->launches;
         SFG_LAUNCH_CHECK(ctx, "k_split");
     }
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));  // d_outs' host source goes out of scope
+    SFG_TRY(sfg_wait(ctx));  // d_outs' host source goes out of scope
     if (n_selected_host)
         for (int g = 0; g < ng; ++g) n_selected_host[g] = b->counts[(size_t)g];
     return SFG_OK;

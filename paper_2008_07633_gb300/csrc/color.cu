@@ -215,7 +215,7 @@ sfg_status sfg_gs_prepare(sfg_ctx* ctx, const sfg_graph* Lc) {
         }
         int hmax = 0;
         SFG_CUDA(ctx, cudaMemcpyAsync(&hmax, maxc, sizeof(int), cudaMemcpyDeviceToHost, st));
-        SFG_CUDA(ctx, cudaStreamSynchronize(st));
+        SFG_TRY(sfg_wait(ctx));
         const int32_t ncolors = hmax + 1;
         uint64_t *k1, *k2;
         uint32_t *v1, *v2;
@@ -237,7 +237,7 @@ sfg_status sfg_gs_prepare(sfg_ctx* ctx, const sfg_graph* Lc) {
         off.assign((size_t)ncolors + 1, 0);
         SFG_CUDA(ctx, cudaMemcpyAsync(off.data(), doff, sizeof(int64_t) * (ncolors + 1),
                                       cudaMemcpyDeviceToHost, st));
-        SFG_CUDA(ctx, cudaStreamSynchronize(st));
+        SFG_TRY(sfg_wait(ctx));
     }
     own.keep = true;
     L->gs_color = color;

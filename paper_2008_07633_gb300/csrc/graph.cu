@@ -995,7 +995,7 @@ static sfg_status build_by_sort(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     if (validate) {
         int herr = 0;
         SFG_CUDA(ctx, cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-        SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        SFG_TRY(sfg_wait(ctx));
         if (herr)
             return sfg_fail(ctx, SFG_EINVAL,
                             "edge list: endpoint outside [0, n) or weight not finite and > 0");
@@ -1094,7 +1094,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     }
     SFG_CUDA(ctx, cudaMemcpyAsync(hw, words, sizeof(unsigned long long) * kWCount, cudaMemcpyDeviceToHost,
                                   ctx->stream));
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     if (validate && hw[kWErr])
         return sfg_fail(ctx, SFG_EINVAL,
                         "edge list: endpoint outside [0, n) or weight not finite and > 0");
@@ -1161,7 +1161,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     SFG_LAUNCH_CHECK(ctx, "k_row_index");
     SFG_CUDA(ctx, cudaMemcpyAsync(hw, words, sizeof(unsigned long long) * kWCount, cudaMemcpyDeviceToHost,
                                   ctx->stream));
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     const int64_t entries = (int64_t)hw[kWNnz], mc = (int64_t)hw[kWEdges];
     g->m = mc;
     SFG_TRY(sfg_alloc(ctx, (void**)&g->eu, sizeof(int32_t) * mc + 16));

@@ -4,16 +4,23 @@
 // the grid size (acquire); with the CTA barriers around it every thread's earlier writes come before
 // any thread's later reads, so plain loads after the barrier see the other CTAs' stores (data that the
 // kernel itself writes must not be read through const __restrict__ pointers). The wait is bounded by the global
-// timer (about two seconds): a run-out sets the error word and the CTA returns (the others' waits then
-// run out too).
+// timer (two seconds): a run-out sets the context's status word, which the host reads at its next wait for
+// the stream (sfg_wait), and the CTA returns; the others' next waits then run out too.
 // Costs 1-2 us on 16-608 CTAs, against 2-3 us from the end of one launch to the work of the next (with full
 // fences around the count instead of release and acquire 0.4 us more).
 #pragma once
 #include <cstdint>
 
+// What a launch's barriers need from the host (sfg_grid_wait).
+struct GridWait {
+    int* status;        // host memory: set when a wait ran out
+    uint64_t limit_ns;
+    unsigned withhold;  // barrier (counted from 1) at which the last CTA does not arrive; 0 unless a test asks
+};
+
 struct GridBar {
     unsigned* count;  // zero at launch; one word per launch
-    int* err;         // set when a wait ran out
+    GridWait wait;
 };
 
 __device__ __forceinline__ uint64_t gridbar_ns() {
@@ -29,23 +36,30 @@ __device__ __forceinline__ bool grid_barrier(const GridBar& b, unsigned& round) 
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned want = (round + 1) * gridDim.x;
-        // release: the CTA's writes (ordered before by the barrier above) before the count
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(b.count) : "memory");
         int ok = 1;
-        uint64_t t0 = 0;
-        for (unsigned spin = 0;; ++spin) {
-            unsigned now;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(b.count) : "memory");
-            if (now >= want) break;
-            if ((spin & 255u) == 255u) {
-                const uint64_t t = gridbar_ns();
-                if (t0 == 0) t0 = t;
-                if (t - t0 > 2000000000ull) {
-                    atomicExch(b.err, 1);
-                    ok = 0;
-                    break;
+        if (b.wait.withhold == round + 1 && blockIdx.x == gridDim.x - 1) {
+            ok = 0;
+        } else {
+            // release: the CTA's writes (ordered before by the barrier above) before the count
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(b.count) : "memory");
+            uint64_t t0 = 0;
+            for (unsigned spin = 0;; ++spin) {
+                unsigned now;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(b.count) : "memory");
+                if (now >= want) break;
+                if ((spin & 255u) == 255u) {
+                    const uint64_t t = gridbar_ns();
+                    if (t0 == 0) t0 = t;
+                    if (t - t0 > b.wait.limit_ns) {
+                        ok = 0;
+                        break;
+                    }
                 }
             }
+        }
+        if (!ok) {
+            *(volatile int*)b.wait.status = 1;
+            __threadfence_system();
         }
         s_bar_ok = ok;
     }

@@ -685,7 +685,7 @@ sfg_status factorise(sfg_ctx* ctx, Scratch& s, const sfg_graph* P, Factor& F) {
         if (nseg > 0)
             SFG_CUDA(ctx, cudaMemcpyAsync(sr.data(), seg_round, sizeof(int32_t) * nseg,
                                           cudaMemcpyDeviceToHost, st));
-        SFG_CUDA(ctx, cudaStreamSynchronize(st));
+        SFG_TRY(sfg_wait(ctx));
         int64_t i = 0;
         for (int r = 0; r < F.rounds; ++r) {
             F.round_seg[r] = i;
@@ -806,7 +806,7 @@ struct Solver {
         SFG_LAUNCH_CHECK(ctx, "k_cg_init");
         double h[8];
         SFG_CUDA(ctx, cudaMemcpyAsync(h, sc, sizeof(double) * 8, cudaMemcpyDeviceToHost, st));
-        SFG_CUDA(ctx, cudaStreamSynchronize(st));
+        SFG_TRY(sfg_wait(ctx));
         bool ok = h[7] != 0.0;
         for (int it = 0; !ok && it < cg_max;) {
             for (int k = 0; k < 16; ++k, ++it) {
@@ -819,7 +819,7 @@ struct Solver {
             }
             SFG_LAUNCH_CHECK(ctx, "core CG");
             SFG_CUDA(ctx, cudaMemcpyAsync(h, sc, sizeof(double) * 8, cudaMemcpyDeviceToHost, st));
-            SFG_CUDA(ctx, cudaStreamSynchronize(st));
+            SFG_TRY(sfg_wait(ctx));
             cg_iters += 16;
             ok = h[7] != 0.0 && h[3] == h[3];
             if (h[7] != 0.0) break;
@@ -1004,7 +1004,7 @@ sfg_status kappa_impl(sfg_ctx* ctx, const sfg_graph* G, const uint8_t* mask, int
     };
     auto rd = [&](double* h, const double* d, int k) -> sfg_status {
         SFG_CUDA(ctx, cudaMemcpyAsync(h, d, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
-        SFG_CUDA(ctx, cudaStreamSynchronize(st));
+        SFG_TRY(sfg_wait(ctx));
         return SFG_OK;
     };
     // v0: seeded, u0 = L_P v0, both scaled to unit L_P-norm
@@ -1146,7 +1146,7 @@ struct CompMean {
         std::vector<int64_t> hs(nseg + 1), hb;
         SFG_CUDA(ctx, cudaMemcpyAsync(hs.data(), seg_start, sizeof(int64_t) * (nseg + 1),
                                       cudaMemcpyDeviceToHost, st));
-        SFG_CUDA(ctx, cudaStreamSynchronize(st));
+        SFG_TRY(sfg_wait(ctx));
         SFG_LAUNCH_CHECK(ctx, "component segments");
         for (int64_t i = 0; i < nseg; ++i)
             if (hs[i + 1] - hs[i] >= kBigSeg) hb.push_back(i);
@@ -1155,7 +1155,7 @@ struct CompMean {
             SFG_TRY(s.get(&big, nbig));
             SFG_CUDA(ctx, cudaMemcpyAsync(big, hb.data(), sizeof(int64_t) * nbig,
                                           cudaMemcpyHostToDevice, st));
-            SFG_CUDA(ctx, cudaStreamSynchronize(st));
+            SFG_TRY(sfg_wait(ctx));
         }
         return SFG_OK;
     }
@@ -1217,7 +1217,7 @@ sfg_status pcg_impl(sfg_ctx* ctx, const sfg_graph* G, const uint8_t* mask, const
         ctx->launches += 2;
         SFG_LAUNCH_CHECK(ctx, "dot");
         SFG_CUDA(ctx, cudaMemcpyAsync(out_host, sc, sizeof(double), cudaMemcpyDeviceToHost, st));
-        SFG_CUDA(ctx, cudaStreamSynchronize(st));
+        SFG_TRY(sfg_wait(ctx));
         return SFG_OK;
     };
     // The recursive residual drifts off range(L_G) by rounding while it shrinks, which would make

@@ -723,7 +723,7 @@ static sfg_status mlp_read_loss(sfg_ctx* ctx, const sfg_mlp* net, const double* 
     SFG_TRY(sfg_host_word(ctx, kSfgHostBuild, &hw));  // pinned: no staging copy
     double* h = reinterpret_cast<double*>(hw);
     SFG_CUDA(ctx, cudaMemcpyAsync(h, loss2, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     *loss_host = h[0];
     return h[1] != 0.0 ? sfg_mlp_check_impl(ctx, net) : SFG_OK;  // reports and clears the word
 }

@@ -47,7 +47,7 @@ __global__ void k_mst_init(int32_t n, int32_t* __restrict__ comp) {
 constexpr int kMstTiles = 2, kMstLong = 32, kMstSorted = 15, kMstAhead = 5;
 constexpr int kMstLanes = 8, kMstGroups = 32 / kMstLanes, kMstItems = 4;
 
-// Words of one launch: barrier count, error, edges taken, last pointer-jumping pass with work left,
+// Words of one launch: barrier count, rounds that ran out, edges taken, last pointer-jumping pass with work left,
 // lengths of the two label lists.
 enum { kMwBar, kMwErr, kMwTree, kMwJump, kMwLabels0, kMwLabels1, kMwCount };
 
@@ -72,6 +72,7 @@ struct MstArgs {
     int32_t* labels[2];         // labels of the components that still had an edge, this round's and the next's
     uint8_t* mask;
     unsigned long long* words;
+    GridWait wait;
 };
 
 // Pointer jumping in place: every node climbs up to kHops parents and stores the ancestor it
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mst(MstArgs A) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % kMstLanes, grp = lane / kMstLanes;
     const int64_t t0 = (int64_t)blockIdx.x * kBlock + threadIdx.x, nt = (int64_t)gridDim.x * kBlock;
     const int64_t items = (int64_t)A.n + A.nseg;
-    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kMwBar), reinterpret_cast<int*>(A.words + kMwErr)};
+    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kMwBar), A.wait};
     unsigned passed = 0;
     for (int64_t p = t0; p < A.n; p += nt) {
         A.comp[p] = (int32_t)p;
@@ -506,7 +507,7 @@ sfg_status sfg_pointer_jump(sfg_ctx* ctx, int32_t n, int32_t* parent) {
         sfg_toc(ctx);
         SFG_LAUNCH_CHECK(ctx, "k_jump_inplace");
         SFG_CUDA(ctx, cudaMemcpyAsync(h, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-        SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        SFG_TRY(sfg_wait(ctx));
         if (!*h) return SFG_OK;
     }
     return sfg_fail(ctx, SFG_ETIMEOUT, "pointer jumping did not converge");
@@ -570,6 +571,7 @@ sfg_status sfg_mst_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* allow, 
     a.key_id = key_id;
     a.key_inv = key_inv;
     a.mask = mask;
+    a.wait = sfg_grid_wait(ctx, "k_mst");
     void* args[] = {(void*)&a};
     const int grid = sfg_grid(ctx, (const void*)k_mst, kBlock, 0, items);
     sfg_tic(ctx, "mst");
@@ -583,7 +585,7 @@ sfg_status sfg_mst_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* allow, 
                                       ctx->stream));
     SFG_CUDA(ctx, cudaMemcpyAsync(hw, a.words, sizeof(unsigned long long) * kMwCount, cudaMemcpyDeviceToHost,
                                   ctx->stream));
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     if (hw[kMwErr]) return sfg_fail(ctx, SFG_ETIMEOUT, "spanning forest did not converge in 64 rounds");
     if (n_tree) *n_tree = (int64_t)hw[kMwTree];
     return SFG_OK;

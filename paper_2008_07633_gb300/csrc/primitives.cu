@@ -293,6 +293,6 @@ sfg_status sfg_radix_sort_pairs(sfg_ctx* ctx, uint64_t** keys, uint32_t** vals,
 
 sfg_status sfg_read_i64(sfg_ctx* ctx, const int64_t* dev, int64_t* host) {
     SFG_CUDA(ctx, cudaMemcpyAsync(host, dev, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     return SFG_OK;
 }

@@ -33,8 +33,8 @@ constexpr int kTkPasses = 6, kTkBins = 2048, kTkUnroll = 8;
 __host__ __device__ constexpr int tk_shift(int pass) { return pass % 3 == 0 ? 21 : pass % 3 == 1 ? 10 : 0; }
 __host__ __device__ constexpr int tk_width(int pass) { return pass % 3 == 2 ? 10 : 11; }
 
-// Words of one launch: barrier count, error, ids out of order.
-enum { kTwBar, kTwErr, kTwOrder, kTwCount };
+// Words of one launch: barrier count, ids out of order.
+enum { kTwBar, kTwOrder, kTwCount };
 
 struct TkArgs {
     int64_t ne, k;
@@ -48,6 +48,7 @@ struct TkArgs {
     int sort_ctas;
     int32_t* tmp;               // k
     int32_t* out;               // k
+    GridWait wait;
 };
 
 struct TkPick {
@@ -175,7 +176,8 @@ __device__ bool tk_sort_ids(const TkArgs& A, const GridBar& bar, unsigned& passe
     return true;  // an even number of passes: the result is in out
 }
 
-// A barrier ran out: no selection; every CTA leaves -1 in its share of the list.
+// A barrier ran out (the status word says so): no selection; every CTA leaves -1 in its share of the list, so
+// that no entry is an unwritten one.
 __device__ void tk_give_up(const TkArgs& A) {
     for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < A.k; i += (int64_t)gridDim.x * kBlock)
         A.out[i] = -1;
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_topk(TkArgs A) {
     __shared__ unsigned h[kTkBins];
     const int tid = threadIdx.x, lane = tid & 31;
     const int64_t t0 = (int64_t)blockIdx.x * kBlock + tid, nt = (int64_t)gridDim.x * kBlock;
-    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kTwBar), reinterpret_cast<int*>(A.words + kTwErr)};
+    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kTwBar), A.wait};
     unsigned passed = 0;
     long long krem = A.k;
     uint32_t word[2] = {0u, 0u};  // the threshold key's score image and complemented id
@@ -316,6 +318,7 @@ sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, 
     a.words = zeroed + (size_t)kTkPasses * kTkBins;
     a.sort_ctas = sort_ctas;
     a.out = list;
+    a.wait = sfg_grid_wait(ctx, "k_topk");
     void* args[] = {(void*)&a};
     sfg_tic(ctx, "topk");
     const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_topk, dim3(grid), dim3(kBlock), args, 0,
@@ -363,7 +366,7 @@ struct SegSel {
     long long krem;
 };
 
-enum { kSwBar, kSwErr, kSwOpen, kSwCount };
+enum { kSwBar, kSwOpen, kSwCount };
 
 struct SegArgs {
     int64_t ne;
@@ -376,6 +379,7 @@ struct SegArgs {
     unsigned* hist;             // nseg x kSgBins, zero at launch
     unsigned long long* words;  // zero at launch
     uint8_t* mask;
+    GridWait wait;
 };
 
 __device__ __forceinline__ int seg_of(const int64_t* __restrict__ off, int nseg, int64_t i) {
@@ -391,7 +395,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_topk_seg(SegArgs A) {
     __shared__ unsigned h[kSgBins];
     __shared__ long long ws[kBlock / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kSwBar), reinterpret_cast<int*>(A.words + kSwErr)};
+    const GridBar bar{reinterpret_cast<unsigned*>(A.words + kSwBar), A.wait};
     unsigned passed = 0;
     const int64_t per = (A.ne + gridDim.x - 1) / gridDim.x;
     const int64_t lo = min(A.ne, (int64_t)blockIdx.x * per), hi = min(A.ne, lo + per);
@@ -504,6 +508,7 @@ sfg_status sfg_topk_segmented_mark(sfg_ctx* ctx, const float* scores, const int3
     a.off = seg_off;
     a.k = k_dev;
     a.mask = mask;
+    a.wait = sfg_grid_wait(ctx, "k_topk_seg");
     void* args[] = {(void*)&a};
     const int grid = sfg_grid(ctx, (const void*)k_topk_seg, kBlock, 0, (ne + 3) / 4);
     sfg_tic(ctx, "topk");

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/sfg.h"
+#include "gridbar.cuh"
 
 // ------------------------------------------------------------------------------------------------
 // Context: device, borrowed stream, last error text, optional per-kernel event timers.
@@ -49,6 +50,9 @@ struct sfg_ctx {
     int64_t fail_alloc_at = -1;            // SFG_FAULT_ALLOC=<n>: the n-th allocation fails
     bool withhold_mma = false;             // SFG_FAULT_MMA_WAIT=1: tensor-core kernels issue no
                                            // MMA, so their bounded completion waits run out
+    int* grid_status = nullptr;            // host word that grid barriers set when a wait runs out
+    std::string fault_grid;                // SFG_FAULT_GRID_WAIT=<kernel>:<n>: at the n-th barrier of
+    unsigned fault_barrier = 0;            // that kernel one CTA does not arrive (waits of 20 ms)
 };
 
 struct sfg_graph {
@@ -207,8 +211,12 @@ sfg_status sfg_scan_i64(sfg_ctx* ctx, const int64_t* in, int64_t* out, int64_t n
 sfg_status sfg_radix_sort_pairs(sfg_ctx* ctx, uint64_t** keys, uint32_t** vals,
                                 uint64_t** keys_alt, uint32_t** vals_alt, int64_t n, int bits);
 // Wait for the context's stream: the last step of every entry point that is documented to synchronise, so
-// that what it made may be used from any stream, and its inputs released, when it returns.
+// that what it made may be used from any stream, and its inputs released, when it returns. Like every wait of
+// the library it reports a grid barrier that has run out since the last one (sfg_grid_check: SFG_ETIMEOUT, once).
 sfg_status sfg_wait(sfg_ctx* ctx);
+sfg_status sfg_grid_check(sfg_ctx* ctx);
+// The barrier limits of a cooperative launch of `kernel`.
+GridWait sfg_grid_wait(const sfg_ctx* ctx, const char* kernel);
 // Copy scalars back (synchronises the stream).
 sfg_status sfg_read_i64(sfg_ctx* ctx, const int64_t* dev, int64_t* host);
 

@@ -530,7 +530,7 @@ sfg_status heavy_prepare(sfg_ctx* ctx, const sfg_graph* Lc) {
     SFG_LAUNCH_CHECK(ctx, "k_heavy_mark");
     int hcount = 0;
     SFG_CUDA(ctx, cudaMemcpyAsync(&hcount, count, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SFG_TRY(sfg_wait(ctx));
     if (hcount == 0) {  // the common case on meshes: one pass over row_ptr, one readback
         L->hv_nseg = 0;
         L->hv_n = 0;
@@ -717,7 +717,7 @@ sfg_status gs_heavy_prepare(sfg_ctx* ctx, const sfg_graph* Lc) {
         SFG_LAUNCH_CHECK(ctx, "k_heavy_gather");
         SFG_CUDA(ctx, cudaMemcpyAsync(h4.data(), dev4, sizeof(int32_t) * 4 * nh, cudaMemcpyDeviceToHost,
                                       ctx->stream));
-        SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        SFG_TRY(sfg_wait(ctx));
     }
     // stable by colour: hv_rows are in id order, so each class keeps increasing ids
     std::vector<int32_t> ord(nh);
@@ -759,7 +759,7 @@ sfg_status gs_heavy_prepare(sfg_ctx* ctx, const sfg_graph* Lc) {
                                   ctx->stream));
     SFG_CUDA(ctx, cudaMemcpyAsync(dseg, gseg.data(), sizeof(int4) * gseg.size(), cudaMemcpyHostToDevice,
                                   ctx->stream));
-    SFG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));  // the host arrays go out of scope
+    SFG_TRY(sfg_wait(ctx));  // the host arrays go out of scope
     L->gh_ready = true;
     return SFG_OK;
 }
@@ -869,7 +869,8 @@ __global__ void k_coef(int32_t n, const double* __restrict__ invdeg, double omeg
 // are swept side by side by the two halves of the grid. Rows, statistics slots and orders of
 // summation are those of k_init, k_jacobi (default shape) and k_finalize, so the bits are theirs.
 // Taken when both halves are resident together (see small_fits) and no row is a hub row: beyond
-// that the separate launches overlap their ends well enough. Filter + score + select of a 17,280-node
+// that the separate launches overlap their ends well enough. A barrier that runs out leaves the results unset
+// and the status word set. Filter + score + select of a 17,280-node
 // mesh (K = 16, 15 steps): 192 us with separate launches, 113 us so.
 // ------------------------------------------------------------------------------------------------
 template <typename T>
@@ -891,7 +892,8 @@ struct SmallArgs {
     float* mu;
     float* mean[2];
     float* scale[2];
-    unsigned* words;              // barrier count and error, zero at launch
+    unsigned* count;              // barrier count, zero at launch
+    GridWait wait;
 };
 
 template <typename T, int LPR>
@@ -902,13 +904,10 @@ __global__ void __launch_bounds__(kBlock, 4) k_small(SmallArgs<T> A) {
     const int side = (int)blockIdx.x >= A.grid ? 1 : 0, cta = (int)blockIdx.x - side * A.grid;
     const int32_t wid = (int32_t)((cta * kBlock + threadIdx.x) >> 5);
     const int32_t ntiles = (A.n + GPW - 1) / GPW;
-    const GridBar bar{A.words, reinterpret_cast<int*>(A.words + 1)};
+    const GridBar bar{A.count, A.wait};
     unsigned passed = 0;
     const int32_t* row_ptr = A.row_ptr[side];
     const int2* colval = A.colval[side];
-    auto give_up = [&] {  // a barrier ran out: the scales, and with them every result, become NaN
-        for (int k = threadIdx.x; k < K; k += kBlock) A.scale[side][k] = __int_as_float(0x7fffffff);
-    };
     // this group's row in tile t
     struct Row { int32_t r, a, b; float cp; };
     auto load_row = [&](int32_t t) {
@@ -926,13 +925,13 @@ __global__ void __launch_bounds__(kBlock, 4) k_small(SmallArgs<T> A) {
     if (side == 0)
         init_rows<T, LPR, true>(A.n, A.seed, A.deg, ((int64_t)cta * kBlock + threadIdx.x) / LPR,
                                 (int64_t)A.grid * kBlock / LPR, A.x0, A.part);
-    if (!grid_barrier(bar, passed)) return give_up();
+    if (!grid_barrier(bar, passed)) return;
     if (side == 0)
         for (int k = cta; k < K; k += A.grid) {
             finalize_column(A.part, A.grid, K, k, A.n, 2, A.mu, nullptr);
             __syncthreads();
         }
-    if (!grid_barrier(bar, passed)) return give_up();
+    if (!grid_barrier(bar, passed)) return;
     const float a_self = (float)(1.0 - A.omega);
     float s1[E], s2[E];
 #pragma unroll
@@ -973,7 +972,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_small(SmallArgs<T> A) {
     for (int t = 1; t < A.steps; ++t) {
         T* nxt = A.buf[side][(t - 1) & 1];
         tile(row, ch, cur, nxt, t == 1, false);
-        if (!grid_barrier(bar, passed)) return give_up();
+        if (!grid_barrier(bar, passed)) return;
         cur = nxt;
     }
     // the last sweep with its statistics, in the tile order of k_jacobi's default shape
@@ -988,13 +987,13 @@ __global__ void __launch_bounds__(kBlock, 4) k_small(SmallArgs<T> A) {
         tile(w, c, cur, last, A.steps == 1, true);
     }
     block_column_partials<LPR, E>(s1, s2, A.part);
-    if (!grid_barrier(bar, passed)) return give_up();
+    if (!grid_barrier(bar, passed)) return;
     for (int k = cta; k < K; k += A.grid) {
         finalize_column(A.part + (size_t)side * A.grid * 2 * K, A.grid, K, k, A.n, 1, A.mean[side], A.scale[side]);
         __syncthreads();
     }
     if (A.sides == 2) return;
-    if (!grid_barrier(bar, passed)) return give_up();
+    if (!grid_barrier(bar, passed)) return;
     if (row.r < A.n) {
         float x[E];
         Vec<T>::load(last + (int64_t)row.r * K + sub * E, x);
@@ -1229,7 +1228,8 @@ struct Smoother {
 
     static sfg_status launch_small(sfg_ctx* ctx, SmallArgs<T>& a) {
         void* args[] = {(void*)&a};
-        SFG_CUDA(ctx, cudaMemsetAsync(a.words, 0, 2 * sizeof(unsigned), ctx->stream));
+        SFG_CUDA(ctx, cudaMemsetAsync(a.count, 0, sizeof(unsigned), ctx->stream));
+        a.wait = sfg_grid_wait(ctx, "k_small");
         sfg_tic(ctx, "small");
         const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_small<T, LPR>, dim3(a.sides * a.grid),
                                                           dim3(kBlock), args, 0, ctx->stream);
@@ -1307,7 +1307,7 @@ struct Smoother {
         SFG_TRY(heavy_prepare(ctx, L));
         if (small_fits(ctx, 1, steps, grid, L, nullptr)) {
             SmallArgs<T> a{};
-            SFG_TRY(s.get(&a.words, 2));
+            SFG_TRY(s.get(&a.count, 1));
             SFG_TRY(s.get(&a.mean[0], K));
             a.n = n, a.grid = grid, a.sides = 1, a.steps = steps, a.omega = omega, a.seed = seed;
             a.deg = L->deg, a.row_ptr[0] = L->row_ptr, a.colval[0] = L->colval, a.invdeg[0] = L->invdeg;
@@ -1483,7 +1483,7 @@ struct Smoother {
         SFG_TRY(heavy_prepare(ctx, LP));
         if (small_fits(ctx, 2, steps, grid, LG, LP)) {
             SmallArgs<T> a{};
-            SFG_TRY(s.get(&a.words, 2));
+            SFG_TRY(s.get(&a.count, 1));
             SFG_TRY(s.get(&a.part, (size_t)2 * grid * 2 * K));
             a.n = n, a.grid = grid, a.sides = 2, a.steps = steps, a.omega = omega, a.seed = seed;
             a.deg = LG->deg, a.x0 = x0, a.mu = mu;

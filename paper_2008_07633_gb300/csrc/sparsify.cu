@@ -337,6 +337,7 @@ extern "C" sfg_status sfg_sparsify_learned(sfg_ctx* ctx, const sfg_graph* G, con
         ++ctx->launches;
         SFG_LAUNCH_CHECK(ctx, "k_set_mask");
         SFG_TRY(sfg_mlp_check_impl(ctx, net));
+        SFG_TRY(sfg_grid_check(ctx));
     }
     if (n_selected_host) SFG_TRY(sfg_count_mask(ctx, mask_out, m, n_selected_host));
     return SFG_OK;
