@@ -1,5 +1,5 @@
 // Context, status, allocation and timing plumbing of libsfg.
-#include <atomic>
+#include <algorithm>
 #include <cstdarg>
 #include <cstdlib>
 #include <cstring>
@@ -34,12 +34,113 @@ static bool alloc_fails(sfg_ctx* ctx) {
     return ctx->fail_alloc_at >= 0 && ctx->alloc_count == ctx->fail_alloc_at;
 }
 
-static sfg_status pool_alloc(sfg_ctx* ctx, void** p, size_t bytes) {
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
-    if (e == cudaErrorMemoryAllocation) {
-        // the pool keeps freed memory; hand it back to the device and try once more
+bool sfg_capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {  // the legacy stream while another one is captured
         cudaGetLastError();
-        sfg_scratch_flush(ctx);
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+constexpr size_t kKeptBlocks = 96;
+constexpr int kKeptDevices = 64;
+constexpr int64_t kKeptShare = 128, kKeptDeviceShare = 32;  // of a device's memory: a context's, all contexts' together
+
+// What the contexts of one device keep together.
+struct KeptDevice {
+    std::mutex mu;  // guards the fields here and the contexts' lists
+    std::once_flag once;
+    int64_t room = 0, all = 0;       // bytes that may still be kept, and before any is
+    std::vector<sfg_ctx*> contexts;
+    cudaStream_t frees = nullptr;    // the library's own: gives blocks back after their event, never on a user's stream
+};
+static KeptDevice kept_devices[kKeptDevices];
+
+static KeptDevice& kept_device(const sfg_ctx* ctx) { return kept_devices[ctx->device]; }
+
+// A context that is not registered (no room for its device's number, no event, no stream of the library's own)
+// keeps nothing.
+static void kept_register(sfg_ctx* ctx) {
+    if (ctx->device >= kKeptDevices) return;
+    KeptDevice& d = kept_device(ctx);
+    std::call_once(d.once, [&d] {
+        size_t unused = 0, total = 0;
+        if (cudaMemGetInfo(&unused, &total) == cudaSuccess &&
+            cudaStreamCreateWithFlags(&d.frees, cudaStreamNonBlocking) == cudaSuccess)
+            d.room = d.all = (int64_t)total / kKeptDeviceShare;
+        else cudaGetLastError();
+    });
+    if (!d.frees || cudaEventCreateWithFlags(&ctx->kept_event, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->kept_event = nullptr;
+        return;
+    }
+    std::lock_guard<std::mutex> lock(d.mu);
+    ctx->kept.reserve(kKeptBlocks);
+    d.contexts.push_back(ctx);
+}
+
+static SfgKept kept_remove(sfg_ctx* ctx, size_t i) {  // with the device's lock
+    const SfgKept b = ctx->kept[i];
+    kept_device(ctx).room += (int64_t)b.bytes;
+    ctx->kept_bytes -= (int64_t)b.bytes;
+    ctx->kept.erase(ctx->kept.begin() + i);
+    return b;
+}
+
+// Gives back what can be waited for without the context's stream, in the order of the event.
+static void kept_release(sfg_ctx* ctx) {  // with the device's lock
+    KeptDevice& d = kept_device(ctx);
+    bool first = true;
+    for (size_t i = ctx->kept.size(); i-- > 0;) {
+        if (!ctx->kept[i].settled) continue;
+        if (first && cudaStreamWaitEvent(d.frees, ctx->kept_event, 0) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        first = false;
+        cudaFreeAsync(kept_remove(ctx, i).p, d.frees);
+    }
+}
+
+// The same in the order of the context's stream, which has to be alive and not captured.
+static void kept_free(sfg_ctx* ctx) {  // with the device's lock
+    for (size_t i = ctx->kept.size(); i-- > 0;) cudaFreeAsync(kept_remove(ctx, i).p, ctx->stream);
+}
+
+// An allocation has failed: everything that any context of the device keeps goes back to the pool.
+static void kept_reclaim(sfg_ctx* ctx) {
+    if (!ctx->kept_event) return;
+    KeptDevice& d = kept_device(ctx);
+    {
+        std::lock_guard<std::mutex> lock(d.mu);
+        if (!sfg_capturing(ctx->stream)) kept_free(ctx);
+        for (sfg_ctx* c : d.contexts) kept_release(c);
+    }
+    cudaStreamSynchronize(d.frees);
+}
+
+static void set_stream(sfg_ctx* ctx, cudaStream_t stream) {
+    unsigned long long id = 0;
+    const bool known = cudaStreamGetId(stream, &id) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    if (ctx->kept_event && (!known || id != ctx->stream_id)) {
+        std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
+        kept_release(ctx);
+    }
+    ctx->stream = stream;
+    ctx->stream_id = id;
+    ctx->stream_keeps = known && ctx->kept_event && stream != cudaStreamPerThread;
+}
+
+static sfg_status pool_alloc(sfg_ctx* ctx, void** p, size_t bytes) {
+    cudaError_t e = ctx->alloc_count == ctx->fail_pool_at ? cudaErrorMemoryAllocation
+                                                          : cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    if (e == cudaErrorMemoryAllocation) {
+        // the contexts keep scratch and the pool freed memory; hand it back to the device and try once more
+        cudaGetLastError();
+        kept_reclaim(ctx);
         cudaStreamSynchronize(ctx->stream);
         cudaMemPoolTrimTo(ctx->pool, 0);
         e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
@@ -63,84 +164,60 @@ sfg_status sfg_alloc(sfg_ctx* ctx, void** p, size_t bytes) {
     return pool_alloc(ctx, p, bytes);
 }
 
-bool sfg_capturing(cudaStream_t stream) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {  // the legacy stream while another one is captured
-        cudaGetLastError();
-        return true;
-    }
-    return st != cudaStreamCaptureStatusNone;
-}
-
-constexpr size_t kKeptBlocks = 96;
-constexpr int kKeptDevices = 64;
-constexpr int64_t kKeptShare = 128, kKeptDeviceShare = 32;  // of a device's memory: a context's, all contexts' together
-static std::atomic<int64_t> kept_room[kKeptDevices];  // bytes that the contexts of a device may still keep
-
-static int64_t kept_all[kKeptDevices];                // the same before any is kept
-
-static void kept_room_init(int device) {  // once per device
-    static std::once_flag once[kKeptDevices];
-    if (device >= kKeptDevices) return;
-    std::call_once(once[device], [device] {
-        size_t unused = 0, total = 0;
-        if (cudaMemGetInfo(&unused, &total) == cudaSuccess) kept_room[device] = kept_all[device] = (int64_t)total / kKeptDeviceShare;
-        else cudaGetLastError();
-    });
-}
-
-static bool kept_reserve(sfg_ctx* ctx, int64_t bytes) {
-    const int device = ctx->device;
-    if (device >= kKeptDevices || ctx->kept_bytes + bytes > kept_all[device] / (kKeptShare / kKeptDeviceShare)) return false;
-    if (kept_room[device].fetch_sub(bytes) < bytes) {
-        kept_room[device].fetch_add(bytes);
-        return false;
-    }
-    ctx->kept_bytes += bytes;
-    return true;
-}
-
-static SfgKept kept_remove(sfg_ctx* ctx, size_t i) {
-    const SfgKept b = ctx->kept[i];
-    kept_room[ctx->device].fetch_add((int64_t)b.bytes);
-    ctx->kept_bytes -= (int64_t)b.bytes;
-    ctx->kept.erase(ctx->kept.begin() + i);
-    return b;
-}
-
-// Frees kept block i in its stream's order; not while that stream is being captured.
-static bool kept_drop(sfg_ctx* ctx, size_t i) {
-    if (sfg_capturing(ctx->kept[i].stream)) return false;
-    const SfgKept b = kept_remove(ctx, i);
-    cudaFreeAsync(b.p, b.stream);
-    return true;
-}
-
-void sfg_scratch_flush(sfg_ctx* ctx) {
-    for (size_t i = ctx->kept.size(); i-- > 0;) kept_drop(ctx, i);
-}
-
 sfg_status sfg_scratch_take(sfg_ctx* ctx, void** p, size_t* bytes) {
     *p = nullptr;
     if (alloc_fails(ctx)) return alloc_injected(ctx);
-    size_t best = 0, size = SIZE_MAX;  // the smallest block that is large enough, if it is not much larger
-    for (size_t i = 0; i < ctx->kept.size(); ++i) {
-        const SfgKept& b = ctx->kept[i];
-        if (b.stream == ctx->stream && b.bytes >= *bytes && b.bytes < size) best = i, size = b.bytes;
+    {
+        std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
+        size_t best = 0, size = SIZE_MAX;  // the smallest block that is large enough, if it is not much larger
+        for (size_t i = 0; i < ctx->kept.size(); ++i) {
+            const size_t b = ctx->kept[i].bytes;
+            if (b >= *bytes && b < size) best = i, size = b;
+        }
+        if (size <= *bytes + *bytes / 4 + 4096) {
+            const SfgKept b = kept_remove(ctx, best);
+            *p = b.p;
+            *bytes = b.bytes;
+            return SFG_OK;
+        }
     }
-    if (size > *bytes + *bytes / 4 + 4096) return pool_alloc(ctx, p, *bytes);
-    const SfgKept b = kept_remove(ctx, best);
-    *p = b.p;
-    *bytes = b.bytes;
-    return SFG_OK;
+    return pool_alloc(ctx, p, *bytes);
 }
 
+// Keeps the block, the oldest ones making room; a block for which even all of the context's own would not make
+// room goes back to the pool at once and leaves them where they are.
 void sfg_scratch_give(sfg_ctx* ctx, void* p, size_t bytes) {
-    if (ctx->kept.size() >= kKeptBlocks) kept_drop(ctx, 0);  // the oldest goes first
-    bool room = ctx->kept.size() < kKeptBlocks && kept_reserve(ctx, (int64_t)bytes);
-    while (!room && !ctx->kept.empty() && kept_drop(ctx, 0)) room = kept_reserve(ctx, (int64_t)bytes);
-    if (room) ctx->kept.push_back({p, bytes, ctx->stream});
-    else sfg_free(ctx, p);
+    KeptDevice& d = kept_device(ctx);
+    const int64_t size = (int64_t)bytes, share = d.all / (kKeptShare / kKeptDeviceShare);
+    void* out[kKeptBlocks];
+    size_t nout = 0;
+    bool kept = false;
+    {
+        std::lock_guard<std::mutex> lock(d.mu);
+        if (size <= share && size <= d.room + ctx->kept_bytes) {
+            while (ctx->kept.size() >= kKeptBlocks || ctx->kept_bytes + size > share || size > d.room)
+                out[nout++] = kept_remove(ctx, 0).p;
+            ctx->kept.push_back({p, bytes, false});  // the list has its room from the start: nothing throws
+            ctx->kept_bytes += size;
+            d.room -= size;
+            ctx->kept_dirty = kept = true;
+        }
+    }
+    for (size_t i = 0; i < nout; ++i) sfg_free(ctx, out[i]);
+    if (!kept) sfg_free(ctx, p);
+}
+
+// At the end of a call: the context's event stands for the last use of everything it keeps. (Nothing is given
+// back while the stream is being captured, so the record is never part of a graph.)
+void sfg_scratch_settle(sfg_ctx* ctx) {
+    ctx->kept_dirty = false;
+    const bool ok = cudaEventRecord(ctx->kept_event, ctx->stream) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
+    for (size_t i = ctx->kept.size(); i-- > 0;) {
+        if (ok) ctx->kept[i].settled = true;
+        else sfg_free(ctx, kept_remove(ctx, i).p);
+    }
 }
 
 void sfg_free(sfg_ctx* ctx, void* p) {
@@ -327,12 +404,10 @@ sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream) {
     SfgDeviceGuard guard(device);
     sfg_ctx* c = new sfg_ctx();
     c->device = device;
-    c->stream = (cudaStream_t)cuda_stream;
     cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (c->num_sms < 1) c->num_sms = 1;
-    kept_room_init(device);
-    c->kept.reserve(kKeptBlocks);  // giving a block back never allocates
     if (const char* f = std::getenv("SFG_FAULT_ALLOC")) c->fail_alloc_at = std::atoll(f);
+    if (const char* f = std::getenv("SFG_FAULT_POOL")) c->fail_pool_at = std::atoll(f);
     if (const char* f = std::getenv("SFG_FAULT_MMA_WAIT")) c->withhold_mma = std::atoi(f) != 0;
     if (const char* f = std::getenv("SFG_FAULT_GRID_WAIT")) {
         const char* colon = std::strchr(f, ':');
@@ -356,6 +431,8 @@ sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream) {
         delete c;
         return SFG_ECUDA;
     }
+    kept_register(c);
+    set_stream(c, (cudaStream_t)cuda_stream);
     *out = c;
     return SFG_OK;
 }
@@ -363,7 +440,10 @@ sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream) {
 sfg_status sfg_ctx_trim(sfg_ctx* ctx) {
     if (!ctx) return SFG_EINVAL;
     SFG_DEVICE(ctx);
-    sfg_scratch_flush(ctx);
+    if (ctx->kept_event) {
+        std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
+        kept_free(ctx);
+    }
     SFG_TRY(sfg_wait(ctx));
     SFG_CUDA(ctx, cudaMemPoolTrimTo(ctx->pool, 0));
     return SFG_OK;
@@ -371,22 +451,28 @@ sfg_status sfg_ctx_trim(sfg_ctx* ctx) {
 
 void sfg_ctx_destroy(sfg_ctx* ctx) {
     if (!ctx) return;
-    SFG_DEVICE(ctx);
+    SfgDeviceGuard guard(ctx->device);
     for (auto& r : ctx->timers) {
         cudaEventDestroy(r.start);
         cudaEventDestroy(r.stop);
     }
     for (auto e : ctx->event_pool) cudaEventDestroy(e);
+    const bool capturing = sfg_capturing(ctx->stream);  // such a stream cannot be waited for
     if (ctx->host_word) {
-        cudaStreamSynchronize(ctx->stream);
+        if (!capturing) cudaStreamSynchronize(ctx->stream);
         cudaFreeHost(ctx->host_word);
     }
-    if (ctx->pool) {
-        sfg_scratch_flush(ctx);
-        // unused memory goes back to the device; memory of live graphs stays valid
-        cudaStreamSynchronize(ctx->stream);
-        cudaMemPoolTrimTo(ctx->pool, 0);
+    if (ctx->kept_event) {
+        KeptDevice& d = kept_device(ctx);
+        std::lock_guard<std::mutex> lock(d.mu);
+        if (capturing) kept_release(ctx);
+        else kept_free(ctx);
+        d.contexts.erase(std::find(d.contexts.begin(), d.contexts.end(), ctx));
+        cudaEventDestroy(ctx->kept_event);
     }
+    // unused memory goes back to the device; memory of live graphs stays valid
+    if (!capturing) cudaStreamSynchronize(ctx->stream);
+    cudaMemPoolTrimTo(ctx->pool, 0);
     status_give(ctx->grid_status);
     delete ctx;
 }
@@ -394,8 +480,7 @@ void sfg_ctx_destroy(sfg_ctx* ctx) {
 sfg_status sfg_ctx_set_stream(sfg_ctx* ctx, void* cuda_stream) {
     if (!ctx) return SFG_EINVAL;
     SFG_DEVICE(ctx);
-    if (ctx->stream != (cudaStream_t)cuda_stream) sfg_scratch_flush(ctx);
-    ctx->stream = (cudaStream_t)cuda_stream;
+    set_stream(ctx, (cudaStream_t)cuda_stream);
     return SFG_OK;
 }
 

@@ -23,11 +23,13 @@ struct sfg_timer_rec {
     cudaEvent_t start, stop;
 };
 
-// A scratch block that a context keeps after the call that used it, free for work on its stream.
+// A scratch block that a context keeps after the call that used it, free for work on its stream. settled: the
+// context's event has been recorded since it was given back, so that its last use can be waited for without
+// the stream.
 struct SfgKept {
     void* p;
     size_t bytes;
-    cudaStream_t stream;
+    bool settled;
 };
 
 struct sfg_ctx {
@@ -44,10 +46,18 @@ struct sfg_ctx {
     std::map<uint32_t, int> tune;          // (K, dtype, degree bucket) -> sweep variant
     std::map<uint32_t, int> score_tune;    // (K, dtype, degree bucket) -> scorer launch shape
     std::map<std::tuple<const void*, int, size_t>, int> occupancy;  // resident CTAs per SM
-    std::vector<SfgKept> kept;             // scratch kept for the next call, oldest first
+    // Scratch kept for the next call, oldest first (guarded by the device's lock: another context that runs
+    // out of memory takes it back). All of it was used on the current stream.
+    std::vector<SfgKept> kept;
     int64_t kept_bytes = 0;
+    bool kept_dirty = false;               // blocks given back since the event was recorded
+    cudaEvent_t kept_event = nullptr;      // NULL: nothing is kept
+    unsigned long long stream_id = 0;      // of the current stream: a handle can name another stream later
+    bool stream_keeps = false;             // not the per-thread default stream, whose handle names many
     int64_t alloc_count = 0;               // for the allocation-failure injection hook
     int64_t fail_alloc_at = -1;            // SFG_FAULT_ALLOC=<n>: the n-th allocation fails
+    int64_t fail_pool_at = -1;             // SFG_FAULT_POOL=<n>: the n-th finds the pool out of memory at
+                                           // its first try, if it comes from the pool
     bool withhold_mma = false;             // SFG_FAULT_MMA_WAIT=1: tensor-core kernels issue no
                                            // MMA, so their bounded completion waits run out
     int* grid_status = nullptr;            // host word that grid barriers set when a wait runs out
@@ -108,7 +118,17 @@ struct SfgDeviceGuard {
     SfgDeviceGuard(const SfgDeviceGuard&) = delete;
     SfgDeviceGuard& operator=(const SfgDeviceGuard&) = delete;
 };
-#define SFG_DEVICE(ctx) SfgDeviceGuard sfg_device_guard_((ctx)->device)
+void sfg_scratch_settle(sfg_ctx* ctx);
+struct SfgCall {
+    SfgDeviceGuard device;
+    sfg_ctx* ctx;
+    explicit SfgCall(sfg_ctx* c) : device(c->device), ctx(c) {}
+    explicit SfgCall(const sfg_ctx* c) : device(c->device), ctx(nullptr) {}
+    ~SfgCall() {
+        if (ctx && ctx->kept_dirty) sfg_scratch_settle(ctx);
+    }
+};
+#define SFG_DEVICE(ctx) SfgCall sfg_call_(ctx)
 
 // ------------------------------------------------------------------------------------------------
 // Status helpers. Every API entry point returns through these so the text lands in ctx.
@@ -139,15 +159,17 @@ sfg_status sfg_alloc(sfg_ctx* ctx, void** p, size_t bytes);
 void sfg_free(sfg_ctx* ctx, void* p);
 
 // Scratch from the blocks the context keeps from its earlier calls, else from the pool; *bytes becomes the
-// block's size. A kept block is reused on the stream it was given back on only. What a context keeps is bounded
-// (kKeptBlocks, and 1/128 of the device's memory; 1/32 over all contexts of a device); sfg_ctx_trim,
-// sfg_ctx_set_stream, sfg_ctx_destroy and an allocation that fails give it back to the pool.
+// block's size. A kept block is reused on the stream it was used on only. What a context keeps is bounded
+// (kKeptBlocks, and 1/128 of the device's memory; 1/32 over all contexts of a device) and goes back to the pool
+// with sfg_ctx_trim, sfg_ctx_set_stream to another stream, sfg_ctx_destroy, and when an allocation of any
+// context on the device fails. An event recorded at the end of each call stands for the last use, so that a
+// change of stream never touches the old one: its owner may have destroyed it, work pending, and its handle
+// may already name another stream (streams are told apart by their ids).
 // Why: the pool took 45-190 us for each of the four large blocks of an end-to-end call on the 128^3 grid, with the
 // GPU idle, and about 1 us for each small one (GB300, all scratch from the pool / kept: that call
 // 7,347 / 7,084 us, two-level 14,170 / 13,970, a 64 x 64 grid 257 / 241, a gradient over 65,536 rows 74 / 61).
 sfg_status sfg_scratch_take(sfg_ctx* ctx, void** p, size_t* bytes);
 void sfg_scratch_give(sfg_ctx* ctx, void* p, size_t bytes);
-void sfg_scratch_flush(sfg_ctx* ctx);
 bool sfg_capturing(cudaStream_t stream);
 
 // Scoped list of scratch allocations released (stream-ordered) at scope exit. A captured call takes and
@@ -156,7 +178,7 @@ struct Scratch {
     sfg_ctx* ctx;
     bool keep;
     std::vector<std::pair<void*, size_t>> ptrs;  // size 0: not to be kept
-    explicit Scratch(sfg_ctx* c) : ctx(c), keep(!sfg_capturing(c->stream)) {}
+    explicit Scratch(sfg_ctx* c) : ctx(c), keep(c->stream_keeps && !sfg_capturing(c->stream)) {}
     ~Scratch() {
         for (auto& q : ptrs) {
             if (!q.first) continue;
