@@ -5,6 +5,9 @@
 #include <cstring>
 #include <mutex>
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include "sfg_internal.cuh"
 
 sfg_status sfg_fail(sfg_ctx* ctx, sfg_status st, const char* fmt, ...) {
@@ -121,6 +124,32 @@ static void kept_reclaim(sfg_ctx* ctx) {
     cudaStreamSynchronize(d.frees);
 }
 
+// The SMs that a stream's kernels can run on: those of its green context, if it has one, else the device's.
+static int stream_sms(const sfg_ctx* ctx, cudaStream_t stream) {
+    static PFN_cuStreamGetGreenCtx_v12040 green_of = nullptr;
+    static PFN_cuGreenCtxGetDevResource_v12040 resource_of = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        auto find = [](const char* name) {
+            void* p = nullptr;
+            cudaDriverEntryPointQueryResult found;
+            if (cudaGetDriverEntryPointByVersion(name, &p, 12040, cudaEnableDefault, &found) != cudaSuccess) {
+                cudaGetLastError();
+                return (void*)nullptr;
+            }
+            return found == cudaDriverEntryPointSuccess ? p : nullptr;
+        };
+        green_of = (PFN_cuStreamGetGreenCtx_v12040)find("cuStreamGetGreenCtx");
+        resource_of = (PFN_cuGreenCtxGetDevResource_v12040)find("cuGreenCtxGetDevResource");
+    });
+    CUgreenCtx green = nullptr;
+    CUdevResource r;
+    if (!green_of || !resource_of || green_of((CUstream)stream, &green) != CUDA_SUCCESS || !green ||
+        resource_of(green, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS)
+        return ctx->num_sms;
+    return std::max(1, std::min(ctx->num_sms, (int)r.sm.smCount));
+}
+
 static void set_stream(sfg_ctx* ctx, cudaStream_t stream) {
     unsigned long long id = 0;
     const bool known = cudaStreamGetId(stream, &id) == cudaSuccess;
@@ -131,6 +160,7 @@ static void set_stream(sfg_ctx* ctx, cudaStream_t stream) {
     }
     ctx->stream = stream;
     ctx->stream_id = id;
+    ctx->stream_sms = stream_sms(ctx, stream);
     ctx->stream_keeps = known && ctx->kept_event && stream != cudaStreamPerThread;
 }
 
@@ -289,7 +319,7 @@ sfg_status sfg_check_dev(sfg_ctx* ctx, const void* p, const char* what) {
     return SFG_OK;
 }
 
-int sfg_grid(sfg_ctx* ctx, const void* kernel, int block, size_t smem, int64_t work_items) {
+static int grid_on(sfg_ctx* ctx, const void* kernel, int block, size_t smem, int64_t work_items, int sms) {
     // resident CTAs per SM, asked once per (kernel, block, shared memory) and context
     const auto key = std::make_tuple(kernel, block, smem);
     auto it = ctx->occupancy.find(key);
@@ -304,10 +334,18 @@ int sfg_grid(sfg_ctx* ctx, const void* kernel, int block, size_t smem, int64_t w
         }
         ctx->occupancy.emplace(key, per_sm);
     }
-    int64_t full = (int64_t)per_sm * ctx->num_sms;
+    int64_t full = (int64_t)per_sm * sms;
     int64_t need = (work_items + block - 1) / block;
     if (need < 1) need = 1;
     return (int)(need < full ? need : full);
+}
+
+int sfg_grid(sfg_ctx* ctx, const void* kernel, int block, size_t smem, int64_t work_items) {
+    return grid_on(ctx, kernel, block, smem, work_items, ctx->num_sms);
+}
+
+int sfg_coop_grid(sfg_ctx* ctx, const void* kernel, int block, int64_t work_items) {
+    return grid_on(ctx, kernel, block, 0, work_items, ctx->stream_sms);
 }
 
 void sfg_tic(sfg_ctx* ctx, const char* name) {

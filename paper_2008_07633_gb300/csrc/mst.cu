@@ -573,7 +573,7 @@ sfg_status sfg_mst_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* allow, 
     a.mask = mask;
     a.wait = sfg_grid_wait(ctx, "k_mst");
     void* args[] = {(void*)&a};
-    const int grid = sfg_grid(ctx, (const void*)k_mst, kBlock, 0, items);
+    const int grid = sfg_coop_grid(ctx, (const void*)k_mst, kBlock, items);
     sfg_tic(ctx, "mst");
     const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_mst, dim3(grid), dim3(kBlock), args, 0,
                                                       ctx->stream);

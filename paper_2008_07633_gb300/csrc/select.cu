@@ -292,7 +292,7 @@ sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, 
                          int64_t k, int32_t* out) {
     if (k == 0) return SFG_OK;
     // at least 1,024 candidates a CTA: fewer CTAs make the barriers cheaper
-    const int grid = sfg_grid(ctx, (const void*)k_topk, kBlock, 0, (ne + 3) / 4);
+    const int grid = sfg_coop_grid(ctx, (const void*)k_topk, kBlock, (ne + 3) / 4);
     const int sort_ctas = (int)std::min<int64_t>(grid, (k + 4095) / 4096);
     Scratch s(ctx);
     // The kept ids are written while other CTAs still read the lists: a list over its own inputs (an
@@ -510,7 +510,7 @@ sfg_status sfg_topk_segmented_mark(sfg_ctx* ctx, const float* scores, const int3
     a.mask = mask;
     a.wait = sfg_grid_wait(ctx, "k_topk_seg");
     void* args[] = {(void*)&a};
-    const int grid = sfg_grid(ctx, (const void*)k_topk_seg, kBlock, 0, (ne + 3) / 4);
+    const int grid = sfg_coop_grid(ctx, (const void*)k_topk_seg, kBlock, (ne + 3) / 4);
     sfg_tic(ctx, "topk");
     const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_topk_seg, dim3(grid), dim3(kBlock), args, 0,
                                                       ctx->stream);

@@ -38,6 +38,7 @@ struct sfg_ctx {
     cudaMemPool_t pool = nullptr;          // the device's stream-ordered pool of the library
     int* host_word = nullptr;              // pinned host ints for flags read after a sync
     int num_sms = 0;
+    int stream_sms = 0;                    // of them, those that the stream's kernels can run on
     std::string last_error;
     bool timing = false;
     std::vector<sfg_timer_rec> timers;     // recorded this session
@@ -218,6 +219,8 @@ sfg_status sfg_check_dev(sfg_ctx* ctx, const void* p, const char* what);
 
 // Grid size for a grid-stride kernel: a whole number of waves over the SMs.
 int sfg_grid(sfg_ctx* ctx, const void* kernel, int block, size_t smem, int64_t work_items);
+// The same for a cooperative launch, whose CTAs have to be resident together: over the SMs of the stream.
+int sfg_coop_grid(sfg_ctx* ctx, const void* kernel, int block, int64_t work_items);
 
 static inline unsigned ceil_div_u(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 

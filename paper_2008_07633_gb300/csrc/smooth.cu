@@ -1223,7 +1223,7 @@ struct Smoother {
         if (steps < 1 || (int64_t)grid * kBlock < (int64_t)LG->n * LPR) return false;
         if (LG->hv_n != 0 || (LP && LP->hv_n != 0)) return false;
         const int64_t lanes = (int64_t)sides * grid * kBlock;
-        return sfg_grid(ctx, (const void*)k_small<T, LPR>, kBlock, 0, lanes) == sides * grid;
+        return sfg_coop_grid(ctx, (const void*)k_small<T, LPR>, kBlock, lanes) == sides * grid;
     }
 
     static sfg_status launch_small(sfg_ctx* ctx, SmallArgs<T>& a) {
