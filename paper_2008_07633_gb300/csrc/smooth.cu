@@ -185,9 +185,10 @@ struct Chunk {
 // acc += sum over slots [s0, s0 + NS) (slots past the chunk ignored at compile time) of
 // w * X[col] for this lane's E columns. All NS gathers are issued before the first is consumed;
 // the weights are taken from the chunk at use time, so only the gathered vectors stay live.
+// Xl without __restrict__: k_gs and k_small gather from blocks that they write.
 template <typename T, int LPR, int NS>
 __device__ __forceinline__ void gather_slots(const Chunk<LPR>& ch, int s0, unsigned gm,
-                                             const T* __restrict__ Xl, float (&acc)[Vec<T>::E]) {
+                                             const T* Xl, float (&acc)[Vec<T>::E]) {
     constexpr int K = LPR * Vec<T>::E, C = Chunk<LPR>::C;
     uint4 xv[NS];
 #pragma unroll
@@ -211,7 +212,7 @@ __device__ __forceinline__ void gather_slots(const Chunk<LPR>& ch, int s0, unsig
 // All slots of a chunk that the tile's longest row needs: warp-uniform batches of 2, 4 or 6.
 template <typename T, int LPR>
 __device__ __forceinline__ void gather_chunk(const Chunk<LPR>& ch, int need, unsigned gm,
-                                             const T* __restrict__ Xl, float (&acc)[Vec<T>::E]) {
+                                             const T* Xl, float (&acc)[Vec<T>::E]) {
     constexpr int C = Chunk<LPR>::C;
     if (need <= 2) {
         if (need > 0) gather_slots<T, LPR, 2>(ch, 0, gm, Xl, acc);
