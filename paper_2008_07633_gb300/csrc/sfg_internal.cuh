@@ -88,6 +88,7 @@ struct sfg_graph {
     // hv_seg[hv_soff[h], hv_soff[h + 1]), each (row, first entry, end entry, 0).
     int32_t hv_n = -1;
     int64_t hv_nseg = 0;
+    bool hv_spread = false;    // hub rows, and the other rows' lengths vary widely (see k_heavy_mark)
     int32_t* hv_rows = nullptr;
     int32_t* hv_soff = nullptr;
     int4* hv_seg = nullptr;

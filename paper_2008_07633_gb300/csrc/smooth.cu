@@ -50,17 +50,26 @@ constexpr int64_t kAheadBytes = 4 << 20;
 enum { kFormTwo, kFormOne, kFormTwoAhead, kFormOneAhead };
 template <typename T, int LPR>
 int plain_form(const sfg_graph* L) {
-    if (L->hv_n > 0) return LPR <= 8 ? kFormOne : kFormTwo;
+    if (L->hv_spread) return LPR <= 8 ? kFormOne : kFormTwo;
     const bool bf16 = sizeof(T) == 2, sparse = L->m < 2 * (int64_t)L->n;
     if (LPR == 1) return kFormOne;
     if (LPR == 4 && bf16) return kFormTwo;
     if (LPR == 8) return bf16 ? kFormOneAhead : sparse ? kFormTwoAhead : kFormOne;
     return kFormTwoAhead;
 }
-// Graphs with hub rows get kHubWaves CTAs a resident slot: their rows differ in length by hundreds, and
-// rows of one length tend to be neighbours (degree order), so CTAs that finish early must find more
-// (2^20-node Chung-Lu graph, K = 32, one wave / eight: 333 / 323 us on L_G, 186 / 154 on its forest,
-// 369 / 241 with two tiles a turn). Meshes lose 10-30% from the extra starts and keep one wave.
+// Graphs with hub rows whose other rows differ in length too get kHubWaves CTAs a resident slot: rows of one
+// length tend to be neighbours (degree order), so CTAs that finish early must find more. The line is the spread
+// of the lengths up to SFG_HEAVY_ROW (longer rows are swept apart), variance over squared mean above 1: 2.3-2.4 on
+// Chung-Lu graphs and 4-6 on their forests, below 0.02 on meshes, power grids and k-NN graphs with a few
+// hubs and 0.2-0.6 on those graphs' forests. Measured (us a sweep: two tiles a turn in one wave, the form of the
+// spread graphs, that of the others; hub rows included):
+//   2^20-node Chung-Lu     K = 4 FP32 224/142/168   K = 16 254/194/253   K = 32 378/326/338   K = 64 552/522/563
+//                          K = 16 BF16 203/142/203  K = 32 264/217/264   K = 64 393/345/358
+//   its forest             K = 32 FP32 249/155/242  K = 32 BF16 229/146/229
+//   60k-node Chung-Lu      K = 32 FP32 81/56/60     K = 32 BF16 85/57/85
+//   128^3 grid, one hub    K = 16 FP32 139/153/133  K = 32 182/225/181    K = 64 328/404/317
+//                          K = 32 BF16 140/173/140  K = 64 210/240/219
+//   300k-node k-NN, one    K = 32 FP32 70/79/68     K = 32 BF16 52/58/52
 constexpr int kHubWaves = 8;
 
 // Gaussian entries 2p and 2p+1 of the counter-based generator (see sfg.h): SplitMix64 output
@@ -468,17 +477,32 @@ __global__ void __launch_bounds__(kBlock) k_heavy_final(int32_t nh, const int32_
     if (STATS) block_column_partials<LPR, E>(s1, s2, part);
 }
 
+// Marks the rows over kHeavy entries; words: how many, and the other rows' summed and summed squared lengths.
 __global__ void k_heavy_mark(int32_t n, const int32_t* __restrict__ row_ptr, int32_t* __restrict__ heavy,
-                             int32_t* __restrict__ nseg, int* __restrict__ count) {
-    int c = 0;
+                             int32_t* __restrict__ nseg, unsigned long long* __restrict__ words) {
+    unsigned long long c = 0, sum = 0, squares = 0;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
         const int32_t d = row_ptr[r + 1] - row_ptr[r];
         heavy[r] = d > kHeavy;
         nseg[r] = d > kHeavy ? (d + kSeg - 1) / kSeg : 0;
-        c += d > kHeavy;
+        if (d > kHeavy) {
+            ++c;
+        } else {
+            sum += (unsigned)d;
+            squares += (unsigned)d * (unsigned)d;
+        }
     }
-    c = __reduce_add_sync(0xffffffffu, c);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        c += __shfl_xor_sync(0xffffffffu, c, o);
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        squares += __shfl_xor_sync(0xffffffffu, squares, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (c) atomicAdd(words, c);
+        if (sum) atomicAdd(words + 1, sum);
+        if (squares) atomicAdd(words + 2, squares);
+    }
 }
 
 __global__ void k_heavy_fill(int32_t n, const int32_t* __restrict__ row_ptr, const int64_t* __restrict__ hoff,
@@ -520,19 +544,19 @@ sfg_status heavy_prepare(sfg_ctx* ctx, const sfg_graph* Lc) {
     Scratch s(ctx);
     int32_t *heavy, *nseg;
     int64_t *hoff, *soff;
-    int* count;
+    unsigned long long* words;
     SFG_TRY(s.get(&heavy, (size_t)n));
     SFG_TRY(s.get(&nseg, (size_t)n));
-    SFG_TRY(s.get(&count, 1));
-    SFG_CUDA(ctx, cudaMemsetAsync(count, 0, sizeof(int), ctx->stream));
+    SFG_TRY(s.get(&words, 3));
+    SFG_CUDA(ctx, cudaMemsetAsync(words, 0, 3 * sizeof(unsigned long long), ctx->stream));
     const int g = sfg_grid(ctx, (const void*)k_heavy_mark, kBlock, 0, n);
-    k_heavy_mark<<<g, kBlock, 0, ctx->stream>>>(n, L->row_ptr, heavy, nseg, count);
+    k_heavy_mark<<<g, kBlock, 0, ctx->stream>>>(n, L->row_ptr, heavy, nseg, words);
     ++ctx->launches;
     SFG_LAUNCH_CHECK(ctx, "k_heavy_mark");
-    int hcount = 0;
-    SFG_CUDA(ctx, cudaMemcpyAsync(&hcount, count, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    unsigned long long got[3] = {0, 0, 0};
+    SFG_CUDA(ctx, cudaMemcpyAsync(got, words, sizeof got, cudaMemcpyDeviceToHost, ctx->stream));
     SFG_TRY(sfg_wait(ctx));
-    if (hcount == 0) {  // the common case on meshes: one pass over row_ptr, one readback
+    if (got[0] == 0) {  // the common case on meshes: one pass over row_ptr, one readback
         L->hv_nseg = 0;
         L->hv_n = 0;
         return SFG_OK;
@@ -563,6 +587,8 @@ sfg_status heavy_prepare(sfg_ctx* ctx, const sfg_graph* Lc) {
         SFG_LAUNCH_CHECK(ctx, "k_heavy_fill");
     }
     L->hv_nseg = ns;
+    // variance over squared mean > 1, as rows * squares > 2 sum^2
+    L->hv_spread = (double)(n - nh) * (double)got[2] > 2.0 * (double)got[1] * (double)got[1];
     L->hv_n = (int32_t)nh;
     return SFG_OK;
 }
@@ -1216,7 +1242,7 @@ struct Smoother {
     static int grid_plain(sfg_ctx* ctx, const void* k, const sfg_graph* L) {
         const int64_t lanes = (int64_t)L->n * LPR;
         const int g = sfg_grid(ctx, k, kBlock, 0, lanes);
-        return L->hv_n > 0 ? (int)std::min<int64_t>((int64_t)g * kHubWaves, (lanes + kBlock - 1) / kBlock) : g;
+        return L->hv_spread ? (int)std::min<int64_t>((int64_t)g * kHubWaves, (lanes + kBlock - 1) / kBlock) : g;
     }
 
     // Whether `sides` copies of one side's grid are resident at once, with one tile a warp and no hub rows.
