@@ -11,6 +11,7 @@
 #include <cmath>
 
 #include "sfg_internal.cuh"
+#include "dot64.cuh"
 
 namespace {
 
@@ -151,9 +152,42 @@ __device__ __forceinline__ bool sums_exact(int lo, int hi, int cnt) {
 }
 __device__ __forceinline__ int exponent_of(float w) { return max(1, (int)((__float_as_uint(w) >> 23) & 0xffu)); }
 
+// A weight widened without the FP64 pipe (dot64.cuh), which the additions need.
+__device__ __forceinline__ double widen_weight(float w) { return is_normal32(w) ? widen_normal(w) : (double)w; }
+
+// FP64 sum of a row's weights in column order by one warp, 32 entries at a time. Where all of them are multiples of
+// the unit of the sum so far and the new sum stays in its binade, no addition rounds, whatever the order: the lanes
+// add them as a tree. Else each lane's weight is added in turn. (An FP64 addition takes a warp about 75 clocks, so
+// a chain of them is what bounds this: a row of 30,000 entries took 1.2 ms in turn, one thread that loads and
+// widens as it adds 2.0 ms.) A tail of zeros changes no sum of positive weights.
+__device__ __forceinline__ double ordered_degree(const int2* __restrict__ row, int32_t len) {
+    const int lane = threadIdx.x & 31;
+    double s = 0.0;
+    float next = lane < len ? __int_as_float(row[lane].y) : 0.f;
+    for (int32_t j0 = 0; j0 < len; j0 += 32) {
+        const int lo = __reduce_min_sync(0xffffffffu, j0 + lane < len ? exponent_of(next) : 255);
+        const double w = widen_weight(next);
+        const int32_t j = j0 + 32 + lane;
+        next = j < len ? __int_as_float(row[j].y) : 0.f;
+        const int es = __double2hiint(s) >> 20;  // s >= 0: its exponent field
+        if (lo + 925 >= es) {  // lowest unit 2^(lo - 150) against 2^(es - 1075)
+            double t = w;
+#pragma unroll
+            for (int q = 16; q > 0; q >>= 1) t += __shfl_xor_sync(0xffffffffu, t, q);
+            t = s + __shfl_sync(0xffffffffu, t, 0);
+            if (__double2hiint(t) >> 20 == es) {
+                s = t;
+                continue;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 32; ++q) s += __shfl_sync(0xffffffffu, w, q);
+    }
+    return s;
+}
+
 // Degrees of the listed rows that have more than SFG_HEAVY_ROW entries, one CTA a row: in parallel
-// where every order gives the column order's bits, else one thread in order (a 4,000-entry row took
-// one thread 0.7 ms).
+// where every order gives the column order's bits, else one warp in order.
 __global__ void __launch_bounds__(kBlock) k_lap_deg_heavy(int32_t nh, const int32_t* __restrict__ hrow,
                                                           const int32_t* __restrict__ row_ptr,
                                                           const int2* __restrict__ colval,
@@ -187,12 +221,13 @@ __global__ void __launch_bounds__(kBlock) k_lap_deg_heavy(int32_t nh, const int3
             ws[warp] = s;
         }
         __syncthreads();
+        const bool exact = sums_exact(slo, shi, b - a);
+        if (!exact && warp == 0) s = ordered_degree(colval + a, b - a);
         if (threadIdx.x == 0) {
-            s = 0.0;
-            if (sums_exact(slo, shi, b - a))
+            if (exact) {
+                s = 0.0;
                 for (int q = 0; q < kBlock / 32; ++q) s += ws[q];
-            else
-                for (int32_t j = a; j < b; ++j) s += (double)__int_as_float(colval[j].y);
+            }
             deg[p] = s;
             invdeg[p] = s > 0.0 ? 1.0 / s : 0.0;
         }
@@ -227,8 +262,8 @@ __global__ void k_lap_f2c(const uint64_t* __restrict__ keys, const uint32_t* __r
 constexpr int kRowSmall = 32, kRowWarp = 256, kRowMid = 1024, kRowBig = 4096, kRowCap = 16384;
 
 // Words the build reads back: input error, longest raw row, rows of the four larger classes, merged
-// rows over SFG_HEAVY_ROW, raw entries, merged entries, canonical edges.
-enum { kWErr, kWMax, kWWarp, kWMid, kWBig, kWLarge, kWHeavy, kWRaw, kWNnz, kWEdges, kWCount };
+// rows over SFG_HEAVY_ROW, raw entries, merged entries, canonical edges; rows left to k_deg_ordered, of up to kRowWarp entries and longer.
+enum { kWErr, kWMax, kWWarp, kWMid, kWBig, kWLarge, kWHeavy, kWRaw, kWNnz, kWEdges, kWDegShort, kWDegLong, kWCount };
 
 // Raw row lengths and each entry's place within its row (slot.x in row u, slot.y in row v; -1 for
 // self-loops and bad edges). A warp whose edges all share an endpoint (a hub's edges in a sorted
@@ -357,14 +392,25 @@ struct RowOut {
     int32_t* up;
     double* deg;
     double* invdeg;
+    int32_t* oshort;  // rows left to k_deg_ordered
+    int32_t* olong;
     unsigned long long* words;
 };
 
-__device__ __forceinline__ void row_finish(const RowOut& o, int64_t r, int32_t nnz, int32_t up, double s) {
-    o.nnz[r] = nnz;
-    o.up[r] = up;
+__device__ __forceinline__ void row_degree(const RowOut& o, int64_t r, double s) {
     o.deg[r] = s;
     o.invdeg[r] = s > 0.0 ? 1.0 / s : 0.0;
+}
+
+__device__ __forceinline__ void row_finish(const RowOut& o, int64_t r, int32_t nnz, int32_t up, double s, bool exact) {
+    o.nnz[r] = nnz;
+    o.up[r] = up;
+    if (exact) {
+        row_degree(o, r, s);
+    } else {
+        const bool longer = nnz > kRowWarp;
+        (longer ? o.olong : o.oshort)[atomicAdd(o.words + (longer ? kWDegLong : kWDegShort), 1ull)] = (int32_t)r;
+    }
     if (nnz > SFG_HEAVY_ROW) atomicAdd(o.words + kWHeavy, 1ull);
 }
 
@@ -523,7 +569,7 @@ __global__ void __launch_bounds__(kBlock, 5)
         t = e;
     }
     for (int t = nnz; t < b - a; ++t) o.rrow[off[r] + t] = -1;
-    row_finish(o, r, nnz, up, s);
+    row_finish(o, r, nnz, up, s, true);
 }
 
 // One warp a listed row of at most kRowWarp raw entries.
@@ -597,23 +643,20 @@ __global__ void __launch_bounds__(kBlock)
         }
         lo = __reduce_min_sync(0xffffffffu, lo);
         hi = __reduce_max_sync(0xffffffffu, hi);
-        if (sums_exact(lo, hi, nnz)) {
+        const bool exact = sums_exact(lo, hi, nnz);
+        if (exact) {
 #pragma unroll
             for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
-        } else if (lane == 0) {
-            s = 0.0;
-            for (int i = 0; i < d; ++i)
-                if (i == 0 || key_col(key[i - 1]) != key_col(key[i])) s += (double)run_weight(key, sw, i, d);
         }
         for (int i = nnz + lane; i < d; i += 32) o.rrow[base + i] = -1;
-        if (lane == 0) row_finish(o, r, nnz, up, s);
+        if (lane == 0) row_finish(o, r, nnz, up, s, exact);
         __syncwarp();  // the next row reuses shared memory
     }
 }
 
 // One CTA a listed row of at most CAP raw entries: bitonic sort of the keys in shared memory.
 // The degree is the FP64 sum in column order; where every partial sum is exact (sums_exact), any
-// order gives the same bits and the CTA adds in parallel, else one thread adds in order.
+// order gives the same bits and the CTA adds in parallel, else k_deg_ordered adds in order.
 template <int THREADS, int CAP>
 __global__ void __launch_bounds__(THREADS)
     k_rows_cta(int32_t nrows, const int32_t* __restrict__ rows, const int32_t* __restrict__ cnt,
@@ -714,7 +757,8 @@ __global__ void __launch_bounds__(THREADS)
         const int nnz = scarry;
         for (int i = nnz + tid; i < d; i += THREADS) o.rrow[base + i] = -1;
         double s = 0.0;
-        if (sums_exact(smin, smax, nnz)) {
+        const bool exact = sums_exact(smin, smax, nnz);
+        if (exact) {
             for (int i = tid; i < nnz; i += THREADS) s += (double)sw[i];
 #pragma unroll
             for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
@@ -723,11 +767,36 @@ __global__ void __launch_bounds__(THREADS)
             s = 0.0;
             if (tid == 0)
                 for (int q = 0; q < THREADS / 32; ++q) s += dsum[q];
-        } else if (tid == 0) {
-            for (int i = 0; i < nnz; ++i) s += (double)sw[i];
         }
-        if (tid == 0) row_finish(o, r, nnz, sup, s);
+        if (tid == 0) row_finish(o, r, nnz, sup, s, exact);
         __syncthreads();  // the next row reuses shared memory
+    }
+}
+
+// Degrees that have to be added in column order, once all rows are sorted: a lane a row up to kRowWarp entries (32
+// rows share each FP64 instruction), a warp a longer row. Added by one thread of the warp or CTA that sorted the row,
+// while the others waited, they made the build of a 2^20-node Chung-Lu graph with weights exp(3 N(0, 1))
+// 3,041 us instead of 2,038 (2,783 with the radix sort of all entries and one thread a row).
+__global__ void __launch_bounds__(kBlock) k_deg_ordered(const int64_t* __restrict__ off, RowOut o) {
+    const int64_t t0 = (int64_t)blockIdx.x * kBlock + threadIdx.x, nt = (int64_t)gridDim.x * kBlock;
+    const int64_t shorter = (int64_t)o.words[kWDegShort], longer = (int64_t)o.words[kWDegLong];
+    for (int64_t i = t0 / 32; i < longer; i += nt / 32) {
+        const int32_t r = o.olong[i];
+        const double s = ordered_degree(o.rcv + off[r], o.nnz[r]);
+        if ((threadIdx.x & 31) == 0) row_degree(o, r, s);
+    }
+    for (int64_t i = t0; i < shorter; i += nt) {
+        const int32_t r = o.oshort[i], len = o.nnz[r];
+        const int2* row = o.rcv + off[r];
+        double s = 0.0;
+        for (int32_t j0 = 0; j0 < len; j0 += 8) {
+            float w[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) w[q] = j0 + q < len ? __int_as_float(row[j0 + q].y) : 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) s += widen_weight(w[q]);
+        }
+        row_degree(o, r, s);
     }
 }
 
@@ -1068,7 +1137,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     *fits = true;
     const int64_t len = 2 * m;
     Scratch s(ctx);
-    int32_t *cnt, *lwarp, *mid, *big, *large, *re, *rrow, *rpos, *nnz, *up, *D, *move;
+    int32_t *cnt, *lwarp, *mid, *big, *large, *re, *rrow, *rpos, *nnz, *up, *D, *move, *oshort, *olong;
     int2 *slot, *rcv;
     uint64_t* raw;
     int64_t *off, *row_off, *up_off;
@@ -1129,7 +1198,9 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
         k_row_place<<<grid_of(ctx, k_row_place, (m + 3) / 4), kBlock, 0, ctx->stream>>>(m, u, v, slot, off, raw);
         ++ctx->launches;
     }
-    const RowOut ro{rcv, re, rrow, rpos, nnz, up, g->deg, g->invdeg, words};
+    SFG_TRY(s.get(&oshort, (size_t)(len / kRowSmall) + 1));
+    SFG_TRY(s.get(&olong, (size_t)(len / kRowWarp) + 1));
+    const RowOut ro{rcv, re, rrow, rpos, nnz, up, g->deg, g->invdeg, oshort, olong, words};
     k_rows_small<<<ceil_div_u(n, kRowsPerWarp * kRowWarps), kBlock, 0, ctx->stream>>>(n, cnt, off, raw, w, ro);
     ++ctx->launches;
     if (nwarp > 0) {
@@ -1152,6 +1223,10 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     if (nmid > 0) SFG_TRY(rows_cta(k_rows_cta<128, kRowMid>, 128, kRowMid, nmid, mid));
     if (nbig > 0) SFG_TRY(rows_cta(k_rows_cta<256, kRowBig>, 256, kRowBig, nbig, big));
     if (nlarge > 0) SFG_TRY(rows_cta(k_rows_cta<1024, kRowCap>, 1024, kRowCap, nlarge, large));
+    if (nwarp + nmid + nbig + nlarge > 0) {
+        k_deg_ordered<<<4 * ctx->num_sms, kBlock, 0, ctx->stream>>>(off, ro);
+        ++ctx->launches;
+    }
     SFG_LAUNCH_CHECK(ctx, "k_rows");
     SFG_TRY(sfg_scan_i32(ctx, nnz, row_off, n));
     SFG_TRY(sfg_scan_i32(ctx, up, up_off, n));
