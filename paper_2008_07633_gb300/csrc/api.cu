@@ -446,6 +446,7 @@ sfg_status sfg_ctx_create(sfg_ctx** out, int device, void* cuda_stream) {
     if (c->num_sms < 1) c->num_sms = 1;
     if (const char* f = std::getenv("SFG_FAULT_ALLOC")) c->fail_alloc_at = std::atoll(f);
     if (const char* f = std::getenv("SFG_FAULT_POOL")) c->fail_pool_at = std::atoll(f);
+    if (const char* f = std::getenv("SFG_BUILD_SORT")) c->build_sorts = std::atoi(f) != 0;
     if (const char* f = std::getenv("SFG_FAULT_MMA_WAIT")) c->withhold_mma = std::atoi(f) != 0;
     if (const char* f = std::getenv("SFG_FAULT_GRID_WAIT")) {
         const char* colon = std::strchr(f, ':');

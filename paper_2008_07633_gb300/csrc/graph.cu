@@ -3,8 +3,8 @@
 //
 // By rows (the usual path): every directed entry (column, input position) is placed in its row by
 // a counting pass and each row is then sorted on chip, so an entry crosses HBM a few times instead
-// of once per radix digit (see build_by_rows). By sort (graphs with a row of more than kRowCap raw
-// entries, or 2m >= 2^31): one stable radix sort of the 2m directed entries keyed by (row, column).
+// of once per radix digit (see build_by_rows; rows too long for that are sorted among themselves). By sort
+// (2m >= 2^31, or too much in such rows): one stable radix sort of the 2m directed entries keyed by (row, column).
 // Both give the CSR rows sorted by column with parallel edges merged by an FP64 sum in input order
 // rounded once to FP32; the upper-triangle entries, in order, are the canonical edge list (edge id
 // = rank among them), and a lower-triangle entry takes the id of its mirror.
@@ -261,9 +261,10 @@ __global__ void k_lap_f2c(const uint64_t* __restrict__ keys, const uint32_t* __r
 // left of the first is the 390 us of counting (atomics on random rows) and 346 us of placing.
 constexpr int kRowSmall = 32, kRowWarp = 256, kRowMid = 1024, kRowBig = 4096, kRowCap = 16384;
 
-// Words the build reads back: input error, longest raw row, rows of the four larger classes, merged
-// rows over SFG_HEAVY_ROW, raw entries, merged entries, canonical edges; rows left to k_deg_ordered, of up to kRowWarp entries and longer.
-enum { kWErr, kWMax, kWWarp, kWMid, kWBig, kWLarge, kWHeavy, kWRaw, kWNnz, kWEdges, kWDegShort, kWDegLong, kWCount };
+// Words the build reads back: input error, rows of the five larger classes, raw entries of the longest class, merged
+// rows over SFG_HEAVY_ROW, raw entries, merged entries, canonical edges; rows left to k_deg_ordered, of up to
+// kRowWarp entries and longer.
+enum { kWErr, kWWarp, kWMid, kWBig, kWLarge, kWLong, kWLongRaw, kWHeavy, kWRaw, kWNnz, kWEdges, kWDegShort, kWDegLong, kWCount };
 
 // Raw row lengths and each entry's place within its row (slot.x in row u, slot.y in row v; -1 for
 // self-loops and bad edges). A warp whose edges all share an endpoint (a hub's edges in a sorted
@@ -321,15 +322,13 @@ __global__ void __launch_bounds__(kBlock)
     }
 }
 
-// The rows of the four larger classes (in no particular order) and the longest row.
+// The rows of the five larger classes (in no particular order) and the raw entries of the longest.
 __global__ void k_row_classify(int32_t n, const int32_t* __restrict__ cnt, int32_t* __restrict__ lwarp,
                                int32_t* __restrict__ mid, int32_t* __restrict__ big, int32_t* __restrict__ large,
-                               unsigned long long* __restrict__ words) {
-    int32_t top = 0;
+                               int32_t* __restrict__ longest, unsigned long long* __restrict__ words) {
     for (int64_t r0 = (int64_t)blockIdx.x * kBlock; r0 < n; r0 += (int64_t)gridDim.x * kBlock) {
         const int64_t r = r0 + threadIdx.x;
         const int32_t c = r < n ? cnt[r] : 0;
-        top = max(top, c);
         const bool w = c > kRowSmall && c <= kRowWarp;
         const unsigned ws = __ballot_sync(0xffffffffu, w);
         if (ws) {
@@ -342,11 +341,13 @@ __global__ void k_row_classify(int32_t n, const int32_t* __restrict__ cnt, int32
         if (c > kRowWarp) {
             if (c <= kRowMid) mid[atomicAdd(words + kWMid, 1ull)] = (int32_t)r;
             else if (c <= kRowBig) big[atomicAdd(words + kWBig, 1ull)] = (int32_t)r;
-            else large[atomicAdd(words + kWLarge, 1ull)] = (int32_t)r;
+            else if (c <= kRowCap) large[atomicAdd(words + kWLarge, 1ull)] = (int32_t)r;
+            else {
+                longest[atomicAdd(words + kWLong, 1ull)] = (int32_t)r;
+                atomicAdd(words + kWLongRaw, (unsigned long long)c);
+            }
         }
     }
-    top = __reduce_max_sync(0xffffffffu, top);
-    if ((threadIdx.x & 31) == 0 && top > 0) atomicMax(words + kWMax, (unsigned long long)top);
 }
 
 __global__ void __launch_bounds__(kBlock)
@@ -800,6 +801,126 @@ __global__ void __launch_bounds__(kBlock) k_deg_ordered(const int64_t* __restric
     }
 }
 
+// ---- rows of more than kRowCap raw entries ----
+// Their entries are gathered from the raw rows as keys (place in the list of rows, column, input position) and sorted
+// by the radix sort, which moves these rows only. While a list with one such row took the sort of all entries,
+// after it had been counted by rows, it took as long as or longer than with the sort alone: a 2^25-node random
+// graph of 2^28 edges and a row of 20,000 entries 117.5 ms (107.8 with the sort alone, now 72.2), a 2^20-node
+// Chung-Lu graph with such a row 2,713 us, now 1,946.
+// pb, cb: bits of an input position and of a column; i0: first listed row of this sort.
+struct LongRows {
+    int32_t i0, cb, pb;
+    const int32_t* rows;
+    const int64_t* start;  // of each listed row's entries among those of all listed rows
+    const int64_t* off;
+};
+
+__global__ void k_long_counts(int32_t nrows, const int32_t* __restrict__ rows, const int32_t* __restrict__ cnt,
+                              int32_t* __restrict__ len) {
+    for (int32_t i = blockIdx.x * kBlock + threadIdx.x; i < nrows; i += gridDim.x * kBlock) len[i] = cnt[rows[i]];
+}
+
+__global__ void k_long_gather(int64_t len, int32_t nrows, LongRows a, const uint64_t* __restrict__ raw,
+                              uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+    const int64_t s0 = a.start[a.i0];
+    for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < len; p += (int64_t)gridDim.x * kBlock) {
+        int32_t lo = 0, hi = nrows;  // last row that starts at or before p
+        while (hi - lo > 1) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (a.start[a.i0 + mid] - s0 <= p) lo = mid; else hi = mid;
+        }
+        const uint64_t k = raw[a.off[a.rows[a.i0 + lo]] + (p - (a.start[a.i0 + lo] - s0))];
+        keys[p] = ((uint64_t)lo << (a.cb + a.pb)) | (k >> 32 << a.pb) | (k & 0xffffffffull);
+        vals[p] = 0u;
+    }
+}
+
+__global__ void k_long_heads(int64_t len, int32_t pb, const uint64_t* __restrict__ keys, uint8_t* __restrict__ head) {
+    for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < len; p += (int64_t)gridDim.x * kBlock)
+        head[p] = p == 0 || keys[p - 1] >> pb != keys[p] >> pb;
+}
+
+// Merged entries and the raw places of the upper ones, as the row kernels write them.
+__global__ void k_long_write(int64_t len, LongRows a, const uint64_t* __restrict__ keys,
+                             const uint8_t* __restrict__ head, const int64_t* __restrict__ run,
+                             const float* __restrict__ w, RowOut o) {
+    const int64_t s0 = a.start[a.i0];
+    const uint64_t pmask = (1ull << a.pb) - 1ull, cmask = (1ull << a.cb) - 1ull;
+    for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < len; p += (int64_t)gridDim.x * kBlock) {
+        const uint64_t k = keys[p], kc = k >> a.pb;
+        const int32_t i = a.i0 + (int32_t)(k >> (a.cb + a.pb)), r = a.rows[i], c = (int32_t)(kc & cmask);
+        const int64_t at = a.off[r] + (run[p + 1] - 1 - run[a.start[i] - s0]);
+        if (c > r) o.rpos[k & pmask] = (int32_t)at;
+        if (!head[p]) continue;
+        double s = (double)w[k & pmask];  // input order, eight entries in flight
+        for (int64_t t = p + 1; t < len && keys[t] >> a.pb == kc; t += 8) {
+            float ww[8];
+            int take = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const uint64_t kk = keys[min(t + q, len - 1)];
+                if (t + q < len && kk >> a.pb == kc) take = q + 1;  // the run's entries are consecutive
+                ww[q] = w[kk & pmask];
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q < take) s += (double)ww[q];
+            if (take < 8) break;
+        }
+        row_entry(o, at, r, ((uint64_t)(uint32_t)c << 32) | (k & pmask), (float)s);
+    }
+}
+
+// One CTA a row: merged length, upper entries, the degree where it may be added in any order, and the rest of the
+// raw row marked unused.
+__global__ void __launch_bounds__(kBlock)
+    k_long_finish(int32_t nrows, LongRows a, const int32_t* __restrict__ cnt, const int64_t* __restrict__ run,
+                  RowOut o) {
+    __shared__ int slo, shi;
+    __shared__ double ws[kBlock / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int32_t i = a.i0 + blockIdx.x; i < a.i0 + nrows; i += gridDim.x) {
+        const int32_t r = a.rows[i], d = cnt[r];
+        const int64_t base = a.off[r], b = a.start[i] - a.start[a.i0];
+        const int32_t nnz = (int32_t)(run[b + d] - run[b]);
+        if (tid == 0) {
+            slo = 255;
+            shi = 0;
+        }
+        __syncthreads();
+        int lo = 255, hi = 0;
+        double s = 0.0;
+        for (int32_t j = tid; j < nnz; j += kBlock) {
+            const float ww = __int_as_float(o.rcv[base + j].y);
+            lo = min(lo, exponent_of(ww));
+            hi = max(hi, exponent_of(ww));
+            s += (double)ww;
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+        if (lane == 0) {
+            atomicMin(&slo, lo);
+            atomicMax(&shi, hi);
+            ws[warp] = s;
+        }
+        __syncthreads();
+        for (int32_t j = nnz + tid; j < d; j += kBlock) o.rrow[base + j] = -1;
+        if (tid == 0) {
+            int32_t first = 0, end = nnz;  // first merged entry above the diagonal
+            while (first < end) {
+                const int32_t mid = (first + end) >> 1;
+                if (o.rcv[base + mid].x > r) end = mid; else first = mid + 1;
+            }
+            s = 0.0;
+            for (int q = 0; q < kBlock / 32; ++q) s += ws[q];
+            row_finish(o, r, nnz, nnz - first, s, sums_exact(slo, shi, nnz));
+        }
+        __syncthreads();  // the next row reuses shared memory
+    }
+}
+
 // row_ptr; D[c] such that an edge whose upper entry sits at raw place p of row c has id p + D[c]; and
 // move[r], from a row's raw places to its final ones.
 __global__ void k_row_index(int32_t n, const int64_t* __restrict__ off, const int64_t* __restrict__ row_off,
@@ -1034,8 +1155,8 @@ static sfg_status row_degrees(sfg_ctx* ctx, sfg_graph* g) {
     return SFG_OK;
 }
 
-// Canonical form by one radix sort of the directed entries: graphs with a row over kRowCap raw
-// entries, and lists whose 2m entries do not fit int32 places.
+// Canonical form by one radix sort of the directed entries: lists whose 2m entries do not fit int32 places, and lists
+// whose longest rows hold much of them (build_by_rows).
 static sfg_status build_by_sort(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
                                 const float* w, bool validate, sfg_graph** out, int32_t* f2c) {
     *out = nullptr;
@@ -1129,15 +1250,73 @@ static sfg_status build_by_sort(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     return SFG_OK;
 }
 
-// Canonical form by rows (see k_row_count). *fits = false (and nothing built) when a raw row is
-// longer than kRowCap. Two host waits: the input check with the longest row, and the merged sizes.
+// The rows of more than kRowCap raw entries: count of them in `longest`, total entries. The row's place in the list
+// shares the 64-bit key with its column and position, so 64 rows (over a million entries) go in one sort, fewer on the
+// largest graphs.
+static sfg_status long_rows(sfg_ctx* ctx, int32_t n, int64_t m, int32_t count, int64_t total, const int32_t* longest,
+                            const int32_t* cnt, const int64_t* off, const uint64_t* raw, const float* w,
+                            const RowOut& o) {
+    Scratch s(ctx);
+    int32_t* len;
+    int64_t *start, *run;
+    uint64_t *keys, *keys2;
+    uint32_t *vals, *vals2;
+    uint8_t* head;
+    SFG_TRY(s.get(&len, count));
+    SFG_TRY(s.get(&start, (size_t)count + 1));
+    k_long_counts<<<grid_of(ctx, k_long_counts, count), kBlock, 0, ctx->stream>>>(count, longest, cnt, len);
+    ++ctx->launches;
+    SFG_TRY(sfg_scan_i32(ctx, len, start, count));
+    LongRows a{0, bits_for(n), 1, longest, start, off};
+    while ((1ll << a.pb) < m) ++a.pb;
+    const int32_t per = 1 << std::min(64 - a.cb - a.pb, 6);  // cb <= 31 and pb <= 30
+    std::vector<int64_t> bounds(1, 0);
+    if (count <= per) {
+        bounds.push_back(total);
+    } else {
+        std::vector<int64_t> host((size_t)count + 1);
+        SFG_CUDA(ctx, cudaMemcpyAsync(host.data(), start, sizeof(int64_t) * host.size(), cudaMemcpyDeviceToHost,
+                                      ctx->stream));
+        SFG_TRY(sfg_wait(ctx));
+        for (int64_t i = per; i < (int64_t)count + per; i += per) bounds.push_back(host[std::min<int64_t>(i, count)]);
+    }
+    int64_t most = 0;
+    for (size_t q = 1; q < bounds.size(); ++q) most = std::max(most, bounds[q] - bounds[q - 1]);
+    SFG_TRY(s.get(&keys, most));
+    SFG_TRY(s.get(&keys2, most));
+    SFG_TRY(s.get(&vals, most));
+    SFG_TRY(s.get(&vals2, most));
+    SFG_TRY(s.get(&head, most));
+    SFG_TRY(s.get(&run, most + 1));
+    for (size_t q = 0; q + 1 < bounds.size(); ++q) {
+        a.i0 = (int32_t)q * per;
+        const int32_t rows = std::min(per, count - a.i0);
+        const int64_t entries = bounds[q + 1] - bounds[q];
+        k_long_gather<<<grid_of(ctx, k_long_gather, entries), kBlock, 0, ctx->stream>>>(entries, rows, a, raw, keys, vals);
+        SFG_LAUNCH_CHECK(ctx, "k_long_gather");
+        SFG_TRY(sfg_radix_sort_pairs(ctx, &keys, &vals, &keys2, &vals2, entries,
+                                     a.cb + a.pb + (rows > 1 ? bits_for(rows) : 0)));
+        k_long_heads<<<grid_of(ctx, k_long_heads, entries), kBlock, 0, ctx->stream>>>(entries, a.pb, keys, head);
+        SFG_TRY(sfg_scan_u8(ctx, head, run, entries));
+        k_long_write<<<grid_of(ctx, k_long_write, entries), kBlock, 0, ctx->stream>>>(entries, a, keys, head, run, w, o);
+        k_long_finish<<<std::min(rows, 4 * ctx->num_sms), kBlock, 0, ctx->stream>>>(rows, a, cnt, run, o);
+        ctx->launches += 4;
+        SFG_LAUNCH_CHECK(ctx, "k_long_write");
+    }
+    return SFG_OK;
+}
+
+// Canonical form by rows (see k_row_count). *fits = false (and nothing built) when rows of more than kRowCap raw
+// entries hold over a quarter of them: the sort of all entries then moves little more than theirs. (GPU time from the
+// list, by rows / by the sort: one row of 500,000 of 6.9M entries 1,590 / 1,800 us, one of 2M of 4M 2,770 / 2,390.)
+// Two host waits: the input check with the sizes of the row classes, and the merged sizes.
 static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
                                 const float* w, bool validate, sfg_graph** out, int32_t* f2c, bool* fits) {
     *out = nullptr;
     *fits = true;
     const int64_t len = 2 * m;
     Scratch s(ctx);
-    int32_t *cnt, *lwarp, *mid, *big, *large, *re, *rrow, *rpos, *nnz, *up, *D, *move, *oshort, *olong;
+    int32_t *cnt, *lwarp, *mid, *big, *large, *longest, *re, *rrow, *rpos, *nnz, *up, *D, *move, *oshort, *olong;
     int2 *slot, *rcv;
     uint64_t* raw;
     int64_t *off, *row_off, *up_off;
@@ -1147,6 +1326,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     SFG_TRY(s.get(&mid, (size_t)(len / kRowWarp) + 1));  // longer rows are at most so many
     SFG_TRY(s.get(&big, (size_t)(len / kRowMid) + 1));
     SFG_TRY(s.get(&large, (size_t)(len / kRowBig) + 1));
+    SFG_TRY(s.get(&longest, (size_t)(len / kRowCap) + 1));
     SFG_TRY(s.get(&slot, m));
     SFG_TRY(s.get(&words, kWCount));
     int* hw32 = nullptr;
@@ -1157,7 +1337,8 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     if (m > 0) {
         auto* count = validate ? k_row_count<false> : k_row_count<true>;
         count<<<grid_of(ctx, count, (m + 3) / 4), kBlock, 0, ctx->stream>>>(n, m, u, v, w, cnt, slot, words);
-        k_row_classify<<<grid_of(ctx, k_row_classify, n), kBlock, 0, ctx->stream>>>(n, cnt, lwarp, mid, big, large, words);
+        k_row_classify<<<grid_of(ctx, k_row_classify, n), kBlock, 0, ctx->stream>>>(n, cnt, lwarp, mid, big, large, longest,
+                                                                                        words);
         ctx->launches += 2;
         SFG_LAUNCH_CHECK(ctx, "k_row_count");
     }
@@ -1167,11 +1348,13 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     if (validate && hw[kWErr])
         return sfg_fail(ctx, SFG_EINVAL,
                         "edge list: endpoint outside [0, n) or weight not finite and > 0");
-    if (hw[kWMax] > (unsigned long long)kRowCap) {
+    const int32_t nwarp = (int32_t)hw[kWWarp], nmid = (int32_t)hw[kWMid], nbig = (int32_t)hw[kWBig], nlarge = (int32_t)hw[kWLarge],
+                  nlong = (int32_t)hw[kWLong];
+    const int64_t long_raw = (int64_t)hw[kWLongRaw];
+    if (long_raw > len / 4) {
         *fits = false;
         return SFG_OK;
     }
-    const int32_t nwarp = (int32_t)hw[kWWarp], nmid = (int32_t)hw[kWMid], nbig = (int32_t)hw[kWBig], nlarge = (int32_t)hw[kWLarge];
 
     sfg_graph* g = new sfg_graph();
     struct Owner { sfg_graph* g; ~Owner() { sfg_graph_free(g); } } own{g};
@@ -1223,7 +1406,8 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     if (nmid > 0) SFG_TRY(rows_cta(k_rows_cta<128, kRowMid>, 128, kRowMid, nmid, mid));
     if (nbig > 0) SFG_TRY(rows_cta(k_rows_cta<256, kRowBig>, 256, kRowBig, nbig, big));
     if (nlarge > 0) SFG_TRY(rows_cta(k_rows_cta<1024, kRowCap>, 1024, kRowCap, nlarge, large));
-    if (nwarp + nmid + nbig + nlarge > 0) {
+    if (nlong > 0) SFG_TRY(long_rows(ctx, n, m, nlong, long_raw, longest, cnt, off, raw, w, ro));
+    if (nwarp + nmid + nbig + nlarge + nlong > 0) {
         k_deg_ordered<<<4 * ctx->num_sms, kBlock, 0, ctx->stream>>>(off, ro);
         ++ctx->launches;
     }
@@ -1276,7 +1460,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
 
 sfg_status sfg_build_graph(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
                            const float* w, bool validate, sfg_graph** out, int32_t* f2c) {
-    if (n > 0 && m < (1ll << 30)) {
+    if (n > 0 && m < (1ll << 30) && !ctx->build_sorts) {
         bool fits = false;
         SFG_TRY(build_by_rows(ctx, n, m, u, v, w, validate, out, f2c, &fits));
         if (fits) return SFG_OK;

@@ -59,6 +59,7 @@ struct sfg_ctx {
     int64_t fail_alloc_at = -1;            // SFG_FAULT_ALLOC=<n>: the n-th allocation fails
     int64_t fail_pool_at = -1;             // SFG_FAULT_POOL=<n>: the n-th finds the pool out of memory at
                                            // its first try, if it comes from the pool
+    bool build_sorts = false;              // SFG_BUILD_SORT=1: graphs are built by the sort of all entries
     bool withhold_mma = false;             // SFG_FAULT_MMA_WAIT=1: tensor-core kernels issue no
                                            // MMA, so their bounded completion waits run out
     int* grid_status = nullptr;            // host word that grid barriers set when a wait runs out
