@@ -417,6 +417,9 @@ static sfg_status batch_build(sfg_ctx* ctx, int ng, const sfg_graph* const* gs, 
 
     // the disjoint union U
     SFG_TRY(sfg_alloc_graph(ctx, n, m, &b->U));
+    b->U->reach = 0.0;
+    for (int g = 0; g < ng; ++g)
+        if (gs[g]->m > 0) b->U->reach += gs[g]->reach * ((double)gs[g]->m / (double)m);
     if (m > 0) {
         k_union_edges<<<grid_of(ctx, k_union_edges, m), kBlock, 0, ctx->stream>>>(
             m, d_desc, ng, b->d_eoff, b->U->eu, b->U->ev, b->U->ew);

@@ -263,8 +263,8 @@ constexpr int kRowSmall = 32, kRowWarp = 256, kRowMid = 1024, kRowBig = 4096, kR
 
 // Words the build reads back: input error, rows of the five larger classes, raw entries of the longest class, merged
 // rows over SFG_HEAVY_ROW, raw entries, merged entries, canonical edges; rows left to k_deg_ordered, of up to
-// kRowWarp entries and longer.
-enum { kWErr, kWWarp, kWMid, kWBig, kWLarge, kWLong, kWLongRaw, kWHeavy, kWRaw, kWNnz, kWEdges, kWDegShort, kWDegLong, kWCount };
+// kRowWarp entries and longer; summed |u - v|.
+enum { kWErr, kWWarp, kWMid, kWBig, kWLarge, kWLong, kWLongRaw, kWHeavy, kWRaw, kWNnz, kWEdges, kWDegShort, kWDegLong, kWReach, kWCount };
 
 // Raw row lengths and each entry's place within its row (slot.x in row u, slot.y in row v; -1 for
 // self-loops and bad edges). A warp whose edges all share an endpoint (a hub's edges in a sorted
@@ -276,7 +276,10 @@ __global__ void __launch_bounds__(kBlock)
                 const float* __restrict__ w, int32_t* __restrict__ cnt, int2* __restrict__ slot,
                 unsigned long long* __restrict__ words) {
     constexpr int Q = 4;
+    __shared__ unsigned long long s_reach;
     const int lane = threadIdx.x & 31;
+    unsigned long long reach = 0;
+    if (threadIdx.x == 0) s_reach = 0ull;
     auto place = [&](int32_t r, bool ok) {
         if (MATCH) {
             const unsigned peers = __match_any_sync(0xffffffffu, ok ? r : -1);
@@ -318,8 +321,15 @@ __global__ void __launch_bounds__(kBlock)
             const bool ok = a[q] >= 0 && a[q] != b[q];
             const int32_t x = place(a[q], ok), y = place(b[q], ok);
             if (e < m) slot[e] = make_int2(x, y);
+            reach += (unsigned)abs(a[q] - b[q]);
         }
     }
+    __syncthreads();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) reach += __shfl_xor_sync(0xffffffffu, reach, o);
+    if (lane == 0 && reach) atomicAdd(&s_reach, reach);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_reach) atomicAdd(words + kWReach, s_reach);
 }
 
 // The rows of the five larger classes (in no particular order) and the raw entries of the longest.
@@ -1421,6 +1431,7 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
     SFG_CUDA(ctx, cudaMemcpyAsync(hw, words, sizeof(unsigned long long) * kWCount, cudaMemcpyDeviceToHost,
                                   ctx->stream));
     SFG_TRY(sfg_wait(ctx));
+    g->reach = m > 0 ? (double)hw[kWReach] / (double)m : 0.0;
     const int64_t entries = (int64_t)hw[kWNnz], mc = (int64_t)hw[kWEdges];
     g->m = mc;
     SFG_TRY(sfg_alloc(ctx, (void**)&g->eu, sizeof(int32_t) * mc + 16));
@@ -1498,6 +1509,7 @@ sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* ma
     sfg_graph* p = nullptr;
     SFG_TRY(sfg_alloc_graph(ctx, g->n, ms, &p));
     struct Owner { sfg_graph* g; ~Owner() { sfg_graph_free(g); } } own{p};
+    p->reach = g->reach;
     int32_t* rest = nullptr;
     if (off_ids) SFG_TRY(s.get(&rest, m - ms));
     if (m > 0) {

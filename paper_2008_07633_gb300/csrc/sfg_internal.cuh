@@ -6,6 +6,7 @@
 
 #include <cstdint>
 #include <algorithm>
+#include <cmath>
 #include <map>
 #include <cstdio>
 #include <string>
@@ -71,6 +72,7 @@ struct sfg_graph {
     int device = -1;           // device that holds the arrays
     int32_t n = 0;
     int64_t m = 0;             // canonical edges
+    double reach = INFINITY;   // mean |u - v| of the edges it was built from (of its supergraph's; infinite: not known)
     int32_t* eu = nullptr;     // [m] canonical edge endpoints, eu < ev, sorted
     int32_t* ev = nullptr;
     float* ew = nullptr;       // [m]

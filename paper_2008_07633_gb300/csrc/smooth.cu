@@ -35,7 +35,9 @@ constexpr int kJNumVariants = 6, kJDefault = 1;
 // sums are per CTA). AHEAD: each tile also prefetches into L2 the rows kAheadBytes after its own, past
 // the rows that the running CTAs gather, so that first touches come from L2; the distance is in the
 // instruction and costs no register. It pays where the gathers leave the L1 pipe room for one more
-// request a row: low degrees (spanning forests) or other widths than 8 FP32 lanes. Measured (GB300, us a
+// request a row: low degrees (spanning forests) or other widths than 8 FP32 lanes. It costs where neighbours are
+// scattered, since every row is then gathered long before or after its turn: graphs whose edges reach over
+// kNearBytes of the block on average keep two tiles a turn. Measured (GB300, us a
 // sweep on the graph, on its spanning forest: two tiles a turn / one tile / two tiles AHEAD / one AHEAD):
 //   128^3 grid K = 4 FP32 (1 lane)       48/48/48/48      42/42/42/41
 //   300k mesh K = 4 FP32                 11/11/11/11      10.9/9.4/10.9/9.6
@@ -46,13 +48,20 @@ constexpr int kJNumVariants = 6, kJDefault = 1;
 //   2048^2 power grid K = 64 BF16 (8)    284/274/298/273  274/268/284/259
 //   1000^2 power grid K = 64 FP32 (16)   124/140/114/132  118/134/107/128
 //   2^20-node Chung-Lu K = 32 FP32       327/325/346/343  212/153/210/154
+// and on scattered graphs (mean reach 45-170 MB; forest not measured):
+//   random, 2^20 nodes, 2M edges K = 32 FP32  106/105/124/123    8M edges K = 64 BF16  314/314/320/320
+//   unsorted k-NN, 2M nodes      K = 64 FP32  939/936/964/959    K = 64 BF16           473/475/509/492
+// (reach of the meshes above: 0.1-1.4 MB; of the k-NN graphs of up to 100,000 nodes in a batch, 16 FP32: about 2 MB,
+// where the prefetch gains 1%).
 constexpr int64_t kAheadBytes = 4 << 20;
+constexpr double kNearBytes = 8 << 20;
 enum { kFormTwo, kFormOne, kFormTwoAhead, kFormOneAhead };
 template <typename T, int LPR>
 int plain_form(const sfg_graph* L) {
     if (L->hv_spread) return LPR <= 8 ? kFormOne : kFormTwo;
     const bool bf16 = sizeof(T) == 2, sparse = L->m < 2 * (int64_t)L->n;
     if (LPR == 1) return kFormOne;
+    if (L->reach * (LPR * 16) > kNearBytes) return kFormTwo;
     if (LPR == 4 && bf16) return kFormTwo;
     if (LPR == 8) return bf16 ? kFormOneAhead : sparse ? kFormTwoAhead : kFormOne;
     return kFormTwoAhead;
