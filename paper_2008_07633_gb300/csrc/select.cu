@@ -33,8 +33,8 @@ constexpr int kTkPasses = 6, kTkBins = 2048, kTkUnroll = 8;
 __host__ __device__ constexpr int tk_shift(int pass) { return pass % 3 == 0 ? 21 : pass % 3 == 1 ? 10 : 0; }
 __host__ __device__ constexpr int tk_width(int pass) { return pass % 3 == 2 ? 10 : 11; }
 
-// Words of one launch: barrier count, ids out of order.
-enum { kTwBar, kTwOrder, kTwCount };
+// Words of one launch: barrier count, ids out of order, all kept ids or'ed.
+enum { kTwBar, kTwOrder, kTwBits, kTwCount };
 
 struct TkArgs {
     int64_t ne, k;
@@ -44,7 +44,7 @@ struct TkArgs {
     unsigned long long* words;  // zero at launch
     unsigned* keep;             // one bit a candidate, written by the kernel from here on
     long long* cta_kept;        // one count a CTA
-    unsigned* cnt;              // digit counts of the id sort, 256 x sort_ctas
+    unsigned* cnt;              // digit counts of the id sort, 256 x sort_ctas, and 256 totals
     int sort_ctas;
     int32_t* tmp;               // k
     int32_t* out;               // k
@@ -115,56 +115,112 @@ __device__ __forceinline__ int tk_scan(int v, int* all) {
     return before + inc - v;
 }
 
-// Stable sort of out[0, k) by id (as unsigned words): four 8-bit digits, CTA c of the first
-// sort_ctas owning one contiguous range.
+// Stable sort of out[0, k) by id (as unsigned words): as many 8-bit digits as the largest id has, CTA c of the first
+// sort_ctas owning one contiguous range. To find the first place of each digit in its range a CTA can read the whole
+// table of counts, sort_ctas words a thread: up to kTkSumRows CTAs that is shorter than another barrier; beyond, the
+// digits' rows of the table are scanned first, a CTA a row. Ids go in tiles of 2,048, a warp ranking 256 consecutive
+// ones by itself, so that a tile costs four CTA barriers. Whole selections of ids in no order (us, with every CTA
+// reading the table and 256 ids a step / so / separate sorting launches): 50,000 of 100,000 kept 114/75/195, 524,288
+// of 2^20 532/227/233, 2^21 of 2^22 1,406/305/333, all of 2^24 3,196/1,065/1,288.
+constexpr int kTkSumRows = 16, kTkSortPer = 8, kTkSortTile = kBlock * kTkSortPer;
+
 __device__ bool tk_sort_ids(const TkArgs& A, const GridBar& bar, unsigned& passed) {
-    __shared__ unsigned base[256], wcnt[kBlock / 32][256];
+    __shared__ unsigned base[256], wcnt[kBlock / 32][256], s_bits;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_bits = 0u;
     const int nc = A.sort_ctas;
     const int64_t per = (A.k + nc - 1) / nc;
     const int64_t lo = min(A.k, (int64_t)blockIdx.x * per), hi = min(A.k, lo + per);
     const bool mine = (int)blockIdx.x < nc;
+    unsigned* totals = A.cnt + (size_t)256 * nc;
     int32_t *from = A.out, *to = A.tmp;
-    for (int shift = 0; shift < 32; shift += 8) {
+    uint32_t bits = 0;
+    for (int shift = 0; shift < 32 && (shift == 0 || bits >> shift); shift += 8) {
         if (mine) {
             base[tid] = 0;
             __syncthreads();
-            for (int64_t i = lo + tid; i < hi; i += kBlock) atomicAdd(&base[((uint32_t)__ldcg(from + i) >> shift) & 0xff], 1u);
+            for (int64_t i0 = lo + tid; i0 < hi; i0 += kBlock * 4) {
+                uint32_t x[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) x[q] = i0 + q * kBlock < hi ? (uint32_t)__ldcg(from + i0 + q * kBlock) : 0u;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (i0 + q * kBlock < hi) atomicAdd(&base[(x[q] >> shift) & 0xff], 1u);
+                    bits |= x[q];
+                }
+            }
+            if (shift == 0) {
+                bits = __reduce_or_sync(0xffffffffu, bits);
+                if (lane == 0) atomicOr(&s_bits, bits);
+            }
             __syncthreads();
+            if (shift == 0 && tid == 0) atomicOr(A.words + kTwBits, (unsigned long long)s_bits);
             A.cnt[(size_t)tid * nc + blockIdx.x] = base[tid];
         }
         if (!grid_barrier(bar, passed)) return false;
+        if (shift == 0) bits = (uint32_t)*(volatile unsigned long long*)(A.words + kTwBits);
+        int all;
+        if (nc > kTkSumRows) {
+            for (int d = blockIdx.x; d < 256; d += gridDim.x) {
+                unsigned carry = 0;
+                for (int c0 = 0; c0 < nc; c0 += kBlock) {
+                    const int c = c0 + tid;
+                    const unsigned v = c < nc ? __ldcg(A.cnt + (size_t)d * nc + c) : 0u;
+                    const unsigned before = carry + (unsigned)tk_scan((int)v, &all);
+                    if (c < nc) A.cnt[(size_t)d * nc + c] = before;
+                    carry += (unsigned)all;
+                }
+                if (tid == 0) totals[d] = carry;
+            }
+            if (!grid_barrier(bar, passed)) return false;
+        }
         if (mine) {
             // first place of digit tid in this CTA's range: smaller digits, then earlier CTAs
             unsigned total = 0, before = 0;
-            for (int c = 0; c < nc; ++c) {
-                const unsigned v = __ldcg(A.cnt + (size_t)tid * nc + c);
-                if (c < (int)blockIdx.x) before += v;
-                total += v;
+            if (nc > kTkSumRows) {
+                total = __ldcg(totals + tid);
+                before = __ldcg(A.cnt + (size_t)tid * nc + blockIdx.x);
+            } else {
+                for (int c = 0; c < nc; ++c) {
+                    const unsigned v = __ldcg(A.cnt + (size_t)tid * nc + c);
+                    if (c < (int)blockIdx.x) before += v;
+                    total += v;
+                }
             }
-            int all;
-            const int first = tk_scan((int)total, &all);
-            base[tid] = (unsigned)first + before;
-            for (int64_t t0 = lo; t0 < hi; t0 += kBlock) {
+            base[tid] = (unsigned)tk_scan((int)total, &all) + before;
+            for (int64_t t0 = lo; t0 < hi; t0 += kTkSortTile) {
+                const int64_t i0 = t0 + warp * (32 * kTkSortPer) + lane;
+                uint32_t x[kTkSortPer];
+                int rank[kTkSortPer];
+#pragma unroll
+                for (int q = 0; q < kTkSortPer; ++q) x[q] = i0 + q * 32 < hi ? (uint32_t)__ldcg(from + i0 + q * 32) : 0u;
 #pragma unroll
                 for (int q = 0; q < kBlock / 32; ++q) wcnt[q][tid] = 0;
                 __syncthreads();
-                const int64_t i = t0 + tid;
-                const bool ok = i < hi;
-                const uint32_t x = ok ? (uint32_t)__ldcg(from + i) : 0u;
-                const int d = ok ? (int)((x >> shift) & 0xff) : 256;
-                const unsigned peers = __match_any_sync(0xffffffffu, d);
-                const int rank = __popc(peers & ((1u << lane) - 1u));
-                if (ok && rank == 0) wcnt[warp][d] = __popc(peers);
-                __syncthreads();
-                if (ok) {
-                    unsigned p = base[d] + rank;
-                    for (int q = 0; q < warp; ++q) p += wcnt[q][d];
-                    to[p] = (int32_t)x;
+#pragma unroll
+                for (int q = 0; q < kTkSortPer; ++q) {
+                    const bool ok = i0 + q * 32 < hi;
+                    const int d = ok ? (int)((x[q] >> shift) & 0xff) : 256;
+                    const unsigned peers = __match_any_sync(0xffffffffu, d);
+                    const unsigned earlier = __popc(peers & ((1u << lane) - 1u));
+                    rank[q] = ok ? (int)(wcnt[warp][d] + earlier) : 0;
+                    __syncwarp();
+                    if (ok && earlier == 0) wcnt[warp][d] += __popc(peers);
+                    __syncwarp();
                 }
                 __syncthreads();
+                unsigned at = base[tid];  // digit tid: the first place of each warp's ids
 #pragma unroll
-                for (int q = 0; q < kBlock / 32; ++q) base[tid] += wcnt[q][tid];
+                for (int q = 0; q < kBlock / 32; ++q) {
+                    const unsigned c = wcnt[q][tid];
+                    wcnt[q][tid] = at;
+                    at += c;
+                }
+                base[tid] = at;
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < kTkSortPer; ++q)
+                    if (i0 + q * 32 < hi) to[wcnt[warp][(x[q] >> shift) & 0xff] + rank[q]] = (int32_t)x[q];
                 __syncthreads();
             }
         }
@@ -173,7 +229,9 @@ __device__ bool tk_sort_ids(const TkArgs& A, const GridBar& bar, unsigned& passe
         from = to;
         to = t;
     }
-    return true;  // an even number of passes: the result is in out
+    if (from != A.out)  // an odd number of passes
+        for (int64_t i = (int64_t)blockIdx.x * kBlock + tid; i < A.k; i += (int64_t)gridDim.x * kBlock) A.out[i] = __ldcg(from + i);
+    return true;
 }
 
 // A barrier ran out (the status word says so): no selection; every CTA leaves -1 in its share of the list, so
@@ -293,7 +351,7 @@ sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, 
     if (k == 0) return SFG_OK;
     // at least 1,024 candidates a CTA: fewer CTAs make the barriers cheaper
     const int grid = sfg_coop_grid(ctx, (const void*)k_topk, kBlock, (ne + 3) / 4);
-    const int sort_ctas = (int)std::min<int64_t>(grid, (k + 4095) / 4096);
+    const int sort_ctas = (int)std::min<int64_t>(grid, (k + kTkSortTile - 1) / kTkSortTile);
     Scratch s(ctx);
     // The kept ids are written while other CTAs still read the lists: a list over its own inputs (an
     // in-place selection) is made beside them first.
@@ -306,7 +364,7 @@ sfg_status sfg_topk_impl(sfg_ctx* ctx, const float* scores, const int32_t* ids, 
     SFG_TRY(s.get(&zeroed, (size_t)kTkPasses * kTkBins + kTwCount));
     SFG_TRY(s.get(&a.keep, (size_t)(ne + 31) / 32));
     SFG_TRY(s.get(&a.cta_kept, grid));
-    SFG_TRY(s.get(&a.cnt, (size_t)256 * sort_ctas));
+    SFG_TRY(s.get(&a.cnt, (size_t)256 * (sort_ctas + 1)));
     SFG_TRY(s.get(&a.tmp, k));
     SFG_CUDA(ctx, cudaMemsetAsync(zeroed, 0, sizeof(unsigned long long) * ((size_t)kTkPasses * kTkBins + kTwCount),
                                   ctx->stream));
