@@ -130,7 +130,7 @@ __global__ void k_lap_lower(const int2* __restrict__ colval, const int32_t* __re
     }
 }
 
-// Degrees of the rows of at most hmax entries: FP64 sum in column order, one thread a row.
+// Degrees of the rows of at most hmax entries (longer rows: k_lap_deg_heavy): FP64 sum in column order, one thread a row.
 __global__ void k_lap_deg(const int32_t* __restrict__ row_ptr, const int2* __restrict__ colval,
                           int32_t n, int32_t hmax, double* __restrict__ deg, double* __restrict__ invdeg) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
@@ -1147,21 +1147,23 @@ sfg_status sfg_alloc_graph(sfg_ctx* ctx, int32_t n, int64_t m, sfg_graph** out) 
     return SFG_OK;
 }
 
-// Degrees of a graph whose rows are in place. The sweep's heavy-row lists are built with the graph, so
-// that later calls (which may be captured into a CUDA graph) never synchronise for them.
+// Degrees of a graph whose rows are in place, hub rows last: building the sweep's heavy-row lists (here, so that later
+// calls, which may be captured into a CUDA graph, never synchronise for them) can wait for the host, and
+// the other rows' degrees are queued by then.
 static sfg_status row_degrees(sfg_ctx* ctx, sfg_graph* g) {
+    if (g->n > 0) {
+        k_lap_deg<<<grid_of(ctx, k_lap_deg, g->n), kBlock, 0, ctx->stream>>>(g->row_ptr, g->colval, g->n, SFG_HEAVY_ROW,
+                                                                             g->deg, g->invdeg);
+        ++ctx->launches;
+        SFG_LAUNCH_CHECK(ctx, "k_lap_deg");
+    }
     SFG_TRY(sfg_heavy_prepare(ctx, g));
-    if (g->n == 0) return SFG_OK;
-    const int32_t hmax = g->hv_n > 0 ? SFG_HEAVY_ROW : INT32_MAX;
-    k_lap_deg<<<grid_of(ctx, k_lap_deg, g->n), kBlock, 0, ctx->stream>>>(g->row_ptr, g->colval, g->n, hmax, g->deg,
-                                                                         g->invdeg);
-    ++ctx->launches;
     if (g->hv_n > 0) {
         k_lap_deg_heavy<<<std::min(g->hv_n, 8 * ctx->num_sms), kBlock, 0, ctx->stream>>>(g->hv_n, g->hv_rows, g->row_ptr,
                                                                                          g->colval, g->deg, g->invdeg);
         ++ctx->launches;
+        SFG_LAUNCH_CHECK(ctx, "k_lap_deg_heavy");
     }
-    SFG_LAUNCH_CHECK(ctx, "k_lap_deg");
     return SFG_OK;
 }
 
