@@ -56,6 +56,7 @@ struct KeptDevice {
     std::once_flag once;
     int64_t room = 0, all = 0;       // bytes that may still be kept, and before any is
     std::vector<sfg_ctx*> contexts;
+    std::vector<void*> left;         // legacy blocks that lost their place while a capture forbade freeing them
     cudaStream_t frees = nullptr;    // the library's own: gives blocks back after their event, never on a user's stream
 };
 static KeptDevice kept_devices[kKeptDevices];
@@ -81,6 +82,7 @@ static void kept_register(sfg_ctx* ctx) {
     }
     std::lock_guard<std::mutex> lock(d.mu);
     ctx->kept.reserve(kKeptBlocks);
+    d.left.reserve(kKeptBlocks);
     d.contexts.push_back(ctx);
 }
 
@@ -92,9 +94,19 @@ static SfgKept kept_remove(sfg_ctx* ctx, size_t i) {  // with the device's lock
     return b;
 }
 
+// Frees in the order of the legacy stream; not while another stream's capture forbids its use.
+static void kept_free_legacy(KeptDevice& d, sfg_ctx* ctx) {  // with the device's lock
+    if (sfg_capturing(cudaStreamLegacy)) return;
+    for (void* p : d.left) cudaFreeAsync(p, cudaStreamLegacy);
+    d.left.clear();
+    for (size_t i = ctx->kept.size(); i-- > 0;)
+        if (ctx->kept[i].legacy) cudaFreeAsync(kept_remove(ctx, i).p, cudaStreamLegacy);
+}
+
 // Gives back what can be waited for without the context's stream, in the order of the event.
 static void kept_release(sfg_ctx* ctx) {  // with the device's lock
     KeptDevice& d = kept_device(ctx);
+    kept_free_legacy(d, ctx);
     bool first = true;
     for (size_t i = ctx->kept.size(); i-- > 0;) {
         if (!ctx->kept[i].settled) continue;
@@ -109,7 +121,9 @@ static void kept_release(sfg_ctx* ctx) {  // with the device's lock
 
 // The same in the order of the context's stream, which has to be alive and not captured.
 static void kept_free(sfg_ctx* ctx) {  // with the device's lock
-    for (size_t i = ctx->kept.size(); i-- > 0;) cudaFreeAsync(kept_remove(ctx, i).p, ctx->stream);
+    kept_free_legacy(kept_device(ctx), ctx);
+    for (size_t i = ctx->kept.size(); i-- > 0;)
+        if (!ctx->kept[i].legacy) cudaFreeAsync(kept_remove(ctx, i).p, ctx->stream);
 }
 
 // An allocation has failed: everything that any context of the device keeps goes back to the pool.
@@ -122,6 +136,7 @@ static void kept_reclaim(sfg_ctx* ctx) {
         for (sfg_ctx* c : d.contexts) kept_release(c);
     }
     cudaStreamSynchronize(d.frees);
+    if (!sfg_capturing(cudaStreamLegacy)) cudaStreamSynchronize(cudaStreamLegacy);
 }
 
 // The SMs that a stream's kernels can run on: those of its green context, if it has one, else the device's.
@@ -161,6 +176,7 @@ static void set_stream(sfg_ctx* ctx, cudaStream_t stream) {
     ctx->stream = stream;
     ctx->stream_id = id;
     ctx->stream_sms = stream_sms(ctx, stream);
+    ctx->on_legacy = stream == nullptr || stream == cudaStreamLegacy;
     ctx->stream_keeps = known && ctx->kept_event && stream != cudaStreamPerThread;
 }
 
@@ -201,8 +217,8 @@ sfg_status sfg_scratch_take(sfg_ctx* ctx, void** p, size_t* bytes) {
         std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
         size_t best = 0, size = SIZE_MAX;  // the smallest block that is large enough, if it is not much larger
         for (size_t i = 0; i < ctx->kept.size(); ++i) {
-            const size_t b = ctx->kept[i].bytes;
-            if (b >= *bytes && b < size) best = i, size = b;
+            const SfgKept& b = ctx->kept[i];
+            if (b.legacy == ctx->on_legacy && b.bytes >= *bytes && b.bytes < size) best = i, size = b.bytes;
         }
         if (size <= *bytes + *bytes / 4 + 4096) {
             const SfgKept b = kept_remove(ctx, best);
@@ -225,12 +241,16 @@ void sfg_scratch_give(sfg_ctx* ctx, void* p, size_t bytes) {
     {
         std::lock_guard<std::mutex> lock(d.mu);
         if (size <= share && size <= d.room + ctx->kept_bytes) {
-            while (ctx->kept.size() >= kKeptBlocks || ctx->kept_bytes + size > share || size > d.room)
-                out[nout++] = kept_remove(ctx, 0).p;
-            ctx->kept.push_back({p, bytes, false});  // the list has its room from the start: nothing throws
+            while (ctx->kept.size() >= kKeptBlocks || ctx->kept_bytes + size > share || size > d.room) {
+                const SfgKept b = kept_remove(ctx, 0);
+                if (b.legacy == ctx->on_legacy) out[nout++] = b.p;
+                else d.left.push_back(b.p);
+            }
+            ctx->kept.push_back({p, bytes, ctx->on_legacy, false});  // the list has its room from the start: nothing throws
             ctx->kept_bytes += size;
             d.room -= size;
-            ctx->kept_dirty = kept = true;
+            kept = true;
+            ctx->kept_dirty = !ctx->on_legacy;
         }
     }
     for (size_t i = 0; i < nout; ++i) sfg_free(ctx, out[i]);
@@ -245,6 +265,7 @@ void sfg_scratch_settle(sfg_ctx* ctx) {
     if (!ok) cudaGetLastError();
     std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
     for (size_t i = ctx->kept.size(); i-- > 0;) {
+        if (ctx->kept[i].legacy) continue;
         if (ok) ctx->kept[i].settled = true;
         else sfg_free(ctx, kept_remove(ctx, i).p);
     }
@@ -506,6 +527,7 @@ void sfg_ctx_destroy(sfg_ctx* ctx) {
         std::lock_guard<std::mutex> lock(d.mu);
         if (capturing) kept_release(ctx);
         else kept_free(ctx);
+        while (!ctx->kept.empty()) d.left.push_back(kept_remove(ctx, 0).p);
         d.contexts.erase(std::find(d.contexts.begin(), d.contexts.end(), ctx));
         cudaEventDestroy(ctx->kept_event);
     }

@@ -24,12 +24,13 @@ struct sfg_timer_rec {
     cudaEvent_t start, stop;
 };
 
-// A scratch block that a context keeps after the call that used it, free for work on its stream. settled: the
-// context's event has been recorded since it was given back, so that its last use can be waited for without
-// the stream.
+// A scratch block that a context keeps after the call that used it, free for work on its stream. legacy: used on the
+// legacy default stream, which is always there. settled: the context's event has been recorded since the block was
+// given back, so that its last use can be waited for without the stream.
 struct SfgKept {
     void* p;
     size_t bytes;
+    bool legacy;
     bool settled;
 };
 
@@ -49,13 +50,14 @@ struct sfg_ctx {
     std::map<uint32_t, int> score_tune;    // (K, dtype, degree bucket) -> scorer launch shape
     std::map<std::tuple<const void*, int, size_t>, int> occupancy;  // resident CTAs per SM
     // Scratch kept for the next call, oldest first (guarded by the device's lock: another context that runs
-    // out of memory takes it back). All of it was used on the current stream.
+    // out of memory takes it back). What is not marked legacy was used on the current stream.
     std::vector<SfgKept> kept;
     int64_t kept_bytes = 0;
     bool kept_dirty = false;               // blocks given back since the event was recorded
     cudaEvent_t kept_event = nullptr;      // NULL: nothing is kept
     unsigned long long stream_id = 0;      // of the current stream: a handle can name another stream later
     bool stream_keeps = false;             // not the per-thread default stream, whose handle names many
+    bool on_legacy = false;                // the current stream is the legacy default stream
     int64_t alloc_count = 0;               // for the allocation-failure injection hook
     int64_t fail_alloc_at = -1;            // SFG_FAULT_ALLOC=<n>: the n-th allocation fails
     int64_t fail_pool_at = -1;             // SFG_FAULT_POOL=<n>: the n-th finds the pool out of memory at
@@ -169,7 +171,8 @@ void sfg_free(sfg_ctx* ctx, void* p);
 // with sfg_ctx_trim, sfg_ctx_set_stream to another stream, sfg_ctx_destroy, and when an allocation of any
 // context on the device fails. An event recorded at the end of each call stands for the last use, so that a
 // change of stream never touches the old one: its owner may have destroyed it, work pending, and its handle
-// may already name another stream (streams are told apart by their ids).
+// may already name another stream (streams are told apart by their ids). The legacy default stream cannot be
+// destroyed and needs no event, which a call of 50 us would feel (1-2 us).
 // Why: the pool took 45-190 us for each of the four large blocks of an end-to-end call on the 128^3 grid, with the
 // GPU idle, and about 1 us for each small one (GB300, all scratch from the pool / kept: that call
 // 7,347 / 7,084 us, two-level 14,170 / 13,970, a 64 x 64 grid 257 / 241, a gradient over 65,536 rows 74 / 61).

@@ -90,10 +90,26 @@ def unused(S, ctx):
     return torch.cuda.mem_get_info()[0]
 
 
-def test_an_allocation_takes_back_what_idle_contexts_keep(S, monkeypatch):
+def test_between_the_legacy_stream_and_others(S):
+    home, side = torch.cuda.current_stream(), torch.cuda.Stream()
+    ctx = S.sfg_ctx_create(0)
+    g = graph(S, ctx, 500)
+    want = [S.sfg_smooth(ctx, g, 64, 6, seed=i).clone() for i in range(10)]
+    got = [torch.empty_like(x) for x in want]
+    torch.cuda.synchronize()
+    for i, out in enumerate(got):  # neither stream waits for the other
+        ctx.set_stream(side if i % 2 else home)
+        S.sfg_smooth(ctx, g, 64, 6, seed=i, out=out)
+    ctx.set_stream(home)
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(got, want))
+
+
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_an_allocation_takes_back_what_idle_contexts_keep(S, monkeypatch, own_stream):
     other = S.sfg_ctx_create(0)
     small = graph(S, other, 40)
-    idle, g = kept(S)
+    idle, g = kept(S, torch.cuda.Stream() if own_stream else None)
     before = unused(S, other)                     # the idle context's blocks stay
     monkeypatch.setenv("SFG_FAULT_POOL", "3")
     ctx = S.sfg_ctx_create(0)
