@@ -9,6 +9,7 @@
 // rounded once to FP32; the upper-triangle entries, in order, are the canonical edge list (edge id
 // = rank among them), and a lower-triangle entry takes the id of its mirror.
 #include <cmath>
+#include <type_traits>
 
 #include "sfg_internal.cuh"
 #include "dot64.cuh"
@@ -951,16 +952,18 @@ __global__ void k_row_index(int32_t n, const int64_t* __restrict__ off, const in
     }
 }
 
-// Edge ids, the edge list, and (MOVE) the entries themselves at their final places. An upper entry's
-// id comes from its own place, a lower entry's from its mirror's.
-template <bool MOVE>
+// Edge ids, the edge list and, where anything was merged or dropped, the entries themselves at their final places
+// (else the sorted rows are the CSR rows). An upper entry's id comes from its own place, a lower entry's
+// from its mirror's.
 __global__ void __launch_bounds__(kBlock)
-    k_entries_write(int64_t len, const int32_t* __restrict__ rrow, const int2* __restrict__ rcv,
+    k_entries_write(int64_t listed, const unsigned long long* __restrict__ words, const int32_t* __restrict__ rrow, const int2* __restrict__ rcv,
                     const int32_t* __restrict__ re, const int32_t* __restrict__ rpos,
                     const int32_t* __restrict__ D, const int32_t* __restrict__ move, int2* __restrict__ colval,
                     int32_t* __restrict__ eid, int32_t* __restrict__ eu, int32_t* __restrict__ ev,
                     float* __restrict__ ew) {
     constexpr int Q = 4;  // entries in flight a thread
+    const int64_t len = (int64_t)words[kWRaw];  // raw places end where the rows do: self-loops were never placed
+    const bool moved = (int64_t)words[kWNnz] != listed;
     for (int64_t j0 = (int64_t)blockIdx.x * (kBlock * Q) + threadIdx.x; j0 < len; j0 += (int64_t)gridDim.x * (kBlock * Q)) {
         int32_t r[Q], e[Q], id[Q];
         int2 cv[Q];
@@ -982,7 +985,7 @@ __global__ void __launch_bounds__(kBlock)
         for (int q = 0; q < Q; ++q) {
             if (r[q] < 0) continue;
             int64_t dst = j0 + q * kBlock;
-            if (MOVE) {
+            if (moved) {
                 dst += move[r[q]];
                 colval[dst] = cv[q];
             }
@@ -1318,10 +1321,31 @@ static sfg_status long_rows(sfg_ctx* ctx, int32_t n, int64_t m, int32_t count, i
     return SFG_OK;
 }
 
+// Lists of up to so many edges get arrays for all of them before the merged sizes are known (a second wait of the
+// host otherwise, 5-15 us of idle GPU); more than a quarter left unused goes back.
+constexpr int64_t kEarlyEdges = 1 << 24;
+
+static sfg_status fit_edges(sfg_ctx* ctx, sfg_graph* g, int64_t room, int64_t mc, int64_t entries) {
+    if (mc >= room - room / 4) return SFG_OK;
+    auto fit = [&](auto** p, int64_t count) -> sfg_status {
+        void* q = nullptr;
+        SFG_TRY(sfg_alloc(ctx, &q, sizeof(**p) * (size_t)count + 16));
+        const cudaError_t e = cudaMemcpyAsync(q, *p, sizeof(**p) * (size_t)count, cudaMemcpyDeviceToDevice, ctx->stream);
+        sfg_free(ctx, *p);
+        *p = static_cast<std::remove_reference_t<decltype(*p)>>(q);
+        return e == cudaSuccess ? SFG_OK : sfg_cuda_fail(ctx, e, "graph arrays");
+    };
+    SFG_TRY(fit(&g->eu, mc));
+    SFG_TRY(fit(&g->ev, mc));
+    SFG_TRY(fit(&g->ew, mc));
+    SFG_TRY(fit(&g->colval, entries));
+    return fit(&g->eid, entries);
+}
+
 // Canonical form by rows (see k_row_count). *fits = false (and nothing built) when rows of more than kRowCap raw
 // entries hold over a quarter of them: the sort of all entries then moves little more than theirs. (GPU time from the
 // list, by rows / by the sort: one row of 500,000 of 6.9M entries 1,590 / 1,800 us, one of 2M of 4M 2,770 / 2,390.)
-// Two host waits: the input check with the sizes of the row classes, and the merged sizes.
+// Two host waits: the input check with the sizes of the row classes, and the merged sizes (see kEarlyEdges).
 static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u, const int32_t* v,
                                 const float* w, bool validate, sfg_graph** out, int32_t* f2c, bool* fits) {
     *out = nullptr;
@@ -1430,28 +1454,27 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
         n, off, row_off, up_off, nnz, up, g->row_ptr, D, move, words);
     ++ctx->launches;
     SFG_LAUNCH_CHECK(ctx, "k_row_index");
-    SFG_CUDA(ctx, cudaMemcpyAsync(hw, words, sizeof(unsigned long long) * kWCount, cudaMemcpyDeviceToHost,
-                                  ctx->stream));
-    SFG_TRY(sfg_wait(ctx));
-    g->reach = m > 0 ? (double)hw[kWReach] / (double)m : 0.0;
-    const int64_t entries = (int64_t)hw[kWNnz], mc = (int64_t)hw[kWEdges];
-    g->m = mc;
+    // A new list gets room for all its entries, so that the host need not wait for the merged sizes before the last
+    // kernel can be queued: the one wait left is that for the whole build.
+    const bool early = validate && m <= kEarlyEdges;
+    int64_t entries = len, mc = m;
+    auto read_sizes = [&]() -> sfg_status {
+        SFG_CUDA(ctx, cudaMemcpyAsync(hw, words, sizeof(unsigned long long) * kWCount, cudaMemcpyDeviceToHost, ctx->stream));
+        SFG_TRY(sfg_wait(ctx));
+        entries = (int64_t)hw[kWNnz];
+        mc = (int64_t)hw[kWEdges];
+        return SFG_OK;
+    };
+    if (!early) SFG_TRY(read_sizes());
     SFG_TRY(sfg_alloc(ctx, (void**)&g->eu, sizeof(int32_t) * mc + 16));
     SFG_TRY(sfg_alloc(ctx, (void**)&g->ev, sizeof(int32_t) * mc + 16));
     SFG_TRY(sfg_alloc(ctx, (void**)&g->ew, sizeof(float) * mc + 16));
     SFG_TRY(sfg_alloc(ctx, (void**)&g->eid, sizeof(int32_t) * entries + 16));
-    const bool moved = entries != len;  // else nothing was merged or dropped: the sorted rows are the CSR rows
-    if (!moved && len > 0) {
-        s.release(rcv);
-        g->colval = rcv;
-    } else {
-        SFG_TRY(sfg_alloc(ctx, (void**)&g->colval, sizeof(int2) * entries + 16));
-    }
+    int2* moved = nullptr;  // the entries if they are moved
+    if (early || entries != len || len == 0) SFG_TRY(s.get(&moved, (size_t)entries + 2));
     if (entries > 0) {
-        auto* write = moved ? k_entries_write<true> : k_entries_write<false>;
-        // raw places end where the rows do: self-loops were never placed
-        write<<<grid_of(ctx, write, (len + 3) / 4), kBlock, 0, ctx->stream>>>(
-            (int64_t)hw[kWRaw], rrow, rcv, re, rpos, D, move, g->colval, g->eid, g->eu, g->ev, g->ew);
+        k_entries_write<<<grid_of(ctx, k_entries_write, (len + 3) / 4), kBlock, 0, ctx->stream>>>(
+            len, words, rrow, rcv, re, rpos, D, move, moved, g->eid, g->eu, g->ev, g->ew);
         ++ctx->launches;
     }
     if (f2c && m > 0) {
@@ -1459,6 +1482,12 @@ static sfg_status build_by_rows(sfg_ctx* ctx, int32_t n, int64_t m, const int32_
         ++ctx->launches;
     }
     SFG_LAUNCH_CHECK(ctx, "k_entries_write");
+    if (early) SFG_TRY(read_sizes());
+    g->colval = entries != len || len == 0 ? moved : rcv;
+    s.release(g->colval);
+    if (early) SFG_TRY(fit_edges(ctx, g, m, mc, entries));
+    g->m = mc;
+    g->reach = m > 0 ? (double)hw[kWReach] / (double)m : 0.0;
     // the sweep's heavy-row lists are built with the graph, so that later calls (which may be
     // captured into a CUDA graph) never synchronise for them
     if (hw[kWHeavy] == 0) {
