@@ -77,7 +77,8 @@ SFG_API void sfg_ctx_destroy(sfg_ctx* ctx);
  * keeps scratch blocks of its last calls (at most 1/128 of the device's memory, and the contexts
  * of a device together 1/32) for its next call on the same stream. sfg_ctx_trim synchronises the context stream and
  * returns what the context keeps and the pool's unused memory to the device (an allocation that
- * fails takes back what all contexts of the device keep, trims and retries once). sfg_ctx_set_stream to another
+ * fails takes back what it and the contexts of the device that are not in a call keep, trims and retries once).
+ * sfg_ctx_set_stream to another
  * stream gives the kept blocks back to the pool once the work that used them is done; it does not touch the
  * stream that the context leaves, which may have been destroyed. */
 SFG_API sfg_status sfg_ctx_trim(sfg_ctx* ctx);

@@ -52,9 +52,10 @@ constexpr int64_t kKeptShare = 128, kKeptDeviceShare = 32;  // of a device's mem
 
 // What the contexts of one device keep together.
 struct KeptDevice {
-    std::mutex mu;  // guards the fields here and the contexts' lists
+    std::mutex mu;  // guards the two lists
     std::once_flag once;
-    int64_t room = 0, all = 0;       // bytes that may still be kept, and before any is
+    std::atomic<int64_t> room{0};    // bytes that may still be kept
+    int64_t all = 0;                 // the same before any is
     std::vector<sfg_ctx*> contexts;
     std::vector<void*> left;         // legacy blocks that lost their place while a capture forbade freeing them
     cudaStream_t frees = nullptr;    // the library's own: gives blocks back after their event, never on a user's stream
@@ -86,27 +87,26 @@ static void kept_register(sfg_ctx* ctx) {
     d.contexts.push_back(ctx);
 }
 
-static SfgKept kept_remove(sfg_ctx* ctx, size_t i) {  // with the device's lock
+// From here on to sfg_scratch_settle: with the context's lock.
+static SfgKept kept_remove(sfg_ctx* ctx, size_t i) {
     const SfgKept b = ctx->kept[i];
-    kept_device(ctx).room += (int64_t)b.bytes;
+    kept_device(ctx).room.fetch_add((int64_t)b.bytes);
     ctx->kept_bytes -= (int64_t)b.bytes;
     ctx->kept.erase(ctx->kept.begin() + i);
     return b;
 }
 
 // Frees in the order of the legacy stream; not while another stream's capture forbids its use.
-static void kept_free_legacy(KeptDevice& d, sfg_ctx* ctx) {  // with the device's lock
+static void kept_free_legacy(sfg_ctx* ctx) {
     if (sfg_capturing(cudaStreamLegacy)) return;
-    for (void* p : d.left) cudaFreeAsync(p, cudaStreamLegacy);
-    d.left.clear();
     for (size_t i = ctx->kept.size(); i-- > 0;)
         if (ctx->kept[i].legacy) cudaFreeAsync(kept_remove(ctx, i).p, cudaStreamLegacy);
 }
 
 // Gives back what can be waited for without the context's stream, in the order of the event.
-static void kept_release(sfg_ctx* ctx) {  // with the device's lock
+static void kept_release(sfg_ctx* ctx) {
     KeptDevice& d = kept_device(ctx);
-    kept_free_legacy(d, ctx);
+    kept_free_legacy(ctx);
     bool first = true;
     for (size_t i = ctx->kept.size(); i-- > 0;) {
         if (!ctx->kept[i].settled) continue;
@@ -120,20 +120,32 @@ static void kept_release(sfg_ctx* ctx) {  // with the device's lock
 }
 
 // The same in the order of the context's stream, which has to be alive and not captured.
-static void kept_free(sfg_ctx* ctx) {  // with the device's lock
-    kept_free_legacy(kept_device(ctx), ctx);
+static void kept_free(sfg_ctx* ctx) {
+    kept_free_legacy(ctx);
     for (size_t i = ctx->kept.size(); i-- > 0;)
         if (!ctx->kept[i].legacy) cudaFreeAsync(kept_remove(ctx, i).p, ctx->stream);
 }
 
-// An allocation has failed: everything that any context of the device keeps goes back to the pool.
+// Blocks that lost their context or place while a capture forbade freeing them.
+static void kept_free_left(KeptDevice& d) {  // with the device's lock
+    if (d.left.empty() || sfg_capturing(cudaStreamLegacy)) return;
+    for (void* p : d.left) cudaFreeAsync(p, cudaStreamLegacy);
+    d.left.clear();
+}
+
+// An allocation has failed: everything that this context and those not in a call keep goes back to the pool.
 static void kept_reclaim(sfg_ctx* ctx) {
     if (!ctx->kept_event) return;
     KeptDevice& d = kept_device(ctx);
+    if (!sfg_capturing(ctx->stream)) kept_free(ctx);
     {
         std::lock_guard<std::mutex> lock(d.mu);
-        if (!sfg_capturing(ctx->stream)) kept_free(ctx);
-        for (sfg_ctx* c : d.contexts) kept_release(c);
+        kept_free_left(d);
+        for (sfg_ctx* c : d.contexts) {
+            if (c == ctx || c->kept_lock.exchange(1, std::memory_order_acquire)) continue;
+            kept_release(c);
+            c->kept_lock.store(0, std::memory_order_release);
+        }
     }
     cudaStreamSynchronize(d.frees);
     if (!sfg_capturing(cudaStreamLegacy)) cudaStreamSynchronize(cudaStreamLegacy);
@@ -169,10 +181,7 @@ static void set_stream(sfg_ctx* ctx, cudaStream_t stream) {
     unsigned long long id = 0;
     const bool known = cudaStreamGetId(stream, &id) == cudaSuccess;
     if (!known) cudaGetLastError();
-    if (ctx->kept_event && (!known || id != ctx->stream_id)) {
-        std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
-        kept_release(ctx);
-    }
+    if (ctx->kept_event && (!known || id != ctx->stream_id)) kept_release(ctx);
     ctx->stream = stream;
     ctx->stream_id = id;
     ctx->stream_sms = stream_sms(ctx, stream);
@@ -213,19 +222,16 @@ sfg_status sfg_alloc(sfg_ctx* ctx, void** p, size_t bytes) {
 sfg_status sfg_scratch_take(sfg_ctx* ctx, void** p, size_t* bytes) {
     *p = nullptr;
     if (alloc_fails(ctx)) return alloc_injected(ctx);
-    {
-        std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
-        size_t best = 0, size = SIZE_MAX;  // the smallest block that is large enough, if it is not much larger
-        for (size_t i = 0; i < ctx->kept.size(); ++i) {
-            const SfgKept& b = ctx->kept[i];
-            if (b.legacy == ctx->on_legacy && b.bytes >= *bytes && b.bytes < size) best = i, size = b.bytes;
-        }
-        if (size <= *bytes + *bytes / 4 + 4096) {
-            const SfgKept b = kept_remove(ctx, best);
-            *p = b.p;
-            *bytes = b.bytes;
-            return SFG_OK;
-        }
+    size_t best = 0, size = SIZE_MAX;  // the smallest block that is large enough, if it is not much larger
+    for (size_t i = 0; i < ctx->kept.size(); ++i) {
+        const SfgKept& b = ctx->kept[i];
+        if (b.legacy == ctx->on_legacy && b.bytes >= *bytes && b.bytes < size) best = i, size = b.bytes;
+    }
+    if (size <= *bytes + *bytes / 4 + 4096) {
+        const SfgKept b = kept_remove(ctx, best);
+        *p = b.p;
+        *bytes = b.bytes;
+        return SFG_OK;
     }
     return pool_alloc(ctx, p, *bytes);
 }
@@ -235,26 +241,28 @@ sfg_status sfg_scratch_take(sfg_ctx* ctx, void** p, size_t* bytes) {
 void sfg_scratch_give(sfg_ctx* ctx, void* p, size_t bytes) {
     KeptDevice& d = kept_device(ctx);
     const int64_t size = (int64_t)bytes, share = d.all / (kKeptShare / kKeptDeviceShare);
-    void* out[kKeptBlocks];
-    size_t nout = 0;
-    bool kept = false;
-    {
-        std::lock_guard<std::mutex> lock(d.mu);
-        if (size <= share && size <= d.room + ctx->kept_bytes) {
-            while (ctx->kept.size() >= kKeptBlocks || ctx->kept_bytes + size > share || size > d.room) {
-                const SfgKept b = kept_remove(ctx, 0);
-                if (b.legacy == ctx->on_legacy) out[nout++] = b.p;
-                else d.left.push_back(b.p);
-            }
-            ctx->kept.push_back({p, bytes, ctx->on_legacy, false});  // the list has its room from the start: nothing throws
-            ctx->kept_bytes += size;
-            d.room -= size;
-            kept = true;
-            ctx->kept_dirty = !ctx->on_legacy;
+    if (size > share || size > d.room.load() + ctx->kept_bytes) return sfg_free(ctx, p);
+    auto reserve = [&] {
+        if (ctx->kept.size() >= kKeptBlocks || ctx->kept_bytes + size > share) return false;
+        if (d.room.fetch_sub(size) >= size) return true;
+        d.room.fetch_add(size);
+        return false;
+    };
+    bool room = reserve();
+    while (!room && !ctx->kept.empty()) {
+        const SfgKept b = kept_remove(ctx, 0);
+        if (b.legacy == ctx->on_legacy) {
+            sfg_free(ctx, b.p);
+        } else {
+            std::lock_guard<std::mutex> lock(d.mu);
+            d.left.push_back(b.p);
         }
+        room = reserve();
     }
-    for (size_t i = 0; i < nout; ++i) sfg_free(ctx, out[i]);
-    if (!kept) sfg_free(ctx, p);
+    if (!room) return sfg_free(ctx, p);
+    ctx->kept.push_back({p, bytes, ctx->on_legacy, false});  // the list has its room from the start: nothing throws
+    ctx->kept_bytes += size;
+    ctx->kept_dirty = !ctx->on_legacy;
 }
 
 // At the end of a call: the context's event stands for the last use of everything it keeps. (Nothing is given
@@ -263,7 +271,6 @@ void sfg_scratch_settle(sfg_ctx* ctx) {
     ctx->kept_dirty = false;
     const bool ok = cudaEventRecord(ctx->kept_event, ctx->stream) == cudaSuccess;
     if (!ok) cudaGetLastError();
-    std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
     for (size_t i = ctx->kept.size(); i-- > 0;) {
         if (ctx->kept[i].legacy) continue;
         if (ok) ctx->kept[i].settled = true;
@@ -501,8 +508,9 @@ sfg_status sfg_ctx_trim(sfg_ctx* ctx) {
     if (!ctx) return SFG_EINVAL;
     SFG_DEVICE(ctx);
     if (ctx->kept_event) {
-        std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
         kept_free(ctx);
+        std::lock_guard<std::mutex> lock(kept_device(ctx).mu);
+        kept_free_left(kept_device(ctx));
     }
     SFG_TRY(sfg_wait(ctx));
     SFG_CUDA(ctx, cudaMemPoolTrimTo(ctx->pool, 0));
@@ -524,11 +532,15 @@ void sfg_ctx_destroy(sfg_ctx* ctx) {
     }
     if (ctx->kept_event) {
         KeptDevice& d = kept_device(ctx);
-        std::lock_guard<std::mutex> lock(d.mu);
+        {   // no other context takes from this one any more
+            std::lock_guard<std::mutex> lock(d.mu);
+            d.contexts.erase(std::find(d.contexts.begin(), d.contexts.end(), ctx));
+        }
         if (capturing) kept_release(ctx);
         else kept_free(ctx);
+        std::lock_guard<std::mutex> lock(d.mu);
         while (!ctx->kept.empty()) d.left.push_back(kept_remove(ctx, 0).p);
-        d.contexts.erase(std::find(d.contexts.begin(), d.contexts.end(), ctx));
+        kept_free_left(d);
         cudaEventDestroy(ctx->kept_event);
     }
     // unused memory goes back to the device; memory of live graphs stays valid

@@ -6,6 +6,7 @@
 
 #include <cstdint>
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <map>
 #include <cstdio>
@@ -49,8 +50,11 @@ struct sfg_ctx {
     std::map<uint32_t, int> tune;          // (K, dtype, degree bucket) -> sweep variant
     std::map<uint32_t, int> score_tune;    // (K, dtype, degree bucket) -> scorer launch shape
     std::map<std::tuple<const void*, int, size_t>, int> occupancy;  // resident CTAs per SM
-    // Scratch kept for the next call, oldest first (guarded by the device's lock: another context that runs
-    // out of memory takes it back). What is not marked legacy was used on the current stream.
+    // Scratch kept for the next call, oldest first. What is not marked legacy was used on the current stream. A call
+    // on the context holds kept_lock throughout; another context that runs out of memory takes the blocks of
+    // contexts that are not in a call (it never waits for the lock).
+    std::atomic<int> kept_lock{0};
+    int call_depth = 0;                    // entry points call one another
     std::vector<SfgKept> kept;
     int64_t kept_bytes = 0;
     bool kept_dirty = false;               // blocks given back since the event was recorded
@@ -129,11 +133,18 @@ void sfg_scratch_settle(sfg_ctx* ctx);
 struct SfgCall {
     SfgDeviceGuard device;
     sfg_ctx* ctx;
-    explicit SfgCall(sfg_ctx* c) : device(c->device), ctx(c) {}
+    explicit SfgCall(sfg_ctx* c) : device(c->device), ctx(c) {
+        if (c->call_depth++ == 0)
+            while (c->kept_lock.exchange(1, std::memory_order_acquire)) {}  // held for some frees at most
+    }
     explicit SfgCall(const sfg_ctx* c) : device(c->device), ctx(nullptr) {}
     ~SfgCall() {
-        if (ctx && ctx->kept_dirty) sfg_scratch_settle(ctx);
+        if (!ctx) return;
+        if (ctx->kept_dirty) sfg_scratch_settle(ctx);
+        if (--ctx->call_depth == 0) ctx->kept_lock.store(0, std::memory_order_release);
     }
+    SfgCall(const SfgCall&) = delete;
+    SfgCall& operator=(const SfgCall&) = delete;
 };
 #define SFG_DEVICE(ctx) SfgCall sfg_call_(ctx)
 

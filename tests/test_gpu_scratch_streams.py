@@ -149,3 +149,36 @@ def test_repeated_contexts_give_all_their_room_back(S):
     idle, g = kept(S)
     before = unused(S, other)
     assert unused(S, idle) - before >= 80 << 20   # the last one still kept its blocks
+
+
+def test_taking_back_beside_contexts_at_work(S, monkeypatch):
+    bad, stop = [], threading.Event()
+    ref_ctx = S.sfg_ctx_create(0)
+    refs = {side: S.sfg_smooth(ref_ctx, graph(S, ref_ctx, side), 32, 4, seed=side).clone() for side in (30, 200, 500)}
+    torch.cuda.synchronize()
+
+    def work(own_stream):
+        stream = torch.cuda.Stream() if own_stream else torch.cuda.current_stream()
+        ctx = S.sfg_ctx_create(0, stream)
+        with torch.cuda.stream(stream):
+            graphs = {side: graph(S, ctx, side) for side in refs}
+            while not stop.is_set():
+                for side, g in graphs.items():
+                    if not torch.equal(S.sfg_smooth(ctx, g, 32, 4, seed=side), refs[side]):
+                        bad.append(side)
+        stream.synchronize()
+
+    threads = [threading.Thread(target=work, args=(o,)) for o in (False, True, True)]
+    [t.start() for t in threads]
+    for n in range(1, 40):
+        monkeypatch.setenv("SFG_FAULT_POOL", str(n))
+        ctx = S.sfg_ctx_create(0)
+        g = graph(S, ctx, 200)
+        if not torch.equal(S.sfg_smooth(ctx, g, 32, 4, seed=200), refs[200]):
+            bad.append(("reclaiming", n))
+        g.close()
+        ctx.close()
+    monkeypatch.delenv("SFG_FAULT_POOL")
+    stop.set()
+    [t.join() for t in threads]
+    assert not bad
