@@ -70,8 +70,8 @@ struct sfg_ctx {
     bool withhold_mma = false;             // SFG_FAULT_MMA_WAIT=1: tensor-core kernels issue no
                                            // MMA, so their bounded completion waits run out
     int* grid_status = nullptr;            // host word that grid barriers set when a wait runs out
-    std::string fault_grid;                // SFG_FAULT_GRID_WAIT=<kernel>:<n>: at the n-th barrier of
-    unsigned fault_barrier = 0;            // that kernel one CTA does not arrive (waits of 20 ms)
+    std::string fault_grid;                // SFG_FAULT_GRID_WAIT=<kernel>:<n>: the waits of that kernel's
+    unsigned fault_barrier = 0;            // n-th barrier run out (after 20 ms)
 };
 
 struct sfg_graph {

@@ -1,5 +1,4 @@
-"""A grid barrier that runs out (one CTA is told not to arrive, the others' waits end after 20 ms) is reported by
-every caller: by the call itself where it synchronises, else by the next call that does, once; and the
+"""A grid barrier that runs out (its waits are told to go on until their limit, 20 ms) is reported by every caller: by the call itself where it synchronises, else by the next call that does, once; and the
 context stays usable. No entry of a selection that gave up is an unwritten one."""
 import numpy as np
 import pytest
@@ -13,7 +12,7 @@ ETIMEOUT = 4
 
 @pytest.fixture()
 def at(monkeypatch):
-    """A context whose launches of `kernel` withhold an arrival at their n-th barrier, and a graph."""
+    """A context whose launches of `kernel` run out of their n-th barrier's waits, and a graph."""
     import paper_2008_07633_gb300.sfg as S
 
     spec = gen.grid2d(60, 50, seed=4)
