@@ -118,11 +118,12 @@ __device__ __forceinline__ int tk_scan(int v, int* all) {
 // Stable sort of out[0, k) by id (as unsigned words): as many 8-bit digits as the largest id has, CTA c of the first
 // sort_ctas owning one contiguous range. To find the first place of each digit in its range a CTA can read the whole
 // table of counts, sort_ctas words a thread: up to kTkSumRows CTAs that is shorter than another barrier; beyond, the
-// digits' rows of the table are scanned first, a CTA a row. Ids go in tiles of 2,048, a warp ranking 256 consecutive
-// ones by itself, so that a tile costs four CTA barriers. Whole selections of ids in no order (us, with every CTA
-// reading the table and 256 ids a step / so / separate sorting launches): 50,000 of 100,000 kept 114/75/195, 524,288
-// of 2^20 532/227/233, 2^21 of 2^22 1,406/305/333, all of 2^24 3,196/1,065/1,288.
-constexpr int kTkSumRows = 16, kTkSortPer = 8, kTkSortTile = kBlock * kTkSortPer;
+// digits' rows of the table are scanned first, a CTA a row. Ids go in tiles of 1,024, a warp ranking 128 consecutive
+// ones by itself, so that a tile costs four CTA barriers (tiles of 2,048 spill and take 3-10% longer below 2^20 kept).
+// Whole selections of ids in no order (us, with every CTA reading the table and 256 ids a step / so / separate
+// sorting launches): 50,000 of 100,000 kept 113/72/195, 524,288 of 2^20 533/215/233, 2^21 of 2^22 1,406/299/333, all of
+// 2^24 3,097/1,020/1,288.
+constexpr int kTkSumRows = 16, kTkSortPer = 4, kTkSortTile = kBlock * kTkSortPer;
 
 __device__ bool tk_sort_ids(const TkArgs& A, const GridBar& bar, unsigned& passed) {
     __shared__ unsigned base[256], wcnt[kBlock / 32][256], s_bits;
