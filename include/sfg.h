@@ -177,7 +177,8 @@ SFG_API sfg_status sfg_jacobi(sfg_ctx* ctx, const sfg_graph* L, int K, int steps
 /* Tile-shape autotuning of the sweep and the scorer (not in the paper). Variant v of the plain
  * sweep: a warp sweeps TPI = {1, 2, 4, 1, 2, 4}[v] consecutive row tiles before its grid-stride
  * jump, with {4, 4, 4, 3, 3, 3}[v] CTAs per SM requested from the compiler; without an entry the
- * shape follows from the width, the storage and the degrees. Shape s
+ * shape follows from the width, the storage, the degrees and how far the edges reach, and variants 0 and 1
+ * prefetch rows ahead of the tile on graphs where that shape does. Shape s
  * of the scorer (sfg_score_edges, sfg_filter_score and the batched forms): a warp scores
  * {1, 2, 1}[s] edge tiles per iteration with {4, 2, 4}[s] CTAs per SM, shape 2 reading rows with
  * loads cached in L2 only; default s = 0 below an average degree of 8, else 1. sfg_autotune times all sweep variants on L (three sweeps each) and both
@@ -240,8 +241,9 @@ SFG_API sfg_status sfg_spanning_tree(sfg_ctx* ctx, const sfg_graph* g, const uin
  * ------------------------------------------------------------------------------------------- */
 
 /* delta_out[e] = 1 - (X_p . X_q)^2 / (||X_p||^2 ||X_q||^2) for every canonical edge e = (p, q)
- * (the algebraic-distance affinity quoted in Sec. 3.2), evaluated in FP64 without fused
- * multiply-add, in increasing k order, from the FP32 block X (n x K). A zero row gives 1. */
+ * (the algebraic-distance affinity quoted in Sec. 3.2), evaluated in FP64 with every product and
+ * sum rounded separately, in increasing k order, from the FP32 block X (n x K). (Products of widened
+ * FP32 entries are exact, so a fused multiply-add gives these bits.) A zero row gives 1. */
 SFG_API sfg_status sfg_affinity(sfg_ctx* ctx, const sfg_graph* L, const float* X, int K,
                         double* delta_out);
 

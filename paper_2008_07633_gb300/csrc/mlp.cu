@@ -539,11 +539,10 @@ __global__ void __launch_bounds__(128, 2)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(kTColsTmem) : "memory");
 }
 
-// grad[i] = sum over CTAs (in order) of part[cta][i] in FP64, as eight interleaved sums added in turn;
-// loss2 (may be NULL) = (sum of squared errors / ne,
+// grad[i] = sum over CTAs (in order) of part[cta][i], in FP64 as eight interleaved sums that are then added in
+// turn: a fixed order, not that of the CTAs; loss2 (may be NULL) = (sum of squared errors / ne,
 // the network's error word). One CTA takes 32 entries; its kFoldWays threads per entry each add every
-// kFoldWays-th partial (32 consecutive floats a warp) and the sums are added in thread order, so
-// the order is fixed. Bound by load latency: 304 partials a thread, one after the other, on 21 CTAs
+// kFoldWays-th partial (32 consecutive floats a warp) and their sums are added in thread order. Bound by load latency: 304 partials a thread, one after the other, on 21 CTAs
 // took 49.6 us for 65,536 rows; 38 partials a thread on 167 CTAs take 5 us.
 constexpr int kFoldWays = 8;
 __global__ void __launch_bounds__(32 * kFoldWays)

@@ -222,9 +222,9 @@ struct Scratch {
 };
 
 // The context's pinned host ints (allocated on first use): a stream-ordered copy into one costs no
-// synchronisation, and the host reads it after the next one. Slots: 0 spanning-forest round
-// flag, 1 pointer-jumping flag, 3 breadth-first flag; from kSfgHostBuild on, the 64-bit words of a
-// graph build.
+// synchronisation, and the host reads it after the next one. Slots: 1 pointer-jumping flag, 3
+// breadth-first flag; from kSfgHostBuild on, 64-bit words read back together (a graph build's, a
+// spanning forest's, a network's loss).
 constexpr int kSfgHostBuild = 8, kSfgHostWords = 64;
 sfg_status sfg_host_word(sfg_ctx* ctx, int slot, int** out);
 
