@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 def partial_stream(sms):
-    """A stream on about `sms` SMs, by the driver's calls."""
+    """A stream on about `sms` SMs, made through the CUDA driver API."""
     torch.zeros(1, device="cuda")
     cu = ctypes.CDLL("libcuda.so.1")
 
