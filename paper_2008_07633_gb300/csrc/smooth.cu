@@ -37,7 +37,8 @@ constexpr int kJNumVariants = 6, kJDefault = 1;
 // instruction and costs no register. It pays where the gathers leave the L1 pipe room for one more
 // request a row: low degrees (spanning forests) or other widths than 8 FP32 lanes. It costs where neighbours are
 // scattered, since every row is then gathered long before or after its turn: graphs whose edges reach over
-// kNearBytes of the block on average keep two tiles a turn. Measured (GB300, us a
+// kNearBytes of the block on average take one tile a turn (four lanes of BF16 two; 16 lanes on forests two with
+// the prefetch, which loses nothing there). Measured (GB300, us a
 // sweep on the graph, on its spanning forest: two tiles a turn / one tile / two tiles AHEAD / one AHEAD):
 //   128^3 grid K = 4 FP32 (1 lane)       48/48/48/48      42/42/42/41
 //   300k mesh K = 4 FP32                 11/11/11/11      10.9/9.4/10.9/9.6
@@ -48,9 +49,12 @@ constexpr int kJNumVariants = 6, kJDefault = 1;
 //   2048^2 power grid K = 64 BF16 (8)    284/274/298/273  274/268/284/259
 //   1000^2 power grid K = 64 FP32 (16)   124/140/114/132  118/134/107/128
 //   2^20-node Chung-Lu K = 32 FP32       327/325/346/343  212/153/210/154
-// and on scattered graphs (mean reach 45-170 MB; forest not measured):
+// and on scattered graphs (mean reach 10-170 MB; the last are forests without hub rows):
 //   random, 2^20 nodes, 2M edges K = 32 FP32  106/105/124/123    8M edges K = 64 BF16  314/314/320/320
+//           8M edges             K = 16 FP32  163/159/163/160    16M edges K = 32 BF16 319/341/320/342
 //   unsorted k-NN, 2M nodes      K = 64 FP32  939/936/964/959    K = 64 BF16           473/475/509/492
+//   2^18-node Chung-Lu forest    K = 32 FP32  76/46/77/46        K = 64 BF16           78/48/73/48
+//   forest of 8M random edges    K = 64 FP32  164/169/162        of the k-NN graph     318/329/314
 // (reach of the meshes above: 0.1-1.4 MB; of the k-NN graphs of up to 100,000 nodes in a batch, 16 FP32: about 2 MB,
 // where the prefetch gains 1%).
 constexpr int64_t kAheadBytes = 4 << 20;
@@ -61,8 +65,8 @@ int plain_form(const sfg_graph* L) {
     if (L->hv_spread) return LPR <= 8 ? kFormOne : kFormTwo;
     const bool bf16 = sizeof(T) == 2, sparse = L->m < 2 * (int64_t)L->n;
     if (LPR == 1) return kFormOne;
-    if (L->reach * (LPR * 16) > kNearBytes) return kFormTwo;
     if (LPR == 4 && bf16) return kFormTwo;
+    if (L->reach * (LPR * 16) > kNearBytes && !(LPR == 16 && sparse)) return kFormOne;
     if (LPR == 8) return bf16 ? kFormOneAhead : sparse ? kFormTwoAhead : kFormOne;
     return kFormTwoAhead;
 }
