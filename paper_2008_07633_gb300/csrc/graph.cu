@@ -1510,6 +1510,9 @@ sfg_status sfg_build_graph(sfg_ctx* ctx, int32_t n, int64_t m, const int32_t* u,
     return build_by_sort(ctx, n, m, u, v, w, validate, out, f2c);
 }
 
+// 36 bytes an edge at most stay unused (2.4 MB); a second wait costs 10 of 65 us.
+constexpr int64_t kEarlySubEdges = 1 << 16;
+
 sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* mask,
                              sfg_graph** out, int32_t** off_ids) {
     *out = nullptr;
@@ -1525,7 +1528,9 @@ sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* ma
     SFG_TRY(s.get(&jpop, jwords));
     SFG_TRY(s.get(&ewoff, ewords + 1));
     SFG_TRY(s.get(&jwoff, jwords + 1));
-    int64_t ms = 0;
+    // Small subgraphs get room for all of g's edges, so that the one host wait is that for the whole build.
+    const bool early = !off_ids && m <= kEarlySubEdges;
+    int64_t ms = early ? m : 0;
     if (m > 0) {
         k_sub_bits<false><<<grid_of(ctx, k_sub_bits<false>, (m + 3) / 4), kBlock, 0, ctx->stream>>>(m, nullptr, mask, ebits, epop);
         SFG_TRY(sfg_scan_i32(ctx, epop, ewoff, ewords));
@@ -1533,7 +1538,7 @@ sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* ma
         SFG_TRY(sfg_scan_i32(ctx, jpop, jwoff, jwords));
         ctx->launches += 2;
         SFG_LAUNCH_CHECK(ctx, "k_sub_bits");
-        SFG_TRY(sfg_read_i64(ctx, ewoff + ewords, &ms));
+        if (!early) SFG_TRY(sfg_read_i64(ctx, ewoff + ewords, &ms));
     } else {
         SFG_CUDA(ctx, cudaMemsetAsync(jwoff, 0, sizeof(int64_t), ctx->stream));
     }
@@ -1559,6 +1564,7 @@ sfg_status sfg_subgraph_impl(sfg_ctx* ctx, const sfg_graph* g, const uint8_t* ma
         p->hv_n = 0;
     }
     SFG_TRY(row_degrees(ctx, p));
+    if (early && m > 0) SFG_TRY(sfg_read_i64(ctx, ewoff + ewords, &p->m));
     if (off_ids) {
         s.release(rest);
         *off_ids = rest;
